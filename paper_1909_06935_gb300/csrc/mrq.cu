@@ -1,13 +1,13 @@
 // mrq.cu - GB300 (sm_103a) kernels and host runtime of the stochastic SC-NEVPT2(s) /
 // SC-MRCI(s) local-estimator path (arXiv:1909.06935), behind the C ABI of include/mrq.h.
 //
-// Hot path (one warp per walker, persistent over steps):
-//   classify the walker (label, Sec. II A) -> enumerate every single and double excitation that
-//   stays in CAS u FOIS as a union of rectangular class blocks -> per lane: <n|H|m> by
-//   Slater-Condon, psi_s(m) by a hash probe (m in the CAS) or reach-back O(m) = <m|H|phi0>
-//   (Eq. 6-7, Sec. II D) -> rates Gamma_nm = |H_nm psi_s(m)/psi_s(n)|, E_L (Eq. 5), the H_D
-//   numerator (Eq. 16) -> warp reductions -> accumulate with weight 1/S -> move by the
-//   first-reaction (competing exponential clocks) form of Gillespie's algorithm.
+// Hot path (mrq_walk.cuh), per step and distinct determinant of the walkers:
+//   classify it (label, Sec. II A) -> enumerate every single and double excitation that stays in
+//   CAS u FOIS -> per lane: <n|H|m> by Slater-Condon, psi_s(m) by a hash probe (m in the CAS) or
+//   reach-back O(m) = <m|H|phi0> (Eq. 6-7, Sec. II D) -> rates Gamma_nm = |H_nm psi_s(m)/psi_s(n)|,
+//   E_L (Eq. 5), the H_D numerator (Eq. 16) -> fixed-order sums -> accumulate with weight 1/S ->
+//   every walker moves by the first-reaction (competing exponential clocks) form of Gillespie's
+//   algorithm.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -42,8 +42,7 @@ struct Walker {
 
 static_assert(sizeof(SysDev) % sizeof(int) == 0, "SysDev is copied word by word");
 
-struct WarpSh {
-    SysDev sys;                      // the walker's system, read by every lane (kept out of local memory)
+struct WarpLists {
     unsigned char ol[2][MRQ_MAXN];   // occupied orbitals per spin, ascending (core|active|virtual)
     unsigned char el[2][MRQ_MAXN];   // empty orbitals per spin
     short os[2][4], es[2][4];        // class starts: [spin][class], [3] = count
@@ -72,7 +71,7 @@ __device__ __forceinline__ void tri_decode(int op, int& i, int& j) {
 
 // Build occupied/empty lists (class-partitioned) and the valid excitation blocks of det d.
 template <int W>
-__device__ void build_lists(const SysDev& S, const unsigned long long (&d)[2][W], WarpSh& sh, int h, int p,
+__device__ void build_lists(const SysDev& S, const unsigned long long (&d)[2][W], WarpLists& sh, int h, int p,
                             int lane) {
     const int n = S.n;
     for (int sg = 0; sg < 2; sg++) {
@@ -196,7 +195,7 @@ __device__ __forceinline__ void pair_decode(int op, bool same, int k1, int k2, b
 }
 
 // decode neighbour `loc` of block `desc` into removed r1<=r2 and added a1<=a2 spin orbitals
-__device__ __forceinline__ void decode_exc(const WarpSh& sh, int n, unsigned desc, int loc, int& kind, int& r1,
+__device__ __forceinline__ void decode_exc(const WarpLists& sh, int n, unsigned desc, int loc, int& kind, int& r1,
                                            int& r2, int& a1, int& a2) {
     kind = desc & 3;
     int sg = (desc >> 2) & 1, X1 = (desc >> 4) & 3, X2 = (desc >> 6) & 3, Y1 = (desc >> 8) & 3,
@@ -256,7 +255,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 
 // <d|H|d> and <d|H_D|d> (lane-parallel over occupied pairs); label >= 0 required for H_D
 template <int W>
-__device__ void diagonals(const SysDev& S, const WarpSh& sh, const unsigned long long (&d)[2][W], int lane,
+__device__ void diagonals(const SysDev& S, const WarpLists& sh, const unsigned long long (&d)[2][W], int lane,
                           double& hnn, double& hdnn) {
     const int na_ = sh.os[0][3], nb_ = sh.os[1][3], N = na_ + nb_;
     double h = 0.0, hd = 0.0;
@@ -290,8 +289,6 @@ __device__ void diagonals(const SysDev& S, const WarpSh& sh, const unsigned long
 
 // ============================================================================ the walk
 
-enum { MODE_STEP = 0, MODE_DEBUG = 1 };
-
 #include "mrq_cas.cuh"
 
 // The walkers of one launch: one or several systems, each with its own walker array; slot numbers
@@ -302,84 +299,7 @@ struct WalkSet {
     const long long* offsets;
     int nsys;
     long long nslots;
-    long long max_seg = 0;        // the most slots of one system (host side: sizes the slot sort)
 };
-
-__device__ __forceinline__ void slot_owner(const WalkSet& ws, long long slot, int& sys, long long& local) {
-    int lo = 0, hi = ws.nsys - 1;
-    while (lo < hi) {                       // last system whose first slot is <= slot
-        const int mid = (lo + hi + 1) >> 1;
-        if (ws.offsets[mid] <= slot) lo = mid;
-        else hi = mid - 1;
-    }
-    sys = lo;
-    local = slot - ws.offsets[lo];
-}
-
-// sort key of a walker slot: system, label, then the active occupation (truncated), and the slot
-template <int W>
-__global__ void k_walker_keys(const WalkSet ws, unsigned long long* __restrict__ keys) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= ws.nslots) return;
-    int sys;
-    long long local;
-    slot_owner(ws, i, sys, local);
-    const Walker wk = ws.walkers[sys][local];
-    const SysDev& S = ws.systems[sys];
-    unsigned long long d[2][W];
-#pragma unroll
-    for (int sg = 0; sg < 2; sg++)
-#pragma unroll
-        for (int w = 0; w < W; w++) d[sg][w] = wk.d[sg][w];
-    int h, p;
-    const long long l = det_label<W>(S, d, h, p);
-    const unsigned long long act = hash_key(S, active_bits<W>(S, d[0]), active_bits<W>(S, d[1]));
-    keys[i] = ((unsigned long long)(l & 0xFFFFFF) << 24) | (act & 0xFFFFFFull);
-}
-
-// Per-system bitonic sort of the slots by key (ties by slot): block b orders the slots of system b,
-// [offsets[b], offsets[b+1]), in shared memory padded to a power of two; a system with fewer than
-// 64 or more than MRQ_SORT_MAX slots keeps its slot order.  order[] receives global slot numbers.
-#define MRQ_SORT_MAX 16384
-__global__ void __launch_bounds__(1024) k_sort_slots(const unsigned long long* __restrict__ keys,
-                                                     const long long* __restrict__ offsets, unsigned* __restrict__ order) {
-    extern __shared__ __align__(16) unsigned char sort_smem[];
-    const long long lo = offsets[blockIdx.x];
-    const int n = (int)(offsets[blockIdx.x + 1] - lo);
-    if (n < 64 || n > MRQ_SORT_MAX) {
-        for (int i = threadIdx.x; i < n; i += blockDim.x) order[lo + i] = (unsigned)(lo + i);
-        return;
-    }
-    const int npad = 1 << (32 - __clz(n - 1));
-    unsigned long long* sk = reinterpret_cast<unsigned long long*>(sort_smem);
-    unsigned* si = reinterpret_cast<unsigned*>(sk + npad);
-    for (int i = threadIdx.x; i < npad; i += blockDim.x) {
-        sk[i] = i < n ? keys[lo + i] : ~0ull;
-        si[i] = i < n ? (unsigned)(lo + i) : 0xFFFFFFFFu;
-    }
-    __syncthreads();
-    for (int k = 2; k <= npad; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < npad; i += blockDim.x) {
-                const int ixj = i ^ j;
-                if (ixj > i) {
-                    const bool up = (i & k) == 0;
-                    const unsigned long long a = sk[i], b = sk[ixj];
-                    const bool swap = up ? (a > b || (a == b && si[i] > si[ixj])) : (a < b || (a == b && si[i] < si[ixj]));
-                    if (swap) {
-                        sk[i] = b;
-                        sk[ixj] = a;
-                        const unsigned t = si[i];
-                        si[i] = si[ixj];
-                        si[ixj] = t;
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    }
-    for (int i = threadIdx.x; i < n; i += blockDim.x) order[lo + i] = si[i];
-}
 
 #include "mrq_walk.cuh"
 
@@ -727,7 +647,9 @@ __global__ void k_race_screen(const unsigned long long* __restrict__ k, const do
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float btf = isinf(tbest[i]) ? INFINITY : (float)tbest[i];
-    pass[i] = race_may_win(k[i], abs_f32_of(rate[i]), btf) ? 1 : 0;
+    const float gf = abs_f32_of(rate[i]);
+    pass[i] = race_pass((unsigned)(k[i] >> 21), gf > 0.0f ? gf : INFINITY, race_scale(btf * 1.0001f, 1.0f)) &&
+              race_may_win(k[i], gf, btf * 1.0001f);
     exact[i] = race_clock_f64(k[i], rate[i]);
 }
 
@@ -1024,10 +946,10 @@ struct mrq_ctx {
     Walker** d_bwptr = nullptr;
     long long* d_boff = nullptr;
     int bcap = 0;
-    unsigned long long* d_sort_keys = nullptr;   // walker-slot ordering by determinant
-    unsigned* d_sort_idx = nullptr;
-    long long sort_cap = 0;
-    size_t sort_smem = 0;
+    // workspace of this context's walk launches (WalkScratch), kept between calls
+    unsigned char* d_work = nullptr;
+    size_t work_cap = 0;
+    WalkScratch work{};
     double* d_partial = nullptr;
     long long partial_cap = 0;
     mrq_result* d_res = nullptr;
@@ -1035,25 +957,24 @@ struct mrq_ctx {
     SysDev* d_sys = nullptr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     // launch configuration (mrq_set_launch, mrq_tune_batch)
-    int wpb = 0;                     // warps per walker block (0: chosen from the system's work units)
-    int max_nw = MRQ_MAXNW;          // most warps per walker whose candidate lists fit shared memory
+    int wpb = 0;                     // warps per walk block (0: MRQ_MAXNW)
+    int max_nw = MRQ_MAXNW;          // most warps per block whose candidate lists fit shared memory
     int spl = 0;                     // steps per launch (0: every advance is one launch)
     int use_graph = 0;               // batches replay one reporting interval from a CUDA graph
     struct GraphKey {
-        const void *sys = nullptr, *wptr = nullptr, *off = nullptr, *keys = nullptr;
+        const void *sys = nullptr, *wptr = nullptr, *off = nullptr, *work = nullptr;
         long long nslots = 0;
-        int k = 0, wpb = 0, spl = 0, cap = 0, gstride = 0;
+        int k = 0, wpb = 0, spl = 0, cap = 0, gstride = 0, ns = 0;
         bool operator==(const GraphKey& o) const {
-            return sys == o.sys && wptr == o.wptr && off == o.off && keys == o.keys && nslots == o.nslots &&
-                   k == o.k && wpb == o.wpb && spl == o.spl && cap == o.cap && gstride == o.gstride;
+            return sys == o.sys && wptr == o.wptr && off == o.off && work == o.work && nslots == o.nslots &&
+                   k == o.k && wpb == o.wpb && spl == o.spl && cap == o.cap && gstride == o.gstride && ns == o.ns;
         }
     };
-    // per determinant width, warps per walker (8, 4, 2, 1) and occupancy class (resident walk blocks
-    // per SM, 4-1) of a batch launch
-    static constexpr int NSLOT = 32;
+    // per determinant width and warps per block (8, 4, 2, 1) of a batch launch
+    static constexpr int NSLOT = 8;
     cudaGraphExec_t gexec[NSLOT] = {};
     GraphKey gkey[NSLOT];
-    int smem_sm = 0, smem_rsv = 0;   // shared memory per SM and reserved per block (bytes)
+    int n_sm = 0;                    // SMs of the device
     long long graph_replays = 0;
     long long* d_nbpre = nullptr;    // debug records: neighbour offsets of a determinant's units
     long long nbpre_cap = 0;
@@ -1073,7 +994,7 @@ struct mrq_ctx {
     int probe_limit = 0, cap_limit = 0;
     int cand_cap_full = 1;           // the candidate-list capacity the loaded system needs
     double l2_fraction = 0.0;        // mrq_set_l2_window: share of the persisting-L2 carve-out for the tables
-    int walk_minb = 2;               // resident walk blocks per SM of the kernel build in use (2, 3, 4)
+    int eval_minb = 2, eval_blocks = 0;   // k_eval: build in use (resident blocks per SM) and grid
 };
 
 static int fail(mrq_ctx* c, int code, const char* fmt, ...) {
@@ -1202,8 +1123,8 @@ static int check_err_flag(mrq_ctx* ctx, int* flag_out) {
     return 0;
 }
 
-// launch-time options of a walk: warps (walkers) per block, whether to accumulate, and whether the
-// one-time set-up (buffer growth, function attributes) has been done already (inside a stream capture)
+// launch-time options of a walk: warps per block, whether to accumulate, and whether the one-time
+// set-up (workspace growth, function attributes) has been done already (inside a stream capture)
 struct WalkLaunch {
     int wpb = 8;
     int accumulate = 1;
@@ -1211,98 +1132,145 @@ struct WalkLaunch {
     cudaAccessPolicyWindow l2win = {};   // num_bytes 0: no persisting-L2 window
 };
 
-// scratch and shared memory of the per-system slot sort; max_seg = the most slots of one system
-static int walk_sort_prepare(mrq_ctx* ctx, long long nslots, long long max_seg) {
-    if (nslots > ctx->sort_cap) {
-        dfree(ctx->d_sort_keys);
-        dfree(ctx->d_sort_idx);
-        CK(cudaMalloc(&ctx->d_sort_keys, sizeof(unsigned long long) * nslots));
-        CK(cudaMalloc(&ctx->d_sort_idx, sizeof(unsigned) * nslots));
-        ctx->sort_cap = nslots;
+// what a walk set's systems need: the largest candidate-list capacity, single-excitation operator and
+// slice count among them
+struct WalkNeed {
+    int cap = 1, gstride = 0, ns = 1;
+    void add(const SysDev& s) {
+        cap = std::max(cap, s.cand_cap);
+        gstride = std::max(gstride, s.gstride);
+        ns = std::max(ns, s.nslice);
     }
-    long long npad = 64;
-    while (npad < std::min<long long>(max_seg, MRQ_SORT_MAX)) npad <<= 1;
-    const size_t ssm = (size_t)npad * (sizeof(unsigned long long) + sizeof(unsigned));
-    CK(cudaFuncSetAttribute(k_sort_slots, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm));
-    ctx->sort_smem = ssm;
+};
+
+// Workspace of a launch over nslots walkers.  A launch takes its walkers in segments of at most
+// `seg` slots, so that the workspace stays below about 1 GiB whatever the number of walkers.
+#define MRQ_WORK_BYTES (1LL << 30)
+static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, long long* seg_out) {
+    const long long per = 12 * 4 + 3 * 4 + (long long)sizeof(TaskGroup) + (long long)sizeof(GroupMeta) +
+                          8LL * need.gstride + 24LL * need.ns + (long long)sizeof(RaceBest) + 4;
+    const long long seg = std::min(nslots, std::max(256LL, std::min(1LL << 20, MRQ_WORK_BYTES / per)));
+    *seg_out = seg;
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = off;
+        off += (bytes + 255) / 256 * 256;
+        return at;
+    };
+    const size_t rep = take(16 * seg), cnt = take(16 * seg), start = take(16 * seg), tab = take(4 * seg), pos = take(4 * seg),
+                 mem = take(4 * seg), tg = take(sizeof(TaskGroup) * seg), meta = take(sizeof(GroupMeta) * seg),
+                 gops = take(8 * (size_t)need.gstride * seg), part = take(24 * (size_t)need.ns * seg),
+                 best = take(sizeof(RaceBest) * seg), bound = take(4 * seg), ctl = take(16);
+    if (off > ctx->work_cap) {
+        CK(cudaStreamSynchronize(ctx->stream));
+        dfree(ctx->d_work);
+        ctx->work_cap = 0;
+        CK(cudaMalloc(&ctx->d_work, off));
+        ctx->work_cap = off;
+    }
+    unsigned char* const b = ctx->d_work;
+    WalkScratch& w = ctx->work;
+    w.rep = (int*)(b + rep);
+    w.cnt = (int*)(b + cnt);
+    w.start = (int*)(b + start);
+    w.tab_of = (int*)(b + tab);
+    w.pos_of = (int*)(b + pos);
+    w.members = (int*)(b + mem);
+    w.tg = (TaskGroup*)(b + tg);
+    w.meta = (GroupMeta*)(b + meta);
+    w.gops = (double*)(b + gops);
+    w.part = (double*)(b + part);
+    w.best = (RaceBest*)(b + best);
+    w.bound = (unsigned*)(b + bound);
+    w.ctl = (int*)(b + ctl);
+    w.gstride = need.gstride;
+    w.ns_max = need.ns;
+    // walkers per task group: 32 when there are many, fewer for small launches, so that the walkers of
+    // a crowded determinant spread over more warps
+    w.tgw = (int)std::max(4LL, std::min<long long>(MRQ_TGW, seg / 128));
     return 0;
 }
 
 template <int W, int B>
-static int walk_fits(mrq_ctx* ctx, size_t smem, int threads, bool& fits) {
-    CK(cudaFuncSetAttribute(k_walk2<W, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int nb = 0;
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_walk2<W, B>, threads, smem));
-    fits = nb >= B;
+static int eval_fits(mrq_ctx* ctx, size_t smem, int threads, int& blocks) {
+    CK(cudaFuncSetAttribute(k_eval<W, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_eval<W, B>, threads, smem));
     return 0;
 }
 
-// the walk kernel's build for this launch: the most resident blocks per SM (4, 3 or 2, fewer
-// registers each) that the block's shared memory allows
-static int walk_attr_prepare(mrq_ctx* ctx, int W, size_t smem, int threads) {
-    bool f4 = false, f3 = false, f2 = false;
+// k_eval's build for this launch: the most resident warps per SM (4, 3 or 2 blocks' worth of MRQ_MAXNW
+// warps, fewer registers each) that the block's shared memory allows, and a grid that fills the chip once
+static int eval_prepare(mrq_ctx* ctx, int W, int nw, int cap) {
+    const size_t smem = nw * eval_warp_bytes(cap), lsm = nw * cand_list_bytes(cap);
+    int b4 = 0, b3 = 0, b2 = 0;
+    const int full = MRQ_MAXNW / nw;             // blocks that hold MRQ_MAXNW warps
     if (W == 1) {
-        if (int r = walk_fits<1, 4>(ctx, smem, threads, f4)) return r;
-        if (int r = walk_fits<1, 3>(ctx, smem, threads, f3)) return r;
-        if (int r = walk_fits<1, 2>(ctx, smem, threads, f2)) return r;
+        if (int r = eval_fits<1, 4>(ctx, smem, 32 * nw, b4)) return r;
+        if (int r = eval_fits<1, 3>(ctx, smem, 32 * nw, b3)) return r;
+        if (int r = eval_fits<1, 2>(ctx, smem, 32 * nw, b2)) return r;
+        CK(cudaFuncSetAttribute(k_move<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm));
     } else {
-        if (int r = walk_fits<2, 2>(ctx, smem, threads, f2)) return r;
+        if (int r = eval_fits<2, 3>(ctx, smem, 32 * nw, b3)) return r;
+        if (int r = eval_fits<2, 2>(ctx, smem, 32 * nw, b2)) return r;
+        CK(cudaFuncSetAttribute(k_move<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm));
     }
-    ctx->walk_minb = f4 ? 4 : (f3 ? 3 : 2);
+    ctx->eval_minb = b4 >= 4 * full ? 4 : (b3 >= 3 * full ? 3 : 2);
+    const int b = ctx->eval_minb == 4 ? b4 : (ctx->eval_minb == 3 ? b3 : b2);
+    ctx->eval_blocks = std::max(1, b) * ctx->n_sm;
     return 0;
 }
 
-// warps per walker block when the caller leaves the choice to the library: enough warps to share a
-// CAS walker's work units, fewer for small systems whose units would leave warps idle
-static int auto_warps(const SysDev& s) {
-    const int u = s.unit_off[8];
-    return u >= 512 ? 8 : (u >= 128 ? 4 : 2);
-}
-// warps per walker of a context's launches: the requested (or automatic) number, at most the most
-// whose per-warp candidate lists fit shared memory (large active spaces run with fewer warps)
-static int warps_of(const mrq_ctx* ctx) {
-    return std::min(ctx->wpb > 0 ? ctx->wpb : auto_warps(ctx->hsys), ctx->max_nw);
-}
+// warps per block of a context's launches: the requested (or default) number, at most the most whose
+// candidate lists fit shared memory (large active spaces run with fewer warps)
+static int warps_of(const mrq_ctx* ctx) { return std::min(ctx->wpb > 0 ? ctx->wpb : MRQ_MAXNW, ctx->max_nw); }
 
-// nsteps walker steps of a walk set: per step, order the slots by determinant (when the slot count
-// allows a one-block sort), one block of L.wpb warps per walker slot (k_walk2), then the
-// deterministic accumulation of the step's records (k_accum); `ctx` provides the stream and the
-// sort scratch.  cap / gstride: the largest candidate-list capacity and single-operator size of
-// the set's systems.
-static int launch_walk(mrq_ctx* ctx, int W, const WalkSet& ws, int nsteps, int cap, int gstride,
+// nsteps walker steps of a walk set (the five kernels of mrq_walk.cuh per step); `ctx` provides the
+// stream and the workspace.
+static int launch_walk(mrq_ctx* ctx, int W, const WalkSet& ws, int nsteps, const WalkNeed& need,
                        const WalkLaunch& L = WalkLaunch()) {
     const int nw = std::min(L.wpb, MRQ_MAXNW);
-    const size_t smem = cta_smem_bytes(nw, cap, gstride);
-    const long long nslots = ws.nslots;
-    if (!L.captured) {
-        if (int r = walk_sort_prepare(ctx, nslots, ws.max_seg)) return r;
-        if (int r = walk_attr_prepare(ctx, W, smem, 32 * nw)) return r;
+    const size_t wbytes = eval_warp_bytes(need.cap), lbytes = cand_list_bytes(need.cap);
+    long long seg = 0;
+    if (int r = work_prepare(ctx, ws.nslots, need, &seg)) return r;
+    if (!L.captured)
+        if (int r = eval_prepare(ctx, W, nw, need.cap)) return r;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ctx->eval_blocks);
+    cfg.blockDim = dim3(32 * nw);
+    cfg.dynamicSmemBytes = nw * wbytes;
+    cfg.stream = ctx->stream;
+    cudaLaunchAttribute attr[1];
+    if (L.l2win.num_bytes > 0) {            // keep the walk's hottest table resident in L2
+        attr[0].id = cudaLaunchAttributeAccessPolicyWindow;
+        attr[0].val.accessPolicyWindow = L.l2win;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
     }
     for (int step = 0; step < nsteps; step++) {
-        // order every system's slots by determinant (walkers on one determinant in neighbouring blocks)
-        const unsigned nb = (unsigned)((nslots + 255) / 256);
-        if (W == 1) k_walker_keys<1><<<nb, 256, 0, ctx->stream>>>(ws, ctx->d_sort_keys);
-        else k_walker_keys<2><<<nb, 256, 0, ctx->stream>>>(ws, ctx->d_sort_keys);
-        k_sort_slots<<<(unsigned)ws.nsys, 1024, ctx->sort_smem, ctx->stream>>>(ctx->d_sort_keys, ws.offsets,
-                                                                              ctx->d_sort_idx);
-        CK(cudaGetLastError());
-        const unsigned* order = ctx->d_sort_idx;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)nslots);
-        cfg.blockDim = dim3(32 * nw);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = ctx->stream;
-        cudaLaunchAttribute attr[1];
-        if (L.l2win.num_bytes > 0) {            // keep the walk's hottest table resident in L2
-            attr[0].id = cudaLaunchAttributeAccessPolicyWindow;
-            attr[0].val.accessPolicyWindow = L.l2win;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
+        for (long long s0 = 0; s0 < ws.nslots; s0 += seg) {
+            WalkScratch sc = ctx->work;
+            sc.seg0 = s0;
+            sc.seg1 = std::min(ws.nslots, s0 + seg);
+            const long long n = sc.seg1 - sc.seg0;
+            if (ws.nsys > 1) CK(cudaMemsetAsync(sc.ctl, 0, 3 * sizeof(int), ctx->stream));
+            const unsigned gp = (unsigned)std::min<long long>(n, 8LL * ctx->n_sm);
+            const unsigned gm = (unsigned)std::min<long long>((n + nw - 1) / nw, 4LL * ctx->n_sm);
+            if (W == 1) {
+                k_group<1><<<(unsigned)ws.nsys, 1024, 0, ctx->stream>>>(ws, sc);
+                k_prep<1><<<gp, 128, 0, ctx->stream>>>(ws, sc);
+                if (ctx->eval_minb == 4) CK(cudaLaunchKernelEx(&cfg, k_eval<1, 4>, ws, sc, (int)wbytes, need.cap));
+                else if (ctx->eval_minb == 3) CK(cudaLaunchKernelEx(&cfg, k_eval<1, 3>, ws, sc, (int)wbytes, need.cap));
+                else CK(cudaLaunchKernelEx(&cfg, k_eval<1, 2>, ws, sc, (int)wbytes, need.cap));
+                k_move<1><<<gm, 32 * nw, nw * lbytes, ctx->stream>>>(ws, sc, L.accumulate, (int)lbytes, need.cap);
+            } else {
+                k_group<2><<<(unsigned)ws.nsys, 1024, 0, ctx->stream>>>(ws, sc);
+                k_prep<2><<<gp, 128, 0, ctx->stream>>>(ws, sc);
+                if (ctx->eval_minb >= 3) CK(cudaLaunchKernelEx(&cfg, k_eval<2, 3>, ws, sc, (int)wbytes, need.cap));
+                else CK(cudaLaunchKernelEx(&cfg, k_eval<2, 2>, ws, sc, (int)wbytes, need.cap));
+                k_move<2><<<gm, 32 * nw, nw * lbytes, ctx->stream>>>(ws, sc, L.accumulate, (int)lbytes, need.cap);
+            }
+            CK(cudaGetLastError());
         }
-        if (W == 2) CK(cudaLaunchKernelEx(&cfg, k_walk2<2, 2>, ws, order, L.accumulate));
-        else if (ctx->walk_minb == 4) CK(cudaLaunchKernelEx(&cfg, k_walk2<1, 4>, ws, order, L.accumulate));
-        else if (ctx->walk_minb == 3) CK(cudaLaunchKernelEx(&cfg, k_walk2<1, 3>, ws, order, L.accumulate));
-        else CK(cudaLaunchKernelEx(&cfg, k_walk2<1, 2>, ws, order, L.accumulate));
         if (L.accumulate) {
             k_accum<<<dim3((unsigned)ws.nsys, 2), 1024, 0, ctx->stream>>>(ws);
             CK(cudaGetLastError());
@@ -1369,6 +1337,10 @@ static int walk_plan(mrq_ctx* ctx, SysDev& s) {
         off += npairs * nch;
     }
     s.unit_off[8] = (int)off;
+    // slices of a determinant's units: about four units each, so that a step on a few hundred
+    // determinants is some 10^5 warp tasks and one on a few still spreads over the chip
+    s.nslice = 32;
+    while (s.nslice < MRQ_NS_MAX && s.nslice * 4 < off) s.nslice <<= 1;
     s.cas_nb_total = total;
     if (off > (1LL << 30) || total > (1LL << 40))
         return fail(ctx, MRQ_TOO_LARGE, "active space too large for the walk's work plan");
@@ -1401,11 +1373,12 @@ static int walk_plan(mrq_ctx* ctx, SysDev& s) {
     s.gstride = 2 * s.nca * s.nav;
     s.cand_cap = (int)cap;
     ctx->cand_cap_full = (int)cap;
-    // the most warps per walker (8, 4, 2 or 1) whose candidate lists and operator fit one block's
-    // shared memory; beyond one warp the active space is too large for the walk
+    // the most warps per block (8, 4, 2 or 1) whose candidate lists fit its shared memory; beyond one
+    // warp the active space is too large for the walk
     ctx->max_nw = 0;
     for (int nw = MRQ_MAXNW; nw >= 1 && ctx->max_nw == 0; nw >>= 1)
-        if (cta_smem_bytes(nw, (int)cap, s.gstride) <= 227 * 1024) ctx->max_nw = nw;
+        if (debug_smem_bytes(nw, (int)cap, s.gstride) <= 227 * 1024 && nw * eval_warp_bytes((int)cap) <= 227 * 1024)
+            ctx->max_nw = nw;
     if (ctx->max_nw == 0)
         return fail(ctx, MRQ_TOO_LARGE, "active space too large for the shared-memory candidate lists");
     return 0;
@@ -1454,8 +1427,7 @@ int mrq_create(mrq_ctx** out, int device) {
     }
     ctx->own_stream = true;
     cudaMemset(ctx->d_err, 0, sizeof(int));
-    if (cudaDeviceGetAttribute(&ctx->smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device) != cudaSuccess ||
-        cudaDeviceGetAttribute(&ctx->smem_rsv, cudaDevAttrReservedSharedMemoryPerBlock, device) != cudaSuccess) {
+    if (cudaDeviceGetAttribute(&ctx->n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
         mrq_destroy(ctx);
         return MRQ_CUDA_ERROR;
     }
@@ -1476,8 +1448,7 @@ void mrq_destroy(mrq_ctx* ctx) {
     dfree(ctx->d_err);
     dfree(ctx->d_sys);
     dfree(ctx->d_res);
-    dfree(ctx->d_sort_keys);
-    dfree(ctx->d_sort_idx);
+    dfree(ctx->d_work);
     dfree(ctx->d_wptr);
     dfree(ctx->d_woff);
     dfree(ctx->d_bsys);
@@ -1765,7 +1736,7 @@ int mrq_debug_local(mrq_ctx* ctx, int64_t n, const uint64_t* dets, mrq_local* lo
     if (int r = push_sys(ctx)) return r;
     const int cap = ctx->hsys.cand_cap;
     const int nw = std::min(warps_of(ctx), MRQ_MAXNW);
-    const size_t smem = cta_smem_bytes(nw, cap, ctx->hsys.gstride);
+    const size_t smem = debug_smem_bytes(nw, cap, ctx->hsys.gstride);
     // neighbour offsets of the CAS units, for the records
     const long long stride = nb ? std::max(1, ctx->hsys.unit_off[8]) : 0;
     if (nb && n * stride > ctx->nbpre_cap) {
@@ -1885,14 +1856,14 @@ int mrq_walkers_advance(mrq_ctx* ctx, int64_t n_steps) {
     }
     CK(cudaEventRecord(ctx->evs[k], ctx->stream));
     WalkSet ws{ctx->d_sys, ctx->d_wptr, ctx->d_woff, 1, ctx->nwalk};
-    ws.max_seg = ctx->nwalk;
+    WalkNeed need;
+    need.add(ctx->hsys);
     WalkLaunch L;
     L.wpb = warps_of(ctx);
     if (int r = l2_window(ctx, L.l2win)) return r;
     const int64_t spl = ctx->spl > 0 ? ctx->spl : n_steps;
     for (int64_t done = 0; done < n_steps; done += spl)
-        if (int r = launch_walk(ctx, ctx->W, ws, (int)std::min<int64_t>(spl, n_steps - done), ctx->hsys.cand_cap,
-                                ctx->hsys.gstride, L))
+        if (int r = launch_walk(ctx, ctx->W, ws, (int)std::min<int64_t>(spl, n_steps - done), need, L))
             return r;
     CK(cudaGetLastError());
     CK(cudaEventRecord(ctx->evs[k + 1], ctx->stream));
@@ -2037,23 +2008,11 @@ static int batch_check(mrq_ctx* const* ctxs, int n) {
     return 0;
 }
 
-// the batch's systems of determinant width W: device tables in the lead context, walker arrays
-// from `walkers` (the contexts' own, or the tuner's scratch copies)
-// occupancy class of a system in a batch launch: the walk blocks per SM (1-4) its own shared
-// memory allows; a batch launches each class separately, so that small systems are not held to the
-// occupancy of the largest one
-static int batch_class(const mrq_ctx* lead, const mrq_ctx* c, int nw) {
-    if (c->W != 1) return 2;
-    const long long per = (long long)cta_smem_bytes(std::min(nw, c->max_nw), c->hsys.cand_cap, c->hsys.gstride) +
-                          lead->smem_rsv;
-    const long long b = per > 0 ? (long long)lead->smem_sm / per : 1;
-    return (int)std::max(1LL, std::min(4LL, b));
-}
-
-// the systems of one batch launch: width W, warps per walker nw_eff (the requested nw, at most
-// what each system's candidate lists allow) and occupancy class cls (0: every class)
-static int batch_tables(mrq_ctx* const* ctxs, int n, int W, Walker* const* walkers, WalkSet& ws, int& cap,
-                        int& gstride, int cls = 0, int nw = MRQ_MAXNW, int nw_eff = 0) {
+// the batch's systems of determinant width W whose launches take nw_eff warps per block (the requested
+// nw, at most what each system's candidate lists allow): device tables in the lead context, walker
+// arrays from `walkers` (the contexts' own, or the tuner's scratch copies)
+static int batch_tables(mrq_ctx* const* ctxs, int n, int W, Walker* const* walkers, WalkSet& ws, WalkNeed& need, int nw,
+                        int nw_eff) {
     mrq_ctx* ctx = ctxs[0];
     if (n > ctx->bcap) {
         dfree(ctx->d_bsys);
@@ -2067,20 +2026,15 @@ static int batch_tables(mrq_ctx* const* ctxs, int n, int W, Walker* const* walke
     std::vector<SysDev> sys;
     std::vector<Walker*> wp;
     std::vector<long long> off(1, 0);
-    cap = 1;
+    need = WalkNeed();
     for (int i = 0; i < n; i++) {
-        if (ctxs[i]->W != W) continue;
-        if (nw_eff > 0 && std::min(nw, ctxs[i]->max_nw) != nw_eff) continue;
-        if (cls > 0 && batch_class(ctx, ctxs[i], nw) != cls) continue;
+        if (ctxs[i]->W != W || std::min(nw, ctxs[i]->max_nw) != nw_eff) continue;
         sys.push_back(ctxs[i]->hsys);
         wp.push_back(walkers[i]);
         off.push_back(off.back() + ctxs[i]->nwalk);
-        cap = std::max(cap, ctxs[i]->hsys.cand_cap);
+        need.add(ctxs[i]->hsys);
     }
     ws = WalkSet{ctx->d_bsys, ctx->d_bwptr, ctx->d_boff, (int)sys.size(), off.back()};
-    for (size_t k = 0; k + 1 < off.size(); k++) ws.max_seg = std::max(ws.max_seg, off[k + 1] - off[k]);
-    gstride = 0;
-    for (const SysDev& sd : sys) gstride = std::max(gstride, sd.gstride);
     if (sys.empty()) return 0;
     const int k = (int)sys.size();
     CK(cudaMemcpy(ctx->d_bsys, sys.data(), sizeof(SysDev) * k, cudaMemcpyHostToDevice));
@@ -2089,39 +2043,38 @@ static int batch_tables(mrq_ctx* const* ctxs, int n, int W, Walker* const* walke
     return 0;
 }
 
-// n_steps steps of one width's walk set: launches of `spl` steps (the reporting interval), each
-// one sort + one walk, replayed from a CUDA graph when the lead context asks for it
-static int batch_run(mrq_ctx* ctx, int W, const WalkSet& ws, int cap, int gstride, int64_t n_steps, int wpb,
-                     int64_t spl, int accumulate, bool graph, int slot = -1) {
-    if (slot < 0) slot = W - 1;
+// n_steps steps of one width's walk set: launches of `spl` steps (the reporting interval), replayed
+// from a CUDA graph when the lead context asks for it
+static int batch_run(mrq_ctx* ctx, int W, const WalkSet& ws, const WalkNeed& need, int64_t n_steps, int wpb, int64_t spl,
+                     int accumulate, bool graph, int slot) {
     WalkLaunch L;
     L.wpb = wpb;
     L.accumulate = accumulate;
     if (spl <= 0 || spl > n_steps) spl = n_steps;
     const int64_t nfull = n_steps / spl, rem = n_steps % spl;
     if (graph && nfull > 0) {
-        if (int r = walk_sort_prepare(ctx, ws.nslots, ws.max_seg)) return r;
-        if (int r = walk_attr_prepare(ctx, W, cta_smem_bytes(std::min(wpb, MRQ_MAXNW), cap, gstride),
-                                      32 * std::min(wpb, MRQ_MAXNW)))
-            return r;
+        long long seg = 0;
+        if (int r = work_prepare(ctx, ws.nslots, need, &seg)) return r;
+        if (int r = eval_prepare(ctx, W, std::min(wpb, MRQ_MAXNW), need.cap)) return r;
         mrq_ctx::GraphKey key;
         key.sys = ws.systems;
         key.wptr = ws.walkers;
         key.off = ws.offsets;
-        key.keys = ctx->d_sort_keys;
+        key.work = ctx->d_work;
         key.nslots = ws.nslots;
         key.k = ws.nsys;
         key.wpb = wpb;
         key.spl = (int)spl;
-        key.cap = cap;
-        key.gstride = gstride;
+        key.cap = need.cap;
+        key.gstride = need.gstride;
+        key.ns = need.ns;
         cudaGraphExec_t& ex = ctx->gexec[slot];
         if (!ex || !(ctx->gkey[slot] == key)) {
             if (ex) CK(cudaGraphExecDestroy(ex));
             ex = nullptr;
             CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
             L.captured = true;
-            const int r = launch_walk(ctx, W, ws, (int)spl, cap, gstride, L);
+            const int r = launch_walk(ctx, W, ws, (int)spl, need, L);
             cudaGraph_t g = nullptr;
             const cudaError_t e = cudaStreamEndCapture(ctx->stream, &g);
             if (r || e != cudaSuccess) {
@@ -2141,10 +2094,10 @@ static int batch_run(mrq_ctx* ctx, int W, const WalkSet& ws, int cap, int gstrid
         L.captured = false;
     } else {
         for (int64_t i = 0; i < nfull; i++)
-            if (int r = launch_walk(ctx, W, ws, (int)spl, cap, gstride, L)) return r;
+            if (int r = launch_walk(ctx, W, ws, (int)spl, need, L)) return r;
     }
     if (rem > 0)
-        if (int r = launch_walk(ctx, W, ws, (int)rem, cap, gstride, L)) return r;
+        if (int r = launch_walk(ctx, W, ws, (int)rem, need, L)) return r;
     return 0;
 }
 
@@ -2159,17 +2112,12 @@ int mrq_batch_advance(mrq_ctx* const* ctxs, int n, int64_t n_steps) {
     for (int i = 0; i < n; i++) CK(cudaStreamSynchronize(ctxs[i]->stream));
     std::vector<Walker*> own(n);
     for (int i = 0; i < n; i++) own[i] = ctxs[i]->d_walk;
-    // one launch sequence per determinant width, warps per walker and occupancy class
+    // one launch sequence per determinant width and warps per block
     for (int slot = 0; slot < mrq_ctx::NSLOT; slot++) {
-        const int W = 1 + slot / 16, nw_eff = MRQ_MAXNW >> ((slot / 4) % 4), cls = 4 - slot % 4;
-        int nw = lead->wpb;
-        if (nw <= 0)
-            for (int i = 0; i < n; i++)
-                if (ctxs[i]->W == W) nw = std::max(nw, auto_warps(ctxs[i]->hsys));
+        const int W = 1 + slot / 4, nw_eff = MRQ_MAXNW >> (slot % 4), nw = lead->wpb > 0 ? lead->wpb : MRQ_MAXNW;
         WalkSet ws;
-        int cap = 1;
-        int gstride = 0;
-        if (int r = batch_tables(ctxs, n, W, own.data(), ws, cap, gstride, cls, nw, nw_eff)) return r;
+        WalkNeed need;
+        if (int r = batch_tables(ctxs, n, W, own.data(), ws, need, nw, nw_eff)) return r;
         if (ws.nsys == 0) continue;
         const size_t q = (size_t)ctx->launches * 2;
         while (ctx->evs.size() < q + 2) {
@@ -2178,7 +2126,7 @@ int mrq_batch_advance(mrq_ctx* const* ctxs, int n, int64_t n_steps) {
             ctx->evs.push_back(ev);
         }
         CK(cudaEventRecord(ctx->evs[q], ctx->stream));
-        if (int r = batch_run(ctx, W, ws, cap, gstride, n_steps, nw_eff, lead->spl, 1, lead->use_graph != 0, slot))
+        if (int r = batch_run(ctx, W, ws, need, n_steps, nw_eff, lead->spl, 1, lead->use_graph != 0, slot))
             return r;
         CK(cudaEventRecord(ctx->evs[q + 1], ctx->stream));
         ctx->launches++;
@@ -2244,13 +2192,12 @@ int mrq_tune_batch(mrq_ctx* const* ctxs, int n, int64_t trial_steps, mrq_tune_re
             if (int r = restore()) return r;
             CK(cudaEventRecord(ctx->ev0, ctx->stream));
             for (int slot = 0; slot < mrq_ctx::NSLOT; slot++) {
-                const int W = 1 + slot / 16, nw_eff = MRQ_MAXNW >> ((slot / 4) % 4), cls = 4 - slot % 4;
+                const int W = 1 + slot / 4, nw_eff = MRQ_MAXNW >> (slot % 4);
                 WalkSet ws;
-                int cap = 1;
-                int gstride = 0;
-                if (int r = batch_tables(ctxs, n, W, scratch.data(), ws, cap, gstride, cls, wpb, nw_eff)) return r;
+                WalkNeed need;
+                if (int r = batch_tables(ctxs, n, W, scratch.data(), ws, need, wpb, nw_eff)) return r;
                 if (ws.nsys == 0) continue;
-                if (int r = batch_run(ctx, W, ws, cap, gstride, trial_steps, nw_eff, spl, 0, false, slot)) return r;
+                if (int r = batch_run(ctx, W, ws, need, trial_steps, nw_eff, spl, 0, false, slot)) return r;
                 if (int r_ = sync_stream(ctx)) return r_;
             }
             CK(cudaEventRecord(ctx->ev1, ctx->stream));
@@ -2454,18 +2401,6 @@ int mrq_debug_set_limits(mrq_ctx* ctx, int max_probe, int cand_cap) {
     }
     return 0;
 }
-
-#ifdef MRQ_PHASE_TIMING
-// timing builds only: the walk's per-phase SM cycles since the last call (ten counters)
-int mrq_phase_times(unsigned long long* out10) {
-    cudaDeviceSynchronize();
-    cudaMemcpyFromSymbol(out10, g_phase, sizeof(unsigned long long) * 10);
-    unsigned long long z[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-    cudaMemcpyToSymbol(g_phase, z, sizeof z);
-    return 0;
-}
-#endif
-
 
 int mrq_read_walkers(mrq_ctx* ctx, uint64_t* dets, double* psi) {
     if (!ctx) return MRQ_INVALID_ARG;

@@ -69,6 +69,7 @@ struct SysDev {
     int cas_units;           // units covering those (MRQ_CAS_CH each)
     int unit_off[9];         // first unit of pair class k = 3 ka + kb (k < 8); unit_off[8] = all units
     int nch[8];              // chunks per (X_a, Y_a) pair of class k
+    int nslice;              // warp tasks a determinant's units are split into (a power of two)
     int gstride;             // doubles of the walker's single-excitation operator, 2 nca nav
     int hb_on;               // heat-bath cutoff in force (hb_eps > 0)
     const unsigned short* colex;       // pair decode table: colex[j(j-1)/2 + i] = i | j << 8, i < j < 128
@@ -93,7 +94,6 @@ struct NoCtr {
     __device__ __forceinline__ void pr(int = 1) {}
     __device__ __forceinline__ void cand() {}
     __device__ __forceinline__ void term(int = 1) {}
-    __device__ __forceinline__ void mark(int) {}     // phase boundary (timing builds only)
 };
 struct Ctr {
     unsigned long long gathers = 0, probes = 0, cands = 0, terms = 0;
@@ -101,7 +101,6 @@ struct Ctr {
     __device__ __forceinline__ void pr(int k = 1) { probes += k; }
     __device__ __forceinline__ void cand() { cands++; }
     __device__ __forceinline__ void term(int k = 1) { terms += k; }   // H_mk phi0(k) products summed
-    __device__ __forceinline__ void mark(int) {}
 };
 
 // ------------------------------------------------------------------ small helpers

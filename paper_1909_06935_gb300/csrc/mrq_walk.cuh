@@ -1,8 +1,20 @@
-// The walk step as one thread block per walker (included by mrq.cu after mrq_cas.cuh).
+// The walk step, by distinct determinants (included by mrq.cu after mrq_cas.cuh).
 //
-// A walker's local evaluation (Eq. 5, Eq. 16, the reach-back overlaps of Eq. 6-7) is split into
-// work units that the block's warps take in a fixed interleaved order (warp w: units w, w + NW,
-// ...), so every sum is formed in the same order on every run: the step is deterministic.
+// A walker's local evaluation (Eq. 5, Eq. 16, the reach-back overlaps of Eq. 6-7) depends on its
+// determinant only, and the walkers of a system crowd on few of them: at 56 orbitals 4,096 walkers
+// in the steady state sit on about 340 determinants of the CAS and 250 of the first-order space.
+// So a step
+//   k_group   finds the distinct determinants (a hash table over the walkers) and cuts each one's
+//             walkers into task groups of at most MRQ_TGW;
+//   k_prep    makes the determinant's constants: its diagonals and its single-excitation operator;
+//   k_eval    evaluates the neighbours once per task group, in work units spread over the whole
+//             chip: the sums S, E_L and the H_D numerator, and for every walker of the group the
+//             move race (its own Philox clocks against the shared rates);
+//   k_move    adds the units' sums, takes each walker's winner, and looks up psi_s there;
+//   k_accum   adds the step records into the accumulators.
+// Every sum is formed in an order that depends on the determinant and its system alone, and the
+// race's winner does not depend on any order, so a walker's step is the same whatever walkers
+// share its determinant, alone or in a batch, and whatever the launch configuration.
 //
 //  * CAS walkers: the neighbours inside the CAS (spin-resolved blocks of active singles and
 //    doubles), then every pair (X_a, Y_a) of active electrons removed / active holes filled.  A
@@ -16,131 +28,69 @@
 // neighbours splits each neighbour's candidate list over f lanes (f a power of two) and reduces
 // the f partial sums with shuffles, so short groups keep the lanes busy.
 //
-// The per-neighbour arithmetic is kept to a few FP64 operations: t = H_nm psi_s(m) is summed as
-// |t| and t, and 1/psi_s(n) is applied once per walker (S = |1/psi_n| sum |t|, E_L = H_nn +
-// (1/psi_n) sum t); the race screens candidates in FP32 (no logarithm: 1 - u against
-// -expm1(-Gamma t_best)) and takes the exact FP64 clock only where a candidate can win.
+// Per neighbour t = H_nm psi_s(m) is summed as |t| and t, and 1/psi_s(n) is applied once per
+// determinant (S = |1/psi_n| sum |t|, E_L = H_nn + (1/psi_n) sum t).
 
 #ifndef MRQ_MAXNW
-#define MRQ_MAXNW 8           // warps per walker block (at most)
+#define MRQ_MAXNW 8           // warps per block (at most)
 #endif
-#define MRQ_VW 8              // virtual warps: the fixed partition of a walker's units (MRQ_MAXNW <= MRQ_VW)
+#define MRQ_VW 8              // virtual warps of the debug evaluation (MRQ_MAXNW <= MRQ_VW)
 #define MRQ_CAS_CH 128        // neighbours per unit inside the CAS
-#define MRQ_FOIS_CH 128       // neighbours per unit of a FOIS walker
+#define MRQ_FOIS_CH 32        // neighbours per unit of a FOIS walker: one round (their reach-back is long)
 #define MRQ_UNIT_NB 1024      // neighbours per unit of an (X_a, Y_a) pair (pairs are cut into chunks)
-// The walk kernel is compiled for 2, 3 and 4 resident blocks of MRQ_MAXNW warps per SM (128, 80
-// and 64 registers); the runtime takes the most blocks the launch's shared memory allows.  More
-// resident warps hide more of the gathers' latency: at 56 orbitals (45 KB per block) four blocks
-// beat three and three beat two (224, 243 and 263 ms per step); five blocks at 48 registers spill
-// too much (268 ms).
+#define MRQ_TGW 32            // walkers per task group (at most): one per lane when they are read and moved
+#define MRQ_NS_MAX 512        // slices of a determinant's units (at most): one warp task each
 
-// the walker block's shared state (dynamic shared memory starts with it)
+// constants of a CAS determinant
 struct CasWalker {
     unsigned long long AOn, AEn, keyn;
     int cntO, cntE;
     double phin, c0, inv_psin;
-    float inv_psin_f;
 };
 
-struct CtaSh {
-    WarpSh L;                       // the walker's system (L.sys) and occupied / empty lists
-    double wsum[3][MRQ_VW];         // per virtual warp sum |t|, sum t, sum t_D
-    double wbt[MRQ_MAXNW];          // per-warp best clock, its psi_s and excitation
-    double wbpsi[MRQ_MAXNW];
-    unsigned wbexc[MRQ_MAXNW];
-    unsigned long long ctr[4];      // debug counters: gathers, probes, candidates, terms
-    double hnn, hdnn;
-    long long nbase_fois;
-    int units;
-    int pad_;
-    // per-thread race state (best exact clock, its psi_s, FP32 image and excitation): kept in shared
-    // memory rather than registers, since it changes only when a candidate beats the lane's best
-    double rbt[MRQ_MAXNW * 32];
-    double rbpsi[MRQ_MAXNW * 32];
-    float rbtf[MRQ_MAXNW * 32];
-    unsigned rbexc[MRQ_MAXNW * 32];
-    // the walker's determinant and CAS constants, read by the work units from shared memory (the
-    // same for every thread; registers stay free for the neighbour loops)
-    CasWalker cw;
-    unsigned long long nsh[4];
-};
-
-__device__ __forceinline__ CtaSh& cta_sh() {
-    extern __shared__ __align__(16) unsigned char smem_dyn[];
-    return *reinterpret_cast<CtaSh*>(smem_dyn);
-}
-
-__host__ __device__ __forceinline__ size_t cta_list_bytes(int cap) {
+__host__ __device__ __forceinline__ size_t cand_list_bytes(int cap) {
     return ((size_t)cap * sizeof(double) + (size_t)cap * sizeof(unsigned) + 15) / 16 * 16;
 }
-__host__ __device__ __forceinline__ size_t cta_smem_bytes(int nw, int cap, int gstride) {
-    return (sizeof(CtaSh) + 15) / 16 * 16 + ((size_t)gstride * sizeof(double) + 15) / 16 * 16 +
-           (size_t)nw * cta_list_bytes(cap);
-}
 
-#ifdef MRQ_PHASE_TIMING
-// Phase clock of a timing build (compiled with -DMRQ_PHASE_TIMING only): per-warp SM cycles spent
-// in 0 set-up, 1 CAS-internal units, 2 pair-unit overhead, 3 candidate lists, 4 neighbour decode
-// and H_nm, 5 reach-back sums, 6 rates / labels / race, 7 FOIS units, 8 block reductions.
-__device__ unsigned long long g_phase[10];
-struct PhCtr : NoCtr {
-    long long t = 0;
-    long long acc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-    __device__ __forceinline__ void mark(int k) {
-        const long long u = clock64();
-        if (t) acc[k] += u - t;
-        t = u;
-    }
-};
-#endif
-
-// per-lane running sums of a walker's step (scaled by 1/psi_s(n) once at the end); the lane's race
-// state is in shared memory (CtaSh::rbt ...)
-struct LaneAcc2 {
-    double sA, sT, sD;     // sum |t|, sum t, sum t_D   (t = H_nm psi_s(m), t_D = (H_D)_nm psi_s(m))
+// the race's best candidate of a walker: FP32 clock, excitation, and t of its neighbour (16 bytes,
+// replaced by one 128-bit compare-and-swap)
+struct __align__(16) RaceBest {
+    unsigned clk;             // FP32 image of the clock
+    unsigned exc;             // excitation code, 0xFFFFFFFF: none yet
+    double t;                 // H_nm psi_s(m)
 };
 
-__device__ __forceinline__ void acc2_init(LaneAcc2& a) {
-    a.sA = a.sT = a.sD = 0.0;
-    CtaSh& cs = cta_sh();
-    cs.rbt[threadIdx.x] = INFINITY;
-    cs.rbtf[threadIdx.x] = INFINITY;
-    cs.rbexc[threadIdx.x] = 0xFFFFFFFFu;
-    cs.rbpsi[threadIdx.x] = 0.0;
-}
+// a run of walkers on one determinant
+struct TaskGroup {
+    int sys, first, count;    // members[first .. first + count): walkers of system sys
+    int group;                // the determinant's index (its operator, constants and partial sums)
+    int primary;              // the group of the determinant that stores its sums
+    int pad;
+};
 
-// the exact FP64 clock, kept out of the hot loop's code (few candidates pass the screen)
-__device__ __noinline__ double race_clock_cold(unsigned long long k53, double g) { return race_clock_f64(k53, g); }
+struct GroupMeta {
+    unsigned long long d[2][2];
+    double psi, hnn, hdnn;
+    long long label;
+    int h, p;
+};
 
-// one neighbour m: sums and the race (Sec. II B first-reaction form).  t = H_nm psi_s(m).
-template <int MODE>
-__device__ __forceinline__ void lane_post2(const SysDev& S, LaneAcc2& a, double t, double tD, double psim,
-                                           double inv_psin, float inv_psin_f, unsigned exc, unsigned step,
-                                           unsigned wid) {
-    a.sA += fabs(t);
-    a.sT += t;
-    a.sD += tD;
-    if (MODE == MODE_STEP) {
-        if ((__double_as_longlong(t) << 1) != 0) {          // t != 0, without an FP64 compare
-            const unsigned long long k53 = race_bits(S.seed, exc, step, wid);
-            CtaSh& cs = cta_sh();
-            const int me = threadIdx.x;
-            if (race_may_win(k53, abs_f32_of(t) * inv_psin_f, cs.rbtf[me])) {
-                const double g = fabs(t * inv_psin);
-                if (g > 0.0) {
-                    const double tc = race_clock_cold(k53, g);
-                    const double bt = cs.rbt[me];
-                    if (tc < bt || (tc == bt && exc < cs.rbexc[me])) {
-                        cs.rbt[me] = tc;
-                        cs.rbtf[me] = (float)tc;
-                        cs.rbexc[me] = exc;
-                        cs.rbpsi[me] = psim;
-                    }
-                }
-            }
-        }
-    }
-}
+// device workspace of a walk launch, sized for the slots [seg0, seg1) of the walk set
+struct WalkScratch {
+    int *rep, *cnt, *start;   // determinant tables, 4 entries per slot: first walker, walkers, first member
+    int *tab_of, *pos_of;     // per slot: table entry and place in it
+    int* members;             // walkers (local index) by determinant
+    TaskGroup* tg;
+    GroupMeta* meta;
+    double* gops;             // single-excitation operators, gstride doubles per determinant
+    double* part;             // [determinant][ns_max][3] partial sums
+    RaceBest* best;           // per slot
+    unsigned* bound;          // per slot: FP32 bits of an upper bound of the best clock
+    int* ctl;                 // task groups, determinants, next warp task
+    long long gstride;
+    int ns_max, tgw;
+    long long seg0, seg1;
+};
 
 __device__ __forceinline__ void write_rec(mrq_neighbour* rec, const unsigned long long* m, int W, double hnm,
                                           double hd, double om, double psim, double gamma, unsigned exc) {
@@ -172,9 +122,6 @@ __device__ __forceinline__ void det_words(const unsigned long long (&m)[2][W], u
 __device__ __forceinline__ unsigned exc_code(int r1, int r2, int a1, int a2) {
     return (unsigned)r1 | ((unsigned)r2 << 8) | ((unsigned)a1 << 16) | ((unsigned)a2 << 24);
 }
-
-// ------------------------------------------------------------------ per-walker constants (CAS)
-
 
 // spin-resolved candidate blocks: R' (ne electrons of m's active occupation) and A' (nf holes),
 // alpha(R') - alpha(A') = dsp; block b takes alpha(R') = ib[b]; its index is decoded by multiplying
@@ -241,11 +188,11 @@ __device__ __forceinline__ void cand_decode(const SysDev& S, const CandPlan& P, 
 }
 
 // build the candidate list of group (c, v, sc, sv) of active remnant (AOm, AEm): singles [0, n1) as
-// codes, doubles [n1, count) as (signed weight, table base); the candidate k = n is left out.  Kept
+// codes, doubles [n1, count) as (signed weight, table base); the candidate of key keyn (the walker) is left out.  Kept
 // out of line: it runs once per group, and its registers and code then stay out of the neighbour
 // loop that follows (1.8 % faster at 56 orbitals)
 template <int W, class C>
-__device__ __noinline__ int build_group_list(const SysDev& S, const CasWalker& cw,
+__device__ __noinline__ int build_group_list(const SysDev& S, unsigned long long keyn,
                                                 const unsigned long long (&mref)[2][W], unsigned long long AOm,
                                                 unsigned long long AEm, int c, int v, int sc, int sv, int rxc0,
                                                 int rxc1, int ryv0, int ryv1, int par_ref, double* cphi,
@@ -272,7 +219,7 @@ __device__ __noinline__ int build_group_list(const SysDev& S, const CasWalker& c
                 const unsigned long long kact = (AOm & ~Rb) | Ab;
                 const unsigned long long key = hash_key(S, (unsigned)kact, (unsigned)(kact >> 32));
                 ctr.cand();
-                if (key == cw.keyn) valid = false;
+                if (key == keyn) valid = false;
                 else {
                     phi = hash_lookup(S, key, ctr);
                     valid = (__double_as_longlong(phi) << 1) != 0;      // phi != 0 without an FP64 compare
@@ -375,82 +322,78 @@ __device__ __forceinline__ int cas_unit_count(const SysDev& S, const CasWalker& 
 
 // neighbours inside the CAS: spin-resolved blocks (alpha singles, beta singles, alpha-alpha,
 // beta-beta, alpha-beta doubles) of the walker's active electrons / holes
-template <int W, int MODE, class C>
-__device__ __noinline__ LaneAcc2 cas_internal_unit(const SysDev& S, const CasWalker& cw, const unsigned long long (&n)[2][W], int u,
-                                  LaneAcc2 acc, unsigned step, unsigned wid, int lane, mrq_neighbour* nbout,
-                                  long long nbase, long long max_nb, C& ctr) {
+template <int W, class Sink, class C>
+__device__ __noinline__ void cas_internal_unit(const SysDev& S, const CasWalker& cw, const unsigned long long (&n)[2][W],
+                                               int u, int lane, Sink& sink, C& ctr) {
     const unsigned long long oa = cw.AOn & 0xFFFFFFFFull, ob = cw.AOn & ~0xFFFFFFFFull;
     const unsigned long long ea = cw.AEn & 0xFFFFFFFFull, eb = cw.AEn & ~0xFFFFFFFFull;
     const int coa = __popcll(oa), cob = __popcll(ob), cea = __popcll(ea), ceb = __popcll(eb);
     const int b0 = coa * cea, b1 = b0 + cob * ceb, b2 = b1 + nsub(coa, 2) * nsub(cea, 2),
               b3 = b2 + nsub(cob, 2) * nsub(ceb, 2), b4 = b3 + coa * cea * cob * ceb;
     const int i0 = u * MRQ_CAS_CH, i1 = min(b4, i0 + MRQ_CAS_CH);
-    for (int idx = i0 + lane; idx < i1; idx += 32) {
-        unsigned long long Xb, Yb;
-        int r;
-        if (idx < b0) {
-            r = 1;
-            Xb = subset_bits(S.colex, oa, coa, 1, idx / cea);
-            Yb = subset_bits(S.colex, ea, cea, 1, idx % cea);
-        } else if (idx < b1) {
-            const int x = idx - b0;
-            r = 1;
-            Xb = subset_bits(S.colex, ob, cob, 1, x / ceb);
-            Yb = subset_bits(S.colex, eb, ceb, 1, x % ceb);
-        } else if (idx < b2) {
-            const int x = idx - b1, ny = nsub(cea, 2);
-            r = 2;
-            Xb = subset_bits(S.colex, oa, coa, 2, x / ny);
-            Yb = subset_bits(S.colex, ea, cea, 2, x % ny);
-        } else if (idx < b3) {
-            const int x = idx - b2, ny = nsub(ceb, 2);
-            r = 2;
-            Xb = subset_bits(S.colex, ob, cob, 2, x / ny);
-            Yb = subset_bits(S.colex, eb, ceb, 2, x % ny);
-        } else {
-            int x = idx - b3;
-            r = 2;
-            const int yb = x % ceb;
-            x /= ceb;
-            const int xb = x % cob;
-            x /= cob;
-            const int ya = x % cea, xa = x / cea;
-            Xb = subset_bits(S.colex, oa, coa, 1, xa) | subset_bits(S.colex, ob, cob, 1, xb);
-            Yb = subset_bits(S.colex, ea, cea, 1, ya) | subset_bits(S.colex, eb, ceb, 1, yb);
-        }
-        int rem[2], add[2];
-        act_list(S, Xb, rem);
-        act_list(S, Yb, add);
+    for (int base = i0; base < i1; base += 32) {
+        const bool valid = base + lane < i1;
+        const int idx = base + lane;
         unsigned long long m[2][W];
 #pragma unroll
         for (int sg = 0; sg < 2; sg++)
 #pragma unroll
             for (int w = 0; w < W; w++) m[sg][w] = n[sg][w];
-        apply_exc<W>(m, S, rem, add, r);
-        const double hnm = r == 1 ? single_elem<W>(S, n, rem[0], add[0], ctr)
-                                  : double_elem_tab<W>(S, n, rem[0], rem[1], add[0], add[1], ctr);
-        const unsigned long long km = (cw.AOn & ~Xb) | Yb;
-        ctr.cand();
-        const double om = hash_lookup(S, hash_key(S, (unsigned)km, (unsigned)(km >> 32)), ctr);
-        const unsigned exc = r == 1 ? exc_code(rem[0], rem[0], add[0], add[0]) : exc_code(rem[0], rem[1], add[0], add[1]);
-        const double psim = cw.c0 * om;
-        const double t = hnm * psim;
-        lane_post2<MODE>(S, acc, t, 0.0, psim, cw.inv_psin, cw.inv_psin_f, exc, step, wid);
-        if (MODE == MODE_DEBUG && nbout != nullptr && nbase + (idx - i0) < max_nb) {
-            unsigned long long w4[4];
-            det_words<W>(m, w4);
-            write_rec(nbout + nbase + (idx - i0), w4, W, hnm, 0.0, om, psim, fabs(t * cw.inv_psin), exc);
+        double hnm = 0.0, om = 0.0, psim = 0.0;
+        unsigned exc = 0;
+        if (valid) {
+            unsigned long long Xb = 0, Yb = 0;
+            int r;
+            if (idx < b0) {
+                r = 1;
+                Xb = subset_bits(S.colex, oa, coa, 1, idx / cea);
+                Yb = subset_bits(S.colex, ea, cea, 1, idx % cea);
+            } else if (idx < b1) {
+                const int x = idx - b0;
+                r = 1;
+                Xb = subset_bits(S.colex, ob, cob, 1, x / ceb);
+                Yb = subset_bits(S.colex, eb, ceb, 1, x % ceb);
+            } else if (idx < b2) {
+                const int x = idx - b1, ny = nsub(cea, 2);
+                r = 2;
+                Xb = subset_bits(S.colex, oa, coa, 2, x / ny);
+                Yb = subset_bits(S.colex, ea, cea, 2, x % ny);
+            } else if (idx < b3) {
+                const int x = idx - b2, ny = nsub(ceb, 2);
+                r = 2;
+                Xb = subset_bits(S.colex, ob, cob, 2, x / ny);
+                Yb = subset_bits(S.colex, eb, ceb, 2, x % ny);
+            } else {
+                int x = idx - b3;
+                r = 2;
+                const int yb = x % ceb;
+                x /= ceb;
+                const int xb = x % cob;
+                x /= cob;
+                const int ya = x % cea, xa = x / cea;
+                Xb = subset_bits(S.colex, oa, coa, 1, xa) | subset_bits(S.colex, ob, cob, 1, xb);
+                Yb = subset_bits(S.colex, ea, cea, 1, ya) | subset_bits(S.colex, eb, ceb, 1, yb);
+            }
+            int rem[2], add[2];
+            act_list(S, Xb, rem);
+            act_list(S, Yb, add);
+            apply_exc<W>(m, S, rem, add, r);
+            hnm = r == 1 ? single_elem<W>(S, n, rem[0], add[0], ctr)
+                                      : double_elem_tab<W>(S, n, rem[0], rem[1], add[0], add[1], ctr);
+            const unsigned long long km = (cw.AOn & ~Xb) | Yb;
+            ctr.cand();
+            om = hash_lookup(S, hash_key(S, (unsigned)km, (unsigned)(km >> 32)), ctr);
+            exc = r == 1 ? exc_code(rem[0], rem[0], add[0], add[0]) : exc_code(rem[0], rem[1], add[0], add[1]);
+            psim = cw.c0 * om;
         }
+        sink.template post<W>(valid, idx - i0, m, hnm, 0.0, om, psim, exc);
     }
-    return acc;
 }
 
 // one (X_a, Y_a) pair chunk [lo, hi) of a CAS walker
-template <int W, int MODE, class C>
+template <int W, class Sink, class C>
 __device__ void cas_pair_unit(const SysDev& S, const CasWalker& cw, const double* __restrict__ gops, double* cphi,
-                              unsigned* ccode, const unsigned long long (&n)[2][W], int u, LaneAcc2& acc,
-                              unsigned step, unsigned wid, int lane, mrq_neighbour* nbout, long long nbase,
-                              long long max_nb, C& ctr) {
+                              unsigned* ccode, const unsigned long long (&n)[2][W], int u, int lane, Sink& sink, C& ctr) {
     int k = 0;
     while (k < 7 && u >= S.unit_off[k + 1]) k++;
     const int ka = k / 3, kb = k % 3, nch = S.nch[k];
@@ -471,7 +414,6 @@ __device__ void cas_pair_unit(const SysDev& S, const CasWalker& cw, const double
     const int ya1 = (kb == 2) ? act_so(S, 63 - __clzll(Yb)) : 0;
     const int nc = S.nc, nv = S.nv, voff = S.nc + S.na;
     int base = 0;
-    ctr.mark(2);
     for (int r = max(1, max(ka, kb)); r <= 2; r++) {
         const int c = r - ka, v = r - kb;
         if (c == 0 && v == 0) continue;
@@ -491,10 +433,8 @@ __device__ void cas_pair_unit(const SysDev& S, const CasWalker& cw, const double
                 int n1;
                 // floor(q / nvc) = high word of q * ceil(2^64 / nvc), exact for q < 2^32 (nvc > 1)
                 const unsigned long long mvc = ~0ull / (unsigned long long)nvc + 1ull;
-                ctr.mark(2);
-                const int count = build_group_list<W>(S, cw, mref, AOm, AEm, c, v, sc, sv, rxc0, rxc1, ryv0, ryv1,
+                const int count = build_group_list<W>(S, cw.keyn, mref, AOm, AEm, c, v, sc, sv, rxc0, rxc1, ryv0, ryv1,
                                                       par_ref, cphi, ccode, n1, lane, ctr);
-                ctr.mark(3);
                 for (int qb = q0; qb < q1; qb += 32) {
                     const int nr = min(32, q1 - qb);
                     const int f = split_of(nr), lf = __ffs(f) - 1;
@@ -510,7 +450,6 @@ __device__ void cas_pair_unit(const SysDev& S, const CasWalker& cw, const double
                     int par;
                     lane_offsets(S, c, v, xc0, xc1, yv0, yv1, offd, offx, par);
                     double hnm = 0.0, a0 = 0.0, a1 = 0.0;
-                    ctr.mark(4);
                     if (valid) {
                         if (part == 0) {
                             if (r == 1) {
@@ -524,7 +463,6 @@ __device__ void cas_pair_unit(const SysDev& S, const CasWalker& cw, const double
                             }
                             a0 = neg_if(hnm * cw.phin, par);        // the k = n term
                         }
-                        ctr.mark(4);
                         for (int e = part; e < n1; e += f)
                             a1 = fma(cphi[e], neg_if(sgl_elem_code<W>(S, gops, m, ccode[e], v, yv0, c, xc0, r, rm0,
                                                                        rm1, ad0, ad1, ctr), par), a1);
@@ -551,30 +489,22 @@ __device__ void cas_pair_unit(const SysDev& S, const CasWalker& cw, const double
                     }
                     double s = a0 + a1;
                     for (int o = f >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                    ctr.mark(5);
-                    if (valid && part == 0) {
+                    double om = 0.0, psim = 0.0;
+                    unsigned exc = 0;
+                    const bool mine = valid && part == 0;
+                    if (mine) {
                         ctr.term(count + 1);
-                        const double om = neg_if(s, par);
+                        om = neg_if(s, par);
                         const int h0 = xc0 >= S.n ? nc + (xc0 - S.n) : xc0;
                         const int h1 = xc1 >= S.n ? nc + (xc1 - S.n) : xc1;
                         const int p0 = yv0 >= S.n ? nv + (yv0 - S.n - voff) : yv0 - voff;
                         const int p1 = yv1 >= S.n ? nv + (yv1 - S.n - voff) : yv1 - voff;
                         const long long lm = set_rank(c, h0, h1, 2 * nc) * S.nPs + set_rank(v, p0, p1, 2 * nv);
                         ctr.g();
-                        const double psim = __ldg(S.c + lm) * om;
-                        const double t = hnm * psim;
-                        const unsigned exc = r == 1 ? exc_code(rm0, rm0, ad0, ad0) : exc_code(rm0, rm1, ad0, ad1);
-                        lane_post2<MODE>(S, acc, t, 0.0, psim, cw.inv_psin, cw.inv_psin_f, exc, step, wid);
-                        if (MODE == MODE_DEBUG && nbout != nullptr) {
-                            const long long ri = nbase + (base + q) - lo;
-                            if (ri < max_nb) {
-                                unsigned long long w4[4];
-                                det_words<W>(m, w4);
-                                write_rec(nbout + ri, w4, W, hnm, 0.0, om, psim, fabs(t * cw.inv_psin), exc);
-                            }
-                        }
+                        psim = __ldg(S.c + lm) * om;
+                        exc = r == 1 ? exc_code(rm0, rm0, ad0, ad0) : exc_code(rm0, rm1, ad0, ad1);
                     }
-                    ctr.mark(6);
+                    sink.template post<W>(mine, base + q - lo, m, hnm, 0.0, om, psim, exc);
                 }
                 __syncwarp();
             }
@@ -586,309 +516,697 @@ __device__ void cas_pair_unit(const SysDev& S, const CasWalker& cw, const double
 // ------------------------------------------------------------------ FOIS units
 
 // neighbours [i0, i1) of the class-block enumeration, reach-back per lane
-template <int W, int MODE, class C>
-__device__ __noinline__ LaneAcc2 fois_unit(const SysDev& S, const WarpSh& sh, const double* __restrict__ gops,
-                          const unsigned long long (&n)[2][W], long long ln,
-                          double c0, double inv_psin, float inv_psin_f, unsigned long long self_key, double phi_self,
-                          int i0, int i1, LaneAcc2 acc, unsigned step, unsigned wid, int lane, mrq_neighbour* nbout,
-                          long long nbase, long long max_nb, C& ctr) {
-    for (int idx = i0 + lane; idx < i1; idx += 32) {
-        int lo = 0, hi = sh.nb - 1;          // block of idx: last b with bstart[b] <= idx
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (sh.bstart[mid] <= idx) lo = mid;
-            else hi = mid - 1;
-        }
-        const unsigned desc = sh.bdesc[lo];
-        int kind, r1, r2, a1, a2;
-        decode_exc(sh, S.n, desc, idx - sh.bstart[lo], kind, r1, r2, a1, a2);
+template <int W, class Sink, class C>
+__device__ __noinline__ void fois_unit(const SysDev& S, const WarpLists& sh, const double* __restrict__ gops,
+                                       const unsigned long long (&n)[2][W], long long ln, double c0,
+                                       unsigned long long self_key, double phi_self, int i0, int i1, int lane,
+                                       Sink& sink, C& ctr) {
+    for (int base = i0; base < i1; base += 32) {
+        const int idx = base + lane;
+        const bool valid = idx < i1;
         unsigned long long m[2][W];
 #pragma unroll
         for (int sg = 0; sg < 2; sg++)
 #pragma unroll
             for (int w = 0; w < W; w++) m[sg][w] = n[sg][w];
-        {
-            int s1 = r1 >= S.n, s2 = a1 >= S.n;
-            flip_reg<W>(m, s1, r1 - s1 * S.n);
-            flip_reg<W>(m, s2, a1 - s2 * S.n);
-            if (kind != 0) {
-                int s3 = r2 >= S.n, s4 = a2 >= S.n;
-                flip_reg<W>(m, s3, r2 - s3 * S.n);
-                flip_reg<W>(m, s4, a2 - s4 * S.n);
+        double hnm = 0.0, hd = 0.0, om = 0.0, psim = 0.0;
+        unsigned exc = 0;
+        if (valid) {
+            int lo = 0, hi = sh.nb - 1;          // block of idx: last b with bstart[b] <= idx
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (sh.bstart[mid] <= idx) lo = mid;
+                else hi = mid - 1;
+            }
+            const unsigned desc = sh.bdesc[lo];
+            int kind, r1, r2, a1, a2;
+            decode_exc(sh, S.n, desc, idx - sh.bstart[lo], kind, r1, r2, a1, a2);
+            {
+                int s1 = r1 >= S.n, s2 = a1 >= S.n;
+                flip_reg<W>(m, s1, r1 - s1 * S.n);
+                flip_reg<W>(m, s2, a1 - s2 * S.n);
+                if (kind != 0) {
+                    int s3 = r2 >= S.n, s4 = a2 >= S.n;
+                    flip_reg<W>(m, s3, r2 - s3 * S.n);
+                    flip_reg<W>(m, s4, a2 - s4 * S.n);
+                }
+            }
+            if (kind != 0) hnm = hb_screen(S, double_elem<W>(S, n, r1, r2, a1, a2, ctr));
+            else if (gops != nullptr && in_walker_block(S, r1, a1))
+                hnm = single_from_walker<W>(S, SglFromWalker{gops, 0, 0, 0, 0, 0}, n, r1, a1, ctr);
+            else hnm = single_elem<W>(S, n, r1, a1, ctr);
+            int hm, pm;
+            const long long lm = det_label<W>(S, m, hm, pm);
+            if (lm == 0) {
+                ctr.cand();
+                om = hash_lookup(S, hash_key(S, active_bits<W>(S, m[0]), active_bits<W>(S, m[1])), ctr);
+                psim = c0 * om;
+            } else {
+                om = reach_back<W>(S, m, ctr, self_key, hnm * phi_self,
+                                   SglFromWalker{gops, kind == 0 ? 1 : 2, r1, r2, a1, a2});
+                ctr.g();
+                psim = __ldg(S.c + lm) * om;
+            }
+            const bool same = ln > 0 && active_only(desc);
+            hd = same ? ((kind == 0) ? hd_single_elem<W>(S, n, r1, a1, ctr) : hnm) : 0.0;
+            exc = exc_code(r1, r2, a1, a2);
+        }
+        sink.template post<W>(valid, idx, m, hnm, hd, om, psim, exc);
+    }
+}
+
+// overlap O(m) = <m|H|phi0> (Eq. 6-7) of one first-order determinant m by a whole warp: m's
+// candidate list as of a group of one neighbour, the list's terms split over the lanes
+template <int W>
+__device__ __noinline__ double reach_back_warp(const SysDev& S, const unsigned long long (&m)[2][W], double* cphi,
+                                               unsigned* ccode, int lane) {
+    int c = 0, v = 0, xc[2] = {0, 0}, yv[2] = {0, 0}, sc = 0, sv = 0;
+#pragma unroll
+    for (int sg = 0; sg < 2; sg++) {
+        unsigned long long hm = ~m[sg][0] & S.mcore[0];
+        while (hm) {
+            const int i = __ffsll(hm) - 1;
+            hm &= hm - 1;
+            if (c == 0) xc[0] = sg * S.n + i;
+            else xc[1] = sg * S.n + i;
+            c++;
+            sc += sg == 0;
+        }
+#pragma unroll
+        for (int w = 0; w < W; w++) {
+            unsigned long long pm = m[sg][w] & S.mvirt[w];
+            while (pm) {
+                const int a = 64 * w + __ffsll(pm) - 1;
+                pm &= pm - 1;
+                if (v == 0) yv[0] = sg * S.n + a;
+                else yv[1] = sg * S.n + a;
+                v++;
+                sv += sg == 0;
             }
         }
-        double hnm;
-        if (kind != 0) hnm = hb_screen(S, double_elem<W>(S, n, r1, r2, a1, a2, ctr));
-        else if (gops != nullptr && in_walker_block(S, r1, a1))
-            hnm = single_from_walker<W>(S, SglFromWalker{gops, 0, 0, 0, 0, 0}, n, r1, a1, ctr);
-        else hnm = single_elem<W>(S, n, r1, a1, ctr);
-        int hm, pm;
-        const long long lm = det_label<W>(S, m, hm, pm);
-        double om, psim;
-        if (lm == 0) {
-            ctr.cand();
-            om = hash_lookup(S, hash_key(S, active_bits<W>(S, m[0]), active_bits<W>(S, m[1])), ctr);
-            psim = c0 * om;
-        } else {
-            om = reach_back<W>(S, m, ctr, self_key, hnm * phi_self,
-                               SglFromWalker{gops, kind == 0 ? 1 : 2, r1, r2, a1, a2});
+    }
+    const unsigned ao0 = active_bits<W>(S, m[0]), ao1 = active_bits<W>(S, m[1]);
+    const unsigned amask = (S.na >= 32) ? 0xFFFFFFFFu : ((1u << S.na) - 1u);
+    const unsigned long long AOm = (unsigned long long)ao0 | ((unsigned long long)ao1 << 32);
+    const unsigned long long AEm = (unsigned long long)(~ao0 & amask) | ((unsigned long long)(~ao1 & amask) << 32);
+    unsigned offd, offx;
+    int par, n1;
+    lane_offsets(S, c, v, xc[0], xc[1], yv[0], yv[1], offd, offx, par);
+    NoCtr ctr;
+    const int count = build_group_list<W>(S, MRQ_EMPTY_KEY, m, AOm, AEm, c, v, sc, sv, xc[0], xc[1], yv[0], yv[1], par,
+                                          cphi, ccode, n1, lane, ctr);
+    double s = 0.0;
+    for (int e = lane; e < n1; e += 32)
+        s = fma(cphi[e], neg_if(sgl_elem_code<W>(S, nullptr, m, ccode[e], v, yv[0], c, xc[0], 0, 0, 0, 0, 0, ctr), par), s);
+    for (int e = n1 + lane; e < count; e += 32) {
+        const unsigned p0 = ccode[e];
+        s = fma(cphi[e], __ldg(S.tab + (p0 & 0x7FFFFFFFu) + ((p0 & 0x80000000u) ? offx : offd)), s);
+    }
+    s = warp_sum(s);
+    __syncwarp();
+    return neg_if(s, par);
+}
+
+// ------------------------------------------------------------------ a determinant's constants
+
+// the determinant's single-excitation operator G_yx(n) = h_yx + sum_{j in n} [(yx|jj) - delta (yj|jx)]
+// for y in core + active, x in active + virtual (not both active), by a whole block: the full-core
+// operator hc, n's active electrons, minus n's core holes, plus its virtual electrons
+template <int W, class C>
+__device__ void walker_operator(const SysDev& S, const unsigned long long (&n)[2][W], bool cas, double* gops, C& ctr) {
+    const unsigned ao0 = active_bits<W>(S, n[0]), ao1 = active_bits<W>(S, n[1]);
+    const unsigned long long AOn = (unsigned long long)ao0 | ((unsigned long long)ao1 << 32);
+    int nh = 0, np = 0, hso[2] = {0, 0}, pso[2] = {0, 0};
+    if (!cas) {
+#pragma unroll
+        for (int sg = 0; sg < 2; sg++) {
+            unsigned long long hm = ~(sg ? n[1][0] : n[0][0]) & S.mcore[0];
+            while (hm) {
+                const int i = __ffsll(hm) - 1;
+                hm &= hm - 1;
+                if (nh == 0) hso[0] = sg * S.n + i;
+                else hso[1] = sg * S.n + i;
+                nh++;
+            }
+#pragma unroll
+            for (int w = 0; w < W; w++) {
+                unsigned long long pm = (sg ? n[1][w] : n[0][w]) & S.mvirt[w];
+                while (pm) {
+                    const int a = 64 * w + __ffsll(pm) - 1;
+                    pm &= pm - 1;
+                    if (np == 0) pso[0] = sg * S.n + a;
+                    else pso[1] = sg * S.n + a;
+                    np++;
+                }
+            }
+        }
+    }
+    const int blk = S.nca * S.nav;
+    for (int t = threadIdx.x; t < 2 * blk; t += blockDim.x) {
+        const int sg = t >= blk, rem = t - sg * blk;
+        const int y = rem / S.nav, xo = rem - y * S.nav, x = S.nc + xo;
+        if (y >= S.nc && xo < S.na) continue;
+        ctr.g();
+        double v = __ldg(S.hc + y * S.n + x);
+        unsigned long long bits = AOn;
+        while (bits) {
+            const int b = __ffsll(bits) - 1;
+            bits &= bits - 1;
+            const int j = S.nc + (b & 31);
+            v += eri_g(S, y, x, j, j);
             ctr.g();
-            psim = __ldg(S.c + lm) * om;
+            if ((b >= 32) == (sg == 1)) {
+                v -= eri_g(S, y, j, j, x);
+                ctr.g();
+            }
         }
-        const bool same = ln > 0 && active_only(desc);
-        const double hd = same ? ((kind == 0) ? hd_single_elem<W>(S, n, r1, a1, ctr) : hnm) : 0.0;
-        const unsigned exc = exc_code(r1, r2, a1, a2);
-        const double t = hnm * psim;
-        lane_post2<MODE>(S, acc, t, hd * psim, psim, inv_psin, inv_psin_f, exc, step, wid);
-        if (MODE == MODE_DEBUG && nbout != nullptr && nbase + idx < max_nb) {
-            unsigned long long w4[4];
-            det_words<W>(m, w4);
-            write_rec(nbout + nbase + idx, w4, W, hnm, hd, om, psim, fabs(t * inv_psin), exc);
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            if (k < nh) {
+                v -= g_corr(S, sg, x, y, hso[k]);
+                ctr.g(2);
+            }
+            if (k < np) {
+                v += g_corr(S, sg, x, y, pso[k]);
+                ctr.g(2);
+            }
         }
-    }
-    return acc;
-}
-
-// ------------------------------------------------------------------ one walker step per block
-
-template <class C>
-__device__ __forceinline__ void ctr_flush(CtaSh& cs, const C& ctr, int lane) {}
-template <>
-__device__ __forceinline__ void ctr_flush<Ctr>(CtaSh& cs, const Ctr& ctr, int lane) {
-    unsigned long long v[4] = {ctr.gathers, ctr.probes, ctr.cands, ctr.terms};
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-        unsigned long long x = v[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (lane == 0) atomicAdd(&cs.ctr[k], x);
+        gops[t] = v;
     }
 }
 
-struct StepOut {
-    double S, EL, num, hnn, hdnn;
-    long long nnb;
-    unsigned bexc;
-    double bpsi;
+template <int W>
+__device__ __forceinline__ CasWalker cas_constants(const SysDev& S, const unsigned long long (&n)[2][W], double psin) {
+    CasWalker cw;
+    const unsigned ao0 = active_bits<W>(S, n[0]), ao1 = active_bits<W>(S, n[1]);
+    const unsigned amask = (S.na >= 32) ? 0xFFFFFFFFu : ((1u << S.na) - 1u);
+    cw.AOn = (unsigned long long)ao0 | ((unsigned long long)ao1 << 32);
+    cw.AEn = (unsigned long long)(~ao0 & amask) | ((unsigned long long)(~ao1 & amask) << 32);
+    cw.keyn = hash_key(S, ao0, ao1);
+    cw.cntO = __popcll(cw.AOn);
+    cw.cntE = __popcll(cw.AEn);
+    cw.c0 = __ldg(S.c);
+    cw.phin = psin / cw.c0;
+    cw.inv_psin = 1.0 / psin;
+    return cw;
+}
+
+// ------------------------------------------------------------------ the move race
+
+// Philox4x32-10 of counter (exc, step, walker, 0): after two rounds the state is a mix of words that
+// depend on the excitation alone and words that depend on the walker alone, so both halves are made
+// once (race_walker_words per walker and task, the excitation's per neighbour) and a clock costs the
+// last eight rounds, of which the last needs one product: 15 products instead of 20.
+#define PHILOX_M0 0xD2511F53u
+#define PHILOX_M1 0xCD9E8D57u
+#define PHILOX_W0 0x9E3779B9u
+#define PHILOX_W1 0xBB67AE85u
+
+struct WarpTask {
+    SysDev sys;                         // the system of the task's walkers
+    CasWalker cw;
+    unsigned long long nsh[4];
+    double inv_psin;
+    float inv_f;                        // FP32 |1/psi_s(n)| (INFINITY when FP32 cannot carry it)
+    int qn;                             // neighbours waiting in the queue
+    uint4 wp[MRQ_TGW];                  // per walker: Philox words (x, y) and screen scale (w, FP32)
+    unsigned wid[MRQ_TGW], step[MRQ_TGW], slot[MRQ_TGW];
+    float bnd[MRQ_TGW];                 // upper bound of the best clock
+    double qt[64];                      // queued neighbours: t and excitation
+    unsigned qe[64];
 };
 
-// The local evaluation of determinant n (psi_s(n) = psin, label ln, (h, p)) by the whole block.
-// Returns on every thread; the winner of the race is valid in MODE_STEP.
-template <int W, int MODE, class C>
-__device__ StepOut block_local(CtaSh& cs, unsigned char* lists, const unsigned long long (&n)[2][W], double psin,
-                               long long ln, int h, int p, unsigned step, unsigned wid, mrq_neighbour* nbout,
-                               long long max_nb, long long* nb_prefix, C& ctr) {
-    const SysDev& S = cs.L.sys;
-    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const double c0 = __ldg(S.c);
-    const double inv_psin = psin != 0.0 ? 1.0 / psin : 0.0;
-    const float inv_psin_f = abs_f32_of(inv_psin);
-    double* gops = reinterpret_cast<double*>(lists);
-    unsigned char* wl = lists + ((size_t)S.gstride * sizeof(double) + 15) / 16 * 16 + (size_t)wi * cta_list_bytes(S.cand_cap);
-    double* cphi = reinterpret_cast<double*>(wl);
-    unsigned* ccode = reinterpret_cast<unsigned*>(cphi + S.cand_cap);
-    if (wi == 0) build_lists<W>(S, n, cs.L, ln == 0 ? 0 : h, ln == 0 ? 0 : p, lane);
-    CasWalker cw;
-    const bool cas = ln == 0 && psin != 0.0;
-    int units;
-    if (cas) {
-        const unsigned ao0 = active_bits<W>(S, n[0]), ao1 = active_bits<W>(S, n[1]);
-        const unsigned amask = (S.na >= 32) ? 0xFFFFFFFFu : ((1u << S.na) - 1u);
-        cw.AOn = (unsigned long long)ao0 | ((unsigned long long)ao1 << 32);
-        cw.AEn = (unsigned long long)(~ao0 & amask) | ((unsigned long long)(~ao1 & amask) << 32);
-        cw.keyn = hash_key(S, ao0, ao1);
-        cw.cntO = __popcll(cw.AOn);
-        cw.cntE = __popcll(cw.AEn);
-        cw.c0 = c0;
-        cw.phin = psin / c0;
-        cw.inv_psin = inv_psin;
-        cw.inv_psin_f = inv_psin_f;
-        units = S.unit_off[8];
-        if (threadIdx.x == 0) cs.cw = cw;
+// the screen's scale of a walker whose best clock is at most `bound`: a neighbour of rate Gamma =
+// |t / psi_n| can win only if w = 1 - u < -expm1(-Gamma bound) <= Gamma bound, i.e. if the top 32
+// bits of w, as an integer, are below |t| x this scale.  The factor 1.0001 covers the FP32 roundings,
+// the floor keeps the scale in the normal range (a larger scale only lets more through).
+__device__ __forceinline__ float race_scale(float bound, float inv_f) {
+    return fmaxf(bound * inv_f * 1.0001f * 4294967296.0f, 1e-30f);
+}
+
+// the screen on the top 32 bits x of the draw (gf: FP32 rate, or |t| when the scale holds 1/psi_n;
+// negative: no neighbour, INFINITY: a rate FP32 cannot carry)
+__device__ __forceinline__ bool race_pass(unsigned x, float gf, float scale) { return (float)(~x) <= gf * scale; }
+
+__device__ __forceinline__ uint4 race_walker_words(unsigned long long seed, unsigned step, unsigned wid) {
+    const unsigned kx = (unsigned)seed, ky = (unsigned)(seed >> 32);
+    const unsigned x1 = __umulhi(PHILOX_M1, wid) ^ step ^ kx, y1 = PHILOX_M1 * wid;      // round 1
+    uint4 r;
+    r.x = y1 ^ (kx + PHILOX_W0);                                                         // round 2
+    r.y = __umulhi(PHILOX_M0, x1) ^ (ky + PHILOX_W1);
+    r.z = PHILOX_M0 * x1;
+    r.w = 0u;
+    return r;
+}
+
+__device__ __forceinline__ bool atomic_cas128(RaceBest* at, const RaceBest& cmp, const RaceBest& val, RaceBest& old) {
+    const unsigned long long c0 = (unsigned long long)cmp.clk | ((unsigned long long)cmp.exc << 32);
+    const unsigned long long v0 = (unsigned long long)val.clk | ((unsigned long long)val.exc << 32);
+    const unsigned long long c1 = (unsigned long long)__double_as_longlong(cmp.t);
+    const unsigned long long v1 = (unsigned long long)__double_as_longlong(val.t);
+    unsigned long long o0, o1;
+    asm volatile("{\n\t.reg .b128 c, v, d;\n\t"
+                 "mov.b128 c, {%2, %3};\n\tmov.b128 v, {%4, %5};\n\t"
+                 "atom.global.cas.b128 d, [%6], c, v;\n\t"
+                 "mov.b128 {%0, %1}, d;\n\t}"
+                 : "=l"(o0), "=l"(o1)
+                 : "l"(c0), "l"(c1), "l"(v0), "l"(v1), "l"(at)
+                 : "memory");
+    old.clk = (unsigned)o0;
+    old.exc = (unsigned)(o0 >> 32);
+    old.t = __longlong_as_double((long long)o1);
+    return o0 == c0 && o1 == c1;
+}
+
+// whether two FP32 clocks (relative error below 1e-5) leave the order of the exact ones open
+__device__ __forceinline__ bool clocks_near(float a, float b) { return !(a < b * 0.9999f) && !(b < a * 0.9999f); }
+
+// Lanes whose neighbour passed walker j's screen: of those that also pass the closer screen
+// (race_may_win) take the smallest clock, settle near ties by
+// the exact FP64 clocks (then the smaller excitation), and replace the walker's best if it is beaten.
+// Runs a handful of times per walker and step.
+__device__ __noinline__ void race_slow(WarpTask& wt, RaceBest* best, unsigned* bound, int j, double t, unsigned exc,
+                                       bool pass, int lane) {
+    const unsigned long long seed = wt.sys.seed;
+    const unsigned step = wt.step[j], wid = wt.wid[j];
+    const unsigned long long k = race_bits(seed, exc, step, wid);
+    const double g = fabs(t * wt.inv_psin);
+    const float gf = abs_f32_of(g);
+    const bool ok = pass && g > 0.0 && race_may_win(k, gf, wt.bnd[j]);
+    float a = INFINITY;
+    if (ok) {
+        const float w = (float)(9007199254740991ull - k) * 1.1102230246251565e-16f;
+        if (gf > 0.0f) a = (w > 0.5f ? -logf((float)(k + 1) * 1.1102230246251565e-16f) : -log1pf(-w)) / gf;
+        else a = (float)race_clock_f64(k, g);
     }
-    // the walker's single-excitation operator G_yx(n) = h_yx + sum_{j in n} [(yx|jj) - delta (yj|jx)]
-    // for y in core + active, x in active + virtual (not both active), by the whole block: the
-    // full-core operator hc, n's active electrons, minus n's core holes, plus its virtual electrons
-    if (psin != 0.0) {
-        const unsigned ao0 = active_bits<W>(S, n[0]), ao1 = active_bits<W>(S, n[1]);
-        const unsigned long long AOn = (unsigned long long)ao0 | ((unsigned long long)ao1 << 32);
-        int nh = 0, np = 0, hso[2] = {0, 0}, pso[2] = {0, 0};
-        if (!cas) {
+    float amin = a;
 #pragma unroll
-            for (int sg = 0; sg < 2; sg++) {
-                unsigned long long hm = ~(sg ? n[1][0] : n[0][0]) & S.mcore[0];
-                while (hm) {
-                    const int i = __ffsll(hm) - 1;
-                    hm &= hm - 1;
-                    if (nh == 0) hso[0] = sg * S.n + i;
-                    else hso[1] = sg * S.n + i;
-                    nh++;
-                }
+    for (int o = 16; o > 0; o >>= 1) amin = fminf(amin, __shfl_xor_sync(0xffffffffu, amin, o));
+    unsigned near = __ballot_sync(0xffffffffu, ok && !(amin < a * 0.9999f));
+    if (near == 0u) return;
+    int src = __ffs(near) - 1;
+    if (near & (near - 1u)) {
+        double tc = INFINITY;
+        unsigned e = 0xFFFFFFFFu;
+        if (near >> lane & 1u) {
+            tc = race_clock_f64(k, g);
+            e = exc;
+        }
+        double tm = tc;
+        unsigned em = e;
 #pragma unroll
-                for (int w = 0; w < W; w++) {
-                    unsigned long long pm = (sg ? n[1][w] : n[0][w]) & S.mvirt[w];
-                    while (pm) {
-                        const int a = 64 * w + __ffsll(pm) - 1;
-                        pm &= pm - 1;
-                        if (np == 0) pso[0] = sg * S.n + a;
-                        else pso[1] = sg * S.n + a;
-                        np++;
-                    }
-                }
+        for (int o = 16; o > 0; o >>= 1) {
+            const double t2 = __shfl_xor_sync(0xffffffffu, tm, o);
+            const unsigned e2 = __shfl_xor_sync(0xffffffffu, em, o);
+            if (t2 < tm || (t2 == tm && e2 < em)) {
+                tm = t2;
+                em = e2;
             }
         }
-        const int blk = S.nca * S.nav;
-        for (int t = threadIdx.x; t < 2 * blk; t += blockDim.x) {
-            const int sg = t >= blk, rem = t - sg * blk;
-            const int y = rem / S.nav, xo = rem - y * S.nav, x = S.nc + xo;
-            if (y >= S.nc && xo < S.na) continue;
-            ctr.g();
-            double v = __ldg(S.hc + y * S.n + x);
-            unsigned long long bits = AOn;
-            while (bits) {
-                const int b = __ffsll(bits) - 1;
-                bits &= bits - 1;
-                const int j = S.nc + (b & 31);
-                v += eri_g(S, y, x, j, j);
-                ctr.g();
-                if ((b >= 32) == (sg == 1)) {
-                    v -= eri_g(S, y, j, j, x);
-                    ctr.g();
+        src = __ffs(__ballot_sync(0xffffffffu, (near >> lane & 1u) && tc == tm && e == em)) - 1;
+        if (src < 0) src = __ffs(near) - 1;
+    }
+    float b = 0.0f;
+    if (lane == src) {
+        RaceBest mine, cur, old;
+        mine.clk = __float_as_uint(a);
+        mine.exc = exc;
+        mine.t = t;
+        const int slot = (int)wt.slot[j];
+        RaceBest* at = best + slot;
+        {
+            unsigned lo, hi;
+            asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(cur.clk), "=r"(cur.exc), "=r"(lo), "=r"(hi)
+                         : "l"(at));
+            cur.t = __hiloint2double((int)hi, (int)lo);
+        }
+        for (;;) {                                      // every turn but the last, another warp's candidate won
+            bool better = cur.exc == 0xFFFFFFFFu;
+            if (!better) {
+                const float ca = __uint_as_float(cur.clk);
+                if (!clocks_near(a, ca)) better = a < ca;
+                else {
+                    const double tm = race_clock_f64(k, g);
+                    const double tb = race_clock_f64(race_bits(seed, cur.exc, step, wid), fabs(cur.t * wt.inv_psin));
+                    better = tm < tb || (tm == tb && exc < cur.exc);
                 }
             }
+            if (!better) break;
+            if (atomic_cas128(at, cur, mine, old)) break;
+            cur = old;
+        }
+        const float up = a * 1.0001f;
+        b = fminf(up, __uint_as_float(atomicMin(bound + slot, __float_as_uint(up))));
+    }
+    b = __shfl_sync(0xffffffffu, b, src);
+    if (lane == 0) {
+        wt.bnd[j] = b;
+        wt.wp[j].w = __float_as_uint(race_scale(b, wt.inv_f));
+    }
+    __syncwarp();
+}
+
+// 32 neighbours (one per lane; t = 0: none) against the clocks of the task's walkers.  Bound by the
+// integer pipe: about 45 instructions per neighbour and walker.
+__device__ __noinline__ void race_round(WarpTask& wt, RaceBest* best, unsigned* bound, double t, unsigned exc, int count,
+                                        int lane) {
+    float gf = -1.0f;                                   // t = 0 never passes
+    if ((__double_as_longlong(t) << 1) != 0) {
+        gf = abs_f32_of(t);
+        if (gf == 0.0f) gf = INFINITY;                  // outside FP32: the exact clock decides
+    }
+    const unsigned kx = (unsigned)wt.sys.seed, ky = (unsigned)(wt.sys.seed >> 32);
+    const unsigned z1 = __umulhi(PHILOX_M0, exc) ^ ky, w1 = PHILOX_M0 * exc;
+    const unsigned e1 = __umulhi(PHILOX_M1, z1), e2 = PHILOX_M1 * z1;
+    for (int j = 0; j < count; j++) {
+        const uint4 a = wt.wp[j];
+        unsigned c0 = e1 ^ a.x, c1 = e2, c2 = w1 ^ a.y, c3 = a.z;
 #pragma unroll
-            for (int k = 0; k < 2; k++) {
-                if (k < nh) {
-                    v -= g_corr(S, sg, x, y, hso[k]);
-                    ctr.g(2);
-                }
-                if (k < np) {
-                    v += g_corr(S, sg, x, y, pso[k]);
-                    ctr.g(2);
-                }
+        for (int r = 2; r < 9; r++) {
+            const unsigned long long p0 = (unsigned long long)PHILOX_M0 * c0, p1 = (unsigned long long)PHILOX_M1 * c2;
+            c0 = (unsigned)(p1 >> 32) ^ c1 ^ (kx + (unsigned)r * PHILOX_W0);
+            c1 = (unsigned)p1;
+            c2 = (unsigned)(p0 >> 32) ^ c3 ^ (ky + (unsigned)r * PHILOX_W1);
+            c3 = (unsigned)p0;
+        }
+        const unsigned x = __umulhi(PHILOX_M1, c2) ^ c1 ^ (kx + 9u * PHILOX_W0);
+        const bool pass = race_pass(x, gf, __uint_as_float(a.w));
+        if (__any_sync(0xffffffffu, pass)) race_slow(wt, best, bound, j, t, exc, pass, lane);
+    }
+}
+
+// neighbours of a walk step: queued so that the sums and the race run with full lanes
+struct StepSink {
+    WarpTask& wt;
+    RaceBest* best;
+    unsigned* bound;
+    int count, lane;
+    double sA, sT, sD;        // sum |t|, sum t, sum t_D   (t = H_nm psi_s(m), t_D = (H_D)_nm psi_s(m))
+    template <int W>
+    __device__ __forceinline__ void post(bool valid, int, const unsigned long long (&)[2][W], double hnm, double hd,
+                                         double, double psim, unsigned exc) {
+        const double t = hnm * psim;
+        const bool on = valid && (__double_as_longlong(t) << 1) != 0;
+        if (on) sD += hd * psim;
+        const unsigned m = __ballot_sync(0xffffffffu, on);
+        int qn = wt.qn;
+        if (on) {
+            const int at = qn + __popc(m & ((1u << lane) - 1u));
+            wt.qt[at] = t;
+            wt.qe[at] = exc;
+        }
+        qn += __popc(m);
+        __syncwarp();
+        if (qn >= 32) {
+            take(wt.qt[lane], wt.qe[lane]);
+            qn -= 32;
+            const double t2 = wt.qt[32 + lane];
+            const unsigned e2 = wt.qe[32 + lane];
+            __syncwarp();
+            if (lane < qn) {
+                wt.qt[lane] = t2;
+                wt.qe[lane] = e2;
             }
-            gops[t] = v;
+        }
+        if (lane == 0) wt.qn = qn;
+        __syncwarp();
+    }
+    __device__ __forceinline__ void take(double t, unsigned exc) {
+        sA += fabs(t);
+        sT += t;
+        race_round(wt, best, bound, t, exc, count, lane);
+    }
+    __device__ __forceinline__ void finish() {
+        const int qn = wt.qn;
+        if (qn > 0) take(lane < qn ? wt.qt[lane] : 0.0, lane < qn ? wt.qe[lane] : 0u);
+    }
+};
+
+// the debug evaluation's neighbours: sums, and records when asked for
+struct DebugSink {
+    mrq_neighbour* nbout;
+    long long nbase, max_nb;
+    double inv_psin;
+    double sA, sT, sD;
+    template <int W>
+    __device__ __forceinline__ void post(bool valid, int ri, const unsigned long long (&m)[2][W], double hnm, double hd,
+                                         double om, double psim, unsigned exc) {
+        if (!valid) return;
+        const double t = hnm * psim;
+        sA += fabs(t);
+        sT += t;
+        sD += hd * psim;
+        if (nbout != nullptr && nbase + ri < max_nb) {
+            unsigned long long w4[4];
+            det_words<W>(m, w4);
+            write_rec(nbout + nbase + ri, w4, W, hnm, hd, om, psim, fabs(t * inv_psin), exc);
         }
     }
+};
+
+// ------------------------------------------------------------------ kernels of a walk step
+
+template <int W>
+__device__ __forceinline__ void load_det(const Walker* w, unsigned long long (&n)[2][W]) {
+#pragma unroll
+    for (int sg = 0; sg < 2; sg++)
+#pragma unroll
+        for (int k = 0; k < W; k++) n[sg][k] = w->d[sg][k];
+}
+
+__device__ __forceinline__ void copy_sys(SysDev* dst, const SysDev* src, int t, int nt) {
+    for (int k = t; k < (int)(sizeof(SysDev) / sizeof(int)); k += nt)
+        reinterpret_cast<int*>(dst)[k] = reinterpret_cast<const int*>(src)[k];
+}
+
+// Distinct determinants of the walkers of system blockIdx.x (slots of the segment), by one block: an
+// open-addressing table whose entries hold the first walker seen on a determinant (full determinants
+// are compared, so a hash collision costs a probe only).  The table has at least twice as many entries
+// as walkers, so a probe always ends.  Task groups and members come out in no fixed order; nothing
+// computed from them depends on it.
+template <int W>
+__global__ void __launch_bounds__(1024) k_group(const WalkSet ws, const WalkScratch sc) {
+    const int sys = blockIdx.x;
+    const long long off = ws.offsets[sys];
+    const long long lo = max(off, sc.seg0) - off, hi = min(ws.offsets[sys + 1], sc.seg1) - off;
+    const int n = (int)max(0LL, hi - lo);
+    const Walker* const wk = ws.walkers[sys] + lo;
+    const int base = (int)(off + lo - sc.seg0);          // first slot of the system in the segment
+    __shared__ int s_members;
     if (threadIdx.x == 0) {
+        s_members = 0;
+        if (gridDim.x == 1) sc.ctl[0] = sc.ctl[1] = sc.ctl[2] = 0;
+    }
+    int tsz = 2;
+    while (tsz < 2 * n) tsz <<= 1;
+    int* const rep = sc.rep + 4LL * base;
+    int* const cnt = sc.cnt + 4LL * base;
+    int* const start = sc.start + 4LL * base;
+    if (n > 0)
+        for (int k = threadIdx.x; k < tsz; k += blockDim.x) {
+            rep[k] = -1;
+            cnt[k] = 0;
+        }
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        unsigned long long d[2][W];
+        load_det<W>(wk + i, d);
+        unsigned long long hh = 0;
 #pragma unroll
         for (int sg = 0; sg < 2; sg++)
 #pragma unroll
-            for (int w = 0; w < W; w++) cs.nsh[sg * W + w] = n[sg][w];
-    }
-    const unsigned long long(&nsh)[2][W] = *reinterpret_cast<const unsigned long long(*)[2][W]>(cs.nsh);
-    __syncthreads();
-    ctr.mark(0);
-    const int total_fois = cas ? 0 : cs.L.bstart[cs.L.nb];
-    if (!cas) units = (total_fois + MRQ_FOIS_CH - 1) / MRQ_FOIS_CH;
-    // neighbour offsets of the units (debug records only)
-    if (MODE == MODE_DEBUG && nbout != nullptr && cas) {
-        for (int u = threadIdx.x; u < units; u += blockDim.x) nb_prefix[u] = cas_unit_count(S, cw, u);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            long long run = 0;
-            for (int u = 0; u < units; u++) {
-                const long long c = nb_prefix[u];
-                nb_prefix[u] = run;
-                run += c;
-            }
-        }
-        __syncthreads();
-    }
-    LaneAcc2 acc;
-    acc2_init(acc);
-    const unsigned long long self_key =
-        ln == 0 ? hash_key(S, active_bits<W>(S, n[0]), active_bits<W>(S, n[1])) : MRQ_EMPTY_KEY;
-    const double phi_self = ln == 0 ? psin / c0 : 0.0;
-    // MRQ_VW virtual warps: virtual warp v owns units v, v + MRQ_VW, ...; warp wi runs virtual warps
-    // wi, wi + nw, ... one after the other and stores each one's sums.  The sums (and so S, E_L and
-    // the numerator) are then the same whatever the number of warps per walker.
-    for (int vw = wi; vw < MRQ_VW; vw += nw) {
-        acc.sA = acc.sT = acc.sD = 0.0;
-        for (int u = vw; u < units; u += MRQ_VW) {
-            if (cas) {
-                const long long nbase = (MODE == MODE_DEBUG && nbout != nullptr) ? nb_prefix[u] : 0;
-                if (u < S.cas_units) {
-                    acc = cas_internal_unit<W, MODE>(S, cs.cw, nsh, u, acc, step, wid, lane, nbout, nbase, max_nb, ctr);
-                    ctr.mark(1);
-                } else {
-                    cas_pair_unit<W, MODE>(S, cs.cw, gops, cphi, ccode, nsh, u, acc, step, wid, lane, nbout, nbase,
-                                           max_nb, ctr);
-                    ctr.mark(2);
-                }
-            } else {
-                const int i0 = u * MRQ_FOIS_CH, i1 = min(total_fois, i0 + MRQ_FOIS_CH);
-                acc = fois_unit<W, MODE>(S, cs.L, psin != 0.0 ? gops : nullptr, nsh, ln, c0, inv_psin, inv_psin_f,
-                                         self_key, phi_self, i0, i1, acc, step, wid, lane, nbout, 0, max_nb, ctr);
-                ctr.mark(7);
-            }
-        }
-        const double sA = warp_sum(acc.sA), sT = warp_sum(acc.sT), sD = warp_sum(acc.sD);
-        if (lane == 0) {
-            cs.wsum[0][vw] = sA;
-            cs.wsum[1][vw] = sT;
-            cs.wsum[2][vw] = sD;
-        }
-    }
-    // the race's winner: smallest clock, then smallest excitation id (order-independent)
-    {
-        const double bt_me = cs.rbt[threadIdx.x];
-        const unsigned be_me = cs.rbexc[threadIdx.x];
-        double t = bt_me;
-        unsigned e = be_me;
+            for (int w = 0; w < W; w++) hh = mix64(hh ^ d[sg][w]);
+        int k = (int)(hh & (unsigned long long)(tsz - 1));
+        for (int probe = 0; probe < tsz; probe++) {
+            const int prev = atomicCAS(rep + k, -1, i);
+            bool same = prev < 0 || prev == i;
+            if (!same) {
+                unsigned long long o[2][W];
+                load_det<W>(wk + prev, o);
+                same = true;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double t2 = __shfl_xor_sync(0xffffffffu, t, o);
-            const unsigned e2 = __shfl_xor_sync(0xffffffffu, e, o);
-            if (t2 < t || (t2 == t && e2 < e)) {
-                t = t2;
-                e = e2;
+                for (int sg = 0; sg < 2; sg++)
+#pragma unroll
+                    for (int w = 0; w < W; w++) same = same && o[sg][w] == d[sg][w];
             }
+            if (same) break;
+            k = (k + 1) & (tsz - 1);
         }
-        const unsigned win = __ballot_sync(0xffffffffu, be_me == e && bt_me == t);
-        const int src = win ? __ffs(win) - 1 : 0;
-        const double bpsi = cs.rbpsi[(threadIdx.x & ~31u) + src];
-        if (lane == 0) {
-            cs.wbt[wi] = t;
-            cs.wbexc[wi] = e;
-            cs.wbpsi[wi] = bpsi;
-        }
+        sc.tab_of[base + i] = k;
+        sc.pos_of[base + i] = atomicAdd(cnt + k, 1);
     }
-    ctr_flush(cs, ctr, lane);
-    if (wi == 0) {
-        double hnn, hdnn;
-        diagonals<W>(S, cs.L, n, lane, hnn, hdnn);
-        if (lane == 0) {
-            cs.hnn = hnn;
-            cs.hdnn = hdnn;
+    __syncthreads();
+    for (int k = threadIdx.x; k < (n > 0 ? tsz : 0); k += blockDim.x) {
+        const int c = cnt[k];
+        if (c == 0) continue;
+        const int st = atomicAdd(&s_members, c);
+        start[k] = st;
+        const int ntg = (c + sc.tgw - 1) / sc.tgw;
+        const int at = atomicAdd(sc.ctl + 0, ntg), grp = atomicAdd(sc.ctl + 1, 1);
+        for (int q = 0; q < ntg; q++) {
+            TaskGroup t;
+            t.sys = sys;
+            t.first = base + st + q * sc.tgw;
+            t.count = min(sc.tgw, c - q * sc.tgw);
+            t.group = grp;
+            t.primary = q == 0;
+            t.pad = 0;
+            sc.tg[at + q] = t;
         }
     }
     __syncthreads();
-    ctr.mark(8);
-    StepOut o;
-    double A = 0.0, T = 0.0, D = 0.0, bt = INFINITY, bpsi = 0.0;
-    unsigned be = 0xFFFFFFFFu;
-    for (int k = 0; k < MRQ_VW; k++) {
-        A += cs.wsum[0][k];
-        T += cs.wsum[1][k];
-        D += cs.wsum[2][k];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        sc.members[base + start[sc.tab_of[base + i]] + sc.pos_of[base + i]] = (int)lo + i;
+        RaceBest b;
+        b.clk = 0x7F800000u;
+        b.exc = 0xFFFFFFFFu;
+        b.t = 0.0;
+        sc.best[base + i] = b;
+        sc.bound[base + i] = 0x7F800000u;
     }
-    for (int k = 0; k < nw; k++) {
-        if (cs.wbt[k] < bt || (cs.wbt[k] == bt && cs.wbexc[k] < be)) {
-            bt = cs.wbt[k];
-            be = cs.wbexc[k];
-            bpsi = cs.wbpsi[k];
+}
+
+// Constants of every distinct determinant, one block each: label, diagonals, single-excitation operator
+template <int W>
+__global__ void __launch_bounds__(128) k_prep(const WalkSet ws, const WalkScratch sc) {
+    __shared__ SysDev S;
+    __shared__ WarpLists lists;
+    int cur = -1;
+    const int ntg = sc.ctl[0];
+    for (int g = blockIdx.x; g < ntg; g += gridDim.x) {
+        const TaskGroup tg = sc.tg[g];
+        if (!tg.primary) continue;
+        __syncthreads();
+        if (tg.sys != cur) {
+            copy_sys(&S, ws.systems + tg.sys, threadIdx.x, blockDim.x);
+            cur = tg.sys;
+            __syncthreads();
+        }
+        const Walker* const wk = ws.walkers[tg.sys] + sc.members[tg.first];
+        unsigned long long n[2][W];
+        load_det<W>(wk, n);
+        int h, p;
+        const long long ln = det_label<W>(S, n, h, p);
+        if (threadIdx.x < 32 && ln >= 0) {
+            double hnn, hdnn;
+            build_lists<W>(S, n, lists, h, p, threadIdx.x);
+            diagonals<W>(S, lists, n, threadIdx.x, hnn, hdnn);
+            if (threadIdx.x == 0) {
+                GroupMeta m;
+                m.d[0][0] = m.d[0][1] = m.d[1][0] = m.d[1][1] = 0;
+#pragma unroll
+                for (int sg = 0; sg < 2; sg++)
+#pragma unroll
+                    for (int w = 0; w < W; w++) m.d[sg][w] = n[sg][w];
+                m.psi = wk->psi;
+                m.hnn = hnn;
+                m.hdnn = hdnn;
+                m.label = ln;
+                m.h = h;
+                m.p = p;
+                sc.meta[tg.group] = m;
+            }
+        } else if (threadIdx.x == 0) {
+            sc.meta[tg.group].label = -1;
+        }
+        NoCtr ctr;
+        if (ln >= 0 && wk->psi != 0.0) walker_operator<W>(S, n, ln == 0, sc.gops + (long long)tg.group * sc.gstride, ctr);
+    }
+}
+
+// Work units of every task group, as warp tasks (task group, slice): slice s of a determinant owns
+// units s, s + nslice, ...  Warps take tasks from a counter, so long and short tasks level out; the
+// slices of one determinant run all over the chip.
+template <int W, int MINB>
+__global__ void __launch_bounds__(MRQ_MAXNW * 32, MINB) k_eval(const WalkSet ws, const WalkScratch sc, int wbytes, int cap) {
+    extern __shared__ __align__(16) unsigned char smem_dyn[];
+    const int lane = threadIdx.x & 31;
+    unsigned char* const mine = smem_dyn + (size_t)(threadIdx.x >> 5) * wbytes;
+    WarpTask& wt = *reinterpret_cast<WarpTask*>(mine);
+    WarpLists& lists = *reinterpret_cast<WarpLists*>(mine + (sizeof(WarpTask) + 15) / 16 * 16);
+    double* const cphi = reinterpret_cast<double*>(&lists);      // CAS tasks: candidate list in the lists' place
+    unsigned* const ccode = reinterpret_cast<unsigned*>(cphi + cap);
+    const SysDev& S = wt.sys;
+    int cur = -1;
+    const int ntg = sc.ctl[0];
+    const long long ntask = (long long)ntg * sc.ns_max;
+    NoCtr ctr;
+    for (;;) {
+        int id = 0;
+        if (lane == 0) id = atomicAdd(sc.ctl + 2, 1);
+        id = __shfl_sync(0xffffffffu, id, 0);
+        if (id >= ntask) break;
+        const int slice = id / ntg, g = id - slice * ntg;
+        const TaskGroup tg = sc.tg[g];
+        __syncwarp();
+        if (tg.sys != cur) {
+            copy_sys(&wt.sys, ws.systems + tg.sys, lane, 32);
+            cur = tg.sys;
+            __syncwarp();
+        }
+        if (slice >= S.nslice) continue;
+        const GroupMeta* const meta = sc.meta + tg.group;
+        const long long ln = meta->label;
+        const double psin = meta->psi;
+        double* const part = sc.part + ((long long)tg.group * sc.ns_max + slice) * 3;
+        if (ln < 0 || !(psin != 0.0)) {
+            if (lane < 3 && tg.primary) part[lane] = 0.0;
+            continue;
+        }
+        unsigned long long(&n)[2][W] = *reinterpret_cast<unsigned long long(*)[2][W]>(wt.nsh);
+        if (lane == 0) {
+#pragma unroll
+            for (int sg = 0; sg < 2; sg++)
+#pragma unroll
+                for (int w = 0; w < W; w++) n[sg][w] = meta->d[sg][w];
+        }
+        __syncwarp();
+        const float inv_f = abs_f32_of(1.0 / psin);
+        if (lane < tg.count) {
+            const int i = sc.members[tg.first + lane];
+            const Walker* const wk = ws.walkers[tg.sys] + i;
+            const int slot = (int)(ws.offsets[tg.sys] + i - sc.seg0);
+            const unsigned step = wk->step, wid = wk->wid;
+            uint4 a = race_walker_words(S.seed, step, wid);
+            const float b = __uint_as_float(__ldcg(sc.bound + slot));
+            a.w = __float_as_uint(race_scale(b, inv_f > 0.0f ? inv_f : INFINITY));
+            wt.bnd[lane] = b;
+            wt.wp[lane] = a;
+            wt.wid[lane] = wid;
+            wt.step[lane] = step;
+            wt.slot[lane] = (unsigned)slot;
+        }
+        if (lane == 0) {
+            wt.inv_psin = 1.0 / psin;
+            wt.inv_f = inv_f > 0.0f ? inv_f : INFINITY;
+            wt.qn = 0;
+            if (ln == 0) wt.cw = cas_constants<W>(S, n, psin);
+        }
+        __syncwarp();
+        StepSink sink{wt, sc.best, sc.bound, tg.count, lane, 0.0, 0.0, 0.0};
+        const double* const gops = sc.gops + (long long)tg.group * sc.gstride;
+        if (ln == 0) {
+            const int units = S.unit_off[8];
+            for (int u = slice; u < units; u += S.nslice) {
+                if (u < S.cas_units) cas_internal_unit<W>(S, wt.cw, n, u, lane, sink, ctr);
+                else cas_pair_unit<W>(S, wt.cw, gops, cphi, ccode, n, u, lane, sink, ctr);
+            }
+        } else {
+            build_lists<W>(S, n, lists, meta->h, meta->p, lane);
+            const int total = lists.bstart[lists.nb], units = (total + MRQ_FOIS_CH - 1) / MRQ_FOIS_CH;
+            for (int u = slice; u < units; u += S.nslice)
+                fois_unit<W>(S, lists, gops, n, ln, __ldg(S.c), MRQ_EMPTY_KEY, 0.0, u * MRQ_FOIS_CH,
+                             min(total, (u + 1) * MRQ_FOIS_CH), lane, sink, ctr);
+        }
+        sink.finish();
+        const double sA = warp_sum(sink.sA), sT = warp_sum(sink.sT), sD = warp_sum(sink.sD);
+        if (lane == 0 && tg.primary) {
+            part[0] = sA;
+            part[1] = sT;
+            part[2] = sD;
         }
     }
-    o.S = fabs(inv_psin) * A;
-    o.hnn = cs.hnn;
-    o.hdnn = cs.hdnn;
-    o.EL = o.hnn + inv_psin * T;
-    o.num = ln > 0 ? o.hdnn + inv_psin * D : 0.0;
-    o.nnb = cas ? (long long)S.cas_nb_total : (long long)total_fois;
-    o.bexc = be;
-    o.bpsi = bpsi;
-    return o;
 }
 
 // apply the excitation code of the race's winner to n
@@ -907,70 +1225,86 @@ __device__ __forceinline__ void apply_code(unsigned long long (&m)[2][W], const 
     }
 }
 
-// One walker step per block: slot blockIdx.x (or order[blockIdx.x]) of the walk set.  The step's
-// contribution goes into the walker's record; k_accum adds the records into the accumulators.
-template <int W, int MINB>
-__global__ void __launch_bounds__(MRQ_MAXNW * 32, MINB) k_walk2(const WalkSet ws, const unsigned* __restrict__ order,
-                                                             int accumulate) {
+// The step's end, one warp per task group: the determinant's sums over its slices (in slice order
+// within a lane, then a fixed tree), each walker's record (k_accum adds them) and move, and psi_s at
+// the new determinant - a function of that determinant alone, so that walkers that meet on it agree
+// bit for bit.
+template <int W>
+__global__ void __launch_bounds__(MRQ_MAXNW * 32) k_move(const WalkSet ws, const WalkScratch sc, int accumulate, int lbytes,
+                                                         int cap) {
     extern __shared__ __align__(16) unsigned char smem_dyn[];
-    CtaSh& cs = *reinterpret_cast<CtaSh*>(smem_dyn);
-    unsigned char* lists = smem_dyn + (sizeof(CtaSh) + 15) / 16 * 16;
-    const long long s0 = blockIdx.x;
-    if (s0 >= ws.nslots) return;
-    const long long slot = order ? (long long)order[s0] : s0;
-    int sys;
-    long long local;
-    slot_owner(ws, slot, sys, local);
-    Walker* const walkers = ws.walkers[sys];
-    {
-        const int* src = reinterpret_cast<const int*>(ws.systems + sys);
-        int* dst = reinterpret_cast<int*>(&cs.L.sys);
-        for (int k = threadIdx.x; k < (int)(sizeof(SysDev) / sizeof(int)); k += blockDim.x) dst[k] = src[k];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    double* const cphi = reinterpret_cast<double*>(smem_dyn + (size_t)warp * lbytes);
+    unsigned* const ccode = reinterpret_cast<unsigned*>(cphi + cap);
+    const int ntg = sc.ctl[0];
+    for (int g = blockIdx.x * nw + warp; g < ntg; g += gridDim.x * nw) {
+        const TaskGroup tg = sc.tg[g];
+        const SysDev& S = ws.systems[tg.sys];
+        const GroupMeta meta = sc.meta[tg.group];
+        const double inv_psin = meta.psi != 0.0 ? 1.0 / meta.psi : 0.0;
+        double A = 0.0, T = 0.0, D = 0.0;
+        const double* const part = sc.part + (long long)tg.group * sc.ns_max * 3;
+        for (int k = lane; k < S.nslice; k += 32) {
+            A += part[3 * k];
+            T += part[3 * k + 1];
+            D += part[3 * k + 2];
+        }
+        A = warp_sum(A);
+        T = warp_sum(T);
+        D = warp_sum(D);
+        const double rate = fabs(inv_psin) * A;
+        unsigned long long m[2][W];
+#pragma unroll
+        for (int sg = 0; sg < 2; sg++)
+#pragma unroll
+            for (int w = 0; w < W; w++) m[sg][w] = meta.d[sg][w];
+        Walker* wk = nullptr;
+        bool moved = false;
+        long long lm = 0;
+        if (lane < tg.count) {
+            const int i = sc.members[tg.first + lane];
+            wk = ws.walkers[tg.sys] + i;
+            wk->rl = -1;
+            const RaceBest b = sc.best[ws.offsets[tg.sys] + i - sc.seg0];
+            if (meta.label < 0 || !(rate > 0.0) || b.exc == 0xFFFFFFFFu) {
+                atomicOr(S.err, meta.label < 0 ? MRQ_ERR_LABEL : MRQ_ERR_NOMOVE);
+            } else {
+                moved = true;
+                if (accumulate && (long long)wk->step >= S.burn_in) {
+                    wk->rl = meta.label;
+                    wk->rtype = 3 * meta.h + meta.p;
+                    wk->rw = 1.0 / rate;
+                    wk->rEL = meta.hnn + inv_psin * T;
+                    wk->rnum = meta.label > 0 ? meta.hdnn + inv_psin * D : 0.0;
+                }
+                apply_code<W>(m, S, b.exc);
+                int h, p;
+                lm = det_label<W>(S, m, h, p);
+            }
+        }
+        double psi = 0.0;
+        if (moved && lm == 0) psi = __ldg(S.c) * hash_lookup(S, hash_key(S, active_bits<W>(S, m[0]), active_bits<W>(S, m[1])));
+        unsigned todo = __ballot_sync(0xffffffffu, moved && lm > 0);
+        while (todo) {
+            const int src = __ffs(todo) - 1;
+            todo &= todo - 1;
+            unsigned long long x[2][W];
+#pragma unroll
+            for (int sg = 0; sg < 2; sg++)
+#pragma unroll
+                for (int w = 0; w < W; w++) x[sg][w] = __shfl_sync(0xffffffffu, m[sg][w], src);
+            const double o = reach_back_warp<W>(S, x, cphi, ccode, lane);
+            if (lane == src) psi = __ldg(S.c + lm) * o;
+        }
+        if (moved) {
+#pragma unroll
+            for (int sg = 0; sg < 2; sg++)
+#pragma unroll
+                for (int w = 0; w < W; w++) wk->d[sg][w] = m[sg][w];
+            wk->psi = psi;
+            wk->step++;
+        }
     }
-    __syncthreads();
-    const SysDev& S = cs.L.sys;
-    Walker wk = walkers[local];
-    unsigned long long n[2][W];
-#pragma unroll
-    for (int sg = 0; sg < 2; sg++)
-#pragma unroll
-        for (int w = 0; w < W; w++) n[sg][w] = wk.d[sg][w];
-    int h, p;
-    const long long ln = det_label<W>(S, n, h, p);
-#ifdef MRQ_PHASE_TIMING
-    PhCtr nc;
-    nc.mark(9);
-#else
-    NoCtr nc;
-#endif
-    StepOut o;
-    if (ln >= 0) o = block_local<W, MODE_STEP>(cs, lists, n, wk.psi, ln, h, p, wk.step, wk.wid, nullptr, 0, nullptr, nc);
-#ifdef MRQ_PHASE_TIMING
-    if ((threadIdx.x & 31) == 0)
-        for (int k = 0; k < 10; k++) atomicAdd(&g_phase[k], (unsigned long long)nc.acc[k]);
-#endif
-    if (threadIdx.x != 0) return;
-    wk.rl = -1;
-    if (ln < 0 || !(o.S > 0.0) || o.bexc == 0xFFFFFFFFu) {
-        atomicOr(S.err, ln < 0 ? MRQ_ERR_LABEL : MRQ_ERR_NOMOVE);
-        walkers[local] = wk;
-        return;
-    }
-    if (accumulate && (long long)wk.step >= S.burn_in) {
-        wk.rl = ln;
-        wk.rtype = 3 * h + p;
-        wk.rw = 1.0 / o.S;
-        wk.rEL = o.EL;
-        wk.rnum = o.num;
-    }
-    apply_code<W>(n, S, o.bexc);
-#pragma unroll
-    for (int sg = 0; sg < 2; sg++)
-#pragma unroll
-        for (int w = 0; w < W; w++) wk.d[sg][w] = n[sg][w];
-    wk.psi = o.bpsi;
-    wk.step++;
-    walkers[local] = wk;
 }
 
 // Accumulate the last step's walker records (Eq. 12, Eq. 16; weight w = 1/S): one warp per
@@ -1038,7 +1372,29 @@ __global__ void __launch_bounds__(1024) k_accum(const WalkSet ws) {
     }
 }
 
-// local quantities of arbitrary determinants (parity): one block per determinant, the walk's code
+// ------------------------------------------------------------------ debug evaluation (parity)
+
+// shared state of a debug block (dynamic shared memory: this, the operator, one list per warp)
+struct DebugSh {
+    SysDev sys;
+    WarpLists lists;
+    double wsum[3][MRQ_VW];
+    unsigned long long ctr[4];      // gathers, probes, candidates, terms
+    double hnn, hdnn;
+    CasWalker cw;
+    unsigned long long nsh[4];
+};
+
+__host__ __device__ __forceinline__ size_t debug_smem_bytes(int nw, int cap, int gstride) {
+    return (sizeof(DebugSh) + 15) / 16 * 16 + ((size_t)gstride * sizeof(double) + 15) / 16 * 16 +
+           (size_t)nw * cand_list_bytes(cap);
+}
+__host__ __device__ __forceinline__ size_t eval_warp_bytes(int cap) {
+    const size_t l = cand_list_bytes(cap);
+    return (sizeof(WarpTask) + 15) / 16 * 16 + (l > sizeof(WarpLists) ? l : (sizeof(WarpLists) + 15) / 16 * 16);
+}
+
+// local quantities of arbitrary determinants: one block per determinant, the walk's unit code
 template <int W>
 __global__ void __launch_bounds__(MRQ_MAXNW * 32, 2) k_debug2(const SysDev* __restrict__ sys,
                                                               const unsigned long long* __restrict__ dets, long long ndet,
@@ -1046,18 +1402,14 @@ __global__ void __launch_bounds__(MRQ_MAXNW * 32, 2) k_debug2(const SysDev* __re
                                                               mrq_neighbour* __restrict__ nb, long long* nb_prefix,
                                                               int prefix_stride) {
     extern __shared__ __align__(16) unsigned char smem_dyn[];
-    CtaSh& cs = *reinterpret_cast<CtaSh*>(smem_dyn);
-    unsigned char* lists = smem_dyn + (sizeof(CtaSh) + 15) / 16 * 16;
+    DebugSh& cs = *reinterpret_cast<DebugSh*>(smem_dyn);
     const long long i = blockIdx.x;
     if (i >= ndet) return;
-    {
-        const int* src = reinterpret_cast<const int*>(sys);
-        int* dst = reinterpret_cast<int*>(&cs.L.sys);
-        for (int k = threadIdx.x; k < (int)(sizeof(SysDev) / sizeof(int)); k += blockDim.x) dst[k] = src[k];
-        if (threadIdx.x < 4) cs.ctr[threadIdx.x] = 0;
-    }
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    copy_sys(&cs.sys, sys, threadIdx.x, blockDim.x);
+    if (threadIdx.x < 4) cs.ctr[threadIdx.x] = 0;
     __syncthreads();
-    const SysDev& S = cs.L.sys;
+    const SysDev& S = cs.sys;
     unsigned long long n[2][W];
 #pragma unroll
     for (int w = 0; w < W; w++) {
@@ -1079,22 +1431,98 @@ __global__ void __launch_bounds__(MRQ_MAXNW * 32, 2) k_debug2(const SysDev* __re
     if (ln == 0) psin = __ldg(S.c) * hash_lookup(S, hash_key(S, active_bits<W>(S, n[0]), active_bits<W>(S, n[1])), nc0);
     else psin = __ldg(S.c + ln) * reach_back<W>(S, n, nc0);
     Ctr ctr;
-    mrq_neighbour* rec = nb ? nb + i * max_nb : nullptr;
-    const StepOut o = block_local<W, MODE_DEBUG>(cs, lists, n, psin, ln, h, p, 0, 0, rec, max_nb,
-                                                 nb_prefix ? nb_prefix + i * (long long)prefix_stride : nullptr, ctr);
+    mrq_neighbour* const rec = nb ? nb + i * max_nb : nullptr;
+    long long* const prefix = nb_prefix ? nb_prefix + i * (long long)prefix_stride : nullptr;
+    unsigned char* const lists = smem_dyn + (sizeof(DebugSh) + 15) / 16 * 16;
+    double* const gops = reinterpret_cast<double*>(lists);
+    double* const cphi = reinterpret_cast<double*>(lists + ((size_t)S.gstride * sizeof(double) + 15) / 16 * 16 +
+                                                   (size_t)wi * cand_list_bytes(S.cand_cap));
+    unsigned* const ccode = reinterpret_cast<unsigned*>(cphi + S.cand_cap);
+    const double c0 = __ldg(S.c), inv_psin = psin != 0.0 ? 1.0 / psin : 0.0;
+    const bool cas = ln == 0 && psin != 0.0;
+    if (wi == 0) {
+        double hnn, hdnn;
+        build_lists<W>(S, n, cs.lists, h, p, lane);
+        diagonals<W>(S, cs.lists, n, lane, hnn, hdnn);
+        if (lane == 0) {
+            cs.hnn = hnn;
+            cs.hdnn = hdnn;
+            if (cas) cs.cw = cas_constants<W>(S, n, psin);
+#pragma unroll
+            for (int sg = 0; sg < 2; sg++)
+#pragma unroll
+                for (int w = 0; w < W; w++) cs.nsh[sg * W + w] = n[sg][w];
+        }
+    }
+    if (psin != 0.0) walker_operator<W>(S, n, cas, gops, ctr);
+    const unsigned long long(&nsh)[2][W] = *reinterpret_cast<const unsigned long long(*)[2][W]>(cs.nsh);
+    __syncthreads();
+    const int total_fois = cas ? 0 : cs.lists.bstart[cs.lists.nb];
+    const int units = cas ? S.unit_off[8] : (total_fois + MRQ_FOIS_CH - 1) / MRQ_FOIS_CH;
+    if (rec != nullptr && cas) {              // neighbour offsets of the units
+        for (int u = threadIdx.x; u < units; u += blockDim.x) prefix[u] = cas_unit_count(S, cs.cw, u);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            long long run = 0;
+            for (int u = 0; u < units; u++) {
+                const long long c = prefix[u];
+                prefix[u] = run;
+                run += c;
+            }
+        }
+        __syncthreads();
+    }
+    const unsigned long long self_key =
+        ln == 0 ? hash_key(S, active_bits<W>(S, n[0]), active_bits<W>(S, n[1])) : MRQ_EMPTY_KEY;
+    const double phi_self = ln == 0 ? psin / c0 : 0.0;
+    for (int vw = wi; vw < MRQ_VW; vw += nw) {
+        DebugSink sink{rec, 0, max_nb, inv_psin, 0.0, 0.0, 0.0};
+        for (int u = vw; u < units; u += MRQ_VW) {
+            if (cas) {
+                sink.nbase = rec != nullptr ? prefix[u] : 0;
+                if (u < S.cas_units) cas_internal_unit<W>(S, cs.cw, nsh, u, lane, sink, ctr);
+                else cas_pair_unit<W>(S, cs.cw, gops, cphi, ccode, nsh, u, lane, sink, ctr);
+            } else {
+                fois_unit<W>(S, cs.lists, psin != 0.0 ? gops : nullptr, nsh, ln, c0, self_key, phi_self, u * MRQ_FOIS_CH,
+                             min(total_fois, (u + 1) * MRQ_FOIS_CH), lane, sink, ctr);
+            }
+        }
+        const double sA = warp_sum(sink.sA), sT = warp_sum(sink.sT), sD = warp_sum(sink.sD);
+        if (lane == 0) {
+            cs.wsum[0][vw] = sA;
+            cs.wsum[1][vw] = sT;
+            cs.wsum[2][vw] = sD;
+        }
+    }
+    {
+        unsigned long long v[4] = {ctr.gathers, ctr.probes, ctr.cands, ctr.terms};
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            unsigned long long x = v[k];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            if (lane == 0) atomicAdd(&cs.ctr[k], x);
+        }
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
+        double A = 0.0, T = 0.0, D = 0.0;
+        for (int k = 0; k < MRQ_VW; k++) {
+            A += cs.wsum[0][k];
+            T += cs.wsum[1][k];
+            D += cs.wsum[2][k];
+        }
         r.n_gathers = (long long)cs.ctr[0];
         r.n_probes = (long long)cs.ctr[1];
         r.n_candidates = (long long)cs.ctr[2];
         r.n_terms = (long long)cs.ctr[3];
-        r.S = o.S;
-        r.e_local = o.EL;
-        r.num = o.num;
-        r.h_nn = o.hnn;
-        r.hd_nn = o.hdnn;
+        r.S = fabs(inv_psin) * A;
+        r.e_local = cs.hnn + inv_psin * T;
+        r.num = ln > 0 ? cs.hdnn + inv_psin * D : 0.0;
+        r.h_nn = cs.hnn;
+        r.hd_nn = cs.hdnn;
         r.psi = psin;
-        r.n_neighbours = o.nnb;
+        r.n_neighbours = cas ? (long long)S.cas_nb_total : (long long)total_fois;
         out[i] = r;
     }
 }
