@@ -408,6 +408,18 @@ __global__ void k_build_tab(const SysDev* __restrict__ sys, double* __restrict__
     }
 }
 
+// terms of the single-excitation operator (SysDev::sgl)
+__global__ void k_build_sgl(const SysDev* __restrict__ sys, double* __restrict__ sgl) {
+    const SysDev S = *sys;
+    const int blk = S.nca * S.nav, half = S.na * blk;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < half; t += gridDim.x * blockDim.x) {
+        const int j = S.nc + t / blk, y = (t % blk) / S.nav, x = S.nc + t % S.nav;
+        const double d = eri_g(S, y, x, j, j);
+        sgl[t] = d - eri_g(S, y, j, j, x);
+        sgl[half + t] = d;
+    }
+}
+
 // hc_pq = h_pq + sum_i [2(pq|ii) - (pi|iq)]
 __global__ void k_core_fock(const SysDev* __restrict__ sys, double* hc) {
     const SysDev S = *sys;
@@ -907,7 +919,7 @@ struct mrq_ctx {
     int n = 0, nc = 0, na = 0, nv = 0, W = 1, nalpha = 0, nbeta = 0;
     double e_nuc = 0.0;
     long long neri = 0;
-    double *d_h1 = nullptr, *d_eri = nullptr, *d_eri4 = nullptr, *d_tab = nullptr, *d_hc = nullptr,
+    double *d_h1 = nullptr, *d_eri = nullptr, *d_eri4 = nullptr, *d_tab = nullptr, *d_sgl = nullptr, *d_hc = nullptr,
            *d_eps = nullptr, *d_gamma = nullptr;
     unsigned short* d_colex = nullptr;
     long long nHs = 0, nPs = 0, nlab = 0;
@@ -949,6 +961,7 @@ struct mrq_ctx {
     // workspace of this context's walk launches (WalkScratch), kept between calls
     unsigned char* d_work = nullptr;
     size_t work_cap = 0;
+    long long row_worst = 0;         // doubles of one CAS determinant's rows when none is shared
     WalkScratch work{};
     double* d_partial = nullptr;
     long long partial_cap = 0;
@@ -964,10 +977,10 @@ struct mrq_ctx {
     struct GraphKey {
         const void *sys = nullptr, *wptr = nullptr, *off = nullptr, *work = nullptr;
         long long nslots = 0;
-        int k = 0, wpb = 0, spl = 0, cap = 0, gstride = 0, ns = 0;
+        int k = 0, wpb = 0, spl = 0, cap = 0, gstride = 0, ns = 0, nref = 0;
         bool operator==(const GraphKey& o) const {
             return sys == o.sys && wptr == o.wptr && off == o.off && work == o.work && nslots == o.nslots &&
-                   k == o.k && wpb == o.wpb && spl == o.spl && cap == o.cap && gstride == o.gstride && ns == o.ns;
+                   k == o.k && wpb == o.wpb && spl == o.spl && cap == o.cap && gstride == o.gstride && ns == o.ns && nref == o.nref;
         }
     };
     // per determinant width and warps per block (8, 4, 2, 1) of a batch launch
@@ -994,7 +1007,7 @@ struct mrq_ctx {
     int probe_limit = 0, cap_limit = 0;
     int cand_cap_full = 1;           // the candidate-list capacity the loaded system needs
     double l2_fraction = 0.0;        // mrq_set_l2_window: share of the persisting-L2 carve-out for the tables
-    int eval_minb = 2, eval_blocks = 0;   // k_eval: build in use (resident blocks per SM) and grid
+    int rows_minb = 2, rows_blocks = 0;   // k_rows: build in use (resident blocks per SM) and grid
 };
 
 static int fail(mrq_ctx* c, int code, const char* fmt, ...) {
@@ -1082,6 +1095,7 @@ static void free_hamiltonian(mrq_ctx* c) {
     dfree(c->d_eri);
     dfree(c->d_eri4);
     dfree(c->d_tab);
+    dfree(c->d_sgl);
     dfree(c->d_hc);
     dfree(c->d_eps);
     dfree(c->d_gamma);
@@ -1135,56 +1149,94 @@ struct WalkLaunch {
 // what a walk set's systems need: the largest candidate-list capacity, single-excitation operator and
 // slice count among them
 struct WalkNeed {
-    int cap = 1, gstride = 0, ns = 1;
-    void add(const SysDev& s) {
+    int cap = 1, gstride = 0, ns = 1, nref = 1;
+    long long row_worst = 1;
+    void add(const mrq_ctx* c) {
+        const SysDev& s = c->hsys;
+        nref = std::max(nref, s.ref_off[8]);
+        row_worst = std::max(row_worst, c->row_worst);
         cap = std::max(cap, s.cand_cap);
         gstride = std::max(gstride, s.gstride);
         ns = std::max(ns, s.nslice);
     }
 };
 
-// Workspace of a launch over nslots walkers.  A launch takes its walkers in segments of at most
-// `seg` slots, so that the workspace stays below about 1 GiB whatever the number of walkers.
+// Workspace of a launch over nslots walkers.  A launch takes its walkers in segments, and a segment's
+// CAS determinants in waves, so that the workspace stays below MRQ_WORK_BYTES and MRQ_ROW_BYTES whatever
+// the number of walkers: a segment's arrays hold one entry per walker, a wave's row buffer the worst
+// case that none of its determinants share a row.  When the device cannot give that much, waves shrink.
 #define MRQ_WORK_BYTES (1LL << 30)
+#define MRQ_ROW_BYTES (4LL << 30)
 static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, long long* seg_out) {
-    const long long per = 12 * 4 + 3 * 4 + (long long)sizeof(TaskGroup) + (long long)sizeof(GroupMeta) +
-                          8LL * need.gstride + 24LL * need.ns + (long long)sizeof(RaceBest) + 4;
+    const long long per = 12 * 4 + 3 * 4 + 2 * (long long)sizeof(TaskGroup) + (long long)sizeof(GroupMeta) +
+                          8LL * need.gstride + 24LL * (need.ns + MRQ_INT_SLICES) + (long long)sizeof(RaceBest) + 4;
     const long long seg = std::min(nslots, std::max(256LL, std::min(1LL << 20, MRQ_WORK_BYTES / per)));
     *seg_out = seg;
-    size_t off = 0;
-    auto take = [&](size_t bytes) {
-        const size_t at = off;
-        off += (bytes + 255) / 256 * 256;
-        return at;
-    };
-    const size_t rep = take(16 * seg), cnt = take(16 * seg), start = take(16 * seg), tab = take(4 * seg), pos = take(4 * seg),
-                 mem = take(4 * seg), tg = take(sizeof(TaskGroup) * seg), meta = take(sizeof(GroupMeta) * seg),
-                 gops = take(8 * (size_t)need.gstride * seg), part = take(24 * (size_t)need.ns * seg),
-                 best = take(sizeof(RaceBest) * seg), bound = take(4 * seg), ctl = take(16);
-    if (off > ctx->work_cap) {
-        CK(cudaStreamSynchronize(ctx->stream));
-        dfree(ctx->d_work);
-        ctx->work_cap = 0;
-        CK(cudaMalloc(&ctx->d_work, off));
-        ctx->work_cap = off;
-    }
-    unsigned char* const b = ctx->d_work;
+    const long long per_group = 8 * need.row_worst + 33LL * need.nref;
+    long long groups = std::max(1LL, std::min(seg, MRQ_ROW_BYTES / per_group));
+    groups = std::min(groups, std::max(1LL, (1LL << 29) / need.nref));           // reference indices and the table: 32 bits
     WalkScratch& w = ctx->work;
-    w.rep = (int*)(b + rep);
-    w.cnt = (int*)(b + cnt);
-    w.start = (int*)(b + start);
-    w.tab_of = (int*)(b + tab);
-    w.pos_of = (int*)(b + pos);
-    w.members = (int*)(b + mem);
-    w.tg = (TaskGroup*)(b + tg);
-    w.meta = (GroupMeta*)(b + meta);
-    w.gops = (double*)(b + gops);
-    w.part = (double*)(b + part);
-    w.best = (RaceBest*)(b + best);
-    w.bound = (unsigned*)(b + bound);
-    w.ctl = (int*)(b + ctl);
+    for (;; groups = (groups + 1) / 2) {
+        long long tsz = 2;
+        while (tsz < 2 * groups * need.nref) tsz <<= 1;
+        size_t off = 0;
+        auto take = [&](size_t bytes) {
+            const size_t at = off;
+            off += (bytes + 255) / 256 * 256;
+            return at;
+        };
+        const size_t nr = (size_t)groups * need.nref;
+        const size_t rep = take(16 * seg), cnt = take(16 * seg), start = take(16 * seg), tab = take(4 * seg),
+                     pos = take(4 * seg), mem = take(4 * seg), tgc = take(sizeof(TaskGroup) * seg),
+                     tgf = take(sizeof(TaskGroup) * seg), meta = take(sizeof(GroupMeta) * seg),
+                     gops = take(8 * (size_t)need.gstride * seg), part = take(24 * (size_t)(need.ns + MRQ_INT_SLICES) * seg),
+                     best = take(sizeof(RaceBest) * seg), bound = take(4 * seg), ctl = take(4 * CTL_N), ao = take(8 * nr),
+                     cls = take(nr), rrep = take(4 * nr), roff = take(8 * nr), tbl = take(4 * tsz), ul = take(4 * nr),
+                     rows = take(8 * (size_t)need.row_worst * groups);
+        if (off > ctx->work_cap) {
+            CK(cudaStreamSynchronize(ctx->stream));
+            dfree(ctx->d_work);
+            ctx->work_cap = 0;
+            const cudaError_t e = cudaMalloc(&ctx->d_work, off);
+            if (e == cudaErrorMemoryAllocation && groups > 1) {
+                cudaGetLastError();
+                ctx->d_work = nullptr;
+                continue;
+            }
+            CK(e);
+            ctx->work_cap = off;
+        }
+        unsigned char* const b = ctx->d_work;
+        w.rep = (int*)(b + rep);
+        w.cnt = (int*)(b + cnt);
+        w.start = (int*)(b + start);
+        w.tab_of = (int*)(b + tab);
+        w.pos_of = (int*)(b + pos);
+        w.members = (int*)(b + mem);
+        w.tgc = (TaskGroup*)(b + tgc);
+        w.tgf = (TaskGroup*)(b + tgf);
+        w.meta = (GroupMeta*)(b + meta);
+        w.gops = (double*)(b + gops);
+        w.part = (double*)(b + part);
+        w.best = (RaceBest*)(b + best);
+        w.bound = (unsigned*)(b + bound);
+        w.ctl = (int*)(b + ctl);
+        w.ref_ao = (unsigned long long*)(b + ao);
+        w.ref_cls = b + cls;
+        w.ref_rep = (int*)(b + rrep);
+        w.row_off = (long long*)(b + roff);
+        w.table = (int*)(b + tbl);
+        w.ulist = (int*)(b + ul);
+        w.rows = (double*)(b + rows);
+        w.table_size = (int)tsz;
+        break;
+    }
+    w.nref_max = need.nref;
+    w.wave_groups = (int)groups;
+    w.wave0 = 0;
     w.gstride = need.gstride;
     w.ns_max = need.ns;
+    w.nseg = seg;
     // walkers per task group: 32 when there are many, fewer for small launches, so that the walkers of
     // a crowded determinant spread over more warps
     w.tgw = (int)std::max(4LL, std::min<long long>(MRQ_TGW, seg / 128));
@@ -1192,52 +1244,77 @@ static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, lo
 }
 
 template <int W, int B>
-static int eval_fits(mrq_ctx* ctx, size_t smem, int threads, int& blocks) {
-    CK(cudaFuncSetAttribute(k_eval<W, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_eval<W, B>, threads, smem));
+static int rows_fits(mrq_ctx* ctx, size_t smem, int threads, int& blocks) {
+    CK(cudaFuncSetAttribute(k_rows<W, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_rows<W, B>, threads, smem));
     return 0;
 }
 
-// k_eval's build for this launch: the most resident warps per SM (4, 3 or 2 blocks' worth of MRQ_MAXNW
-// warps, fewer registers each) that the block's shared memory allows, and a grid that fills the chip once
-static int eval_prepare(mrq_ctx* ctx, int W, int nw, int cap) {
-    const size_t smem = nw * eval_warp_bytes(cap), lsm = nw * cand_list_bytes(cap);
-    int b4 = 0, b3 = 0, b2 = 0;
-    const int full = MRQ_MAXNW / nw;             // blocks that hold MRQ_MAXNW warps
+// k_rows' build for this launch: the most resident warps per SM (4 or 2 blocks' worth of MRQ_MAXNW warps)
+// that the candidate lists in shared memory allow, and a grid that fills the chip once
+static int rows_prepare(mrq_ctx* ctx, int W, int nw, int cap) {
+    const size_t smem = nw * rows_warp_bytes(cap), lsm = nw * cand_list_bytes(cap);
+    int b4 = 0, b2 = 0;
     if (W == 1) {
-        if (int r = eval_fits<1, 4>(ctx, smem, 32 * nw, b4)) return r;
-        if (int r = eval_fits<1, 3>(ctx, smem, 32 * nw, b3)) return r;
-        if (int r = eval_fits<1, 2>(ctx, smem, 32 * nw, b2)) return r;
+        if (int r = rows_fits<1, 4>(ctx, smem, 32 * nw, b4)) return r;
+        if (int r = rows_fits<1, 2>(ctx, smem, 32 * nw, b2)) return r;
         CK(cudaFuncSetAttribute(k_move<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm));
     } else {
-        if (int r = eval_fits<2, 3>(ctx, smem, 32 * nw, b3)) return r;
-        if (int r = eval_fits<2, 2>(ctx, smem, 32 * nw, b2)) return r;
+        if (int r = rows_fits<2, 4>(ctx, smem, 32 * nw, b4)) return r;
+        if (int r = rows_fits<2, 2>(ctx, smem, 32 * nw, b2)) return r;
         CK(cudaFuncSetAttribute(k_move<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm));
     }
-    ctx->eval_minb = b4 >= 4 * full ? 4 : (b3 >= 3 * full ? 3 : 2);
-    const int b = ctx->eval_minb == 4 ? b4 : (ctx->eval_minb == 3 ? b3 : b2);
-    ctx->eval_blocks = std::max(1, b) * ctx->n_sm;
+    ctx->rows_minb = b4 > b2 ? 4 : 2;
+    ctx->rows_blocks = std::max(1, std::max(b4, b2)) * ctx->n_sm;
     return 0;
 }
 
-// warps per block of a context's launches: the requested (or default) number, at most the most whose
-// candidate lists fit shared memory (large active spaces run with fewer warps)
+// warps per block of a context's k_rows and k_move launches: the requested (or default) number, at most
+// the most whose candidate lists fit shared memory (large active spaces run with fewer warps)
 static int warps_of(const mrq_ctx* ctx) { return std::min(ctx->wpb > 0 ? ctx->wpb : MRQ_MAXNW, ctx->max_nw); }
 
-// nsteps walker steps of a walk set (the five kernels of mrq_walk.cuh per step); `ctx` provides the
-// stream and the workspace.
+template <int W>
+static int launch_segment(mrq_ctx* ctx, const WalkSet& ws, WalkScratch sc, const WalkNeed& need, int nw, int accumulate,
+                          cudaLaunchConfig_t cfg) {
+    const long long n = sc.seg1 - sc.seg0;
+    const int sms = ctx->n_sm;
+    const cudaStream_t st = ctx->stream;
+    const size_t lbytes = cand_list_bytes(need.cap), rbytes = rows_warp_bytes(need.cap);
+    if (ws.nsys > 1) CK(cudaMemsetAsync(sc.ctl, 0, sizeof(int) * CTL_N, st));
+    k_group<W><<<(unsigned)ws.nsys, 1024, 0, st>>>(ws, sc);
+    k_prep<W><<<(unsigned)std::min<long long>(n, 8LL * sms), 128, 0, st>>>(ws, sc);
+    k_int<W><<<(unsigned)std::min<long long>(n, 3LL * sms), 256, 0, st>>>(ws, sc);
+    k_fois<W, 3><<<3 * sms, 256, 0, st>>>(ws, sc);
+    for (long long g = 0; g < n; g += sc.wave_groups) {
+        sc.wave0 = (int)g;
+        k_refs<W><<<(unsigned)std::min<long long>(n, 8LL * sms), 256, 0, st>>>(ws, sc);
+        k_insert<<<8 * sms, 256, 0, st>>>(ws, sc);
+        cfg.gridDim = dim3((unsigned)ctx->rows_blocks);
+        cfg.blockDim = dim3(32 * nw);
+        cfg.dynamicSmemBytes = nw * rbytes;
+        if (ctx->rows_minb == 4) CK(cudaLaunchKernelEx(&cfg, k_rows<W, 4>, ws, sc, (int)rbytes, need.cap));
+        else CK(cudaLaunchKernelEx(&cfg, k_rows<W, 2>, ws, sc, (int)rbytes, need.cap));
+        cfg.gridDim = dim3(4u * sms);
+        cfg.blockDim = dim3(256);
+        cfg.dynamicSmemBytes = 0;
+        CK(cudaLaunchKernelEx(&cfg, k_pairs<W, 4>, ws, sc));
+    }
+    k_move<W><<<(unsigned)std::min<long long>((n + nw - 1) / nw, 4LL * sms), 32 * nw, nw * lbytes, st>>>(
+        ws, sc, accumulate, (int)lbytes, need.cap);
+    CK(cudaGetLastError());
+    return 0;
+}
+
+// nsteps walker steps of a walk set (the kernels of mrq_walk.cuh per step); `ctx` provides the stream
+// and the workspace.
 static int launch_walk(mrq_ctx* ctx, int W, const WalkSet& ws, int nsteps, const WalkNeed& need,
                        const WalkLaunch& L = WalkLaunch()) {
     const int nw = std::min(L.wpb, MRQ_MAXNW);
-    const size_t wbytes = eval_warp_bytes(need.cap), lbytes = cand_list_bytes(need.cap);
     long long seg = 0;
     if (int r = work_prepare(ctx, ws.nslots, need, &seg)) return r;
     if (!L.captured)
-        if (int r = eval_prepare(ctx, W, nw, need.cap)) return r;
+        if (int r = rows_prepare(ctx, W, nw, need.cap)) return r;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)ctx->eval_blocks);
-    cfg.blockDim = dim3(32 * nw);
-    cfg.dynamicSmemBytes = nw * wbytes;
     cfg.stream = ctx->stream;
     cudaLaunchAttribute attr[1];
     if (L.l2win.num_bytes > 0) {            // keep the walk's hottest table resident in L2
@@ -1251,25 +1328,9 @@ static int launch_walk(mrq_ctx* ctx, int W, const WalkSet& ws, int nsteps, const
             WalkScratch sc = ctx->work;
             sc.seg0 = s0;
             sc.seg1 = std::min(ws.nslots, s0 + seg);
-            const long long n = sc.seg1 - sc.seg0;
-            if (ws.nsys > 1) CK(cudaMemsetAsync(sc.ctl, 0, 3 * sizeof(int), ctx->stream));
-            const unsigned gp = (unsigned)std::min<long long>(n, 8LL * ctx->n_sm);
-            const unsigned gm = (unsigned)std::min<long long>((n + nw - 1) / nw, 4LL * ctx->n_sm);
-            if (W == 1) {
-                k_group<1><<<(unsigned)ws.nsys, 1024, 0, ctx->stream>>>(ws, sc);
-                k_prep<1><<<gp, 128, 0, ctx->stream>>>(ws, sc);
-                if (ctx->eval_minb == 4) CK(cudaLaunchKernelEx(&cfg, k_eval<1, 4>, ws, sc, (int)wbytes, need.cap));
-                else if (ctx->eval_minb == 3) CK(cudaLaunchKernelEx(&cfg, k_eval<1, 3>, ws, sc, (int)wbytes, need.cap));
-                else CK(cudaLaunchKernelEx(&cfg, k_eval<1, 2>, ws, sc, (int)wbytes, need.cap));
-                k_move<1><<<gm, 32 * nw, nw * lbytes, ctx->stream>>>(ws, sc, L.accumulate, (int)lbytes, need.cap);
-            } else {
-                k_group<2><<<(unsigned)ws.nsys, 1024, 0, ctx->stream>>>(ws, sc);
-                k_prep<2><<<gp, 128, 0, ctx->stream>>>(ws, sc);
-                if (ctx->eval_minb >= 3) CK(cudaLaunchKernelEx(&cfg, k_eval<2, 3>, ws, sc, (int)wbytes, need.cap));
-                else CK(cudaLaunchKernelEx(&cfg, k_eval<2, 2>, ws, sc, (int)wbytes, need.cap));
-                k_move<2><<<gm, 32 * nw, nw * lbytes, ctx->stream>>>(ws, sc, L.accumulate, (int)lbytes, need.cap);
-            }
-            CK(cudaGetLastError());
+            if (int r = W == 1 ? launch_segment<1>(ctx, ws, sc, need, nw, L.accumulate, cfg)
+                               : launch_segment<2>(ctx, ws, sc, need, nw, L.accumulate, cfg))
+                return r;
         }
         if (L.accumulate) {
             k_accum<<<dim3((unsigned)ws.nsys, 2), 1024, 0, ctx->stream>>>(ws);
@@ -1318,6 +1379,7 @@ static int walk_plan(mrq_ctx* ctx, SysDev& s) {
     long long off = (cas_nb + MRQ_CAS_CH - 1) / MRQ_CAS_CH;
     s.cas_nb = (int)cas_nb;
     s.cas_units = (int)off;
+    long long nref = 0;
     for (int k = 0; k < 8; k++) {
         const int ka = k / 3, kb = k % 3;
         const long long npairs = nsub_h(cntO, ka) * nsub_h(cntE, kb);
@@ -1335,8 +1397,12 @@ static int walk_plan(mrq_ctx* ctx, SysDev& s) {
         s.nch[k] = (int)nch;
         s.unit_off[k] = (int)off;
         off += npairs * nch;
+        s.ref_off[k] = (int)nref;
+        nref += npairs * (ka + kb == 1 ? 2 : 1);
     }
     s.unit_off[8] = (int)off;
+    s.ref_off[8] = (int)nref;
+    ctx->row_worst = total - cas_nb + 4 * nref;
     // slices of a determinant's units: about four units each, so that a step on a few hundred
     // determinants is some 10^5 warp tasks and one on a few still spreads over the chip
     s.nslice = 32;
@@ -1377,7 +1443,7 @@ static int walk_plan(mrq_ctx* ctx, SysDev& s) {
     // warp the active space is too large for the walk
     ctx->max_nw = 0;
     for (int nw = MRQ_MAXNW; nw >= 1 && ctx->max_nw == 0; nw >>= 1)
-        if (debug_smem_bytes(nw, (int)cap, s.gstride) <= 227 * 1024 && nw * eval_warp_bytes((int)cap) <= 227 * 1024)
+        if (debug_smem_bytes(nw, (int)cap, s.gstride) <= 227 * 1024 && nw * rows_warp_bytes((int)cap) <= 227 * 1024)
             ctx->max_nw = nw;
     if (ctx->max_nw == 0)
         return fail(ctx, MRQ_TOO_LARGE, "active space too large for the shared-memory candidate lists");
@@ -1520,6 +1586,7 @@ int mrq_load_hamiltonian(mrq_ctx* ctx, int n_core, int n_act, int n_virt, int n_
     CK(cudaMalloc(&ctx->d_eri4, sizeof(double) * npair * n * n));
     const long long nca = n_core + n_act, nav = n_act + n_virt;
     CK(cudaMalloc(&ctx->d_tab, sizeof(double) * 2 * std::max(1LL, nca * nca * nav * nav)));
+    CK(cudaMalloc(&ctx->d_sgl, sizeof(double) * 2 * std::max(1LL, n_act * nca * nav)));
     CK(cudaMalloc(&ctx->d_hc, sizeof(double) * n * n));
     CK(cudaMalloc(&ctx->d_eps, sizeof(double) * n));
     CK(cudaMalloc(&ctx->d_gamma, sizeof(double) * std::max(1, n_act * n_act)));
@@ -1558,6 +1625,7 @@ int mrq_load_hamiltonian(mrq_ctx* ctx, int n_core, int n_act, int n_virt, int n_
     s.eri = ctx->d_eri;
     s.eri4 = ctx->d_eri4;
     s.tab = ctx->d_tab;
+    s.sgl = ctx->d_sgl;
     s.nca = (int)nca;
     s.nav = (int)nav;
     s.tab_half = (unsigned)(nca * nca * nav * nav);
@@ -1575,6 +1643,8 @@ int mrq_load_hamiltonian(mrq_ctx* ctx, int n_core, int n_act, int n_virt, int n_
     k_expand_eri<<<1216, 256, 0, ctx->stream>>>(ctx->d_eri, ctx->d_eri4, n);
     CK(cudaGetLastError());
     k_build_tab<<<2432, 256, 0, ctx->stream>>>(ctx->d_sys, ctx->d_tab);
+    CK(cudaGetLastError());
+    k_build_sgl<<<304, 256, 0, ctx->stream>>>(ctx->d_sys, ctx->d_sgl);
     CK(cudaGetLastError());
     k_core_fock<<<(n * n + 127) / 128, 128, 0, ctx->stream>>>(ctx->d_sys, ctx->d_hc);
     CK(cudaGetLastError());
@@ -1857,7 +1927,7 @@ int mrq_walkers_advance(mrq_ctx* ctx, int64_t n_steps) {
     CK(cudaEventRecord(ctx->evs[k], ctx->stream));
     WalkSet ws{ctx->d_sys, ctx->d_wptr, ctx->d_woff, 1, ctx->nwalk};
     WalkNeed need;
-    need.add(ctx->hsys);
+    need.add(ctx);
     WalkLaunch L;
     L.wpb = warps_of(ctx);
     if (int r = l2_window(ctx, L.l2win)) return r;
@@ -2032,7 +2102,7 @@ static int batch_tables(mrq_ctx* const* ctxs, int n, int W, Walker* const* walke
         sys.push_back(ctxs[i]->hsys);
         wp.push_back(walkers[i]);
         off.push_back(off.back() + ctxs[i]->nwalk);
-        need.add(ctxs[i]->hsys);
+        need.add(ctxs[i]);
     }
     ws = WalkSet{ctx->d_bsys, ctx->d_bwptr, ctx->d_boff, (int)sys.size(), off.back()};
     if (sys.empty()) return 0;
@@ -2055,7 +2125,7 @@ static int batch_run(mrq_ctx* ctx, int W, const WalkSet& ws, const WalkNeed& nee
     if (graph && nfull > 0) {
         long long seg = 0;
         if (int r = work_prepare(ctx, ws.nslots, need, &seg)) return r;
-        if (int r = eval_prepare(ctx, W, std::min(wpb, MRQ_MAXNW), need.cap)) return r;
+        if (int r = rows_prepare(ctx, W, std::min(wpb, MRQ_MAXNW), need.cap)) return r;
         mrq_ctx::GraphKey key;
         key.sys = ws.systems;
         key.wptr = ws.walkers;
@@ -2068,6 +2138,7 @@ static int batch_run(mrq_ctx* ctx, int W, const WalkSet& ws, const WalkNeed& nee
         key.cap = need.cap;
         key.gstride = need.gstride;
         key.ns = need.ns;
+        key.nref = need.nref;
         cudaGraphExec_t& ex = ctx->gexec[slot];
         if (!ex || !(ctx->gkey[slot] == key)) {
             if (ex) CK(cudaGraphExecDestroy(ex));

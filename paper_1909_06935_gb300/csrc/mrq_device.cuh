@@ -70,6 +70,10 @@ struct SysDev {
     int unit_off[9];         // first unit of pair class k = 3 ka + kb (k < 8); unit_off[8] = all units
     int nch[8];              // chunks per (X_a, Y_a) pair of class k
     int nslice;              // warp tasks a determinant's units are split into (a power of two)
+    int ref_off[9];          // first row reference of pair class k; ref_off[8] = all of a CAS determinant's
+    // terms of the single-excitation operator, [j][y][x - n_core] for an active j: (yx|jj) - (yj|jx) (j of
+    // the electron's spin), then after n_act blocks (yx|jj) (j of the other)
+    const double* sgl;
     int gstride;             // doubles of the walker's single-excitation operator, 2 nca nav
     int hb_on;               // heat-bath cutoff in force (hb_eps > 0)
     const unsigned short* colex;       // pair decode table: colex[j(j-1)/2 + i] = i | j << 8, i < j < 128

@@ -7,26 +7,27 @@
 //   k_group   finds the distinct determinants (a hash table over the walkers) and cuts each one's
 //             walkers into task groups of at most MRQ_TGW;
 //   k_prep    makes the determinant's constants: its diagonals and its single-excitation operator;
-//   k_eval    evaluates the neighbours once per task group, in work units spread over the whole
-//             chip: the sums S, E_L and the H_D numerator, and for every walker of the group the
-//             move race (its own Philox clocks against the shared rates);
+//   k_int     CAS determinants: the neighbours inside the CAS;
+//   k_refs, k_insert, k_rows
+//             CAS determinants: the overlaps outside the CAS.  O(m) depends on m alone, and the
+//             determinants of a step share most of their active remnants, so the distinct rows
+//             (remnant, core holes, virtual electrons) are found and computed once;
+//   k_pairs   CAS determinants: every (X_a, Y_a) pair's neighbours, elements times rows;
+//   k_fois    first-order determinants: their neighbours, reach-back per lane;
 //   k_move    adds the units' sums, takes each walker's winner, and looks up psi_s there;
 //   k_accum   adds the step records into the accumulators.
+// k_int, k_pairs and k_fois evaluate a determinant's neighbours once per task group, in work units
+// spread over the whole chip, and run the move race of every walker of the group (its own Philox
+// clocks against the shared rates).  They are kernels of their own because the walk is bound by
+// instruction fetch when a warp scheduler's warps run different code (in one kernel 25 of 38 cycles
+// per issue were waits for instructions).
 // Every sum is formed in an order that depends on the determinant and its system alone, and the
 // race's winner does not depend on any order, so a walker's step is the same whatever walkers
 // share its determinant, alone or in a batch, and whatever the launch configuration.
 //
-//  * CAS walkers: the neighbours inside the CAS (spin-resolved blocks of active singles and
-//    doubles), then every pair (X_a, Y_a) of active electrons removed / active holes filled.  A
-//    pair owns the groups (r, spins of the core holes X_c and virtual electrons Y_v) of mrq_cas.cuh,
-//    whose neighbours share one reach-back candidate list; large pairs are cut into chunks of
-//    neighbours.  The unit plan depends only on the system (all CAS determinants have the same
-//    active electron counts), so it is computed on the host at load.
-//  * FOIS walkers: chunks of the class-block enumeration of build_lists, reach-back per lane.
-//
-// Within a unit, rounds of up to 32 neighbours run one neighbour per lane; a round with fewer
-// neighbours splits each neighbour's candidate list over f lanes (f a power of two) and reduces
-// the f partial sums with shuffles, so short groups keep the lanes busy.
+// The units of a CAS determinant - chunks of the neighbours of an (X_a, Y_a) pair of active electrons
+// removed / active holes filled - depend only on the system (all CAS determinants have the same active
+// electron counts), so they are planned on the host at load.
 //
 // Per neighbour t = H_nm psi_s(m) is summed as |t| and t, and 1/psi_s(n) is applied once per
 // determinant (S = |1/psi_n| sum |t|, E_L = H_nn + (1/psi_n) sum t).
@@ -72,22 +73,44 @@ struct GroupMeta {
     unsigned long long d[2][2];
     double psi, hnn, hdnn;
     long long label;
-    int h, p;
+    int h, p, sys, pad;
 };
+
+// counters of a step (WalkScratch::ctl)
+enum {
+    CTL_TGC, CTL_GC,              // CAS task groups, CAS determinants
+    CTL_TGF, CTL_GF,              // first-order task groups, determinants
+    CTL_INT, CTL_PAIRS, CTL_FOIS, CTL_ROWTASK,   // next warp task of each kernel
+    CTL_BIG, CTL_SMALL,           // distinct rows of a wave: long ones (from the list's front), short ones
+    CTL_CUR,                      // (64 bits) doubles of the row buffer in use
+    CTL_N = CTL_CUR + 2
+};
+#define MRQ_INT_SLICES 8          // warp tasks of a determinant's neighbours inside the CAS
+#define MRQ_BIG_ROW 1024          // entries of a long row
+#define MRQ_NOROW 255             // a reference without entries
 
 // device workspace of a walk launch, sized for the slots [seg0, seg1) of the walk set
 struct WalkScratch {
     int *rep, *cnt, *start;   // determinant tables, 4 entries per slot: first walker, walkers, first member
     int *tab_of, *pos_of;     // per slot: table entry and place in it
     int* members;             // walkers (local index) by determinant
-    TaskGroup* tg;
-    GroupMeta* meta;
+    TaskGroup *tgc, *tgf;     // CAS and first-order task groups
+    GroupMeta* meta;          // per determinant: CAS ones from the front, first-order ones from the back
     double* gops;             // single-excitation operators, gstride doubles per determinant
-    double* part;             // [determinant][ns_max][3] partial sums
+    double* part;             // [determinant][ns_max + MRQ_INT_SLICES][3] partial sums
     RaceBest* best;           // per slot
     unsigned* bound;          // per slot: FP32 bits of an upper bound of the best clock
-    int* ctl;                 // task groups, determinants, next warp task
-    long long gstride;
+    int* ctl;
+    // rows of a wave of at most wave_groups CAS determinants; a reference is (determinant of the wave,
+    // row number in it), index determinant * nref_max + row number
+    unsigned long long* ref_ao;   // the row's active remnant
+    unsigned char* ref_cls;       // 3 (core holes) + (virtual electrons), MRQ_NOROW
+    int* ref_rep;                 // the reference that owns the row
+    long long* row_off;           // (owners) the row's place in rows
+    int *table, *ulist;           // open addressing over references; the owners
+    double* rows;
+    int table_size, nref_max, wave_groups, wave0;
+    long long gstride, nseg;
     int ns_max, tgw;
     long long seg0, seg1;
 };
@@ -191,7 +214,7 @@ __device__ __forceinline__ void cand_decode(const SysDev& S, const CandPlan& P, 
 // codes, doubles [n1, count) as (signed weight, table base); the candidate of key keyn (the walker) is left out.  Kept
 // out of line: it runs once per group, and its registers and code then stay out of the neighbour
 // loop that follows (1.8 % faster at 56 orbitals)
-template <int W, class C>
+template <int W, bool ROWS, class C>
 __device__ __noinline__ int build_group_list(const SysDev& S, unsigned long long keyn,
                                                 const unsigned long long (&mref)[2][W], unsigned long long AOm,
                                                 unsigned long long AEm, int c, int v, int sc, int sv, int rxc0,
@@ -230,7 +253,13 @@ __device__ __noinline__ int build_group_list(const SysDev& S, unsigned long long
                 const int pos = count + __popc(vm & lt);
                 if (pos < S.cand_cap) {
                     if (rr == 1) {
-                        cphi[pos] = phi;
+                        int sgn = 0;
+                        if (ROWS) {     // <k|H|m> changes sign between the group's neighbours as their core parity does
+                            const int x = v ? ryv0 : act_so(S, __ffsll(Rb) - 1), y = c ? rxc0 : act_so(S, __ffsll(Ab) - 1);
+                            const int sx = x >= S.n, px = x - sx * S.n, py = y - sx * S.n;
+                            sgn = popc_sel<W>(mref, sx, min(px, py), max(px, py)) + par_ref;
+                        }
+                        cphi[pos] = neg_if(phi, sgn);
                         ccode[pos] = pack_cand(Rb, Ab, rr);
                     } else {
                         double w;
@@ -433,7 +462,7 @@ __device__ void cas_pair_unit(const SysDev& S, const CasWalker& cw, const double
                 int n1;
                 // floor(q / nvc) = high word of q * ceil(2^64 / nvc), exact for q < 2^32 (nvc > 1)
                 const unsigned long long mvc = ~0ull / (unsigned long long)nvc + 1ull;
-                const int count = build_group_list<W>(S, cw.keyn, mref, AOm, AEm, c, v, sc, sv, rxc0, rxc1, ryv0, ryv1,
+                const int count = build_group_list<W, false>(S, cw.keyn, mref, AOm, AEm, c, v, sc, sv, rxc0, rxc1, ryv0, ryv1,
                                                       par_ref, cphi, ccode, n1, lane, ctr);
                 for (int qb = q0; qb < q1; qb += 32) {
                     const int nr = min(32, q1 - qb);
@@ -613,7 +642,7 @@ __device__ __noinline__ double reach_back_warp(const SysDev& S, const unsigned l
     int par, n1;
     lane_offsets(S, c, v, xc[0], xc[1], yv[0], yv[1], offd, offx, par);
     NoCtr ctr;
-    const int count = build_group_list<W>(S, MRQ_EMPTY_KEY, m, AOm, AEm, c, v, sc, sv, xc[0], xc[1], yv[0], yv[1], par,
+    const int count = build_group_list<W, false>(S, MRQ_EMPTY_KEY, m, AOm, AEm, c, v, sc, sv, xc[0], xc[1], yv[0], yv[1], par,
                                           cphi, ccode, n1, lane, ctr);
     double s = 0.0;
     for (int e = lane; e < n1; e += 32)
@@ -906,9 +935,11 @@ struct StepSink {
     template <int W>
     __device__ __forceinline__ void post(bool valid, int, const unsigned long long (&)[2][W], double hnm, double hd,
                                          double, double psim, unsigned exc) {
-        const double t = hnm * psim;
+        if (valid) sD += hd * psim;
+        push(valid, hnm * psim, exc);
+    }
+    __device__ __forceinline__ void push(bool valid, double t, unsigned exc) {
         const bool on = valid && (__double_as_longlong(t) << 1) != 0;
-        if (on) sD += hd * psim;
         const unsigned m = __ballot_sync(0xffffffffu, on);
         int qn = wt.qn;
         if (on) {
@@ -993,11 +1024,10 @@ __global__ void __launch_bounds__(1024) k_group(const WalkSet ws, const WalkScra
     const int n = (int)max(0LL, hi - lo);
     const Walker* const wk = ws.walkers[sys] + lo;
     const int base = (int)(off + lo - sc.seg0);          // first slot of the system in the segment
+    const SysDev& S = ws.systems[sys];
     __shared__ int s_members;
-    if (threadIdx.x == 0) {
-        s_members = 0;
-        if (gridDim.x == 1) sc.ctl[0] = sc.ctl[1] = sc.ctl[2] = 0;
-    }
+    if (threadIdx.x == 0) s_members = 0;
+    if (gridDim.x == 1 && threadIdx.x < CTL_N) sc.ctl[threadIdx.x] = 0;
     int tsz = 2;
     while (tsz < 2 * n) tsz <<= 1;
     int* const rep = sc.rep + 4LL * base;
@@ -1020,7 +1050,7 @@ __global__ void __launch_bounds__(1024) k_group(const WalkSet ws, const WalkScra
         int k = (int)(hh & (unsigned long long)(tsz - 1));
         for (int probe = 0; probe < tsz; probe++) {
             const int prev = atomicCAS(rep + k, -1, i);
-            bool same = prev < 0 || prev == i;
+            bool same = prev < 0;
             if (!same) {
                 unsigned long long o[2][W];
                 load_det<W>(wk + prev, o);
@@ -1042,17 +1072,25 @@ __global__ void __launch_bounds__(1024) k_group(const WalkSet ws, const WalkScra
         if (c == 0) continue;
         const int st = atomicAdd(&s_members, c);
         start[k] = st;
+        unsigned long long d[2][W];
+        load_det<W>(wk + rep[k], d);
+        bool cas = true;
+#pragma unroll
+        for (int sg = 0; sg < 2; sg++)
+#pragma unroll
+            for (int w = 0; w < W; w++) cas = cas && (d[sg][w] & S.mcore[w]) == S.mcore[w] && (d[sg][w] & S.mvirt[w]) == 0;
         const int ntg = (c + sc.tgw - 1) / sc.tgw;
-        const int at = atomicAdd(sc.ctl + 0, ntg), grp = atomicAdd(sc.ctl + 1, 1);
+        const int at = atomicAdd(sc.ctl + (cas ? CTL_TGC : CTL_TGF), ntg), grp = atomicAdd(sc.ctl + (cas ? CTL_GC : CTL_GF), 1);
+        TaskGroup* const tg = cas ? sc.tgc : sc.tgf;
         for (int q = 0; q < ntg; q++) {
             TaskGroup t;
             t.sys = sys;
             t.first = base + st + q * sc.tgw;
             t.count = min(sc.tgw, c - q * sc.tgw);
-            t.group = grp;
+            t.group = cas ? grp : (int)(sc.nseg - 1 - grp);
             t.primary = q == 0;
             t.pad = 0;
-            sc.tg[at + q] = t;
+            tg[at + q] = t;
         }
     }
     __syncthreads();
@@ -1073,9 +1111,9 @@ __global__ void __launch_bounds__(128) k_prep(const WalkSet ws, const WalkScratc
     __shared__ SysDev S;
     __shared__ WarpLists lists;
     int cur = -1;
-    const int ntg = sc.ctl[0];
+    const int ntc = sc.ctl[CTL_TGC], ntg = ntc + sc.ctl[CTL_TGF];
     for (int g = blockIdx.x; g < ntg; g += gridDim.x) {
-        const TaskGroup tg = sc.tg[g];
+        const TaskGroup tg = g < ntc ? sc.tgc[g] : sc.tgf[g - ntc];
         if (!tg.primary) continue;
         __syncthreads();
         if (tg.sys != cur) {
@@ -1088,10 +1126,12 @@ __global__ void __launch_bounds__(128) k_prep(const WalkSet ws, const WalkScratc
         load_det<W>(wk, n);
         int h, p;
         const long long ln = det_label<W>(S, n, h, p);
-        if (threadIdx.x < 32 && ln >= 0) {
-            double hnn, hdnn;
-            build_lists<W>(S, n, lists, h, p, threadIdx.x);
-            diagonals<W>(S, lists, n, threadIdx.x, hnn, hdnn);
+        if (threadIdx.x < 32) {
+            double hnn = 0.0, hdnn = 0.0;
+            if (ln >= 0) {
+                build_lists<W>(S, n, lists, h, p, threadIdx.x);
+                diagonals<W>(S, lists, n, threadIdx.x, hnn, hdnn);
+            }
             if (threadIdx.x == 0) {
                 GroupMeta m;
                 m.d[0][0] = m.d[0][1] = m.d[1][0] = m.d[1][1] = 0;
@@ -1105,107 +1145,572 @@ __global__ void __launch_bounds__(128) k_prep(const WalkSet ws, const WalkScratc
                 m.label = ln;
                 m.h = h;
                 m.p = p;
+                m.sys = tg.sys;
+                m.pad = 0;
                 sc.meta[tg.group] = m;
             }
-        } else if (threadIdx.x == 0) {
-            sc.meta[tg.group].label = -1;
         }
         NoCtr ctr;
         if (ln >= 0 && wk->psi != 0.0) walker_operator<W>(S, n, ln == 0, sc.gops + (long long)tg.group * sc.gstride, ctr);
     }
 }
 
-// Work units of every task group, as warp tasks (task group, slice): slice s of a determinant owns
-// units s, s + nslice, ...  Warps take tasks from a counter, so long and short tasks level out; the
-// slices of one determinant run all over the chip.
-template <int W, int MINB>
-__global__ void __launch_bounds__(MRQ_MAXNW * 32, MINB) k_eval(const WalkSet ws, const WalkScratch sc, int wbytes, int cap) {
-    extern __shared__ __align__(16) unsigned char smem_dyn[];
+// ---- warp tasks of k_int, k_pairs and k_fois
+
+// the next task of a warp
+__device__ __forceinline__ int next_task(int* counter, int lane) {
+    int id = 0;
+    if (lane == 0) id = atomicAdd(counter, 1);
+    return __shfl_sync(0xffffffffu, id, 0);
+}
+
+// the system of a warp's task, in its shared memory
+__device__ __forceinline__ void task_system(WarpTask& wt, const WalkSet& ws, int sys, int& cur, int lane) {
+    __syncwarp();
+    if (sys != cur) {
+        copy_sys(&wt.sys, ws.systems + sys, lane, 32);
+        cur = sys;
+        __syncwarp();
+    }
+}
+
+// the determinant of a task group and the Philox words and screens of its walkers; false when it cannot
+// be evaluated (outside the first-order space, or psi_s = 0)
+template <int W>
+__device__ __forceinline__ bool task_begin(WarpTask& wt, const WalkSet& ws, const WalkScratch& sc, const TaskGroup& tg,
+                                           int lane) {
+    const GroupMeta* const meta = sc.meta + tg.group;
+    const double psin = meta->psi;
+    if (meta->label < 0 || !(psin != 0.0)) return false;
+    if (lane < 2 * W) wt.nsh[lane] = meta->d[lane / W][lane % W];
+    const double inv = 1.0 / psin;
+    float inv_f = abs_f32_of(inv);
+    if (!(inv_f > 0.0f)) inv_f = INFINITY;
+    if (lane < tg.count) {
+        const int i = sc.members[tg.first + lane];
+        const Walker* const wk = ws.walkers[tg.sys] + i;
+        const int slot = (int)(ws.offsets[tg.sys] + i - sc.seg0);
+        const unsigned step = wk->step, wid = wk->wid;
+        uint4 a = race_walker_words(wt.sys.seed, step, wid);
+        const float b = __uint_as_float(__ldcg(sc.bound + slot));
+        a.w = __float_as_uint(race_scale(b, inv_f));
+        wt.bnd[lane] = b;
+        wt.wp[lane] = a;
+        wt.wid[lane] = wid;
+        wt.step[lane] = step;
+        wt.slot[lane] = (unsigned)slot;
+    }
+    if (lane == 0) {
+        wt.inv_psin = inv;
+        wt.inv_f = inv_f;
+        wt.qn = 0;
+    }
+    __syncwarp();
+    return true;
+}
+
+// partial sums of a task, stored by the determinant's primary group
+__device__ __forceinline__ void task_sums(const WalkScratch& sc, const TaskGroup& tg, int slice, double sA, double sT,
+                                          double sD, int lane) {
+    sA = warp_sum(sA);
+    sT = warp_sum(sT);
+    sD = warp_sum(sD);
+    if (lane == 0 && tg.primary) {
+        double* const p = sc.part + ((long long)tg.group * (sc.ns_max + MRQ_INT_SLICES) + slice) * 3;
+        p[0] = sA;
+        p[1] = sT;
+        p[2] = sD;
+    }
+}
+
+// neighbours inside the CAS.  They carry most of the total rate, so they run first: the later kernels
+// start with nearly final screens.
+template <int W>
+__global__ void __launch_bounds__(256, 3) k_int(const WalkSet ws, const WalkScratch sc) {
+    __shared__ WarpTask tasks[8];
     const int lane = threadIdx.x & 31;
-    unsigned char* const mine = smem_dyn + (size_t)(threadIdx.x >> 5) * wbytes;
-    WarpTask& wt = *reinterpret_cast<WarpTask*>(mine);
-    WarpLists& lists = *reinterpret_cast<WarpLists*>(mine + (sizeof(WarpTask) + 15) / 16 * 16);
-    double* const cphi = reinterpret_cast<double*>(&lists);      // CAS tasks: candidate list in the lists' place
-    unsigned* const ccode = reinterpret_cast<unsigned*>(cphi + cap);
+    WarpTask& wt = tasks[threadIdx.x >> 5];
     const SysDev& S = wt.sys;
     int cur = -1;
-    const int ntg = sc.ctl[0];
-    const long long ntask = (long long)ntg * sc.ns_max;
+    const int ntg = sc.ctl[CTL_TGC];
     NoCtr ctr;
     for (;;) {
-        int id = 0;
-        if (lane == 0) id = atomicAdd(sc.ctl + 2, 1);
-        id = __shfl_sync(0xffffffffu, id, 0);
-        if (id >= ntask) break;
-        const int slice = id / ntg, g = id - slice * ntg;
-        const TaskGroup tg = sc.tg[g];
-        __syncwarp();
-        if (tg.sys != cur) {
-            copy_sys(&wt.sys, ws.systems + tg.sys, lane, 32);
-            cur = tg.sys;
+        const int id = next_task(sc.ctl + CTL_INT, lane);
+        if (id >= ntg * MRQ_INT_SLICES) break;
+        const int slice = id / ntg;
+        const TaskGroup tg = sc.tgc[id - slice * ntg];
+        task_system(wt, ws, tg.sys, cur, lane);
+        double sA = 0.0, sT = 0.0;
+        if (task_begin<W>(wt, ws, sc, tg, lane)) {
+            const unsigned long long(&n)[2][W] = *reinterpret_cast<const unsigned long long(*)[2][W]>(wt.nsh);
+            if (lane == 0) wt.cw = cas_constants<W>(S, n, sc.meta[tg.group].psi);
             __syncwarp();
+            StepSink sink{wt, sc.best, sc.bound, tg.count, lane, 0.0, 0.0, 0.0};
+            for (int u = slice; u < S.cas_units; u += MRQ_INT_SLICES) cas_internal_unit<W>(S, wt.cw, n, u, lane, sink, ctr);
+            sink.finish();
+            sA = sink.sA;
+            sT = sink.sT;
         }
+        task_sums(sc, tg, sc.ns_max + slice, sA, sT, 0.0, lane);
+    }
+}
+
+// neighbours of first-order determinants
+template <int W, int MINB>
+__global__ void __launch_bounds__(256, MINB) k_fois(const WalkSet ws, const WalkScratch sc) {
+    __shared__ WarpTask tasks[8];
+    __shared__ WarpLists lists_sh[8];
+    const int lane = threadIdx.x & 31;
+    WarpTask& wt = tasks[threadIdx.x >> 5];
+    WarpLists& lists = lists_sh[threadIdx.x >> 5];
+    const SysDev& S = wt.sys;
+    int cur = -1;
+    const int ntg = sc.ctl[CTL_TGF];
+    NoCtr ctr;
+    for (;;) {
+        const int id = next_task(sc.ctl + CTL_FOIS, lane);
+        if (id >= (long long)ntg * sc.ns_max) break;
+        const int slice = id / ntg;
+        const TaskGroup tg = sc.tgf[id - slice * ntg];
+        task_system(wt, ws, tg.sys, cur, lane);
         if (slice >= S.nslice) continue;
-        const GroupMeta* const meta = sc.meta + tg.group;
-        const long long ln = meta->label;
-        const double psin = meta->psi;
-        double* const part = sc.part + ((long long)tg.group * sc.ns_max + slice) * 3;
-        if (ln < 0 || !(psin != 0.0)) {
-            if (lane < 3 && tg.primary) part[lane] = 0.0;
-            continue;
-        }
-        unsigned long long(&n)[2][W] = *reinterpret_cast<unsigned long long(*)[2][W]>(wt.nsh);
-        if (lane == 0) {
-#pragma unroll
-            for (int sg = 0; sg < 2; sg++)
-#pragma unroll
-                for (int w = 0; w < W; w++) n[sg][w] = meta->d[sg][w];
-        }
-        __syncwarp();
-        const float inv_f = abs_f32_of(1.0 / psin);
-        if (lane < tg.count) {
-            const int i = sc.members[tg.first + lane];
-            const Walker* const wk = ws.walkers[tg.sys] + i;
-            const int slot = (int)(ws.offsets[tg.sys] + i - sc.seg0);
-            const unsigned step = wk->step, wid = wk->wid;
-            uint4 a = race_walker_words(S.seed, step, wid);
-            const float b = __uint_as_float(__ldcg(sc.bound + slot));
-            a.w = __float_as_uint(race_scale(b, inv_f > 0.0f ? inv_f : INFINITY));
-            wt.bnd[lane] = b;
-            wt.wp[lane] = a;
-            wt.wid[lane] = wid;
-            wt.step[lane] = step;
-            wt.slot[lane] = (unsigned)slot;
-        }
-        if (lane == 0) {
-            wt.inv_psin = 1.0 / psin;
-            wt.inv_f = inv_f > 0.0f ? inv_f : INFINITY;
-            wt.qn = 0;
-            if (ln == 0) wt.cw = cas_constants<W>(S, n, psin);
-        }
-        __syncwarp();
-        StepSink sink{wt, sc.best, sc.bound, tg.count, lane, 0.0, 0.0, 0.0};
-        const double* const gops = sc.gops + (long long)tg.group * sc.gstride;
-        if (ln == 0) {
-            const int units = S.unit_off[8];
-            for (int u = slice; u < units; u += S.nslice) {
-                if (u < S.cas_units) cas_internal_unit<W>(S, wt.cw, n, u, lane, sink, ctr);
-                else cas_pair_unit<W>(S, wt.cw, gops, cphi, ccode, n, u, lane, sink, ctr);
-            }
-        } else {
+        double sA = 0.0, sT = 0.0, sD = 0.0;
+        if (task_begin<W>(wt, ws, sc, tg, lane)) {
+            const unsigned long long(&n)[2][W] = *reinterpret_cast<const unsigned long long(*)[2][W]>(wt.nsh);
+            const GroupMeta* const meta = sc.meta + tg.group;
+            StepSink sink{wt, sc.best, sc.bound, tg.count, lane, 0.0, 0.0, 0.0};
             build_lists<W>(S, n, lists, meta->h, meta->p, lane);
             const int total = lists.bstart[lists.nb], units = (total + MRQ_FOIS_CH - 1) / MRQ_FOIS_CH;
             for (int u = slice; u < units; u += S.nslice)
-                fois_unit<W>(S, lists, gops, n, ln, __ldg(S.c), MRQ_EMPTY_KEY, 0.0, u * MRQ_FOIS_CH,
-                             min(total, (u + 1) * MRQ_FOIS_CH), lane, sink, ctr);
+                fois_unit<W>(S, lists, sc.gops + (long long)tg.group * sc.gstride, n, meta->label, __ldg(S.c), MRQ_EMPTY_KEY,
+                             0.0, u * MRQ_FOIS_CH, min(total, (u + 1) * MRQ_FOIS_CH), lane, sink, ctr);
+            sink.finish();
+            sA = sink.sA;
+            sT = sink.sT;
+            sD = sink.sD;
         }
-        sink.finish();
-        const double sA = warp_sum(sink.sA), sT = warp_sum(sink.sT), sD = warp_sum(sink.sD);
-        if (lane == 0 && tg.primary) {
-            part[0] = sA;
-            part[1] = sT;
-            part[2] = sD;
+        task_sums(sc, tg, slice, sA, sT, sD, lane);
+    }
+}
+
+// ---- rows of a wave of CAS determinants
+
+// entries of the row (c core holes, v virtual electrons) of a remnant with d more active alpha electrons
+// than a CAS determinant: the groups (sc, sv = sc - d) one after the other
+__device__ __forceinline__ int row_len(const SysDev& S, int c, int v, int d) {
+    int len = 0;
+    for (int sc = 0; sc <= c; sc++) {
+        const int sv = sc - d;
+        if (sv < 0 || sv > v) continue;
+        len += shape_count(S.nc, c, sc) * shape_count(S.nv, v, sv);
+    }
+    return len;
+}
+
+// the row references of every determinant of the wave: remnant and class
+template <int W>
+__global__ void __launch_bounds__(256) k_refs(const WalkSet ws, const WalkScratch sc) {
+    const int ng = min(sc.wave_groups, sc.ctl[CTL_GC] - sc.wave0);
+    if (ng <= 0) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        sc.ctl[CTL_PAIRS] = sc.ctl[CTL_ROWTASK] = sc.ctl[CTL_BIG] = sc.ctl[CTL_SMALL] = 0;
+        *reinterpret_cast<unsigned long long*>(sc.ctl + CTL_CUR) = 0ull;
+    }
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < sc.table_size; k += gridDim.x * blockDim.x) sc.table[k] = -1;
+    for (int g = blockIdx.x; g < ng; g += gridDim.x) {
+        const GroupMeta& meta = sc.meta[sc.wave0 + g];
+        const SysDev& S = ws.systems[meta.sys];
+        unsigned long long n[2][W];
+#pragma unroll
+        for (int sg = 0; sg < 2; sg++)
+#pragma unroll
+            for (int w = 0; w < W; w++) n[sg][w] = meta.d[sg][w];
+        const unsigned ao0 = active_bits<W>(S, n[0]), ao1 = active_bits<W>(S, n[1]);
+        const unsigned amask = (S.na >= 32) ? 0xFFFFFFFFu : ((1u << S.na) - 1u);
+        const unsigned long long AO = (unsigned long long)ao0 | ((unsigned long long)ao1 << 32);
+        const unsigned long long AE = (unsigned long long)(~ao0 & amask) | ((unsigned long long)(~ao1 & amask) << 32);
+        const int cntO = __popcll(AO), cntE = __popcll(AE);
+        const long long at = (long long)g * sc.nref_max;
+        for (int q = threadIdx.x; q < sc.nref_max; q += blockDim.x) {
+            unsigned char cls = MRQ_NOROW;
+            if (q < S.ref_off[8]) {
+                int k = 0;
+                while (k < 7 && q >= S.ref_off[k + 1]) k++;
+                const int ka = k / 3, kb = k % 3, two = ka + kb == 1;       // (0,1) and (1,0) pairs own two rows
+                const int loc = q - S.ref_off[k], pair = two ? loc >> 1 : loc;
+                const int r = (ka + kb == 0 || (two && !(loc & 1))) ? 1 : 2;
+                const int nYa = nsub(cntE, kb), xa = pair / nYa, ya = pair - xa * nYa;
+                const unsigned long long Xb = subset_bits(S.colex, AO, cntO, ka, xa);
+                const unsigned long long Yb = subset_bits(S.colex, AE, cntE, kb, ya);
+                const int d = __popcll(Yb & 0xFFFFFFFFull) - __popcll(Xb & 0xFFFFFFFFull);
+                const int c = r - ka, v = r - kb;
+                sc.ref_ao[at + q] = (AO & ~Xb) | Yb;
+                if (row_len(S, c, v, d) > 0) cls = (unsigned char)(3 * c + v);
+            }
+            sc.ref_cls[at + q] = cls;
         }
+    }
+}
+
+// Distinct rows: every reference finds or becomes the owner of its (system, class, remnant) in an
+// open-addressing table with at least twice as many entries as references; owners get a place in the
+// row buffer (which holds the worst case of a wave, every row distinct).
+__global__ void __launch_bounds__(256) k_insert(const WalkSet ws, const WalkScratch sc) {
+    const int ng = min(sc.wave_groups, sc.ctl[CTL_GC] - sc.wave0);
+    if (ng <= 0) return;
+    const int total = ng * sc.nref_max, lane = threadIdx.x & 31;
+    for (int base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31; base < total; base += gridDim.x * blockDim.x) {
+        const int i = base + lane;
+        bool owner = false;
+        int len = 0;
+        if (i < total && sc.ref_cls[i] != MRQ_NOROW) {
+            const int cls = sc.ref_cls[i], sys = sc.meta[sc.wave0 + i / sc.nref_max].sys;
+            const unsigned long long ao = sc.ref_ao[i];
+            int k = (int)(mix64(ao + 0x9E3779B97F4A7C15ull * (unsigned)(9 * sys + cls + 1)) & (unsigned)(sc.table_size - 1));
+            for (int probe = 0; probe < sc.table_size; probe++) {
+                const int prev = atomicCAS(sc.table + k, -1, i);
+                if (prev < 0) {
+                    owner = true;
+                    sc.ref_rep[i] = i;
+                    break;
+                }
+                if (sc.ref_ao[prev] == ao && sc.ref_cls[prev] == cls && sc.meta[sc.wave0 + prev / sc.nref_max].sys == sys) {
+                    sc.ref_rep[i] = prev;
+                    break;
+                }
+                k = (k + 1) & (sc.table_size - 1);
+            }
+            if (owner) {
+                const SysDev& S = ws.systems[sys];
+                const int c = cls / 3, v = cls - 3 * c;
+                len = row_len(S, c, v, __popcll(ao & 0xFFFFFFFFull) - (S.nalpha - S.nc));
+                len = (len + 3) & ~3;                    // rows start on 32-byte sectors
+            }
+        }
+        // one atomic per warp for the places in the buffer and in the task list
+        int x = len;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        const unsigned big = __ballot_sync(0xffffffffu, owner && len >= MRQ_BIG_ROW);
+        const unsigned small = __ballot_sync(0xffffffffu, owner && len < MRQ_BIG_ROW);
+        unsigned long long cur = 0;
+        int nb = 0, ns = 0;
+        if (lane == 31 && x > 0) cur = atomicAdd(reinterpret_cast<unsigned long long*>(sc.ctl + CTL_CUR), (unsigned long long)x);
+        if (lane == 0 && big) nb = atomicAdd(sc.ctl + CTL_BIG, __popc(big));
+        if (lane == 0 && small) ns = atomicAdd(sc.ctl + CTL_SMALL, __popc(small));
+        cur = __shfl_sync(0xffffffffu, cur, 31);
+        nb = __shfl_sync(0xffffffffu, nb, 0);
+        ns = __shfl_sync(0xffffffffu, ns, 0);
+        if (owner) {
+            sc.row_off[i] = (long long)cur + x - len;
+            const unsigned lt = (1u << lane) - 1u;
+            const int all = sc.wave_groups * sc.nref_max;
+            if (len >= MRQ_BIG_ROW) sc.ulist[nb + __popc(big & lt)] = i;
+            else sc.ulist[all - 1 - (ns + __popc(small & lt))] = i;
+        }
+    }
+}
+
+// sum of a row's candidates e0, e0 + stride, ... < count for one neighbour: w T[base + lane part]
+__device__ __forceinline__ double row_doubles(const double* __restrict__ tab, const double* cphi, const unsigned* ccode,
+                                              int e, int count, int st, unsigned offd, unsigned offx) {
+    double a0 = 0.0, a1 = 0.0;
+    for (; e + 3 * st < count; e += 4 * st) {
+        const unsigned p0 = ccode[e], p1 = ccode[e + st], p2 = ccode[e + 2 * st], p3 = ccode[e + 3 * st];
+        const double x0 = __ldg(tab + (p0 & 0x7FFFFFFFu) + ((p0 & 0x80000000u) ? offx : offd));
+        const double x1 = __ldg(tab + (p1 & 0x7FFFFFFFu) + ((p1 & 0x80000000u) ? offx : offd));
+        const double x2 = __ldg(tab + (p2 & 0x7FFFFFFFu) + ((p2 & 0x80000000u) ? offx : offd));
+        const double x3 = __ldg(tab + (p3 & 0x7FFFFFFFu) + ((p3 & 0x80000000u) ? offx : offd));
+        a0 = fma(cphi[e], x0, a0);
+        a1 = fma(cphi[e + st], x1, a1);
+        a0 = fma(cphi[e + 2 * st], x2, a0);
+        a1 = fma(cphi[e + 3 * st], x3, a1);
+    }
+    for (; e < count; e += st) {
+        const unsigned p0 = ccode[e];
+        a0 = fma(cphi[e], __ldg(tab + (p0 & 0x7FFFFFFFu) + ((p0 & 0x80000000u) ? offx : offd)), a0);
+    }
+    return a0 + a1;
+}
+
+// The distinct rows, one warp task each.  Entry q of a group (core choice slow, virtual choice fast)
+// holds c_l O(m) (-1)^(core-hole positions of m): the sign that H_nm of the same neighbour carries too,
+// so k_pairs multiplies the two as they are.  Per group the warp builds the candidate list in shared
+// memory; a single candidate x -> y takes h_yx + sum over the remnant's electrons j of (yx|jj) -
+// (yj|jx) (the neighbour's own hole y and electron x drop out), a double one table read and one FMA.
+// Bound by FP64 (2 FMA per clock and SM): one read and one FMA per candidate.
+template <int W, int MINB>
+__global__ void __launch_bounds__(MRQ_MAXNW * 32, MINB) k_rows(const WalkSet ws, const WalkScratch sc, int lbytes, int cap) {
+    extern __shared__ __align__(16) unsigned char smem_dyn[];
+    const int lane = threadIdx.x & 31;
+    unsigned char* const mine = smem_dyn + (size_t)(threadIdx.x >> 5) * lbytes;
+    SysDev& S = *reinterpret_cast<SysDev*>(mine);
+    double* const cphi = reinterpret_cast<double*>(mine + (sizeof(SysDev) + 15) / 16 * 16);
+    unsigned* const ccode = reinterpret_cast<unsigned*>(cphi + cap);
+    if (sc.ctl[CTL_GC] <= sc.wave0) return;
+    int cur = -1;
+    const int nbig = sc.ctl[CTL_BIG], ntask = nbig + sc.ctl[CTL_SMALL], all = sc.wave_groups * sc.nref_max;
+    NoCtr ctr;
+    for (;;) {
+        const int id = next_task(sc.ctl + CTL_ROWTASK, lane);
+        if (id >= ntask) break;
+        const int i = id < nbig ? sc.ulist[id] : sc.ulist[all - 1 - (id - nbig)];
+        const int sys = sc.meta[sc.wave0 + i / sc.nref_max].sys;
+        __syncwarp();
+        if (sys != cur) {
+            copy_sys(&S, ws.systems + sys, lane, 32);
+            cur = sys;
+            __syncwarp();
+        }
+        const unsigned long long AO = sc.ref_ao[i];
+        const unsigned amask = (S.na >= 32) ? 0xFFFFFFFFu : ((1u << S.na) - 1u);
+        const unsigned long long AE = ~AO & ((unsigned long long)amask | ((unsigned long long)amask << 32));
+        const int c = sc.ref_cls[i] / 3, v = sc.ref_cls[i] - 3 * c;
+        const int d = __popcll(AO & 0xFFFFFFFFull) - (S.nalpha - S.nc);
+        double* row = sc.rows + sc.row_off[i];
+        const int voff = S.nc + S.na;
+        for (int scn = 0; scn <= c; scn++) {
+            const int sv = scn - d;
+            if (sv < 0 || sv > v) continue;
+            const int nvc = shape_count(S.nv, v, sv), ni = shape_count(S.nc, c, scn) * nvc;
+            if (ni == 0) continue;
+            // the group's first neighbour, for the candidates' signs
+            int xc[2] = {0, 0}, yv[2] = {0, 0};
+            shape_decode(S, S.nc, c, scn, 0, 0, xc, S.mag_c);
+            shape_decode(S, S.nv, v, sv, voff, 0, yv, S.mag_v);
+            unsigned long long m[2][W];
+#pragma unroll
+            for (int sg = 0; sg < 2; sg++) {
+                const unsigned long long a = sg ? AO >> 32 : AO & 0xFFFFFFFFull;
+#pragma unroll
+                for (int w = 0; w < W; w++) {
+                    const int sh = S.nc - 64 * w;                      // the active block may straddle a word
+                    m[sg][w] = S.mcore[w] | ((sh >= 0 ? (sh < 64 ? a << sh : 0ull) : (sh > -64 ? a >> -sh : 0ull)) & S.mact[w]);
+                }
+            }
+            for (int k = 0; k < c; k++) flip_reg<W>(m, xc[k] >= S.n, xc[k] - (xc[k] >= S.n ? S.n : 0));
+            for (int k = 0; k < v; k++) flip_reg<W>(m, yv[k] >= S.n, yv[k] - (yv[k] >= S.n ? S.n : 0));
+            unsigned offd, offx;
+            int par, n1;
+            lane_offsets(S, c, v, xc[0], xc[1], yv[0], yv[1], offd, offx, par);
+            const int count = build_group_list<W, true>(S, MRQ_EMPTY_KEY, m, AO, AE, c, v, scn, sv, xc[0], xc[1], yv[0], yv[1],
+                                                        par, cphi, ccode, n1, lane, ctr);
+            const unsigned long long mvc = ~0ull / (unsigned long long)nvc + 1ull;     // q / nvc by its high product
+            for (int qb = 0; qb < ni; qb += 32) {
+                const int nr = min(32, ni - qb), f = split_of(nr), lf = __ffs(f) - 1;
+                const int qi = lane >> lf, part = lane & (f - 1);
+                const int q = qb + min(qi, nr - 1);
+                const int ic = nvc == 1 ? q : (int)__umul64hi((unsigned long long)q, mvc);
+                shape_decode(S, S.nc, c, scn, 0, ic, xc, S.mag_c);
+                shape_decode(S, S.nv, v, sv, voff, q - ic * nvc, yv, S.mag_v);
+                lane_offsets(S, c, v, xc[0], xc[1], yv[0], yv[1], offd, offx, par);
+                double s = 0.0;
+                for (int e = part; e < n1; e += f) {
+                    const unsigned code = ccode[e];
+                    const int x = v ? yv[0] : act_so(S, (int)(code & 127u)), y = c ? xc[0] : act_so(S, (int)((code >> 14) & 127u));
+                    const int sx = x >= S.n, px = x - sx * S.n, py = y - sx * S.n;
+                    double g = __ldg(S.hc + py * S.n + px);
+                    const double* const col = S.sgl + py * S.nav + (px - S.nc);
+                    for (unsigned long long bits = AO; bits; bits &= bits - 1) {
+                        const int b = __ffsll(bits) - 1;
+                        g += __ldg(col + (long long)((b & 31) + (((b >= 32) == (sx == 1)) ? 0 : S.na)) * S.nca * S.nav);
+                    }
+                    s = fma(cphi[e], g, s);
+                }
+                s += row_doubles(S.tab, cphi, ccode, n1 + part, count, f, offd, offx);
+                for (int o = f >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                if (qi < nr && part == 0) {
+                    const int h0 = xc[0] >= S.n ? S.nc + (xc[0] - S.n) : xc[0], h1 = xc[1] >= S.n ? S.nc + (xc[1] - S.n) : xc[1];
+                    const int p0 = yv[0] >= S.n ? S.nv + (yv[0] - S.n - voff) : yv[0] - voff;
+                    const int p1 = yv[1] >= S.n ? S.nv + (yv[1] - S.n - voff) : yv[1] - voff;
+                    row[q] = __ldg(S.c + set_rank(c, h0, h1, 2 * S.nc) * S.nPs + set_rank(v, p0, p1, 2 * S.nv)) * s;
+                }
+            }
+            __syncwarp();
+            row += ni;
+        }
+    }
+}
+
+// The neighbours of the (X_a, Y_a) pairs of CAS determinants.  A group's neighbour is (core choice,
+// virtual choice); its element lies at an affine place of the physicists' table (or of the walker's
+// single-excitation operator, r = 1), its overlap times c_l at its place of the group's row, and its
+// excitation code is affine too, so a neighbour costs two reads, one product and the two sums.  The
+// sign of H_nm (-1)^(core-hole positions) is the same for the whole group.  (No active electron
+// moved and r = 2: the only reference determinant reached is the walker's, t = c_l H_nm^2 phi_0(n).)
+template <int W, int MINB>
+__global__ void __launch_bounds__(256, MINB) k_pairs(const WalkSet ws, const WalkScratch sc) {
+    __shared__ WarpTask tasks[8];
+    const int lane = threadIdx.x & 31;
+    WarpTask& wt = tasks[threadIdx.x >> 5];
+    const SysDev& S = wt.sys;
+    if (sc.ctl[CTL_GC] <= sc.wave0) return;
+    int cur = -1;
+    const int ntg = sc.ctl[CTL_TGC];
+    for (;;) {
+        const int id = next_task(sc.ctl + CTL_PAIRS, lane);
+        if (id >= (long long)ntg * sc.ns_max) break;
+        const int slice = id / ntg;
+        const TaskGroup tg = sc.tgc[id - slice * ntg];
+        if (tg.group < sc.wave0 || tg.group >= sc.wave0 + sc.wave_groups) continue;
+        task_system(wt, ws, tg.sys, cur, lane);
+        if (slice >= S.nslice) continue;
+        StepSink sink{wt, sc.best, sc.bound, tg.count, lane, 0.0, 0.0, 0.0};
+        if (task_begin<W>(wt, ws, sc, tg, lane)) {
+            const unsigned long long(&n)[2][W] = *reinterpret_cast<const unsigned long long(*)[2][W]>(wt.nsh);
+            const unsigned ao0 = active_bits<W>(S, n[0]), ao1 = active_bits<W>(S, n[1]);
+            const unsigned amask = (S.na >= 32) ? 0xFFFFFFFFu : ((1u << S.na) - 1u);
+            const unsigned long long AO = (unsigned long long)ao0 | ((unsigned long long)ao1 << 32);
+            const unsigned long long AE = (unsigned long long)(~ao0 & amask) | ((unsigned long long)(~ao1 & amask) << 32);
+            const int cntO = __popcll(AO), cntE = __popcll(AE), nc = S.nc, nv = S.nv, voff = S.nc + S.na;
+            const long long refs = (long long)(tg.group - sc.wave0) * sc.nref_max;
+            const double phin = sc.meta[tg.group].psi / __ldg(S.c);
+            for (int u = S.cas_units + slice; u < S.unit_off[8]; u += S.nslice) {
+                int k = 0;
+                while (k < 7 && u >= S.unit_off[k + 1]) k++;
+                const int ka = k / 3, kb = k % 3, nch = S.nch[k];
+                const int loc = u - S.unit_off[k], pair = loc / nch, ch = loc - pair * nch;
+                const int nYa = nsub(cntE, kb), xa = pair / nYa, ya = pair - xa * nYa;
+                const unsigned long long Xb = subset_bits(S.colex, AO, cntO, ka, xa);
+                const unsigned long long Yb = subset_bits(S.colex, AE, cntE, kb, ya);
+                const int d = __popcll(Yb & 0xFFFFFFFFull) - __popcll(Xb & 0xFFFFFFFFull);
+                const int tot = pair_total(S, ka, kb, d);
+                const int lo = (int)((long long)ch * tot / nch), hi = (int)((long long)(ch + 1) * tot / nch);
+                const int xa0 = Xb ? act_so(S, __ffsll(Xb) - 1) : 0, xa1 = ka == 2 ? act_so(S, 63 - __clzll(Xb)) : 0;
+                const int ya0 = Yb ? act_so(S, __ffsll(Yb) - 1) : 0, ya1 = kb == 2 ? act_so(S, 63 - __clzll(Yb)) : 0;
+                int base = 0;
+                int ref = S.ref_off[k] + (ka + kb == 1 ? 2 * pair : pair);
+                for (int r = max(1, max(ka, kb)); r <= 2; r++) {
+                    const int c = r - ka, v = r - kb;
+                    if (c == 0 && v == 0) continue;
+                    const bool self = c == 2 && v == 2;
+                    const double* row = sc.rows;
+                    if (!self) {
+                        if (sc.ref_cls[refs + ref] != MRQ_NOROW) row += sc.row_off[sc.ref_rep[refs + ref]];
+                        ref++;
+                    }
+                    for (int scn = 0; scn <= c; scn++) {
+                        const int sv = scn - d;
+                        if (sv < 0 || sv > v) continue;
+                        const int nvc = shape_count(nv, v, sv), ni = shape_count(nc, c, scn) * nvc;
+                        const int q0 = max(lo, base) - base, q1 = min(hi, base + ni) - base;
+                        if (ni > 0 && q0 < q1) {
+                            // the group's first neighbour, and how element and code change from it
+                            int xc0, xc1, yv0, yv1, rm0, rm1, ad0, ad1;
+                            unsigned long long m[2][W];
+                            group_neighbour<W>(S, n, nc, nv, voff, c, scn, v, sv, 0, 0, ka, xa0, xa1, kb, ya0, ya1, r, xc0, xc1,
+                                               yv0, yv1, rm0, rm1, ad0, ad1, m);
+                            const int cp0 = xc0 - (xc0 >= S.n ? S.n : 0), cp1 = xc1 - (xc1 >= S.n ? S.n : 0);
+                            const int vp0 = yv0 - (yv0 >= S.n ? S.n : 0) - voff, vp1 = yv1 - (yv1 >= S.n ? S.n : 0) - voff;
+                            const double* H;
+                            unsigned cs0 = 0, cs1 = 0, vs0 = 0, vs1 = 0, ce0 = 0, ce1 = 0, ve0 = 0, ve1 = 0, hb, eb;
+                            int odd = (c >= 1 ? cp0 : 0) + (c == 2 ? cp1 : 0);
+                            const unsigned sv1 = (unsigned)S.nav, sq = sv1 * sv1, sp = sq * (unsigned)S.nca;
+                            if (r == 1) {
+                                const int sx = rm0 >= S.n, px = rm0 - sx * S.n, py = ad0 - sx * S.n;
+                                H = sc.gops + (long long)tg.group * sc.gstride;
+                                hb = (unsigned)((sx * S.nca + px) * S.nav + (py - nc));
+                                odd += popc_sel<W>(n, sx, min(px, py), max(px, py));
+                                eb = exc_code(rm0, rm0, ad0, ad0);
+                                cs0 = sv1;
+                                vs0 = 1u;
+                                ce0 = 0x101u;
+                                ve0 = 0x1010000u;
+                            } else {
+                                const int s1 = rm0 >= S.n, s2 = rm1 >= S.n;
+                                int p1 = rm0 - s1 * S.n, p2 = rm1 - s2 * S.n;
+                                int a1 = ad0 - (ad0 >= S.n) * S.n, a2 = ad1 - (ad1 >= S.n) * S.n;
+                                int o = popc_sel<W>(n, s1, min(p1, a1), max(p1, a1));
+                                if (s1 == s2) {
+                                    unsigned long long t[W];
+#pragma unroll
+                                    for (int w = 0; w < W; w++) t[w] = s1 ? n[1][w] : n[0][w];
+                                    flip<W>(t, p1);
+                                    flip<W>(t, a1);
+                                    o += popc_between<W>(t, min(p2, a2), max(p2, a2));
+                                } else {
+                                    o += popc_sel<W>(n, s2, min(p2, a2), max(p2, a2));
+                                }
+                                odd += o;
+                                H = S.tab;
+                                eb = exc_code(rm0, rm1, ad0, ad1);
+                                const bool cfirst = c == 2 || (c == 1 && rm0 == xc0), vfirst = v == 2 || (v == 1 && ad0 == yv0);
+                                cs0 = cfirst ? sp : sq;
+                                cs1 = sq;
+                                ce0 = cfirst ? 0x1u : 0x100u;
+                                ce1 = 0x100u;
+                                vs0 = vfirst ? sv1 : 1u;
+                                vs1 = 1u;
+                                ve0 = vfirst ? 0x10000u : 0x1000000u;
+                                ve1 = 0x1000000u;
+                                if (v == 1 && vfirst) {
+                                    // <pq|rs> = <qp|sr>: the virtual index last, so that a warp reads consecutive words
+                                    int t = p1;
+                                    p1 = p2;
+                                    p2 = t;
+                                    t = a1;
+                                    a1 = a2;
+                                    a2 = t;
+                                    cs0 = cfirst ? sq : sp;
+                                    cs1 = sp;                  // (c = 2: the two holes are of opposite spin)
+                                    vs0 = 1u;
+                                }
+                                hb = (s1 == s2 ? S.tab_half : 0u) + (unsigned)p1 * sp + (unsigned)p2 * sq +
+                                     (unsigned)(a1 - nc) * sv1 + (unsigned)(a2 - nc);
+                            }
+                            if (c < 2) cs1 = ce1 = 0u;
+                            if (v < 2) vs1 = ve1 = 0u;
+                            if (c < 1) cs0 = ce0 = 0u;
+                            if (v < 1) vs0 = ve0 = 0u;
+                            hb -= (unsigned)cp0 * cs0 + (unsigned)cp1 * cs1 + (unsigned)vp0 * vs0 + (unsigned)vp1 * vs1;
+                            eb -= (unsigned)cp0 * ce0 + (unsigned)cp1 * ce1 + (unsigned)vp0 * ve0 + (unsigned)vp1 * ve1;
+                            const unsigned long long mvc = ~0ull / (unsigned long long)nvc + 1ull;
+                            for (int qb = q0; qb < q1; qb += 32) {
+                                const bool valid = qb + lane < q1;
+                                const int q = valid ? qb + lane : q1 - 1;
+                                const int ic = nvc == 1 ? q : (int)__umul64hi((unsigned long long)q, mvc), iv = q - ic * nvc;
+                                int i0 = ic, i1 = 0, j0 = iv, j1 = 0;
+                                if (c == 2) {
+                                    if (scn == 1) {
+                                        i0 = S.mag_c ? (int)__umul64hi((unsigned long long)ic, S.mag_c) : ic;
+                                        i1 = ic - i0 * nc;
+                                    } else {
+                                        lex_decode_tab(S.colex, ic, nc, i0, i1);
+                                    }
+                                }
+                                if (v == 2) {
+                                    if (sv == 1) {
+                                        j0 = S.mag_v ? (int)__umul64hi((unsigned long long)iv, S.mag_v) : iv;
+                                        j1 = iv - j0 * nv;
+                                    } else {
+                                        lex_decode_tab(S.colex, iv, nv, j0, j1);
+                                    }
+                                }
+                                const double h = H[hb + (unsigned)i0 * cs0 + (unsigned)i1 * cs1 + (unsigned)j0 * vs0 + (unsigned)j1 * vs1];
+                                const unsigned exc = eb + (unsigned)i0 * ce0 + (unsigned)i1 * ce1 + (unsigned)j0 * ve0 + (unsigned)j1 * ve1;
+                                double t;
+                                if (self) {
+                                    const int h0 = scn == 0 ? nc + i0 : i0, h1 = scn == 2 ? i1 : nc + i1;
+                                    const int p0 = sv == 0 ? nv + j0 : j0, p1 = sv == 2 ? j1 : nv + j1;
+                                    t = h * (h * phin) * __ldg(S.c + set_rank(2, h0, h1, 2 * nc) * S.nPs + set_rank(2, p0, p1, 2 * nv));
+                                } else {
+                                    t = neg_if(h * __ldcg(row + q), odd);
+                                }
+                                if (q1 - qb >= 32) sink.take(t, exc);
+                                else sink.push(valid, t, exc);
+                            }
+                        }
+                        base += ni;
+                        if (!self) row += ni;
+                    }
+                }
+            }
+            sink.finish();
+        }
+        task_sums(sc, tg, slice, sink.sA, sink.sT, 0.0, lane);
     }
 }
 
@@ -1236,18 +1741,22 @@ __global__ void __launch_bounds__(MRQ_MAXNW * 32) k_move(const WalkSet ws, const
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     double* const cphi = reinterpret_cast<double*>(smem_dyn + (size_t)warp * lbytes);
     unsigned* const ccode = reinterpret_cast<unsigned*>(cphi + cap);
-    const int ntg = sc.ctl[0];
+    const int ntc = sc.ctl[CTL_TGC], ntg = ntc + sc.ctl[CTL_TGF];
     for (int g = blockIdx.x * nw + warp; g < ntg; g += gridDim.x * nw) {
-        const TaskGroup tg = sc.tg[g];
+        const TaskGroup tg = g < ntc ? sc.tgc[g] : sc.tgf[g - ntc];
         const SysDev& S = ws.systems[tg.sys];
         const GroupMeta meta = sc.meta[tg.group];
         const double inv_psin = meta.psi != 0.0 ? 1.0 / meta.psi : 0.0;
         double A = 0.0, T = 0.0, D = 0.0;
-        const double* const part = sc.part + (long long)tg.group * sc.ns_max * 3;
+        const double* const part = sc.part + (long long)tg.group * (sc.ns_max + MRQ_INT_SLICES) * 3;
         for (int k = lane; k < S.nslice; k += 32) {
             A += part[3 * k];
             T += part[3 * k + 1];
             D += part[3 * k + 2];
+        }
+        if (g < ntc && lane < MRQ_INT_SLICES) {
+            A += part[3 * (sc.ns_max + lane)];
+            T += part[3 * (sc.ns_max + lane) + 1];
         }
         A = warp_sum(A);
         T = warp_sum(T);
@@ -1389,9 +1898,8 @@ __host__ __device__ __forceinline__ size_t debug_smem_bytes(int nw, int cap, int
     return (sizeof(DebugSh) + 15) / 16 * 16 + ((size_t)gstride * sizeof(double) + 15) / 16 * 16 +
            (size_t)nw * cand_list_bytes(cap);
 }
-__host__ __device__ __forceinline__ size_t eval_warp_bytes(int cap) {
-    const size_t l = cand_list_bytes(cap);
-    return (sizeof(WarpTask) + 15) / 16 * 16 + (l > sizeof(WarpLists) ? l : (sizeof(WarpLists) + 15) / 16 * 16);
+__host__ __device__ __forceinline__ size_t rows_warp_bytes(int cap) {
+    return (sizeof(SysDev) + 15) / 16 * 16 + cand_list_bytes(cap);
 }
 
 // local quantities of arbitrary determinants: one block per determinant, the walk's unit code
