@@ -962,6 +962,7 @@ struct mrq_ctx {
     unsigned char* d_work = nullptr;
     size_t work_cap = 0;
     long long row_worst = 0;         // doubles of one CAS determinant's rows when none is shared
+    int fg_max = 1;                  // groups of a first-order determinant's neighbours (at most)
     WalkScratch work{};
     double* d_partial = nullptr;
     long long partial_cap = 0;
@@ -977,10 +978,10 @@ struct mrq_ctx {
     struct GraphKey {
         const void *sys = nullptr, *wptr = nullptr, *off = nullptr, *work = nullptr;
         long long nslots = 0;
-        int k = 0, wpb = 0, spl = 0, cap = 0, gstride = 0, ns = 0, nref = 0;
+        int k = 0, wpb = 0, spl = 0, cap = 0, gstride = 0, ns = 0, nref = 0, fg = 0;
         bool operator==(const GraphKey& o) const {
             return sys == o.sys && wptr == o.wptr && off == o.off && work == o.work && nslots == o.nslots &&
-                   k == o.k && wpb == o.wpb && spl == o.spl && cap == o.cap && gstride == o.gstride && ns == o.ns && nref == o.nref;
+                   k == o.k && wpb == o.wpb && spl == o.spl && cap == o.cap && gstride == o.gstride && ns == o.ns && nref == o.nref && fg == o.fg;
         }
     };
     // per determinant width and warps per block (8, 4, 2, 1) of a batch launch
@@ -1008,6 +1009,7 @@ struct mrq_ctx {
     int cand_cap_full = 1;           // the candidate-list capacity the loaded system needs
     double l2_fraction = 0.0;        // mrq_set_l2_window: share of the persisting-L2 carve-out for the tables
     int rows_minb = 2, rows_blocks = 0;   // k_rows: build in use (resident blocks per SM) and grid
+    int frows_blocks = 0;            // k_frows' grid
 };
 
 static int fail(mrq_ctx* c, int code, const char* fmt, ...) {
@@ -1149,12 +1151,14 @@ struct WalkLaunch {
 // what a walk set's systems need: the largest candidate-list capacity, single-excitation operator and
 // slice count among them
 struct WalkNeed {
-    int cap = 1, gstride = 0, ns = 1, nref = 1;
-    long long row_worst = 1;
+    int cap = 1, gstride = 0, ns = MRQ_FOIS_SLICES, nref = 1, fg_max = 1;
+    long long row_worst = 1, fois_nb = 1;
     void add(const mrq_ctx* c) {
         const SysDev& s = c->hsys;
         nref = std::max(nref, s.ref_off[8]);
         row_worst = std::max(row_worst, c->row_worst);
+        fg_max = std::max(fg_max, c->fg_max);
+        fois_nb = std::max(fois_nb, s.cas_nb_total + 4);
         cap = std::max(cap, s.cand_cap);
         gstride = std::max(gstride, s.gstride);
         ns = std::max(ns, s.nslice);
@@ -1166,17 +1170,20 @@ struct WalkNeed {
 // the number of walkers: a segment's arrays hold one entry per walker, a wave's row buffer the worst
 // case that none of its determinants share a row.  When the device cannot give that much, waves shrink.
 #define MRQ_WORK_BYTES (1LL << 30)
-#define MRQ_ROW_BYTES (4LL << 30)
+#define MRQ_ROW_BYTES (8LL << 30)
 static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, long long* seg_out) {
     const long long per = 12 * 4 + 3 * 4 + 2 * (long long)sizeof(TaskGroup) + (long long)sizeof(GroupMeta) +
-                          8LL * need.gstride + 24LL * (need.ns + MRQ_INT_SLICES) + (long long)sizeof(RaceBest) + 4;
+                          8LL * need.gstride + 24LL * (need.ns + MRQ_ACT_SLICES) + (long long)sizeof(RaceBest) + 4;
     const long long seg = std::min(nslots, std::max(256LL, std::min(1LL << 20, MRQ_WORK_BYTES / per)));
     *seg_out = seg;
     const long long per_group = 8 * need.row_worst + 33LL * need.nref;
     long long groups = std::max(1LL, std::min(seg, MRQ_ROW_BYTES / per_group));
     groups = std::min(groups, std::max(1LL, (1LL << 29) / need.nref));           // reference indices and the table: 32 bits
+    const long long per_fois = 8 * need.fois_nb + (long long)sizeof(FGroup) * need.fg_max + 8;
+    long long fwave = std::max(1LL, std::min(seg, MRQ_ROW_BYTES / per_fois));
+    fwave = std::min(fwave, std::max(1LL, (1LL << 30) / need.fg_max));           // group indices: 32 bits
     WalkScratch& w = ctx->work;
-    for (;; groups = (groups + 1) / 2) {
+    for (;; groups = (groups + 1) / 2, fwave = (fwave + 1) / 2) {
         long long tsz = 2;
         while (tsz < 2 * groups * need.nref) tsz <<= 1;
         size_t off = 0;
@@ -1189,16 +1196,17 @@ static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, lo
         const size_t rep = take(16 * seg), cnt = take(16 * seg), start = take(16 * seg), tab = take(4 * seg),
                      pos = take(4 * seg), mem = take(4 * seg), tgc = take(sizeof(TaskGroup) * seg),
                      tgf = take(sizeof(TaskGroup) * seg), meta = take(sizeof(GroupMeta) * seg),
-                     gops = take(8 * (size_t)need.gstride * seg), part = take(24 * (size_t)(need.ns + MRQ_INT_SLICES) * seg),
+                     gops = take(8 * (size_t)need.gstride * seg), part = take(24 * (size_t)(need.ns + MRQ_ACT_SLICES) * seg),
                      best = take(sizeof(RaceBest) * seg), bound = take(4 * seg), ctl = take(4 * CTL_N), ao = take(8 * nr),
                      cls = take(nr), rrep = take(4 * nr), roff = take(8 * nr), tbl = take(4 * tsz), ul = take(4 * nr),
-                     rows = take(8 * (size_t)need.row_worst * groups);
+                     fgo = take(8 * fwave), fg = take(sizeof(FGroup) * (size_t)need.fg_max * fwave),
+                     rows = take(8 * std::max((size_t)need.row_worst * groups, (size_t)need.fois_nb * fwave));
         if (off > ctx->work_cap) {
             CK(cudaStreamSynchronize(ctx->stream));
             dfree(ctx->d_work);
             ctx->work_cap = 0;
             const cudaError_t e = cudaMalloc(&ctx->d_work, off);
-            if (e == cudaErrorMemoryAllocation && groups > 1) {
+            if (e == cudaErrorMemoryAllocation && (groups > 1 || fwave > 1)) {
                 cudaGetLastError();
                 ctx->d_work = nullptr;
                 continue;
@@ -1229,11 +1237,16 @@ static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, lo
         w.ulist = (int*)(b + ul);
         w.rows = (double*)(b + rows);
         w.table_size = (int)tsz;
+        w.fg_of = (int2*)(b + fgo);
+        w.fg = (FGroup*)(b + fg);
         break;
     }
     w.nref_max = need.nref;
     w.wave_groups = (int)groups;
     w.wave0 = 0;
+    w.fg_max = need.fg_max;
+    w.fwave = (int)fwave;
+    w.fwave0 = 0;
     w.gstride = need.gstride;
     w.ns_max = need.ns;
     w.nseg = seg;
@@ -1254,18 +1267,24 @@ static int rows_fits(mrq_ctx* ctx, size_t smem, int threads, int& blocks) {
 // that the candidate lists in shared memory allow, and a grid that fills the chip once
 static int rows_prepare(mrq_ctx* ctx, int W, int nw, int cap) {
     const size_t smem = nw * rows_warp_bytes(cap), lsm = nw * cand_list_bytes(cap);
-    int b4 = 0, b2 = 0;
+    const size_t fsm = nw * frows_warp_bytes(cap);
+    int b4 = 0, b2 = 0, bf = 0;
     if (W == 1) {
         if (int r = rows_fits<1, 4>(ctx, smem, 32 * nw, b4)) return r;
         if (int r = rows_fits<1, 2>(ctx, smem, 32 * nw, b2)) return r;
         CK(cudaFuncSetAttribute(k_move<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm));
+        CK(cudaFuncSetAttribute(k_frows<1, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm));
+        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bf, k_frows<1, 3>, 32 * nw, fsm));
     } else {
         if (int r = rows_fits<2, 4>(ctx, smem, 32 * nw, b4)) return r;
         if (int r = rows_fits<2, 2>(ctx, smem, 32 * nw, b2)) return r;
         CK(cudaFuncSetAttribute(k_move<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm));
+        CK(cudaFuncSetAttribute(k_frows<2, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm));
+        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bf, k_frows<2, 3>, 32 * nw, fsm));
     }
     ctx->rows_minb = b4 > b2 ? 4 : 2;
     ctx->rows_blocks = std::max(1, std::max(b4, b2)) * ctx->n_sm;
+    ctx->frows_blocks = std::max(1, bf) * ctx->n_sm;
     return 0;
 }
 
@@ -1279,12 +1298,20 @@ static int launch_segment(mrq_ctx* ctx, const WalkSet& ws, WalkScratch sc, const
     const long long n = sc.seg1 - sc.seg0;
     const int sms = ctx->n_sm;
     const cudaStream_t st = ctx->stream;
-    const size_t lbytes = cand_list_bytes(need.cap), rbytes = rows_warp_bytes(need.cap);
+    const size_t lbytes = cand_list_bytes(need.cap), rbytes = rows_warp_bytes(need.cap), fbytes = frows_warp_bytes(need.cap);
     if (ws.nsys > 1) CK(cudaMemsetAsync(sc.ctl, 0, sizeof(int) * CTL_N, st));
     k_group<W><<<(unsigned)ws.nsys, 1024, 0, st>>>(ws, sc);
     k_prep<W><<<(unsigned)std::min<long long>(n, 8LL * sms), 128, 0, st>>>(ws, sc);
     k_int<W><<<(unsigned)std::min<long long>(n, 3LL * sms), 256, 0, st>>>(ws, sc);
-    k_fois<W, 3><<<3 * sms, 256, 0, st>>>(ws, sc);
+    k_fois_act<W><<<(unsigned)std::min<long long>(4 * n, 3LL * sms), 256, 0, st>>>(ws, sc);
+    cfg.dynamicSmemBytes = 0;
+    for (long long g = 0; g < n; g += sc.fwave) {
+        sc.fwave0 = (int)g;
+        CK(cudaMemsetAsync(sc.ctl + CTL_FOIS, 0, sizeof(int) * (CTL_N - CTL_FOIS), st));
+        k_fgroups<W><<<(unsigned)std::min<long long>(n, 4LL * sms), 256, 0, st>>>(ws, sc);
+        k_frows<W, 3><<<(unsigned)ctx->frows_blocks, 32 * nw, nw * fbytes, st>>>(ws, sc, (int)fbytes, need.cap);
+        k_fois<W, 3><<<3 * sms, 256, 0, st>>>(ws, sc);
+    }
     for (long long g = 0; g < n; g += sc.wave_groups) {
         sc.wave0 = (int)g;
         k_refs<W><<<(unsigned)std::min<long long>(n, 8LL * sms), 256, 0, st>>>(ws, sc);
@@ -1408,6 +1435,22 @@ static int walk_plan(mrq_ctx* ctx, SysDev& s) {
     s.nslice = 32;
     while (s.nslice < MRQ_NS_MAX && s.nslice * 4 < off) s.nslice <<= 1;
     s.cas_nb_total = total;
+    // Groups of a first-order determinant's neighbours: the outer patterns of a pair (X_a, Y_a) of each
+    // class, at most (electrons removed: kinds of the virtual ones x alpha core ones; likewise added),
+    // for any number of active electrons the determinant may have, and the cuts of long groups.  (A
+    // determinant has as many singles and doubles in all as a CAS determinant.)
+    {
+        static const long long per[8] = {66, 45, 12, 45, 18, 6, 12, 6};
+        long long most = 0;
+        for (int o = std::max(0, cntO - 2); o <= std::min(2 * na, cntO + 2); o++) {
+            long long g = 0;
+            for (int k = 0; k < 8; k++) g += nsub_h(o, k / 3) * nsub_h(2 * na - o, k % 3) * per[k];
+            most = std::max(most, g);
+        }
+        most += total / MRQ_FG_NB + 1;
+        if (most > (1LL << 28)) return fail(ctx, MRQ_TOO_LARGE, "active space too large for the walk's work plan");
+        ctx->fg_max = (int)most;
+    }
     if (off > (1LL << 30) || total > (1LL << 40))
         return fail(ctx, MRQ_TOO_LARGE, "active space too large for the walk's work plan");
     // largest candidate list: m's active occupation differs from n's by at most two electrons
@@ -1443,7 +1486,7 @@ static int walk_plan(mrq_ctx* ctx, SysDev& s) {
     // warp the active space is too large for the walk
     ctx->max_nw = 0;
     for (int nw = MRQ_MAXNW; nw >= 1 && ctx->max_nw == 0; nw >>= 1)
-        if (debug_smem_bytes(nw, (int)cap, s.gstride) <= 227 * 1024 && nw * rows_warp_bytes((int)cap) <= 227 * 1024)
+        if (debug_smem_bytes(nw, (int)cap, s.gstride) <= 227 * 1024 && nw * frows_warp_bytes((int)cap) <= 227 * 1024)
             ctx->max_nw = nw;
     if (ctx->max_nw == 0)
         return fail(ctx, MRQ_TOO_LARGE, "active space too large for the shared-memory candidate lists");
@@ -2139,6 +2182,7 @@ static int batch_run(mrq_ctx* ctx, int W, const WalkSet& ws, const WalkNeed& nee
         key.gstride = need.gstride;
         key.ns = need.ns;
         key.nref = need.nref;
+        key.fg = need.fg_max;
         cudaGraphExec_t& ex = ctx->gexec[slot];
         if (!ex || !(ctx->gkey[slot] == key)) {
             if (ex) CK(cudaGraphExecDestroy(ex));

@@ -13,7 +13,9 @@
 //             determinants of a step share most of their active remnants, so the distinct rows
 //             (remnant, core holes, virtual electrons) are found and computed once;
 //   k_pairs   CAS determinants: every (X_a, Y_a) pair's neighbours, elements times rows;
-//   k_fois    first-order determinants: their neighbours, reach-back per lane;
+//   k_fois_act; k_fgroups, k_frows, k_fois
+//             first-order determinants: the neighbours that move active electrons only; the others, by
+//             groups that share an active remnant (k_fgroups finds them, k_frows their overlaps);
 //   k_move    adds the units' sums, takes each walker's winner, and looks up psi_s there;
 //   k_accum   adds the step records into the accumulators.
 // k_int, k_pairs and k_fois evaluate a determinant's neighbours once per task group, in work units
@@ -80,13 +82,29 @@ struct GroupMeta {
 enum {
     CTL_TGC, CTL_GC,              // CAS task groups, CAS determinants
     CTL_TGF, CTL_GF,              // first-order task groups, determinants
-    CTL_INT, CTL_PAIRS, CTL_FOIS, CTL_ROWTASK,   // next warp task of each kernel
+    CTL_INT, CTL_PAIRS, CTL_ACT, CTL_FOIS, CTL_ROWTASK,   // next warp task of each kernel
     CTL_BIG, CTL_SMALL,           // distinct rows of a wave: long ones (from the list's front), short ones
-    CTL_CUR,                      // (64 bits) doubles of the row buffer in use
+    CTL_FG, CTL_FGTASK,           // neighbour groups of a wave of first-order determinants, next task
+    CTL_PAD,
+    CTL_CUR,                      // (64 bits, aligned) doubles of the row buffer in use
     CTL_N = CTL_CUR + 2
 };
-#define MRQ_INT_SLICES 8          // warp tasks of a determinant's neighbours inside the CAS
+#define MRQ_INT_SLICES 8          // warp tasks of a CAS determinant's neighbours inside the CAS
+#define MRQ_ACT_SLICES 32         // warp tasks of a first-order determinant's active-only neighbours
+#define MRQ_FOIS_SLICES 256       // warp tasks of its other neighbours
 #define MRQ_BIG_ROW 1024          // entries of a long row
+#define MRQ_FG_NB 1024            // neighbours of a group of a first-order determinant (longer ones are cut)
+
+// Neighbours of a first-order determinant that share an active remnant and an outer pattern: core
+// electrons out (ac, sac of them alpha) and virtual orbitals entered (bv, sbv) run over all choices, the
+// av virtual electrons that leave (the xs-th, or both) and the bc holes that are filled are fixed.
+struct FGroup {
+    unsigned long long ao;    // the neighbours' active remnant
+    long long off;            // place of their psi_s in the row buffer
+    int det, q0, nq;          // determinant; neighbours q0 ... q0 + nq - 1 of the choices
+    unsigned char c, v, scn, sv;             // their core holes and virtual electrons (and alpha ones)
+    unsigned char ac, sac, bv, sbv, av, bc, xs, ys;
+};
 #define MRQ_NOROW 255             // a reference without entries
 
 // device workspace of a walk launch, sized for the slots [seg0, seg1) of the walk set
@@ -97,7 +115,7 @@ struct WalkScratch {
     TaskGroup *tgc, *tgf;     // CAS and first-order task groups
     GroupMeta* meta;          // per determinant: CAS ones from the front, first-order ones from the back
     double* gops;             // single-excitation operators, gstride doubles per determinant
-    double* part;             // [determinant][ns_max + MRQ_INT_SLICES][3] partial sums
+    double* part;             // [determinant][ns_max + MRQ_ACT_SLICES][3] partial sums (the last ones: k_int, k_fois_act)
     RaceBest* best;           // per slot
     unsigned* bound;          // per slot: FP32 bits of an upper bound of the best clock
     int* ctl;
@@ -110,6 +128,10 @@ struct WalkScratch {
     int *table, *ulist;           // open addressing over references; the owners
     double* rows;
     int table_size, nref_max, wave_groups, wave0;
+    // groups of a wave of at most fwave first-order determinants (fg_max each), in the same row buffer
+    FGroup* fg;
+    int2* fg_of;              // per determinant of the wave: first group, groups
+    int fg_max, fwave, fwave0;
     long long gstride, nseg;
     int ns_max, tgw;
     long long seg0, seg1;
@@ -349,6 +371,43 @@ __device__ __forceinline__ int cas_unit_count(const SysDev& S, const CasWalker& 
     return hi - lo;
 }
 
+// excitations of active electrons into active holes (coa, cob: occupied alpha, beta; cea, ceb: empty)
+__device__ __forceinline__ int active_neighbours(int coa, int cob, int cea, int ceb) {
+    return coa * cea + cob * ceb + nsub(coa, 2) * nsub(cea, 2) + nsub(cob, 2) * nsub(ceb, 2) + coa * cea * cob * ceb;
+}
+
+// the idx-th of them, spin-resolved (alpha singles, beta singles, alpha-alpha, beta-beta, alpha-beta
+// doubles): removed and added active bits; returns the rank
+__device__ __forceinline__ int active_neighbour(const SysDev& S, unsigned long long oa, unsigned long long ob,
+                                                unsigned long long ea, unsigned long long eb, int idx,
+                                                unsigned long long& Xb, unsigned long long& Yb) {
+    const int coa = __popcll(oa), cob = __popcll(ob), cea = __popcll(ea), ceb = __popcll(eb);
+    const int b0 = coa * cea, b1 = b0 + cob * ceb, b2 = b1 + nsub(coa, 2) * nsub(cea, 2),
+              b3 = b2 + nsub(cob, 2) * nsub(ceb, 2);
+    if (idx < b1) {
+        const bool al = idx < b0;
+        const int x = al ? idx : idx - b0, ny = al ? cea : ceb;
+        Xb = subset_bits(S.colex, al ? oa : ob, al ? coa : cob, 1, x / ny);
+        Yb = subset_bits(S.colex, al ? ea : eb, ny, 1, x % ny);
+        return 1;
+    }
+    if (idx < b3) {
+        const bool al = idx < b2;
+        const int x = al ? idx - b1 : idx - b2, ne = al ? cea : ceb, ny = nsub(ne, 2);
+        Xb = subset_bits(S.colex, al ? oa : ob, al ? coa : cob, 2, x / ny);
+        Yb = subset_bits(S.colex, al ? ea : eb, ne, 2, x % ny);
+        return 2;
+    }
+    int x = idx - b3;
+    const int yb = x % ceb;
+    x /= ceb;
+    const int xb = x % cob;
+    x /= cob;
+    Xb = subset_bits(S.colex, oa, coa, 1, x / cea) | subset_bits(S.colex, ob, cob, 1, xb);
+    Yb = subset_bits(S.colex, ea, cea, 1, x % cea) | subset_bits(S.colex, eb, ceb, 1, yb);
+    return 2;
+}
+
 // neighbours inside the CAS: spin-resolved blocks (alpha singles, beta singles, alpha-alpha,
 // beta-beta, alpha-beta doubles) of the walker's active electrons / holes
 template <int W, class Sink, class C>
@@ -356,10 +415,8 @@ __device__ __noinline__ void cas_internal_unit(const SysDev& S, const CasWalker&
                                                int u, int lane, Sink& sink, C& ctr) {
     const unsigned long long oa = cw.AOn & 0xFFFFFFFFull, ob = cw.AOn & ~0xFFFFFFFFull;
     const unsigned long long ea = cw.AEn & 0xFFFFFFFFull, eb = cw.AEn & ~0xFFFFFFFFull;
-    const int coa = __popcll(oa), cob = __popcll(ob), cea = __popcll(ea), ceb = __popcll(eb);
-    const int b0 = coa * cea, b1 = b0 + cob * ceb, b2 = b1 + nsub(coa, 2) * nsub(cea, 2),
-              b3 = b2 + nsub(cob, 2) * nsub(ceb, 2), b4 = b3 + coa * cea * cob * ceb;
-    const int i0 = u * MRQ_CAS_CH, i1 = min(b4, i0 + MRQ_CAS_CH);
+    const int i0 = u * MRQ_CAS_CH;
+    const int i1 = min(active_neighbours(__popcll(oa), __popcll(ob), __popcll(ea), __popcll(eb)), i0 + MRQ_CAS_CH);
     for (int base = i0; base < i1; base += 32) {
         const bool valid = base + lane < i1;
         const int idx = base + lane;
@@ -371,38 +428,8 @@ __device__ __noinline__ void cas_internal_unit(const SysDev& S, const CasWalker&
         double hnm = 0.0, om = 0.0, psim = 0.0;
         unsigned exc = 0;
         if (valid) {
-            unsigned long long Xb = 0, Yb = 0;
-            int r;
-            if (idx < b0) {
-                r = 1;
-                Xb = subset_bits(S.colex, oa, coa, 1, idx / cea);
-                Yb = subset_bits(S.colex, ea, cea, 1, idx % cea);
-            } else if (idx < b1) {
-                const int x = idx - b0;
-                r = 1;
-                Xb = subset_bits(S.colex, ob, cob, 1, x / ceb);
-                Yb = subset_bits(S.colex, eb, ceb, 1, x % ceb);
-            } else if (idx < b2) {
-                const int x = idx - b1, ny = nsub(cea, 2);
-                r = 2;
-                Xb = subset_bits(S.colex, oa, coa, 2, x / ny);
-                Yb = subset_bits(S.colex, ea, cea, 2, x % ny);
-            } else if (idx < b3) {
-                const int x = idx - b2, ny = nsub(ceb, 2);
-                r = 2;
-                Xb = subset_bits(S.colex, ob, cob, 2, x / ny);
-                Yb = subset_bits(S.colex, eb, ceb, 2, x % ny);
-            } else {
-                int x = idx - b3;
-                r = 2;
-                const int yb = x % ceb;
-                x /= ceb;
-                const int xb = x % cob;
-                x /= cob;
-                const int ya = x % cea, xa = x / cea;
-                Xb = subset_bits(S.colex, oa, coa, 1, xa) | subset_bits(S.colex, ob, cob, 1, xb);
-                Yb = subset_bits(S.colex, ea, cea, 1, ya) | subset_bits(S.colex, eb, ceb, 1, yb);
-            }
+                unsigned long long Xb, Yb;
+            const int r = active_neighbour(S, oa, ob, ea, eb, idx, Xb, Yb);
             int rem[2], add[2];
             act_list(S, Xb, rem);
             act_list(S, Yb, add);
@@ -604,12 +631,108 @@ __device__ __noinline__ void fois_unit(const SysDev& S, const WarpLists& sh, con
     }
 }
 
-// overlap O(m) = <m|H|phi0> (Eq. 6-7) of one first-order determinant m by a whole warp: m's
-// candidate list as of a group of one neighbour, the list's terms split over the lanes
+// ------------------------------------------------------------------ overlaps outside the CAS
+//
+// O(m) of a determinant m with active remnant A, c core holes and v virtual electrons (scn, sv of them
+// alpha): the warp builds the candidate list of (A, c, v, scn, sv) once (row_list), and every m of that
+// class sums it with its own orbitals' part of the table index (row_overlap).  The sum's sign is m's
+// up to (-1)^(core-hole positions).
+
+// the candidate list in shared memory; its signs are those of the class's first determinant (core holes
+// and virtual electrons in the lowest orbitals).  Returns the entries, n1 of them singles.
+template <int W, class C>
+__device__ __noinline__ int row_list(const SysDev& S, unsigned long long AO, int c, int v, int scn, int sv, double* cphi,
+                                     unsigned* ccode, int& n1, int lane, C& ctr) {
+    const unsigned amask = (S.na >= 32) ? 0xFFFFFFFFu : ((1u << S.na) - 1u);
+    const unsigned long long AE = ~AO & ((unsigned long long)amask | ((unsigned long long)amask << 32));
+    int xc[2] = {0, 0}, yv[2] = {0, 0};
+    shape_decode(S, S.nc, c, scn, 0, 0, xc, S.mag_c);
+    shape_decode(S, S.nv, v, sv, S.nc + S.na, 0, yv, S.mag_v);
+    unsigned long long m[2][W];
+#pragma unroll
+    for (int sg = 0; sg < 2; sg++) {
+        const unsigned long long a = sg ? AO >> 32 : AO & 0xFFFFFFFFull;
+#pragma unroll
+        for (int w = 0; w < W; w++) {
+            const int sh = S.nc - 64 * w;                      // the active block may straddle a word
+            m[sg][w] = S.mcore[w] | ((sh >= 0 ? (sh < 64 ? a << sh : 0ull) : (sh > -64 ? a >> -sh : 0ull)) & S.mact[w]);
+        }
+    }
+    int par = 0;
+    for (int k = 0; k < c; k++) {
+        const int x = xc[k] - (xc[k] >= S.n ? S.n : 0);
+        flip_reg<W>(m, xc[k] >= S.n, x);
+        par += x;
+    }
+    for (int k = 0; k < v; k++) flip_reg<W>(m, yv[k] >= S.n, yv[k] - (yv[k] >= S.n ? S.n : 0));
+    return build_group_list<W, true>(S, MRQ_EMPTY_KEY, m, AO, AE, c, v, scn, sv, xc[0], xc[1], yv[0], yv[1], par, cphi,
+                                     ccode, n1, lane, ctr);
+}
+
+// candidates e, e + st, ... < count: w T[base + lane part]
+__device__ __forceinline__ double row_doubles(const double* __restrict__ tab, const double* cphi, const unsigned* ccode,
+                                              int e, int count, int st, unsigned offd, unsigned offx) {
+    double a0 = 0.0, a1 = 0.0;
+    for (; e + 3 * st < count; e += 4 * st) {
+        const unsigned p0 = ccode[e], p1 = ccode[e + st], p2 = ccode[e + 2 * st], p3 = ccode[e + 3 * st];
+        const double x0 = __ldg(tab + (p0 & 0x7FFFFFFFu) + ((p0 & 0x80000000u) ? offx : offd));
+        const double x1 = __ldg(tab + (p1 & 0x7FFFFFFFu) + ((p1 & 0x80000000u) ? offx : offd));
+        const double x2 = __ldg(tab + (p2 & 0x7FFFFFFFu) + ((p2 & 0x80000000u) ? offx : offd));
+        const double x3 = __ldg(tab + (p3 & 0x7FFFFFFFu) + ((p3 & 0x80000000u) ? offx : offd));
+        a0 = fma(cphi[e], x0, a0);
+        a1 = fma(cphi[e + st], x1, a1);
+        a0 = fma(cphi[e + 2 * st], x2, a0);
+        a1 = fma(cphi[e + 3 * st], x3, a1);
+    }
+    for (; e < count; e += st) {
+        const unsigned p0 = ccode[e];
+        a0 = fma(cphi[e], __ldg(tab + (p0 & 0x7FFFFFFFu) + ((p0 & 0x80000000u) ? offx : offd)), a0);
+    }
+    return a0 + a1;
+}
+
+// The list's sum for the determinant with core holes xc and virtual electrons yv (sorted), the entries
+// part, part + f, ... of it added over f neighbouring lanes; par is its core parity.  A single candidate
+// x -> y takes h_yx + sum over the remnant's electrons j of (yx|jj) - (yj|jx): m's own hole y and electron
+// x drop out.  A double is one table read and one FMA.
+__device__ __forceinline__ double row_overlap(const SysDev& S, unsigned long long AO, int c, int v, int xc0, int xc1, int yv0,
+                                              int yv1, const double* cphi, const unsigned* ccode, int n1, int count, int part,
+                                              int f, int& par) {
+    unsigned offd, offx;
+    lane_offsets(S, c, v, xc0, xc1, yv0, yv1, offd, offx, par);
+    double s = 0.0;
+    for (int e = part; e < n1; e += f) {
+        const unsigned code = ccode[e];
+        const int x = v ? yv0 : act_so(S, (int)(code & 127u)), y = c ? xc0 : act_so(S, (int)((code >> 14) & 127u));
+        const int sx = x >= S.n, px = x - sx * S.n, py = y - sx * S.n;
+        double g = __ldg(S.hc + py * S.n + px);
+        const double* const col = S.sgl + py * S.nav + (px - S.nc);
+        for (unsigned long long bits = AO; bits; bits &= bits - 1) {
+            const int b = __ffsll(bits) - 1;
+            g += __ldg(col + (long long)((b & 31) + (((b >= 32) == (sx == 1)) ? 0 : S.na)) * S.nca * S.nav);
+        }
+        s = fma(cphi[e], g, s);
+    }
+    s += row_doubles(S.tab, cphi, ccode, n1 + part, count, f, offd, offx);
+    for (int o = f >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+// label of core holes xc and virtual electrons yv (sorted)
+__device__ __forceinline__ long long row_label(const SysDev& S, int c, int v, int xc0, int xc1, int yv0, int yv1) {
+    const int voff = S.nc + S.na;
+    const int h0 = xc0 >= S.n ? S.nc + (xc0 - S.n) : xc0, h1 = xc1 >= S.n ? S.nc + (xc1 - S.n) : xc1;
+    const int p0 = yv0 >= S.n ? S.nv + (yv0 - S.n - voff) : yv0 - voff;
+    const int p1 = yv1 >= S.n ? S.nv + (yv1 - S.n - voff) : yv1 - voff;
+    return set_rank(c, h0, h1, 2 * S.nc) * S.nPs + set_rank(v, p0, p1, 2 * S.nv);
+}
+
+// core holes and virtual electrons of a determinant (at most two each, spin orbitals, sorted)
 template <int W>
-__device__ __noinline__ double reach_back_warp(const SysDev& S, const unsigned long long (&m)[2][W], double* cphi,
-                                               unsigned* ccode, int lane) {
-    int c = 0, v = 0, xc[2] = {0, 0}, yv[2] = {0, 0}, sc = 0, sv = 0;
+__device__ __forceinline__ void outer_orbitals(const SysDev& S, const unsigned long long (&m)[2][W], int& c, int& v, int* xc,
+                                               int* yv) {
+    c = v = 0;
+    xc[0] = xc[1] = yv[0] = yv[1] = 0;
 #pragma unroll
     for (int sg = 0; sg < 2; sg++) {
         unsigned long long hm = ~m[sg][0] & S.mcore[0];
@@ -619,7 +742,6 @@ __device__ __noinline__ double reach_back_warp(const SysDev& S, const unsigned l
             if (c == 0) xc[0] = sg * S.n + i;
             else xc[1] = sg * S.n + i;
             c++;
-            sc += sg == 0;
         }
 #pragma unroll
         for (int w = 0; w < W; w++) {
@@ -630,28 +752,24 @@ __device__ __noinline__ double reach_back_warp(const SysDev& S, const unsigned l
                 if (v == 0) yv[0] = sg * S.n + a;
                 else yv[1] = sg * S.n + a;
                 v++;
-                sv += sg == 0;
             }
         }
     }
-    const unsigned ao0 = active_bits<W>(S, m[0]), ao1 = active_bits<W>(S, m[1]);
-    const unsigned amask = (S.na >= 32) ? 0xFFFFFFFFu : ((1u << S.na) - 1u);
-    const unsigned long long AOm = (unsigned long long)ao0 | ((unsigned long long)ao1 << 32);
-    const unsigned long long AEm = (unsigned long long)(~ao0 & amask) | ((unsigned long long)(~ao1 & amask) << 32);
-    unsigned offd, offx;
-    int par, n1;
-    lane_offsets(S, c, v, xc[0], xc[1], yv[0], yv[1], offd, offx, par);
+}
+
+// O(m) of one first-order determinant by a whole warp
+template <int W>
+__device__ __noinline__ double reach_back_warp(const SysDev& S, const unsigned long long (&m)[2][W], double* cphi,
+                                               unsigned* ccode, int lane) {
+    int c, v, xc[2], yv[2];
+    outer_orbitals<W>(S, m, c, v, xc, yv);
+    const int scn = (c >= 1 && xc[0] < S.n) + (c == 2 && xc[1] < S.n), sv = (v >= 1 && yv[0] < S.n) + (v == 2 && yv[1] < S.n);
+    const unsigned long long AO =
+        (unsigned long long)active_bits<W>(S, m[0]) | ((unsigned long long)active_bits<W>(S, m[1]) << 32);
     NoCtr ctr;
-    const int count = build_group_list<W, false>(S, MRQ_EMPTY_KEY, m, AOm, AEm, c, v, sc, sv, xc[0], xc[1], yv[0], yv[1], par,
-                                          cphi, ccode, n1, lane, ctr);
-    double s = 0.0;
-    for (int e = lane; e < n1; e += 32)
-        s = fma(cphi[e], neg_if(sgl_elem_code<W>(S, nullptr, m, ccode[e], v, yv[0], c, xc[0], 0, 0, 0, 0, 0, ctr), par), s);
-    for (int e = n1 + lane; e < count; e += 32) {
-        const unsigned p0 = ccode[e];
-        s = fma(cphi[e], __ldg(S.tab + (p0 & 0x7FFFFFFFu) + ((p0 & 0x80000000u) ? offx : offd)), s);
-    }
-    s = warp_sum(s);
+    int n1, par;
+    const int count = row_list<W>(S, AO, c, v, scn, sv, cphi, ccode, n1, lane, ctr);
+    const double s = row_overlap(S, AO, c, v, xc[0], xc[1], yv[0], yv[1], cphi, ccode, n1, count, lane, 32, par);
     __syncwarp();
     return neg_if(s, par);
 }
@@ -761,8 +879,8 @@ struct WarpTask {
     uint4 wp[MRQ_TGW];                  // per walker: Philox words (x, y) and screen scale (w, FP32)
     unsigned wid[MRQ_TGW], step[MRQ_TGW], slot[MRQ_TGW];
     float bnd[MRQ_TGW];                 // upper bound of the best clock
-    double qt[64];                      // queued neighbours: t and excitation
-    unsigned qe[64];
+    double qt[96];                      // queued neighbours: t and excitation
+    unsigned qe[96];
 };
 
 // the screen's scale of a walker whose best clock is at most `bound`: a neighbour of rate Gamma =
@@ -810,18 +928,18 @@ __device__ __forceinline__ bool atomic_cas128(RaceBest* at, const RaceBest& cmp,
 // whether two FP32 clocks (relative error below 1e-5) leave the order of the exact ones open
 __device__ __forceinline__ bool clocks_near(float a, float b) { return !(a < b * 0.9999f) && !(b < a * 0.9999f); }
 
-// Lanes whose neighbour passed walker j's screen: of those that also pass the closer screen
-// (race_may_win) take the smallest clock, settle near ties by
+// Some lane's neighbour passed walker j's screen: of those that pass the closer one (race_may_win)
+// take the smallest clock, settle near ties by
 // the exact FP64 clocks (then the smaller excitation), and replace the walker's best if it is beaten.
 // Runs a handful of times per walker and step.
 __device__ __noinline__ void race_slow(WarpTask& wt, RaceBest* best, unsigned* bound, int j, double t, unsigned exc,
-                                       bool pass, int lane) {
+                                       int lane) {
     const unsigned long long seed = wt.sys.seed;
     const unsigned step = wt.step[j], wid = wt.wid[j];
     const unsigned long long k = race_bits(seed, exc, step, wid);
     const double g = fabs(t * wt.inv_psin);
     const float gf = abs_f32_of(g);
-    const bool ok = pass && g > 0.0 && race_may_win(k, gf, wt.bnd[j]);
+    const bool ok = g > 0.0 && race_may_win(k, gf, wt.bnd[j]);
     float a = INFINITY;
     if (ok) {
         const float w = (float)(9007199254740991ull - k) * 1.1102230246251565e-16f;
@@ -896,33 +1014,50 @@ __device__ __noinline__ void race_slow(WarpTask& wt, RaceBest* best, unsigned* b
     __syncwarp();
 }
 
-// 32 neighbours (one per lane; t = 0: none) against the clocks of the task's walkers.  Bound by the
-// integer pipe: about 45 instructions per neighbour and walker.
-__device__ __noinline__ void race_round(WarpTask& wt, RaceBest* best, unsigned* bound, double t, unsigned exc, int count,
-                                        int lane) {
-    float gf = -1.0f;                                   // t = 0 never passes
-    if ((__double_as_longlong(t) << 1) != 0) {
-        gf = abs_f32_of(t);
-        if (gf == 0.0f) gf = INFINITY;                  // outside FP32: the exact clock decides
-    }
+// the FP32 |t| of the screen
+__device__ __forceinline__ float race_rate(double t) {
+    if ((__double_as_longlong(t) << 1) == 0) return -1.0f;          // no neighbour: never passes
+    const float gf = abs_f32_of(t);
+    return gf == 0.0f ? INFINITY : gf;                              // outside FP32: the exact clock decides
+}
+
+// 64 neighbours (two per lane; t = 0: none) against the clocks of the task's walkers; returns the
+// walkers that some neighbour may win.  Bound by the integer pipes: 15 products and about 20 logic
+// operations per neighbour and walker.  Two neighbours per lane share a walker's words and the loop; the
+// rare candidates are settled by the caller, so that the loop holds no call and spills nothing.
+__device__ __noinline__ unsigned race_round(const WarpTask& wt, double t0, unsigned exc0, double t1, unsigned exc1,
+                                            int count) {
+    const float gf0 = race_rate(t0), gf1 = race_rate(t1);
     const unsigned kx = (unsigned)wt.sys.seed, ky = (unsigned)(wt.sys.seed >> 32);
-    const unsigned z1 = __umulhi(PHILOX_M0, exc) ^ ky, w1 = PHILOX_M0 * exc;
-    const unsigned e1 = __umulhi(PHILOX_M1, z1), e2 = PHILOX_M1 * z1;
+    const unsigned za = __umulhi(PHILOX_M0, exc0) ^ ky, wa = PHILOX_M0 * exc0;
+    const unsigned zb = __umulhi(PHILOX_M0, exc1) ^ ky, wb = PHILOX_M0 * exc1;
+    const unsigned ha = __umulhi(PHILOX_M1, za), la = PHILOX_M1 * za;
+    const unsigned hb = __umulhi(PHILOX_M1, zb), lb = PHILOX_M1 * zb;
+    unsigned hits = 0;
     for (int j = 0; j < count; j++) {
         const uint4 a = wt.wp[j];
-        unsigned c0 = e1 ^ a.x, c1 = e2, c2 = w1 ^ a.y, c3 = a.z;
+        unsigned c0 = ha ^ a.x, c1 = la, c2 = wa ^ a.y, c3 = a.z;
+        unsigned d0 = hb ^ a.x, d1 = lb, d2 = wb ^ a.y, d3 = a.z;
 #pragma unroll
         for (int r = 2; r < 9; r++) {
+            const unsigned k0 = kx + (unsigned)r * PHILOX_W0, k1 = ky + (unsigned)r * PHILOX_W1;
             const unsigned long long p0 = (unsigned long long)PHILOX_M0 * c0, p1 = (unsigned long long)PHILOX_M1 * c2;
-            c0 = (unsigned)(p1 >> 32) ^ c1 ^ (kx + (unsigned)r * PHILOX_W0);
+            const unsigned long long q0 = (unsigned long long)PHILOX_M0 * d0, q1 = (unsigned long long)PHILOX_M1 * d2;
+            c0 = (unsigned)(p1 >> 32) ^ c1 ^ k0;
             c1 = (unsigned)p1;
-            c2 = (unsigned)(p0 >> 32) ^ c3 ^ (ky + (unsigned)r * PHILOX_W1);
+            c2 = (unsigned)(p0 >> 32) ^ c3 ^ k1;
             c3 = (unsigned)p0;
+            d0 = (unsigned)(q1 >> 32) ^ d1 ^ k0;
+            d1 = (unsigned)q1;
+            d2 = (unsigned)(q0 >> 32) ^ d3 ^ k1;
+            d3 = (unsigned)q0;
         }
-        const unsigned x = __umulhi(PHILOX_M1, c2) ^ c1 ^ (kx + 9u * PHILOX_W0);
-        const bool pass = race_pass(x, gf, __uint_as_float(a.w));
-        if (__any_sync(0xffffffffu, pass)) race_slow(wt, best, bound, j, t, exc, pass, lane);
+        const unsigned k9 = kx + 9u * PHILOX_W0;
+        const unsigned x = __umulhi(PHILOX_M1, c2) ^ c1 ^ k9, y = __umulhi(PHILOX_M1, d2) ^ d1 ^ k9;
+        const float scale = __uint_as_float(a.w);
+        if (__any_sync(0xffffffffu, race_pass(x, gf0, scale) || race_pass(y, gf1, scale))) hits |= 1u << j;
     }
+    return hits;
 }
 
 // neighbours of a walk step: queued so that the sums and the race run with full lanes
@@ -949,11 +1084,11 @@ struct StepSink {
         }
         qn += __popc(m);
         __syncwarp();
-        if (qn >= 32) {
-            take(wt.qt[lane], wt.qe[lane]);
-            qn -= 32;
-            const double t2 = wt.qt[32 + lane];
-            const unsigned e2 = wt.qe[32 + lane];
+        if (qn >= 64) {
+            take(wt.qt[lane], wt.qe[lane], wt.qt[32 + lane], wt.qe[32 + lane]);
+            qn -= 64;
+            const double t2 = wt.qt[64 + lane];
+            const unsigned e2 = wt.qe[64 + lane];
             __syncwarp();
             if (lane < qn) {
                 wt.qt[lane] = t2;
@@ -963,14 +1098,22 @@ struct StepSink {
         if (lane == 0) wt.qn = qn;
         __syncwarp();
     }
-    __device__ __forceinline__ void take(double t, unsigned exc) {
-        sA += fabs(t);
-        sT += t;
-        race_round(wt, best, bound, t, exc, count, lane);
+    __device__ __forceinline__ void take(double t0, unsigned e0, double t1, unsigned e1) {
+        sA += fabs(t0);
+        sT += t0;
+        sA += fabs(t1);
+        sT += t1;
+        for (unsigned hits = race_round(wt, t0, e0, t1, e1, count); hits; hits &= hits - 1) {
+            const int j = __ffs(hits) - 1;
+            race_slow(wt, best, bound, j, t0, e0, lane);
+            race_slow(wt, best, bound, j, t1, e1, lane);
+        }
     }
     __device__ __forceinline__ void finish() {
         const int qn = wt.qn;
-        if (qn > 0) take(lane < qn ? wt.qt[lane] : 0.0, lane < qn ? wt.qe[lane] : 0u);
+        if (qn > 0)
+            take(lane < qn ? wt.qt[lane] : 0.0, lane < qn ? wt.qe[lane] : 0u, 32 + lane < qn ? wt.qt[32 + lane] : 0.0,
+                 32 + lane < qn ? wt.qe[32 + lane] : 0u);
     }
 };
 
@@ -1216,7 +1359,7 @@ __device__ __forceinline__ void task_sums(const WalkScratch& sc, const TaskGroup
     sT = warp_sum(sT);
     sD = warp_sum(sD);
     if (lane == 0 && tg.primary) {
-        double* const p = sc.part + ((long long)tg.group * (sc.ns_max + MRQ_INT_SLICES) + slice) * 3;
+        double* const p = sc.part + ((long long)tg.group * (sc.ns_max + MRQ_ACT_SLICES) + slice) * 3;
         p[0] = sA;
         p[1] = sT;
         p[2] = sD;
@@ -1255,41 +1398,449 @@ __global__ void __launch_bounds__(256, 3) k_int(const WalkSet ws, const WalkScra
     }
 }
 
-// neighbours of first-order determinants
-template <int W, int MINB>
-__global__ void __launch_bounds__(256, MINB) k_fois(const WalkSet ws, const WalkScratch sc) {
+// ---- first-order determinants
+
+// Neighbours that move active electrons only (the determinant's own label), one per lane: each has an
+// active remnant of its own, so there is no list to share.
+template <int W>
+__global__ void __launch_bounds__(256, 3) k_fois_act(const WalkSet ws, const WalkScratch sc) {
     __shared__ WarpTask tasks[8];
-    __shared__ WarpLists lists_sh[8];
     const int lane = threadIdx.x & 31;
     WarpTask& wt = tasks[threadIdx.x >> 5];
-    WarpLists& lists = lists_sh[threadIdx.x >> 5];
     const SysDev& S = wt.sys;
     int cur = -1;
     const int ntg = sc.ctl[CTL_TGF];
     NoCtr ctr;
     for (;;) {
-        const int id = next_task(sc.ctl + CTL_FOIS, lane);
-        if (id >= (long long)ntg * sc.ns_max) break;
+        const int id = next_task(sc.ctl + CTL_ACT, lane);
+        if (id >= ntg * MRQ_ACT_SLICES) break;
         const int slice = id / ntg;
         const TaskGroup tg = sc.tgf[id - slice * ntg];
         task_system(wt, ws, tg.sys, cur, lane);
-        if (slice >= S.nslice) continue;
-        double sA = 0.0, sT = 0.0, sD = 0.0;
+        StepSink sink{wt, sc.best, sc.bound, tg.count, lane, 0.0, 0.0, 0.0};
         if (task_begin<W>(wt, ws, sc, tg, lane)) {
             const unsigned long long(&n)[2][W] = *reinterpret_cast<const unsigned long long(*)[2][W]>(wt.nsh);
-            const GroupMeta* const meta = sc.meta + tg.group;
-            StepSink sink{wt, sc.best, sc.bound, tg.count, lane, 0.0, 0.0, 0.0};
-            build_lists<W>(S, n, lists, meta->h, meta->p, lane);
-            const int total = lists.bstart[lists.nb], units = (total + MRQ_FOIS_CH - 1) / MRQ_FOIS_CH;
-            for (int u = slice; u < units; u += S.nslice)
-                fois_unit<W>(S, lists, sc.gops + (long long)tg.group * sc.gstride, n, meta->label, __ldg(S.c), MRQ_EMPTY_KEY,
-                             0.0, u * MRQ_FOIS_CH, min(total, (u + 1) * MRQ_FOIS_CH), lane, sink, ctr);
+            const double* const gops = sc.gops + (long long)tg.group * sc.gstride;
+            const double cl = __ldg(S.c + sc.meta[tg.group].label);
+            const unsigned amask = (S.na >= 32) ? 0xFFFFFFFFu : ((1u << S.na) - 1u);
+            const unsigned ao0 = active_bits<W>(S, n[0]), ao1 = active_bits<W>(S, n[1]);
+            const unsigned long long oa = ao0, ob = (unsigned long long)ao1 << 32;
+            const unsigned long long ea = ~ao0 & amask, eb = (unsigned long long)(~ao1 & amask) << 32;
+            const int total = active_neighbours(__popcll(oa), __popcll(ob), __popcll(ea), __popcll(eb));
+            for (int base = 32 * slice; base < total; base += 32 * MRQ_ACT_SLICES) {
+                double t = 0.0;
+                unsigned exc = 0;
+                if (base + lane < total) {
+                    unsigned long long Xb, Yb, m[2][W];
+                    const int r = active_neighbour(S, oa, ob, ea, eb, base + lane, Xb, Yb);
+                    int rem[2], add[2];
+                    act_list(S, Xb, rem);
+                    act_list(S, Yb, add);
+#pragma unroll
+                    for (int sg = 0; sg < 2; sg++)
+#pragma unroll
+                        for (int w = 0; w < W; w++) m[sg][w] = n[sg][w];
+                    apply_exc<W>(m, S, rem, add, r);
+                    const double hnm = r == 1 ? single_elem<W>(S, n, rem[0], add[0], ctr)
+                                              : hb_screen(S, double_elem<W>(S, n, rem[0], rem[1], add[0], add[1], ctr));
+                    const int r2 = r == 1 ? rem[0] : rem[1], a2 = r == 1 ? add[0] : add[1];
+                    const double psim = cl * reach_back<W>(S, m, ctr, MRQ_EMPTY_KEY, 0.0, SglFromWalker{gops, r, rem[0], r2, add[0], a2});
+                    sink.sD += (r == 1 ? hd_single_elem<W>(S, n, rem[0], add[0], ctr) : hnm) * psim;
+                    t = hnm * psim;
+                    exc = exc_code(rem[0], r2, add[0], a2);
+                }
+                sink.push(true, t, exc);
+            }
             sink.finish();
-            sA = sink.sA;
-            sT = sink.sT;
-            sD = sink.sD;
         }
-        task_sums(sc, tg, slice, sA, sT, sD, lane);
+        task_sums(sc, tg, sc.ns_max + slice, sink.sA, sink.sT, sink.sD, lane);
+    }
+}
+
+// A neighbour of a first-order determinant n moves active electrons X_a -> Y_a and outer ones: core
+// electrons X_c and virtual electrons X_v out, core holes Y_c filled, virtual orbitals Y_v entered.  A
+// unit is a pair (X_a, Y_a) - one active remnant - and its groups run over the outer patterns; the
+// neighbours of a group differ in the orbitals of X_c and Y_v only and share one candidate list.
+
+// core holes and virtual electrons of a first-order determinant and what they leave free
+struct FoisOuter {
+    int h, p, ha, pa;                 // holes, virtual electrons, alpha ones
+    int hs[2], ps[2];                 // spin orbitals, sorted
+    int ct[2][2], vt[2][2];           // taken core / virtual positions per spin, ascending (large: none)
+    int fc[2], fv[2];                 // free ones
+};
+
+template <int W>
+__device__ __forceinline__ void fois_outer(const SysDev& S, const unsigned long long (&n)[2][W], FoisOuter& o) {
+    int hs[2], ps[2], h, p;
+    outer_orbitals<W>(S, n, h, p, hs, ps);
+    const int voff = S.nc + S.na, none = 1 << 20;
+    const int ha = (h >= 1 && hs[0] < S.n) + (h == 2 && hs[1] < S.n), pa = (p >= 1 && ps[0] < S.n) + (p == 2 && ps[1] < S.n);
+    o.h = h;
+    o.p = p;
+    o.ha = ha;
+    o.pa = pa;
+    o.hs[0] = hs[0];
+    o.hs[1] = hs[1];
+    o.ps[0] = ps[0];
+    o.ps[1] = ps[1];
+    o.ct[0][0] = ha >= 1 ? hs[0] : none;
+    o.ct[0][1] = ha == 2 ? hs[1] : none;
+    o.ct[1][0] = h - ha >= 1 ? (ha ? hs[1] : hs[0]) - S.n : none;
+    o.ct[1][1] = h - ha == 2 ? hs[1] - S.n : none;
+    o.vt[0][0] = pa >= 1 ? ps[0] - voff : none;
+    o.vt[0][1] = pa == 2 ? ps[1] - voff : none;
+    o.vt[1][0] = p - pa >= 1 ? (pa ? ps[1] : ps[0]) - S.n - voff : none;
+    o.vt[1][1] = p - pa == 2 ? ps[1] - S.n - voff : none;
+    o.fc[0] = S.nc - ha;
+    o.fc[1] = S.nc - (h - ha);
+    o.fv[0] = S.nv - pa;
+    o.fv[1] = S.nv - (p - pa);
+}
+
+// the i-th orbital that is neither a nor b (a < b)
+__device__ __forceinline__ int skip_two(int i, int a, int b) {
+    i += i >= a;
+    i += i >= b;
+    return i;
+}
+
+// choices of cnt orbitals, nal of them alpha, among f0 alpha and f1 beta ones
+__device__ __forceinline__ int free_count(int cnt, int nal, int f0, int f1) {
+    if (cnt == 0) return 1;
+    if (cnt == 1) return nal ? f0 : f1;
+    return nal == 1 ? f0 * f1 : (nal == 2 ? f0 * (f0 - 1) / 2 : f1 * (f1 - 1) / 2);
+}
+
+// the idx-th choice: sorted spin orbitals; `taken` positions of each spin are left out, orbitals start at off
+__device__ __forceinline__ void free_decode(const SysDev& S, int cnt, int nal, const int* f, const int (*taken)[2], int off,
+                                            int idx, int& x0, int& x1) {
+    if (cnt == 1) {
+        const int sg = nal ? 0 : 1;
+        x0 = sg * S.n + off + skip_two(idx, taken[sg][0], taken[sg][1]);
+    } else if (cnt == 2) {
+        int i, j, s0 = 0, s1 = 1;
+        if (nal == 1) {
+            i = idx / f[1];
+            j = idx - i * f[1];
+        } else {
+            s0 = s1 = nal == 2 ? 0 : 1;
+            lex_decode_tab(S.colex, idx, f[s0], i, j);
+        }
+        x0 = s0 * S.n + off + skip_two(i, taken[s0][0], taken[s0][1]);
+        x1 = s1 * S.n + off + skip_two(j, taken[s1][0], taken[s1][1]);
+    }
+}
+
+__device__ __forceinline__ void put2(int x, int& k, int& a, int& b) {
+    if (k == 0) a = x;
+    else b = x;
+    k++;
+}
+
+// Groups of the wave's determinants, one block each: threads take the units in order, count their
+// groups and neighbours, and a block scan gives every group its number, which therefore depends on the
+// determinant alone (the sums of k_fois run in that order).
+template <int W>
+__global__ void __launch_bounds__(256) k_fgroups(const WalkSet ws, const WalkScratch sc) {
+    const int ng = min(sc.fwave, sc.ctl[CTL_GF] - sc.fwave0);
+    __shared__ FoisOuter o;
+    __shared__ int s_sum[2][8], s_base[2];
+    __shared__ long long s_row;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int g = blockIdx.x; g < ng; g += gridDim.x) {
+        const int det = (int)(sc.nseg - 1 - (sc.fwave0 + g));
+        const GroupMeta& meta = sc.meta[det];
+        const SysDev& S = ws.systems[meta.sys];
+        __syncthreads();
+        if (meta.label < 0 || !(meta.psi != 0.0)) {
+            if (threadIdx.x == 0) sc.fg_of[g] = make_int2(0, 0);
+            continue;
+        }
+        unsigned long long n[2][W];
+#pragma unroll
+        for (int sg = 0; sg < 2; sg++)
+#pragma unroll
+            for (int w = 0; w < W; w++) n[sg][w] = meta.d[sg][w];
+        if (threadIdx.x == 0) {
+            fois_outer<W>(S, n, o);
+            s_base[0] = s_base[1] = 0;
+        }
+        const unsigned ao0 = active_bits<W>(S, n[0]), ao1 = active_bits<W>(S, n[1]);
+        const unsigned amask = (S.na >= 32) ? 0xFFFFFFFFu : ((1u << S.na) - 1u);
+        const unsigned long long AO = (unsigned long long)ao0 | ((unsigned long long)ao1 << 32);
+        const unsigned long long AE = (unsigned long long)(~ao0 & amask) | ((unsigned long long)(~ao1 & amask) << 32);
+        const int cntO = __popcll(AO), cntE = __popcll(AE);
+        int units = 0;
+        for (int k = 0; k < 8; k++) units += nsub(cntO, k / 3) * nsub(cntE, k % 3);
+        FGroup* const fg = sc.fg + (long long)g * sc.fg_max;
+        __syncthreads();
+        // pass 0 counts, then the determinant takes its place in the row buffer; pass 1 writes
+        for (int pass = 0; pass < 2; pass++) {
+            for (int u0 = 0; u0 < units; u0 += blockDim.x) {
+                const int u = u0 + threadIdx.x;
+                int ngr = 0, nnb = 0, at = 0, row = 0;
+                for (int emit = 0; emit <= pass; emit++) {
+                    if (emit) {
+                        // exclusive scan of (groups, neighbours) over the block
+                        int x = ngr, y = nnb;
+#pragma unroll
+                        for (int d = 1; d < 32; d <<= 1) {
+                            const int x2 = __shfl_up_sync(0xffffffffu, x, d), y2 = __shfl_up_sync(0xffffffffu, y, d);
+                            if (lane >= d) {
+                                x += x2;
+                                y += y2;
+                            }
+                        }
+                        if (lane == 31) {
+                            s_sum[0][warp] = x;
+                            s_sum[1][warp] = y;
+                        }
+                        __syncthreads();
+                        at = s_base[0] + x - ngr;
+                        row = s_base[1] + y - nnb;
+                        for (int w = 0; w < warp; w++) {
+                            at += s_sum[0][w];
+                            row += s_sum[1][w];
+                        }
+                        __syncthreads();
+                        if (threadIdx.x == blockDim.x - 1) {
+                            s_base[0] = at + ngr;
+                            s_base[1] = row + nnb;
+                        }
+                    }
+                    if (u < units) {
+                        int k = 0, pair = u;
+                        for (; k < 7; k++) {
+                            const int w = nsub(cntO, k / 3) * nsub(cntE, k % 3);
+                            if (pair < w) break;
+                            pair -= w;
+                        }
+                        const int ka = k / 3, kb = k % 3, nYa = nsub(cntE, kb), xa = pair / nYa, ya = pair - xa * nYa;
+                        const unsigned long long Xb = subset_bits(S.colex, AO, cntO, ka, xa);
+                        const unsigned long long Yb = subset_bits(S.colex, AE, cntE, kb, ya);
+                        const int da = __popcll(Xb & 0xFFFFFFFFull) - __popcll(Yb & 0xFFFFFFFFull);
+                        for (int r = max(1, max(ka, kb)); r <= 2; r++) {
+                            const int ko = r - ka, vo = r - kb;              // outer electrons removed / added
+                            if (ko == 0 && vo == 0) continue;                // active only: k_fois_act
+                            const int na_ = min(ko, o.p) + 1, nb_ = min(vo, o.h) + 1;
+                            for (int pat = 0; pat < na_ * nb_ * 4; pat++) {
+                                const int av = (pat >> 2) / nb_, bc = (pat >> 2) - av * nb_, xs = pat & 1, ys = (pat >> 1) & 1;
+                                if ((xs && !(av == 1 && o.p == 2)) || (ys && !(bc == 1 && o.h == 2))) continue;
+                                const int ac = ko - av, bv = vo - bc, c = o.h + ac - bc, v = o.p - av + bv;
+                                if (c > 2 || v > 2) continue;
+                                const int xva = av == 2 ? o.pa : (av == 1 ? o.ps[xs] < S.n : 0);
+                                const int yca = bc == 2 ? o.ha : (bc == 1 ? o.hs[ys] < S.n : 0);
+                                for (int sac = 0; sac <= ac; sac++) {
+                                    const int sbv = da + xva + sac - yca;
+                                    if (sbv < 0 || sbv > bv) continue;
+                                    const int ni = free_count(ac, sac, o.fc[0], o.fc[1]) * free_count(bv, sbv, o.fv[0], o.fv[1]);
+                                    if (!emit) {
+                                        ngr += (ni + MRQ_FG_NB - 1) / MRQ_FG_NB;
+                                        nnb += ni;
+                                        continue;
+                                    }
+                                    for (int q = 0; q < ni; q += MRQ_FG_NB) {
+                                        FGroup f;
+                                        f.ao = (AO & ~Xb) | Yb;
+                                        f.off = s_row + row;
+                                        f.det = det;
+                                        f.q0 = q;
+                                        f.nq = min(MRQ_FG_NB, ni - q);
+                                        f.c = (unsigned char)c;
+                                        f.v = (unsigned char)v;
+                                        f.scn = (unsigned char)(o.ha + sac - yca);
+                                        f.sv = (unsigned char)(o.pa - xva + sbv);
+                                        f.ac = (unsigned char)ac;
+                                        f.sac = (unsigned char)sac;
+                                        f.bv = (unsigned char)bv;
+                                        f.sbv = (unsigned char)sbv;
+                                        f.av = (unsigned char)av;
+                                        f.bc = (unsigned char)bc;
+                                        f.xs = (unsigned char)xs;
+                                        f.ys = (unsigned char)ys;
+                                        fg[at++] = f;
+                                        row += f.nq;
+                                    }
+                                }
+                            }
+                        }
+                    }
+                }
+                if (pass == 0) {
+                    const int x = __reduce_add_sync(0xffffffffu, nnb);
+                    if (lane == 0) atomicAdd(&s_base[1], x);
+                }
+                __syncthreads();
+            }
+            if (pass == 0) {
+                if (threadIdx.x == 0) {
+                    s_row = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(sc.ctl + CTL_CUR),
+                                                 (unsigned long long)((s_base[1] + 3) & ~3));
+                    s_base[1] = 0;
+                }
+                __syncthreads();
+            }
+        }
+        if (threadIdx.x == 0) {
+            sc.fg_of[g] = make_int2(g * sc.fg_max, s_base[0]);
+            atomicMax(sc.ctl + CTL_FG, s_base[0]);
+        }
+    }
+}
+
+// psi_s of the groups' neighbours, a warp task each: the candidate list once, then its sum per neighbour
+// (bound by the building of the short lists' candidates: hash reads and integer work)
+template <int W, int MINB>
+__global__ void __launch_bounds__(MRQ_MAXNW * 32, MINB) k_frows(const WalkSet ws, const WalkScratch sc, int lbytes, int cap) {
+    extern __shared__ __align__(16) unsigned char smem_dyn[];
+    const int lane = threadIdx.x & 31;
+    unsigned char* const mine = smem_dyn + (size_t)(threadIdx.x >> 5) * lbytes;
+    SysDev& S = *reinterpret_cast<SysDev*>(mine);
+    FoisOuter& o = *reinterpret_cast<FoisOuter*>(mine + (sizeof(SysDev) + 15) / 16 * 16);
+    double* const cphi = reinterpret_cast<double*>(mine + (sizeof(SysDev) + 15) / 16 * 16 + (sizeof(FoisOuter) + 15) / 16 * 16);
+    unsigned* const ccode = reinterpret_cast<unsigned*>(cphi + cap);
+    const int ng = min(sc.fwave, sc.ctl[CTL_GF] - sc.fwave0);
+    if (ng <= 0) return;
+    int cur = -1;
+    const long long ntask = (long long)ng * sc.ctl[CTL_FG];
+    NoCtr ctr;
+    for (;;) {
+        const int id = next_task(sc.ctl + CTL_FGTASK, lane);
+        if (id >= ntask) break;
+        const int g = id % ng, k = id / ng;
+        const int2 of = sc.fg_of[g];
+        if (k >= of.y) continue;
+        const FGroup f = sc.fg[of.x + k];
+        const GroupMeta& meta = sc.meta[f.det];
+        __syncwarp();
+        if (meta.sys != cur) {
+            copy_sys(&S, ws.systems + meta.sys, lane, 32);
+            cur = meta.sys;
+            __syncwarp();
+        }
+        if (lane == 0) {
+            unsigned long long n[2][W];
+#pragma unroll
+            for (int sg = 0; sg < 2; sg++)
+#pragma unroll
+                for (int w = 0; w < W; w++) n[sg][w] = meta.d[sg][w];
+            fois_outer<W>(S, n, o);
+        }
+        __syncwarp();
+        double* const row = sc.rows + f.off;
+        if (f.c == 0 && f.v == 0) {                       // a CAS determinant: the group holds one neighbour
+            if (lane == 0) row[0] = __ldg(S.c) * hash_lookup(S, hash_key(S, (unsigned)f.ao, (unsigned)(f.ao >> 32)));
+            continue;
+        }
+        int n1;
+        const int count = row_list<W>(S, f.ao, f.c, f.v, f.scn, f.sv, cphi, ccode, n1, lane, ctr);
+        const int nvc = free_count(f.bv, f.sbv, o.fv[0], o.fv[1]);
+        const int h0 = o.hs[0], h1 = o.hs[1], p0 = o.ps[0], p1 = o.ps[1];
+        const int yc = f.bc == 1 ? (f.ys ? h1 : h0) : -1, xv = f.av == 1 ? (f.xs ? p1 : p0) : -1;
+        for (int qb = 0; qb < f.nq; qb += 32) {
+            const int nr = min(32, f.nq - qb), fl = split_of(nr), lf = __ffs(fl) - 1;
+            const int qi = lane >> lf, part = lane & (fl - 1);
+            const int q = f.q0 + qb + min(qi, nr - 1), ic = q / nvc;
+            int x0 = 0, x1 = 0, y0 = 0, y1 = 0, H0 = 0, H1 = 0, P0 = 0, P1 = 0, i = 0, j = 0, par;
+            free_decode(S, f.ac, f.sac, o.fc, o.ct, 0, ic, x0, x1);
+            free_decode(S, f.bv, f.sbv, o.fv, o.vt, S.nc + S.na, q - ic * nvc, y0, y1);
+            if (o.h >= 1 && f.bc < 2 && yc != h0) put2(h0, i, H0, H1);
+            if (o.h == 2 && f.bc < 2 && yc != h1) put2(h1, i, H0, H1);
+            if (f.ac >= 1) put2(x0, i, H0, H1);
+            if (f.ac == 2) put2(x1, i, H0, H1);
+            if (o.p >= 1 && f.av < 2 && xv != p0) put2(p0, j, P0, P1);
+            if (o.p == 2 && f.av < 2 && xv != p1) put2(p1, j, P0, P1);
+            if (f.bv >= 1) put2(y0, j, P0, P1);
+            if (f.bv == 2) put2(y1, j, P0, P1);
+            if (f.c == 2 && H0 > H1) { const int t = H0; H0 = H1; H1 = t; }
+            if (f.v == 2 && P0 > P1) { const int t = P0; P0 = P1; P1 = t; }
+            const double s = row_overlap(S, f.ao, f.c, f.v, H0, H1, P0, P1, cphi, ccode, n1, count, part, fl, par);
+            if (qi < nr && part == 0) row[qb + qi] = __ldg(S.c + row_label(S, f.c, f.v, H0, H1, P0, P1)) * neg_if(s, par);
+        }
+        __syncwarp();
+    }
+}
+
+// the groups' neighbours: elements times the overlaps of k_frows, and the race
+template <int W, int MINB>
+__global__ void __launch_bounds__(256, MINB) k_fois(const WalkSet ws, const WalkScratch sc) {
+    __shared__ WarpTask tasks[8];
+    __shared__ FoisOuter outer[8];
+    const int lane = threadIdx.x & 31;
+    WarpTask& wt = tasks[threadIdx.x >> 5];
+    FoisOuter& o = outer[threadIdx.x >> 5];
+    const SysDev& S = wt.sys;
+    if (sc.ctl[CTL_GF] <= sc.fwave0) return;
+    int cur = -1;
+    const int ntg = sc.ctl[CTL_TGF];
+    NoCtr ctr;
+    for (;;) {
+        const int id = next_task(sc.ctl + CTL_FOIS, lane);
+        if (id >= ntg * MRQ_FOIS_SLICES) break;
+        const int slice = id / ntg;
+        const TaskGroup tg = sc.tgf[id - slice * ntg];
+        const int g = (int)(sc.nseg - 1 - tg.group) - sc.fwave0;
+        if (g < 0 || g >= sc.fwave) continue;
+        task_system(wt, ws, tg.sys, cur, lane);
+        StepSink sink{wt, sc.best, sc.bound, tg.count, lane, 0.0, 0.0, 0.0};
+        if (task_begin<W>(wt, ws, sc, tg, lane)) {
+            const unsigned long long(&n)[2][W] = *reinterpret_cast<const unsigned long long(*)[2][W]>(wt.nsh);
+            if (lane == 0) fois_outer<W>(S, n, o);
+            __syncwarp();
+            const unsigned long long AO =
+                (unsigned long long)active_bits<W>(S, n[0]) | ((unsigned long long)active_bits<W>(S, n[1]) << 32);
+            const double* const gops = sc.gops + (long long)tg.group * sc.gstride;
+            const int2 of = sc.fg_of[g];
+            for (int k = slice; k < of.y; k += MRQ_FOIS_SLICES) {
+                const FGroup f = sc.fg[of.x + k];
+                const unsigned long long Xb = AO & ~f.ao, Yb = f.ao & ~AO;
+                // the fixed orbitals removed and added
+                int rf0 = 0, rf1 = 0, af0 = 0, af1 = 0, nrf = 0, naf = 0;
+                if (Xb) put2(act_so(S, __ffsll(Xb) - 1), nrf, rf0, rf1);
+                if (Xb & (Xb - 1)) put2(act_so(S, 63 - __clzll(Xb)), nrf, rf0, rf1);
+                if (f.av >= 1) put2(f.av == 1 ? o.ps[f.xs] : o.ps[0], nrf, rf0, rf1);
+                if (f.av == 2) put2(o.ps[1], nrf, rf0, rf1);
+                if (Yb) put2(act_so(S, __ffsll(Yb) - 1), naf, af0, af1);
+                if (Yb & (Yb - 1)) put2(act_so(S, 63 - __clzll(Yb)), naf, af0, af1);
+                if (f.bc >= 1) put2(f.bc == 1 ? o.hs[f.ys] : o.hs[0], naf, af0, af1);
+                if (f.bc == 2) put2(o.hs[1], naf, af0, af1);
+                const int nvc = free_count(f.bv, f.sbv, o.fv[0], o.fv[1]);
+                const bool one = nrf + f.ac == 1;
+                const double* const row = sc.rows + f.off;
+                for (int qb = 0; qb < f.nq; qb += 32) {
+                    const bool on = qb + lane < f.nq;
+                    double t = 0.0;
+                    unsigned exc = 0;
+                    if (on) {
+                        const double psim = __ldcg(row + qb + lane);
+                        const int q = f.q0 + qb + lane, ic = q / nvc;
+                        int x0 = 0, x1 = 0, y0 = 0, y1 = 0, r0 = rf0, r1 = rf1, a0 = af0, a1 = af1, i = nrf, j = naf;
+                        free_decode(S, f.ac, f.sac, o.fc, o.ct, 0, ic, x0, x1);
+                        free_decode(S, f.bv, f.sbv, o.fv, o.vt, S.nc + S.na, q - ic * nvc, y0, y1);
+                        if (f.ac >= 1) put2(x0, i, r0, r1);
+                        if (f.ac == 2) put2(x1, i, r0, r1);
+                        if (f.bv >= 1) put2(y0, j, a0, a1);
+                        if (f.bv == 2) put2(y1, j, a0, a1);
+                        if (one) {
+                            r1 = r0;
+                            a1 = a0;
+                            t = (in_walker_block(S, r0, a0)
+                                     ? single_from_walker<W>(S, SglFromWalker{gops, 0, 0, 0, 0, 0}, n, r0, a0, ctr)
+                                     : single_elem<W>(S, n, r0, a0, ctr)) * psim;
+                        } else {
+                            if (r0 > r1) { const int z = r0; r0 = r1; r1 = z; }
+                            if (a0 > a1) { const int z = a0; a0 = a1; a1 = z; }
+                            t = hb_screen(S, double_elem<W>(S, n, r0, r1, a0, a1, ctr)) * psim;
+                        }
+                        exc = exc_code(r0, r1, a0, a1);
+                    }
+                    sink.push(on, t, exc);
+                }
+            }
+            sink.finish();
+        }
+        task_sums(sc, tg, slice, sink.sA, sink.sT, 0.0, lane);
     }
 }
 
@@ -1414,33 +1965,9 @@ __global__ void __launch_bounds__(256) k_insert(const WalkSet ws, const WalkScra
     }
 }
 
-// sum of a row's candidates e0, e0 + stride, ... < count for one neighbour: w T[base + lane part]
-__device__ __forceinline__ double row_doubles(const double* __restrict__ tab, const double* cphi, const unsigned* ccode,
-                                              int e, int count, int st, unsigned offd, unsigned offx) {
-    double a0 = 0.0, a1 = 0.0;
-    for (; e + 3 * st < count; e += 4 * st) {
-        const unsigned p0 = ccode[e], p1 = ccode[e + st], p2 = ccode[e + 2 * st], p3 = ccode[e + 3 * st];
-        const double x0 = __ldg(tab + (p0 & 0x7FFFFFFFu) + ((p0 & 0x80000000u) ? offx : offd));
-        const double x1 = __ldg(tab + (p1 & 0x7FFFFFFFu) + ((p1 & 0x80000000u) ? offx : offd));
-        const double x2 = __ldg(tab + (p2 & 0x7FFFFFFFu) + ((p2 & 0x80000000u) ? offx : offd));
-        const double x3 = __ldg(tab + (p3 & 0x7FFFFFFFu) + ((p3 & 0x80000000u) ? offx : offd));
-        a0 = fma(cphi[e], x0, a0);
-        a1 = fma(cphi[e + st], x1, a1);
-        a0 = fma(cphi[e + 2 * st], x2, a0);
-        a1 = fma(cphi[e + 3 * st], x3, a1);
-    }
-    for (; e < count; e += st) {
-        const unsigned p0 = ccode[e];
-        a0 = fma(cphi[e], __ldg(tab + (p0 & 0x7FFFFFFFu) + ((p0 & 0x80000000u) ? offx : offd)), a0);
-    }
-    return a0 + a1;
-}
-
 // The distinct rows, one warp task each.  Entry q of a group (core choice slow, virtual choice fast)
 // holds c_l O(m) (-1)^(core-hole positions of m): the sign that H_nm of the same neighbour carries too,
-// so k_pairs multiplies the two as they are.  Per group the warp builds the candidate list in shared
-// memory; a single candidate x -> y takes h_yx + sum over the remnant's electrons j of (yx|jj) -
-// (yj|jx) (the neighbour's own hole y and electron x drop out), a double one table read and one FMA.
+// so k_pairs multiplies the two as they are.
 // Bound by FP64 (2 FMA per clock and SM): one read and one FMA per candidate.
 template <int W, int MINB>
 __global__ void __launch_bounds__(MRQ_MAXNW * 32, MINB) k_rows(const WalkSet ws, const WalkScratch sc, int lbytes, int cap) {
@@ -1466,68 +1993,27 @@ __global__ void __launch_bounds__(MRQ_MAXNW * 32, MINB) k_rows(const WalkSet ws,
             __syncwarp();
         }
         const unsigned long long AO = sc.ref_ao[i];
-        const unsigned amask = (S.na >= 32) ? 0xFFFFFFFFu : ((1u << S.na) - 1u);
-        const unsigned long long AE = ~AO & ((unsigned long long)amask | ((unsigned long long)amask << 32));
         const int c = sc.ref_cls[i] / 3, v = sc.ref_cls[i] - 3 * c;
         const int d = __popcll(AO & 0xFFFFFFFFull) - (S.nalpha - S.nc);
         double* row = sc.rows + sc.row_off[i];
-        const int voff = S.nc + S.na;
         for (int scn = 0; scn <= c; scn++) {
             const int sv = scn - d;
             if (sv < 0 || sv > v) continue;
             const int nvc = shape_count(S.nv, v, sv), ni = shape_count(S.nc, c, scn) * nvc;
             if (ni == 0) continue;
-            // the group's first neighbour, for the candidates' signs
-            int xc[2] = {0, 0}, yv[2] = {0, 0};
-            shape_decode(S, S.nc, c, scn, 0, 0, xc, S.mag_c);
-            shape_decode(S, S.nv, v, sv, voff, 0, yv, S.mag_v);
-            unsigned long long m[2][W];
-#pragma unroll
-            for (int sg = 0; sg < 2; sg++) {
-                const unsigned long long a = sg ? AO >> 32 : AO & 0xFFFFFFFFull;
-#pragma unroll
-                for (int w = 0; w < W; w++) {
-                    const int sh = S.nc - 64 * w;                      // the active block may straddle a word
-                    m[sg][w] = S.mcore[w] | ((sh >= 0 ? (sh < 64 ? a << sh : 0ull) : (sh > -64 ? a >> -sh : 0ull)) & S.mact[w]);
-                }
-            }
-            for (int k = 0; k < c; k++) flip_reg<W>(m, xc[k] >= S.n, xc[k] - (xc[k] >= S.n ? S.n : 0));
-            for (int k = 0; k < v; k++) flip_reg<W>(m, yv[k] >= S.n, yv[k] - (yv[k] >= S.n ? S.n : 0));
-            unsigned offd, offx;
-            int par, n1;
-            lane_offsets(S, c, v, xc[0], xc[1], yv[0], yv[1], offd, offx, par);
-            const int count = build_group_list<W, true>(S, MRQ_EMPTY_KEY, m, AO, AE, c, v, scn, sv, xc[0], xc[1], yv[0], yv[1],
-                                                        par, cphi, ccode, n1, lane, ctr);
+            int n1;
+            const int count = row_list<W>(S, AO, c, v, scn, sv, cphi, ccode, n1, lane, ctr);
             const unsigned long long mvc = ~0ull / (unsigned long long)nvc + 1ull;     // q / nvc by its high product
             for (int qb = 0; qb < ni; qb += 32) {
                 const int nr = min(32, ni - qb), f = split_of(nr), lf = __ffs(f) - 1;
                 const int qi = lane >> lf, part = lane & (f - 1);
                 const int q = qb + min(qi, nr - 1);
                 const int ic = nvc == 1 ? q : (int)__umul64hi((unsigned long long)q, mvc);
+                int xc[2] = {0, 0}, yv[2] = {0, 0}, par;
                 shape_decode(S, S.nc, c, scn, 0, ic, xc, S.mag_c);
-                shape_decode(S, S.nv, v, sv, voff, q - ic * nvc, yv, S.mag_v);
-                lane_offsets(S, c, v, xc[0], xc[1], yv[0], yv[1], offd, offx, par);
-                double s = 0.0;
-                for (int e = part; e < n1; e += f) {
-                    const unsigned code = ccode[e];
-                    const int x = v ? yv[0] : act_so(S, (int)(code & 127u)), y = c ? xc[0] : act_so(S, (int)((code >> 14) & 127u));
-                    const int sx = x >= S.n, px = x - sx * S.n, py = y - sx * S.n;
-                    double g = __ldg(S.hc + py * S.n + px);
-                    const double* const col = S.sgl + py * S.nav + (px - S.nc);
-                    for (unsigned long long bits = AO; bits; bits &= bits - 1) {
-                        const int b = __ffsll(bits) - 1;
-                        g += __ldg(col + (long long)((b & 31) + (((b >= 32) == (sx == 1)) ? 0 : S.na)) * S.nca * S.nav);
-                    }
-                    s = fma(cphi[e], g, s);
-                }
-                s += row_doubles(S.tab, cphi, ccode, n1 + part, count, f, offd, offx);
-                for (int o = f >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                if (qi < nr && part == 0) {
-                    const int h0 = xc[0] >= S.n ? S.nc + (xc[0] - S.n) : xc[0], h1 = xc[1] >= S.n ? S.nc + (xc[1] - S.n) : xc[1];
-                    const int p0 = yv[0] >= S.n ? S.nv + (yv[0] - S.n - voff) : yv[0] - voff;
-                    const int p1 = yv[1] >= S.n ? S.nv + (yv[1] - S.n - voff) : yv[1] - voff;
-                    row[q] = __ldg(S.c + set_rank(c, h0, h1, 2 * S.nc) * S.nPs + set_rank(v, p0, p1, 2 * S.nv)) * s;
-                }
+                shape_decode(S, S.nv, v, sv, S.nc + S.na, q - ic * nvc, yv, S.mag_v);
+                const double s = row_overlap(S, AO, c, v, xc[0], xc[1], yv[0], yv[1], cphi, ccode, n1, count, part, f, par);
+                if (qi < nr && part == 0) row[q] = __ldg(S.c + row_label(S, c, v, xc[0], xc[1], yv[0], yv[1])) * s;
             }
             __syncwarp();
             row += ni;
@@ -1668,9 +2154,7 @@ __global__ void __launch_bounds__(256, MINB) k_pairs(const WalkSet ws, const Wal
                             hb -= (unsigned)cp0 * cs0 + (unsigned)cp1 * cs1 + (unsigned)vp0 * vs0 + (unsigned)vp1 * vs1;
                             eb -= (unsigned)cp0 * ce0 + (unsigned)cp1 * ce1 + (unsigned)vp0 * ve0 + (unsigned)vp1 * ve1;
                             const unsigned long long mvc = ~0ull / (unsigned long long)nvc + 1ull;
-                            for (int qb = q0; qb < q1; qb += 32) {
-                                const bool valid = qb + lane < q1;
-                                const int q = valid ? qb + lane : q1 - 1;
+                            auto element = [&](int q, double& t, unsigned& exc) {
                                 const int ic = nvc == 1 ? q : (int)__umul64hi((unsigned long long)q, mvc), iv = q - ic * nvc;
                                 int i0 = ic, i1 = 0, j0 = iv, j1 = 0;
                                 if (c == 2) {
@@ -1690,8 +2174,7 @@ __global__ void __launch_bounds__(256, MINB) k_pairs(const WalkSet ws, const Wal
                                     }
                                 }
                                 const double h = H[hb + (unsigned)i0 * cs0 + (unsigned)i1 * cs1 + (unsigned)j0 * vs0 + (unsigned)j1 * vs1];
-                                const unsigned exc = eb + (unsigned)i0 * ce0 + (unsigned)i1 * ce1 + (unsigned)j0 * ve0 + (unsigned)j1 * ve1;
-                                double t;
+                                exc = eb + (unsigned)i0 * ce0 + (unsigned)i1 * ce1 + (unsigned)j0 * ve0 + (unsigned)j1 * ve1;
                                 if (self) {
                                     const int h0 = scn == 0 ? nc + i0 : i0, h1 = scn == 2 ? i1 : nc + i1;
                                     const int p0 = sv == 0 ? nv + j0 : j0, p1 = sv == 2 ? j1 : nv + j1;
@@ -1699,8 +2182,18 @@ __global__ void __launch_bounds__(256, MINB) k_pairs(const WalkSet ws, const Wal
                                 } else {
                                     t = neg_if(h * __ldcg(row + q), odd);
                                 }
-                                if (q1 - qb >= 32) sink.take(t, exc);
-                                else sink.push(valid, t, exc);
+                            };
+                            for (int qb = q0; qb < q1; qb += 64) {
+                                double t0, t1;
+                                unsigned e0, e1;
+                                element(min(qb + lane, q1 - 1), t0, e0);
+                                element(min(qb + 32 + lane, q1 - 1), t1, e1);
+                                if (q1 - qb >= 64) {
+                                    sink.take(t0, e0, t1, e1);
+                                } else {
+                                    sink.push(qb + lane < q1, t0, e0);
+                                    if (qb + 32 < q1) sink.push(qb + 32 + lane < q1, t1, e1);
+                                }
                             }
                         }
                         base += ni;
@@ -1748,15 +2241,17 @@ __global__ void __launch_bounds__(MRQ_MAXNW * 32) k_move(const WalkSet ws, const
         const GroupMeta meta = sc.meta[tg.group];
         const double inv_psin = meta.psi != 0.0 ? 1.0 / meta.psi : 0.0;
         double A = 0.0, T = 0.0, D = 0.0;
-        const double* const part = sc.part + (long long)tg.group * (sc.ns_max + MRQ_INT_SLICES) * 3;
-        for (int k = lane; k < S.nslice; k += 32) {
+        const double* const part = sc.part + (long long)tg.group * (sc.ns_max + MRQ_ACT_SLICES) * 3;
+        const int ns = g < ntc ? S.nslice : MRQ_FOIS_SLICES;
+        for (int k = lane; k < ns; k += 32) {
             A += part[3 * k];
             T += part[3 * k + 1];
             D += part[3 * k + 2];
         }
-        if (g < ntc && lane < MRQ_INT_SLICES) {
+        if (lane < (g < ntc ? MRQ_INT_SLICES : MRQ_ACT_SLICES)) {
             A += part[3 * (sc.ns_max + lane)];
             T += part[3 * (sc.ns_max + lane) + 1];
+            D += part[3 * (sc.ns_max + lane) + 2];
         }
         A = warp_sum(A);
         T = warp_sum(T);
@@ -1897,6 +2392,9 @@ struct DebugSh {
 __host__ __device__ __forceinline__ size_t debug_smem_bytes(int nw, int cap, int gstride) {
     return (sizeof(DebugSh) + 15) / 16 * 16 + ((size_t)gstride * sizeof(double) + 15) / 16 * 16 +
            (size_t)nw * cand_list_bytes(cap);
+}
+__host__ __device__ __forceinline__ size_t frows_warp_bytes(int cap) {
+    return (sizeof(SysDev) + 15) / 16 * 16 + (sizeof(FoisOuter) + 15) / 16 * 16 + cand_list_bytes(cap);
 }
 __host__ __device__ __forceinline__ size_t rows_warp_bytes(int cap) {
     return (sizeof(SysDev) + 15) / 16 * 16 + cand_list_bytes(cap);
