@@ -694,6 +694,7 @@ __global__ void k_argmax_abs(const double* c, long long n, long long* out) {
 
 // ============================================================================ finalize (Eq. 14-15)
 
+static const long long FIN_CHUNK = 8192;    // labels per partial sum
 #define FIN_Q 5    // per type: kept ratio, e2, screened count, screened ratio, visited count
 #define FIN_NV (MRQ_NTYPES * FIN_Q)
 
@@ -704,13 +705,44 @@ __device__ __forceinline__ int label_type(long long l, long long nPs, int nc2, i
     return 3 * h + p;
 }
 
-// block (v, chunk): labels of the chunk under variant v (v < G: group v left out; v == G: all)
-__global__ void __launch_bounds__(256) k_fin_labels(const SysDev* __restrict__ sys, double tau, int nchunk,
-                                                    long long chunk, double* partial) {
-    const SysDev S = *sys;
+// The visited labels of every chunk, in label order: list[chunk ...], how many in list[nlab + chunk].
+// A walk visits few of its labels (a few thousand of 256,038 at 56 orbitals), so one pass over the
+// accumulators finds them and the G + 1 jackknife variants read only those.  Bound by the one read
+// of accN (G x labels).
+__global__ void __launch_bounds__(256) k_fin_list(const SysDev* __restrict__ sys, long long chunk, int* __restrict__ list) {
+    const int G = sys->G;
+    const long long L = sys->nlab, lo = blockIdx.x * chunk, hi = min(L, lo + chunk);
+    const double* const accN = sys->accN;
+    __shared__ int s_w[8];
+    int run = 0;
+    for (long long base = lo; base < hi; base += 256) {
+        const long long l = base + threadIdx.x;
+        bool seen = false;
+        if (l > 0 && l < hi)
+            for (int g = 0; g < G; g++) seen = seen || !(accN[(long long)g * L + l] == 0.0);
+        const unsigned m = __ballot_sync(0xffffffffu, seen);
+        if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = __popc(m);
+        __syncthreads();
+        int at = run, all = 0;
+        for (int w = 0; w < 8; w++) {
+            if (w < (int)(threadIdx.x >> 5)) at += s_w[w];
+            all += s_w[w];
+        }
+        if (seen) list[lo + at + __popc(m & ((1u << (threadIdx.x & 31)) - 1u))] = (int)l;
+        run += all;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) list[L + blockIdx.x] = run;
+}
+
+// block (v, chunk): visited labels of the chunk under variant v (v < G: group v left out; v == G: all)
+__global__ void __launch_bounds__(256) k_fin_labels(const SysDev* __restrict__ sys, double tau, int nchunk, long long chunk,
+                                                    const int* __restrict__ list, double* partial) {
+    const SysDev& S = *sys;
     const int v = blockIdx.x / nchunk, ch = blockIdx.x % nchunk;
     const int G = S.G;
     const long long L = S.nlab;
+    const int n = list[L + ch];
     __shared__ double s_n0;
     if (threadIdx.x == 0) {
         double a = 0.0;
@@ -723,9 +755,8 @@ __global__ void __launch_bounds__(256) k_fin_labels(const SysDev* __restrict__ s
     double acc[FIN_NV];
 #pragma unroll
     for (int k = 0; k < FIN_NV; k++) acc[k] = 0.0;
-    const long long lo = (long long)ch * chunk, hi = min(L, lo + chunk);
-    for (long long l = lo + threadIdx.x; l < hi; l += blockDim.x) {
-        if (l == 0) continue;
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+        const long long l = list[(long long)ch * chunk + k];
         double Nl = 0.0, Ul = 0.0;
         for (int g = 0; g < G; g++) {
             Nl += S.accN[(long long)g * L + l];
@@ -751,97 +782,105 @@ __global__ void __launch_bounds__(256) k_fin_labels(const SysDev* __restrict__ s
         for (int tt = 0; tt < MRQ_NTYPES; tt++)
             if (tt == t) {
 #pragma unroll
-                for (int k = 0; k < FIN_Q; k++) acc[tt * FIN_Q + k] += q[k];
+                for (int j = 0; j < FIN_Q; j++) acc[tt * FIN_Q + j] += q[j];
             }
+    }
+    if (n == 0) {                    // no visited label: zeros without the reduction
+        for (int k = threadIdx.x; k < FIN_NV; k += blockDim.x) partial[(long long)blockIdx.x * FIN_NV + k] = 0.0;
+        return;
     }
     block_sum_store<FIN_NV>(acc, partial);
 }
 
-// one block: sum chunk partials in order, jackknife over groups, write the result struct
-__global__ void k_fin_reduce(const SysDev* __restrict__ sys, const double* partial, int nchunk, mrq_result* res) {
-    const SysDev S = *sys;
+// one block: sum chunk partials in order, jackknife over groups, write the result struct.  Warp k makes the
+// sums of the (variant, quantity) pairs k, k + 32, ...; then one thread per reported quantity runs the jackknife.
+__global__ void __launch_bounds__(1024) k_fin_reduce(const SysDev* __restrict__ sys, const double* __restrict__ partial,
+                                                     int nchunk, mrq_result* res) {
+    const SysDev& S = *sys;
     const int G = S.G;
     const long long L = S.nlab;
     __shared__ double vals[65][FIN_NV];   // G <= 64
+    __shared__ double sW[64], sE[64], sN[64];
+    for (int g = threadIdx.x; g < G; g += blockDim.x) {
+        sW[g] = S.accW[g];
+        sE[g] = S.accE[g];
+        sN[g] = S.accN[(long long)g * L];
+    }
     for (int idx = threadIdx.x; idx < (G + 1) * FIN_NV; idx += blockDim.x) {
         int v = idx / FIN_NV, k = idx % FIN_NV;
         double s = 0.0;
+#pragma unroll 8
         for (int c = 0; c < nchunk; c++) s += partial[((long long)v * nchunk + c) * FIN_NV + k];
         vals[v][k] = s;
     }
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    double Wt = 0.0, Et = 0.0, N0t = 0.0;
-    for (int g = 0; g < G; g++) {
-        Wt += S.accW[g];
-        Et += S.accE[g];
-        N0t += S.accN[(long long)g * L];
-    }
     const double c0 = S.c[0];
-    auto scal = [&](int v, double& e2, double& ev, double& a0) {
-        double Wv = Wt - (v < G ? S.accW[v] : 0.0);
-        double Ev = Et - (v < G ? S.accE[v] : 0.0);
-        double N0v = N0t - (v < G ? S.accN[(long long)v * L] : 0.0);
-        e2 = 0.0;
-        for (int t = 0; t < MRQ_NTYPES; t++) e2 += vals[v][t * FIN_Q + 1];
-        ev = Ev / Wv;
-        a0 = c0 * c0 * N0v / Wv;
-    };
-    double e2f, evf, a0f;
-    scal(G, e2f, evf, a0f);
-    res->e0 = S.e0;
-    res->e2 = e2f;
-    res->e_var = evf;
-    res->a0sq = a0f;
-    res->e_mrci_q = evf + (1.0 - a0f) * (evf - S.e0);
-    // jackknife
-    double m_e2 = 0, m_ev = 0, m_a0 = 0, tn_m[MRQ_NTYPES], te_m[MRQ_NTYPES];
-    for (int t = 0; t < MRQ_NTYPES; t++) tn_m[t] = te_m[t] = 0.0;
-    for (int g = 0; g < G; g++) {
-        double a, b, c;
-        scal(g, a, b, c);
-        m_e2 += a; m_ev += b; m_a0 += c;
-        for (int t = 0; t < MRQ_NTYPES; t++) {
-            tn_m[t] += vals[g][t * FIN_Q + 0];
-            te_m[t] += vals[g][t * FIN_Q + 1];
-        }
-    }
-    m_e2 /= G; m_ev /= G; m_a0 /= G;
-    for (int t = 0; t < MRQ_NTYPES; t++) { tn_m[t] /= G; te_m[t] /= G; }
-    double v_e2 = 0, v_ev = 0, v_a0 = 0, tn_v[MRQ_NTYPES], te_v[MRQ_NTYPES];
-    for (int t = 0; t < MRQ_NTYPES; t++) tn_v[t] = te_v[t] = 0.0;
-    for (int g = 0; g < G; g++) {
-        double a, b, c;
-        scal(g, a, b, c);
-        v_e2 += (a - m_e2) * (a - m_e2);
-        v_ev += (b - m_ev) * (b - m_ev);
-        v_a0 += (c - m_a0) * (c - m_a0);
-        for (int t = 0; t < MRQ_NTYPES; t++) {
-            double x = vals[g][t * FIN_Q + 0] - tn_m[t], y = vals[g][t * FIN_Q + 1] - te_m[t];
-            tn_v[t] += x * x;
-            te_v[t] += y * y;
-        }
-    }
     const double f = G > 1 ? (double)(G - 1) / G : NAN;
-    res->e2_sigma = sqrt(f * v_e2);
-    res->e_var_sigma = sqrt(f * v_ev);
-    res->a0sq_sigma = sqrt(f * v_a0);
-    double scr_norm = 0.0, visited = 0.0;
-    long long wsteps = 0;
-    for (int t = 0; t < MRQ_NTYPES; t++) {
-        res->type_norm[t] = vals[G][t * FIN_Q + 0];
-        res->type_e2[t] = vals[G][t * FIN_Q + 1];
-        res->type_screened[t] = vals[G][t * FIN_Q + 2];
-        res->type_norm_sigma[t] = sqrt(f * tn_v[t]);
-        res->type_e2_sigma[t] = sqrt(f * te_v[t]);
-        scr_norm += vals[G][t * FIN_Q + 3];
-        visited += vals[G][t * FIN_Q + 4];
-        res->type_steps[t] = (long long)S.type_steps[t];
-        wsteps += (long long)S.type_steps[t];
+    // quantity q of variant v: 0 E^(2), 1 E_var, 2 a_0^2, then per type its norm and E^(2)
+    auto quantity = [&](int q, int v, double Wt, double Et, double N0t) {
+        if (q == 0) {
+            double e2 = 0.0;
+            for (int t = 0; t < MRQ_NTYPES; t++) e2 += vals[v][t * FIN_Q + 1];
+            return e2;
+        }
+        const double Wv = Wt - (v < G ? sW[v] : 0.0);
+        if (q == 1) return (Et - (v < G ? sE[v] : 0.0)) / Wv;
+        if (q == 2) return c0 * c0 * (N0t - (v < G ? sN[v] : 0.0)) / Wv;
+        return vals[v][(q - 3) / 2 * FIN_Q + (q - 3) % 2];
+    };
+    if (threadIdx.x < 3 + 2 * MRQ_NTYPES) {
+        const int q = threadIdx.x;
+        double Wt = 0.0, Et = 0.0, N0t = 0.0;
+        for (int g = 0; g < G; g++) {
+            Wt += sW[g];
+            Et += sE[g];
+            N0t += sN[g];
+        }
+        const double full = quantity(q, G, Wt, Et, N0t);
+        double m = 0.0, var = 0.0;
+        for (int g = 0; g < G; g++) m += quantity(q, g, Wt, Et, N0t);
+        m /= G;
+        for (int g = 0; g < G; g++) {
+            const double x = quantity(q, g, Wt, Et, N0t);
+            var += (x - m) * (x - m);
+        }
+        const double sigma = sqrt(f * var);
+        if (q == 0) {
+            res->e0 = S.e0;
+            res->e2 = full;
+            res->e2_sigma = sigma;
+        } else if (q == 1) {
+            const double a0 = quantity(2, G, Wt, Et, N0t);
+            res->e_var = full;
+            res->e_var_sigma = sigma;
+            res->e_mrci_q = full + (1.0 - a0) * (full - S.e0);
+        } else if (q == 2) {
+            res->a0sq = full;
+            res->a0sq_sigma = sigma;
+        } else {
+            const int t = (q - 3) / 2;
+            if ((q - 3) % 2 == 0) {
+                res->type_norm[t] = full;
+                res->type_norm_sigma[t] = sigma;
+                res->type_screened[t] = vals[G][t * FIN_Q + 2];
+                res->type_steps[t] = (long long)S.type_steps[t];
+            } else {
+                res->type_e2[t] = full;
+                res->type_e2_sigma[t] = sigma;
+            }
+        }
+    } else if (threadIdx.x == 32) {
+        double scr_norm = 0.0, visited = 0.0;
+        long long wsteps = 0;
+        for (int t = 0; t < MRQ_NTYPES; t++) {
+            scr_norm += vals[G][t * FIN_Q + 3];
+            visited += vals[G][t * FIN_Q + 4];
+            wsteps += (long long)S.type_steps[t];
+        }
+        res->screened_norm = scr_norm;
+        res->n_labels_visited = visited;
+        res->walker_steps = wsteps;
     }
-    res->screened_norm = scr_norm;
-    res->n_labels_visited = visited;
-    res->walker_steps = wsteps;
 }
 
 // ============================================================================ SC-MRCI(s) optimisation (Eq. 8-9)
@@ -946,6 +985,7 @@ struct mrq_ctx {
     double *d_accA = nullptr, *d_accB = nullptr;        // SC-MRCI gradient sums [G][nlab]
     double *d_grad = nullptr, *d_am_m = nullptr, *d_am_v = nullptr, *d_am_vh = nullptr;   // AMSGrad state
     unsigned long long* d_types = nullptr;
+    int* d_flist = nullptr;                             // visited labels of the finalize, by chunk, and their counts
     long long acc_lab = 0;
     int acc_G = 0;
     int* d_err = nullptr;
@@ -970,6 +1010,8 @@ struct mrq_ctx {
     SysDev hsys{};
     SysDev* d_sys = nullptr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+    cudaStream_t side = nullptr;     // second stream of a walk step, forked from and joined to `stream`
+    cudaEvent_t ev_fork = nullptr, ev_prep = nullptr, ev_join = nullptr;
     // launch configuration (mrq_set_launch, mrq_tune_batch)
     int wpb = 0;                     // warps per walk block (0: MRQ_MAXNW)
     int max_nw = MRQ_MAXNW;          // most warps per block whose candidate lists fit shared memory
@@ -1086,6 +1128,7 @@ static void free_walkers(mrq_ctx* c) {
     dfree(c->d_accW);
     dfree(c->d_accE);
     dfree(c->d_types);
+    dfree(c->d_flist);
     dfree(c->d_partial);
     c->nwalk = c->walk_cap = 0;
     c->acc_lab = 0;
@@ -1171,6 +1214,7 @@ struct WalkNeed {
 // case that none of its determinants share a row.  When the device cannot give that much, waves shrink.
 #define MRQ_WORK_BYTES (1LL << 30)
 #define MRQ_ROW_BYTES (8LL << 30)
+#define MRQ_FROW_BYTES (2LL << 30)     // likewise for the first-order determinants
 static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, long long* seg_out) {
     const long long per = 12 * 4 + 3 * 4 + 2 * (long long)sizeof(TaskGroup) + (long long)sizeof(GroupMeta) +
                           8LL * need.gstride + 24LL * (need.ns + MRQ_ACT_SLICES) + (long long)sizeof(RaceBest) + 4;
@@ -1180,7 +1224,7 @@ static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, lo
     long long groups = std::max(1LL, std::min(seg, MRQ_ROW_BYTES / per_group));
     groups = std::min(groups, std::max(1LL, (1LL << 29) / need.nref));           // reference indices and the table: 32 bits
     const long long per_fois = 8 * need.fois_nb + (long long)sizeof(FGroup) * need.fg_max + 8;
-    long long fwave = std::max(1LL, std::min(seg, MRQ_ROW_BYTES / per_fois));
+    long long fwave = std::max(1LL, std::min(seg, MRQ_FROW_BYTES / per_fois));
     fwave = std::min(fwave, std::max(1LL, (1LL << 30) / need.fg_max));           // group indices: 32 bits
     WalkScratch& w = ctx->work;
     for (;; groups = (groups + 1) / 2, fwave = (fwave + 1) / 2) {
@@ -1200,7 +1244,7 @@ static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, lo
                      best = take(sizeof(RaceBest) * seg), bound = take(4 * seg), ctl = take(4 * CTL_N), ao = take(8 * nr),
                      cls = take(nr), rrep = take(4 * nr), roff = take(8 * nr), tbl = take(4 * tsz), ul = take(4 * nr),
                      fgo = take(8 * fwave), fg = take(sizeof(FGroup) * (size_t)need.fg_max * fwave),
-                     rows = take(8 * std::max((size_t)need.row_worst * groups, (size_t)need.fois_nb * fwave));
+                     rows = take(8 * (size_t)need.row_worst * groups), frows = take(8 * (size_t)need.fois_nb * fwave);
         if (off > ctx->work_cap) {
             CK(cudaStreamSynchronize(ctx->stream));
             dfree(ctx->d_work);
@@ -1236,6 +1280,7 @@ static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, lo
         w.table = (int*)(b + tbl);
         w.ulist = (int*)(b + ul);
         w.rows = (double*)(b + rows);
+        w.frows = (double*)(b + frows);
         w.table_size = (int)tsz;
         w.fg_of = (int2*)(b + fgo);
         w.fg = (FGroup*)(b + fg);
@@ -1299,19 +1344,25 @@ static int launch_segment(mrq_ctx* ctx, const WalkSet& ws, WalkScratch sc, const
     const int sms = ctx->n_sm;
     const cudaStream_t st = ctx->stream;
     const size_t lbytes = cand_list_bytes(need.cap), rbytes = rows_warp_bytes(need.cap), fbytes = frows_warp_bytes(need.cap);
+    const cudaStream_t st2 = ctx->side;
     if (ws.nsys > 1) CK(cudaMemsetAsync(sc.ctl, 0, sizeof(int) * CTL_N, st));
     k_group<W><<<(unsigned)ws.nsys, 1024, 0, st>>>(ws, sc);
-    k_prep<W><<<(unsigned)std::min<long long>(n, 8LL * sms), 128, 0, st>>>(ws, sc);
-    k_int<W><<<(unsigned)std::min<long long>(n, 3LL * sms), 256, 0, st>>>(ws, sc);
-    k_fois_act<W><<<(unsigned)std::min<long long>(4 * n, 3LL * sms), 256, 0, st>>>(ws, sc);
-    cfg.dynamicSmemBytes = 0;
+    // side stream: the determinants' constants, the neighbours inside the CAS and of first-order determinants
+    CK(cudaEventRecord(ctx->ev_fork, st));
+    CK(cudaStreamWaitEvent(st2, ctx->ev_fork, 0));
+    k_prep<W><<<(unsigned)std::min<long long>(n, 8LL * sms), 128, 0, st2>>>(ws, sc);
+    CK(cudaEventRecord(ctx->ev_prep, st2));
+    k_int<W><<<(unsigned)std::min<long long>(n, 3LL * sms), 256, 0, st2>>>(ws, sc);
+    k_fois_act<W><<<(unsigned)std::min<long long>(4 * n, 3LL * sms), 256, 0, st2>>>(ws, sc);
     for (long long g = 0; g < n; g += sc.fwave) {
         sc.fwave0 = (int)g;
-        CK(cudaMemsetAsync(sc.ctl + CTL_FOIS, 0, sizeof(int) * (CTL_N - CTL_FOIS), st));
-        k_fgroups<W><<<(unsigned)std::min<long long>(n, 4LL * sms), 256, 0, st>>>(ws, sc);
-        k_frows<W, 3><<<(unsigned)ctx->frows_blocks, 32 * nw, nw * fbytes, st>>>(ws, sc, (int)fbytes, need.cap);
-        k_fois<W, 3><<<3 * sms, 256, 0, st>>>(ws, sc);
+        if (g > 0) CK(cudaMemsetAsync(sc.ctl + CTL_FOIS, 0, sizeof(int) * (CTL_CUR - CTL_FOIS), st2));
+        k_fgroups<W><<<(unsigned)std::min<long long>(n, 4LL * sms), 256, 0, st2>>>(ws, sc);
+        k_frows<W, 3><<<(unsigned)ctx->frows_blocks, 32 * nw, nw * fbytes, st2>>>(ws, sc, (int)fbytes, need.cap);
+        k_fois<W, 3><<<3 * sms, 256, 0, st2>>>(ws, sc);
     }
+    CK(cudaEventRecord(ctx->ev_join, st2));
+    // main stream: the CAS determinants' rows and pairs
     for (long long g = 0; g < n; g += sc.wave_groups) {
         sc.wave0 = (int)g;
         k_refs<W><<<(unsigned)std::min<long long>(n, 8LL * sms), 256, 0, st>>>(ws, sc);
@@ -1321,11 +1372,13 @@ static int launch_segment(mrq_ctx* ctx, const WalkSet& ws, WalkScratch sc, const
         cfg.dynamicSmemBytes = nw * rbytes;
         if (ctx->rows_minb == 4) CK(cudaLaunchKernelEx(&cfg, k_rows<W, 4>, ws, sc, (int)rbytes, need.cap));
         else CK(cudaLaunchKernelEx(&cfg, k_rows<W, 2>, ws, sc, (int)rbytes, need.cap));
+        if (g == 0) CK(cudaStreamWaitEvent(st, ctx->ev_prep, 0));
         cfg.gridDim = dim3(4u * sms);
         cfg.blockDim = dim3(256);
         cfg.dynamicSmemBytes = 0;
         CK(cudaLaunchKernelEx(&cfg, k_pairs<W, 4>, ws, sc));
     }
+    CK(cudaStreamWaitEvent(st, ctx->ev_join, 0));
     k_move<W><<<(unsigned)std::min<long long>((n + nw - 1) / nw, 4LL * sms), 32 * nw, nw * lbytes, st>>>(
         ws, sc, accumulate, (int)lbytes, need.cap);
     CK(cudaGetLastError());
@@ -1432,7 +1485,7 @@ static int walk_plan(mrq_ctx* ctx, SysDev& s) {
     ctx->row_worst = total - cas_nb + 4 * nref;
     // slices of a determinant's units: about four units each, so that a step on a few hundred
     // determinants is some 10^5 warp tasks and one on a few still spreads over the chip
-    s.nslice = 32;
+    s.nslice = 128;
     while (s.nslice < MRQ_NS_MAX && s.nslice * 4 < off) s.nslice <<= 1;
     s.cas_nb_total = total;
     // Groups of a first-order determinant's neighbours: the outer patterns of a pair (X_a, Y_a) of each
@@ -1530,6 +1583,10 @@ int mrq_create(mrq_ctx** out, int device) {
         cudaMalloc(&ctx->d_err, sizeof(int)) != cudaSuccess || cudaMalloc(&ctx->d_sys, sizeof(SysDev)) != cudaSuccess ||
         cudaMalloc(&ctx->d_res, sizeof(mrq_result)) != cudaSuccess || cudaEventCreate(&ctx->ev0) != cudaSuccess ||
         cudaEventCreate(&ctx->ev1) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->ev_prep, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->ev_wait, cudaEventDisableTiming) != cudaSuccess) {
         mrq_destroy(ctx);
         return MRQ_CUDA_ERROR;
@@ -1572,6 +1629,10 @@ void mrq_destroy(mrq_ctx* ctx) {
     if (ctx->ev0) cudaEventDestroy(ctx->ev0);
     if (ctx->ev1) cudaEventDestroy(ctx->ev1);
     if (ctx->ev_wait) cudaEventDestroy(ctx->ev_wait);
+    if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
+    if (ctx->ev_prep) cudaEventDestroy(ctx->ev_prep);
+    if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
+    if (ctx->side) cudaStreamDestroy(ctx->side);
     if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
     delete ctx;
 }
@@ -1906,6 +1967,7 @@ int mrq_walkers_init(mrq_ctx* ctx, const mrq_sample_params* p) {
         dfree(ctx->d_accW);
         dfree(ctx->d_accE);
         dfree(ctx->d_types);
+        dfree(ctx->d_flist);
         CK(cudaMalloc(&ctx->d_accN, sizeof(double) * ctx->nlab * p->n_groups));
         CK(cudaMalloc(&ctx->d_accU, sizeof(double) * ctx->nlab * p->n_groups));
         dfree(ctx->d_accA);
@@ -1915,6 +1977,7 @@ int mrq_walkers_init(mrq_ctx* ctx, const mrq_sample_params* p) {
         CK(cudaMalloc(&ctx->d_accW, sizeof(double) * p->n_groups));
         CK(cudaMalloc(&ctx->d_accE, sizeof(double) * p->n_groups));
         CK(cudaMalloc(&ctx->d_types, sizeof(unsigned long long) * MRQ_NTYPES));
+        CK(cudaMalloc(&ctx->d_flist, sizeof(int) * (ctx->nlab + (ctx->nlab + FIN_CHUNK - 1) / FIN_CHUNK)));
         ctx->acc_lab = ctx->nlab;
         ctx->acc_G = p->n_groups;
     }
@@ -1985,8 +2048,6 @@ int mrq_walkers_advance(mrq_ctx* ctx, int64_t n_steps) {
     return 0;
 }
 
-static const long long FIN_CHUNK = 8192;
-
 static long long fin_scratch_doubles(const mrq_ctx* ctx, int* nchunk) {
     *nchunk = (int)((ctx->nlab + FIN_CHUNK - 1) / FIN_CHUNK);
     return (long long)(ctx->G + 1) * (*nchunk) * FIN_NV;
@@ -1996,9 +2057,10 @@ static long long fin_scratch_doubles(const mrq_ctx* ctx, int* nchunk) {
 // (the device copy of the system is current since mrq_walkers_init pushed it, so nothing is copied
 // in: a copy from pageable host memory would wait for the walk and defeat the deadline)
 static int finalize_with(mrq_ctx* ctx, mrq_result* out, double* scratch, int nchunk) {
-    k_fin_labels<<<(ctx->G + 1) * nchunk, 256, 0, ctx->stream>>>(ctx->d_sys, ctx->tau, nchunk, FIN_CHUNK, scratch);
+    k_fin_list<<<nchunk, 256, 0, ctx->stream>>>(ctx->d_sys, FIN_CHUNK, ctx->d_flist);
+    k_fin_labels<<<(ctx->G + 1) * nchunk, 256, 0, ctx->stream>>>(ctx->d_sys, ctx->tau, nchunk, FIN_CHUNK, ctx->d_flist, scratch);
     CK(cudaGetLastError());
-    k_fin_reduce<<<1, 256, 0, ctx->stream>>>(ctx->d_sys, scratch, nchunk, ctx->d_res);
+    k_fin_reduce<<<1, 1024, 0, ctx->stream>>>(ctx->d_sys, scratch, nchunk, ctx->d_res);
     CK(cudaGetLastError());
     if (int r = sync_stream(ctx)) return r;
     CK(cudaMemcpyAsync(out, ctx->d_res, sizeof(mrq_result), cudaMemcpyDeviceToHost, ctx->stream));
@@ -2417,6 +2479,7 @@ int mrq_load_accumulators(mrq_ctx* ctx, int32_t n_groups, const double* accN, co
         dfree(ctx->d_accW);
         dfree(ctx->d_accE);
         dfree(ctx->d_types);
+        dfree(ctx->d_flist);
         CK(cudaMalloc(&ctx->d_accN, sizeof(double) * ctx->nlab * n_groups));
         CK(cudaMalloc(&ctx->d_accU, sizeof(double) * ctx->nlab * n_groups));
         CK(cudaMalloc(&ctx->d_accA, sizeof(double) * ctx->nlab * n_groups));
@@ -2424,6 +2487,7 @@ int mrq_load_accumulators(mrq_ctx* ctx, int32_t n_groups, const double* accN, co
         CK(cudaMalloc(&ctx->d_accW, sizeof(double) * n_groups));
         CK(cudaMalloc(&ctx->d_accE, sizeof(double) * n_groups));
         CK(cudaMalloc(&ctx->d_types, sizeof(unsigned long long) * MRQ_NTYPES));
+        CK(cudaMalloc(&ctx->d_flist, sizeof(int) * (ctx->nlab + (ctx->nlab + FIN_CHUNK - 1) / FIN_CHUNK)));
         ctx->acc_lab = ctx->nlab;
         ctx->acc_G = n_groups;
     }

@@ -82,11 +82,11 @@ struct GroupMeta {
 enum {
     CTL_TGC, CTL_GC,              // CAS task groups, CAS determinants
     CTL_TGF, CTL_GF,              // first-order task groups, determinants
-    CTL_INT, CTL_PAIRS, CTL_ACT, CTL_FOIS, CTL_ROWTASK,   // next warp task of each kernel
+    CTL_INT, CTL_PAIRS, CTL_ACT, CTL_ROWTASK,   // next warp task of each kernel
     CTL_BIG, CTL_SMALL,           // distinct rows of a wave: long ones (from the list's front), short ones
-    CTL_FG, CTL_FGTASK,           // neighbour groups of a wave of first-order determinants, next task
-    CTL_PAD,
-    CTL_CUR,                      // (64 bits, aligned) doubles of the row buffer in use
+    CTL_FOIS, CTL_FG, CTL_FGTASK, // first-order waves: next task of k_fois, most groups of a determinant, next task
+    CTL_FCUR = 14,                // (64 bits) doubles of the first-order row buffer in use
+    CTL_CUR = 16,                 // (64 bits) doubles of the row buffer in use
     CTL_N = CTL_CUR + 2
 };
 #define MRQ_INT_SLICES 8          // warp tasks of a CAS determinant's neighbours inside the CAS
@@ -128,8 +128,9 @@ struct WalkScratch {
     int *table, *ulist;           // open addressing over references; the owners
     double* rows;
     int table_size, nref_max, wave_groups, wave0;
-    // groups of a wave of at most fwave first-order determinants (fg_max each), in the same row buffer
+    // groups of a wave of at most fwave first-order determinants (fg_max each) and psi_s of their neighbours
     FGroup* fg;
+    double* frows;
     int2* fg_of;              // per determinant of the wave: first group, groups
     int fg_max, fwave, fwave0;
     long long gstride, nseg;
@@ -1225,12 +1226,25 @@ __global__ void __launch_bounds__(1024) k_group(const WalkSet ws, const WalkScra
         const int ntg = (c + sc.tgw - 1) / sc.tgw;
         const int at = atomicAdd(sc.ctl + (cas ? CTL_TGC : CTL_TGF), ntg), grp = atomicAdd(sc.ctl + (cas ? CTL_GC : CTL_GF), 1);
         TaskGroup* const tg = cas ? sc.tgc : sc.tgf;
+        const int det = cas ? grp : (int)(sc.nseg - 1 - grp);
+        GroupMeta m;
+        m.d[0][0] = m.d[0][1] = m.d[1][0] = m.d[1][1] = 0;
+#pragma unroll
+        for (int sg = 0; sg < 2; sg++)
+#pragma unroll
+            for (int w = 0; w < W; w++) m.d[sg][w] = d[sg][w];
+        m.psi = wk[rep[k]].psi;
+        m.hnn = m.hdnn = 0.0;
+        m.label = det_label<W>(S, d, m.h, m.p);
+        m.sys = sys;
+        m.pad = 0;
+        sc.meta[det] = m;
         for (int q = 0; q < ntg; q++) {
             TaskGroup t;
             t.sys = sys;
             t.first = base + st + q * sc.tgw;
             t.count = min(sc.tgw, c - q * sc.tgw);
-            t.group = cas ? grp : (int)(sc.nseg - 1 - grp);
+            t.group = det;
             t.primary = q == 0;
             t.pad = 0;
             tg[at + q] = t;
@@ -1248,7 +1262,7 @@ __global__ void __launch_bounds__(1024) k_group(const WalkSet ws, const WalkScra
     }
 }
 
-// Constants of every distinct determinant, one block each: label, diagonals, single-excitation operator
+// Constants of every distinct determinant, one block each: diagonals, single-excitation operator
 template <int W>
 __global__ void __launch_bounds__(128) k_prep(const WalkSet ws, const WalkScratch sc) {
     __shared__ SysDev S;
@@ -1264,37 +1278,25 @@ __global__ void __launch_bounds__(128) k_prep(const WalkSet ws, const WalkScratc
             cur = tg.sys;
             __syncthreads();
         }
-        const Walker* const wk = ws.walkers[tg.sys] + sc.members[tg.first];
+        GroupMeta& meta = sc.meta[tg.group];
+        const long long ln = meta.label;
+        if (ln < 0) continue;
         unsigned long long n[2][W];
-        load_det<W>(wk, n);
-        int h, p;
-        const long long ln = det_label<W>(S, n, h, p);
+#pragma unroll
+        for (int sg = 0; sg < 2; sg++)
+#pragma unroll
+            for (int w = 0; w < W; w++) n[sg][w] = meta.d[sg][w];
         if (threadIdx.x < 32) {
-            double hnn = 0.0, hdnn = 0.0;
-            if (ln >= 0) {
-                build_lists<W>(S, n, lists, h, p, threadIdx.x);
-                diagonals<W>(S, lists, n, threadIdx.x, hnn, hdnn);
-            }
+            double hnn, hdnn;
+            build_lists<W>(S, n, lists, meta.h, meta.p, threadIdx.x);
+            diagonals<W>(S, lists, n, threadIdx.x, hnn, hdnn);
             if (threadIdx.x == 0) {
-                GroupMeta m;
-                m.d[0][0] = m.d[0][1] = m.d[1][0] = m.d[1][1] = 0;
-#pragma unroll
-                for (int sg = 0; sg < 2; sg++)
-#pragma unroll
-                    for (int w = 0; w < W; w++) m.d[sg][w] = n[sg][w];
-                m.psi = wk->psi;
-                m.hnn = hnn;
-                m.hdnn = hdnn;
-                m.label = ln;
-                m.h = h;
-                m.p = p;
-                m.sys = tg.sys;
-                m.pad = 0;
-                sc.meta[tg.group] = m;
+                meta.hnn = hnn;
+                meta.hdnn = hdnn;
             }
         }
         NoCtr ctr;
-        if (ln >= 0 && wk->psi != 0.0) walker_operator<W>(S, n, ln == 0, sc.gops + (long long)tg.group * sc.gstride, ctr);
+        if (meta.psi != 0.0) walker_operator<W>(S, n, ln == 0, sc.gops + (long long)tg.group * sc.gstride, ctr);
     }
 }
 
@@ -1675,7 +1677,7 @@ __global__ void __launch_bounds__(256) k_fgroups(const WalkSet ws, const WalkScr
             }
             if (pass == 0) {
                 if (threadIdx.x == 0) {
-                    s_row = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(sc.ctl + CTL_CUR),
+                    s_row = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(sc.ctl + CTL_FCUR),
                                                  (unsigned long long)((s_base[1] + 3) & ~3));
                     s_base[1] = 0;
                 }
@@ -1728,7 +1730,7 @@ __global__ void __launch_bounds__(MRQ_MAXNW * 32, MINB) k_frows(const WalkSet ws
             fois_outer<W>(S, n, o);
         }
         __syncwarp();
-        double* const row = sc.rows + f.off;
+        double* const row = sc.frows + f.off;
         if (f.c == 0 && f.v == 0) {                       // a CAS determinant: the group holds one neighbour
             if (lane == 0) row[0] = __ldg(S.c) * hash_lookup(S, hash_key(S, (unsigned)f.ao, (unsigned)(f.ao >> 32)));
             continue;
@@ -1807,7 +1809,7 @@ __global__ void __launch_bounds__(256, MINB) k_fois(const WalkSet ws, const Walk
                 if (f.bc == 2) put2(o.hs[1], naf, af0, af1);
                 const int nvc = free_count(f.bv, f.sbv, o.fv[0], o.fv[1]);
                 const bool one = nrf + f.ac == 1;
-                const double* const row = sc.rows + f.off;
+                const double* const row = sc.frows + f.off;
                 for (int qb = 0; qb < f.nq; qb += 32) {
                     const bool on = qb + lane < f.nq;
                     double t = 0.0;
@@ -2312,8 +2314,9 @@ __global__ void __launch_bounds__(MRQ_MAXNW * 32) k_move(const WalkSet ws, const
 }
 
 // Accumulate the last step's walker records (Eq. 12, Eq. 16; weight w = 1/S): one warp per
-// (system, group), walkers of the group in id order, label-0 (CAS) sums as warp sums in a fixed
-// order and the other labels one lane at a time in lane order - the same result on every run.
+// (system, group), walkers of the group in id order.  The label-0 (CAS) sums are warp sums in a fixed
+// order; other labels are added by their lanes at once, walkers that share a label one after the other
+// in lane order - the same result on every run.
 __global__ void __launch_bounds__(1024) k_accum(const WalkSet ws) {
     const int sys = blockIdx.x;
     const int g = blockIdx.y * 32 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -2323,34 +2326,39 @@ __global__ void __launch_bounds__(1024) k_accum(const WalkSet ws) {
     const long long nw = ws.offsets[sys + 1] - ws.offsets[sys];
     const long long L = S.nlab;
     double n0 = 0.0, a0 = 0.0, b0 = 0.0, wsum = 0.0, esum = 0.0;
+    unsigned count = 0;                       // lane t < MRQ_NTYPES: steps at type t
     const double c0 = S.c[0];
     for (long long base = g; base < nw; base += 32LL * S.G) {
         const long long i = base + (long long)lane * S.G;
         long long l = -1;
         double w = 0.0, EL = 0.0, num = 0.0;
-        int type = 0;
+        int type = -1;
         if (i < nw) {
             l = wk[i].rl;
             w = wk[i].rw;
             EL = wk[i].rEL;
             num = wk[i].rnum;
-            type = wk[i].rtype;
+            if (l >= 0) type = wk[i].rtype;
+        }
+#pragma unroll
+        for (int t = 0; t < MRQ_NTYPES; t++) {
+            const unsigned m = __ballot_sync(0xffffffffu, type == t);
+            if (lane == t) count += __popc(m);
         }
         if (l >= 0) {
             wsum += w;
             esum += w * EL;
-            atomicAdd(S.type_steps + type, 1ull);
         }
         if (l == 0) {
             n0 += w / (c0 * c0);
             a0 += (w * EL) / c0;
             b0 += w / c0;
         }
-        unsigned m = __ballot_sync(0xffffffffu, l > 0);
-        while (m) {
-            const int src = __ffs(m) - 1;
-            m &= m - 1;
-            if (lane == src) {
+        unsigned todo = __ballot_sync(0xffffffffu, l > 0);
+        const unsigned peers = __match_any_sync(0xffffffffu, l) & todo;
+        while (todo) {
+            const bool mine = (todo >> lane & 1u) && (peers & todo & ((1u << lane) - 1u)) == 0u;   // first of its label left
+            if (mine) {
                 const double cl = S.c[l], c2 = cl * cl;
                 const long long at = (long long)g * L + l;
                 S.accN[at] += w / c2;
@@ -2358,6 +2366,7 @@ __global__ void __launch_bounds__(1024) k_accum(const WalkSet ws) {
                 S.accA[at] += (w * EL) / cl;
                 S.accB[at] += w / cl;
             }
+            todo &= ~__ballot_sync(0xffffffffu, mine);
             __syncwarp();
         }
     }
@@ -2366,6 +2375,7 @@ __global__ void __launch_bounds__(1024) k_accum(const WalkSet ws) {
     b0 = warp_sum(b0);
     wsum = warp_sum(wsum);
     esum = warp_sum(esum);
+    if (lane < MRQ_NTYPES && count) atomicAdd(S.type_steps + lane, (unsigned long long)count);
     if (lane == 0) {
         const long long at = (long long)g * L;
         S.accN[at] += n0;
