@@ -450,17 +450,66 @@ __device__ void block_sum_store(double (&v)[NV], double* out) {
     __syncthreads();
 }
 
-// E0 numerator and norm: sum_k c_k^2 H_kk + sum_k sum_{k' active exc} c_k H_kk' c_k'
-// one thread per (reference determinant, excitation) pair, strided; partials per block.
+#define MRQ_REF_BLOCKS 304       // blocks of k_ref_sum
+
+// <k|H|k> of every reference determinant: e_nuc + sum_p [h_pp + 1/2 sum_q ((pp|qq) - delta (pq|qp))], one
+// running sum per determinant (its rounding is that of E0 against the perturbers' energies), one thread
+// each, and every determinant's integrals in the same order, so that a warp's reads coincide or nearly do
 template <int W>
-__global__ void k_ref_energy(const SysDev* __restrict__ sys, const unsigned long long* dets, const double* coeffs,
-                             long long nref, double* partial) {
-    const SysDev S = *sys;
-    double acc[2] = {0.0, 0.0};
-    const int na = S.na;
-    const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long gsz = (long long)gridDim.x * blockDim.x;
-    for (long long i = gtid; i < nref; i += gsz) {
+__global__ void __launch_bounds__(128) k_ref_diag(const SysDev* __restrict__ sys, const unsigned long long* __restrict__ dets,
+                                                  long long nref, double* __restrict__ e) {
+    const SysDev& S = *sys;
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nref) return;
+    unsigned long long d[2][W];
+#pragma unroll
+    for (int w = 0; w < W; w++) {
+        d[0][w] = dets[i * 2 * W + w];
+        d[1][w] = dets[i * 2 * W + W + w];
+    }
+    double hdiag = S.e_nuc;
+#pragma unroll
+    for (int sg = 0; sg < 2; sg++)
+#pragma unroll
+        for (int w = 0; w < W; w++) {
+            unsigned long long om = d[sg][w];
+            while (om) {
+                const int p1 = 64 * w + __ffsll(om) - 1;
+                om &= om - 1;
+                hdiag += __ldg(S.h1 + p1 * S.n + p1);
+#pragma unroll
+                for (int sg2 = 0; sg2 < 2; sg2++)
+#pragma unroll
+                    for (int w2 = 0; w2 < W; w2++) {
+                        unsigned long long om2 = d[sg2][w2];
+                        while (om2) {
+                            const int p2 = 64 * w2 + __ffsll(om2) - 1;
+                            om2 &= om2 - 1;
+                            hdiag += 0.5 * eri_g(S, p1, p1, p2, p2);
+                            if (sg == sg2) hdiag -= 0.5 * eri_g(S, p1, p2, p2, p1);
+                        }
+                    }
+            }
+        }
+    e[i] = hdiag;
+}
+
+// E0 numerator per reference determinant k: e[k] <- c_k^2 H_kk + 2 sum_{k' > k} c_k H_kk' c_k', one warp each,
+// lanes over its active singles and doubles; a pair is taken at the determinant of the smaller key (H is
+// symmetric), which halves the lookups and elements.  Bound by the random reads of the hash table and
+// the integrals.
+template <int W>
+__global__ void __launch_bounds__(256) k_ref_energy(const SysDev* __restrict__ sys, const unsigned long long* __restrict__ dets,
+                                                    const double* __restrict__ coeffs, long long nref, double* __restrict__ e) {
+    __shared__ SysDev S;
+    for (int k = threadIdx.x; k < (int)(sizeof(SysDev) / sizeof(int)); k += blockDim.x)
+        reinterpret_cast<int*>(&S)[k] = reinterpret_cast<const int*>(sys)[k];
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const long long nwarp = (long long)gridDim.x * (blockDim.x >> 5);
+    const unsigned am = (S.na >= 32) ? 0xFFFFFFFFu : ((1u << S.na) - 1u);
+    NoCtr z;
+    for (long long i = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < nref; i += nwarp) {
         unsigned long long d[2][W];
 #pragma unroll
         for (int w = 0; w < W; w++) {
@@ -468,115 +517,64 @@ __global__ void k_ref_energy(const SysDev* __restrict__ sys, const unsigned long
             d[1][w] = dets[i * 2 * W + W + w];
         }
         const double ck = coeffs[i];
-        acc[1] += ck * ck;
-        // diagonal
-        double hdiag = S.e_nuc;
-        for (int sg = 0; sg < 2; sg++)
-            for (int w = 0; w < W; w++) {
-                unsigned long long om = d[sg][w];
-                while (om) {
-                    int p1 = 64 * w + __ffsll(om) - 1;
-                    om &= om - 1;
-                    hdiag += __ldg(S.h1 + p1 * S.n + p1);
-                    for (int sg2 = 0; sg2 < 2; sg2++)
-                        for (int w2 = 0; w2 < W; w2++) {
-                            unsigned long long om2 = d[sg2][w2];
-                            while (om2) {
-                                int p2 = 64 * w2 + __ffsll(om2) - 1;
-                                om2 &= om2 - 1;
-                                hdiag += 0.5 * eri_g(S, p1, p1, p2, p2);
-                                if (sg == sg2) hdiag -= 0.5 * eri_g(S, p1, p2, p2, p1);
-                            }
-                        }
+        const unsigned ao0 = active_bits<W>(S, d[0]), ao1 = active_bits<W>(S, d[1]);
+        const unsigned long long oa = ao0, ob = (unsigned long long)ao1 << 32, AO = oa | ob;
+        const unsigned long long ea = ~ao0 & am, eb = (unsigned long long)(~ao1 & am) << 32;
+        const unsigned long long key = hash_key(S, ao0, ao1);
+        double sum = 0.0;
+        const int total = active_neighbours(__popcll(oa), __popcll(ob), __popcll(ea), __popcll(eb));
+        for (int q = lane; q < total; q += 32) {
+            unsigned long long Xb, Yb;
+            const int r = active_neighbour(S, oa, ob, ea, eb, q, Xb, Yb);
+            const unsigned long long km = (AO & ~Xb) | Yb;
+            const unsigned long long kk = hash_key(S, (unsigned)km, (unsigned)(km >> 32));
+            if (kk < key) continue;
+            const double c = hash_lookup(S, kk);
+            if (c == 0.0) continue;
+            int rem[2], add[2];
+            act_list(S, Xb, rem);
+            act_list(S, Yb, add);
+            double h;
+            if (r == 1) {
+                const int sx = rem[0] >= S.n, px = rem[0] - sx * S.n, py = add[0] - sx * S.n;
+                h = __ldg(S.hc + py * S.n + px);
+                const double* const col = S.sgl + py * S.nav + (px - S.nc);
+                for (unsigned long long bits = AO; bits; bits &= bits - 1) {
+                    const int b = __ffsll(bits) - 1;
+                    h += __ldg(col + (long long)((b & 31) + (((b >= 32) == (sx == 1)) ? 0 : S.na)) * S.nca * S.nav);
                 }
+                h = neg_if(h, popc_sel<W>(d, sx, min(px, py), max(px, py)));
+            } else {
+                h = double_elem<W>(S, d, rem[0], rem[1], add[0], add[1], z);
             }
-        double off = 0.0;
-        const unsigned ao[2] = {active_bits<W>(S, d[0]), active_bits<W>(S, d[1])};
-        const unsigned am = (na >= 32) ? 0xFFFFFFFFu : ((1u << na) - 1u);
-        // singles and same-spin doubles
-        for (int sg = 0; sg < 2; sg++) {
-            unsigned o1 = ao[sg];
-            while (o1) {
-                int t = __ffs(o1) - 1;
-                o1 &= o1 - 1;
-                unsigned e1 = ~ao[sg] & am;
-                while (e1) {
-                    int u = __ffs(e1) - 1;
-                    e1 &= e1 - 1;
-                    unsigned k0 = ao[0], k1 = ao[1];
-                    (sg ? k1 : k0) ^= (1u << t) | (1u << u);
-                    double c = hash_lookup(S, hash_key(S, k0, k1));
-                    NoCtr z;
-                    if (c != 0.0) off += ck * c * single_elem<W>(S, d, sg * S.n + S.nc + t, sg * S.n + S.nc + u, z);
-                }
-                unsigned o2 = o1;   // t2 > t
-                while (o2) {
-                    int t2 = __ffs(o2) - 1;
-                    o2 &= o2 - 1;
-                    unsigned e2 = ~ao[sg] & am;
-                    while (e2) {
-                        int u1 = __ffs(e2) - 1;
-                        e2 &= e2 - 1;
-                        unsigned e3 = e2;
-                        while (e3) {
-                            int u2 = __ffs(e3) - 1;
-                            e3 &= e3 - 1;
-                            unsigned k0 = ao[0], k1 = ao[1];
-                            (sg ? k1 : k0) ^= (1u << t) | (1u << t2) | (1u << u1) | (1u << u2);
-                            double c = hash_lookup(S, hash_key(S, k0, k1));
-                            if (c != 0.0) {
-                                int b = sg * S.n + S.nc;
-                                NoCtr z;
-                                off += ck * c * double_elem<W>(S, d, b + t, b + t2, b + u1, b + u2, z);
-                            }
-                        }
-                    }
-                }
-            }
+            sum += 2.0 * (ck * c) * h;
         }
-        // opposite-spin doubles
-        {
-            unsigned oa = ao[0];
-            while (oa) {
-                int t = __ffs(oa) - 1;
-                oa &= oa - 1;
-                unsigned ea = ~ao[0] & am;
-                while (ea) {
-                    int u = __ffs(ea) - 1;
-                    ea &= ea - 1;
-                    unsigned ob = ao[1];
-                    while (ob) {
-                        int s = __ffs(ob) - 1;
-                        ob &= ob - 1;
-                        unsigned eb = ~ao[1] & am;
-                        while (eb) {
-                            int v = __ffs(eb) - 1;
-                            eb &= eb - 1;
-                            unsigned k0 = ao[0] ^ ((1u << t) | (1u << u));
-                            unsigned k1 = ao[1] ^ ((1u << s) | (1u << v));
-                            double c = hash_lookup(S, hash_key(S, k0, k1));
-                            NoCtr z;
-                            if (c != 0.0)
-                                off += ck * c *
-                                       double_elem<W>(S, d, S.nc + t, S.n + S.nc + s, S.nc + u, S.n + S.nc + v, z);
-                        }
-                    }
-                }
-            }
-        }
-        acc[0] += ck * ck * hdiag + off;
+        sum = warp_sum(sum);
+        if (lane == 0) e[i] = ck * ck * e[i] + sum;
+    }
+}
+
+// sums of the determinants' numerators and of c_k^2, partials per block
+__global__ void __launch_bounds__(128) k_ref_sum(const double* __restrict__ e, const double* __restrict__ coeffs, long long nref,
+                                                 double* partial) {
+    double acc[2] = {0.0, 0.0};
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nref; i += (long long)gridDim.x * blockDim.x) {
+        acc[0] += e[i];
+        acc[1] += coeffs[i] * coeffs[i];
     }
     block_sum_store<2>(acc, partial);
 }
 
-// spin-summed active 1-RDM element gamma_tu (unnormalised): block (t, u) over all determinants
+// spin-summed active 1-RDM element gamma_tu (unnormalised): block (t, u; slice) over a slice of the
+// determinants, partial sums added in order by k_setup_finish
+#define MRQ_RDM_SLICES 16
 template <int W>
-__global__ void k_ref_rdm(const SysDev* __restrict__ sys, const unsigned long long* dets, const double* coeffs,
-                          long long nref, double* gamma_raw) {
-    const SysDev S = *sys;
+__global__ void __launch_bounds__(256) k_ref_rdm(const SysDev* __restrict__ sys, const unsigned long long* __restrict__ dets,
+                                                 const double* __restrict__ coeffs, long long nref, double* partial) {
+    const SysDev& S = *sys;
     const int t = blockIdx.x / S.na, u = blockIdx.x % S.na;
     double acc[1] = {0.0};
-    for (long long i = threadIdx.x; i < nref; i += blockDim.x) {
+    for (long long i = (long long)blockIdx.y * blockDim.x + threadIdx.x; i < nref; i += (long long)gridDim.y * blockDim.x) {
         unsigned long long d[2][W];
 #pragma unroll
         for (int w = 0; w < W; w++) {
@@ -599,7 +597,6 @@ __global__ void k_ref_rdm(const SysDev* __restrict__ sys, const unsigned long lo
             if (c != 0.0) acc[0] += ck * c * sgn_single<W>(d[sg], S.nc + u, S.nc + t);
         }
     }
-    // single block per (t,u): reduce and store
     __shared__ double red[32];
     double x = warp_sum(acc[0]);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
@@ -607,48 +604,68 @@ __global__ void k_ref_rdm(const SysDev* __restrict__ sys, const unsigned long lo
     if (threadIdx.x == 0) {
         double s = 0.0;
         for (int w = 0; w < (int)(blockDim.x + 31) / 32; w++) s += red[w];
-        gamma_raw[blockIdx.x] = s;
+        partial[(long long)blockIdx.x * gridDim.y + blockIdx.y] = s;
     }
 }
 
 // reduce E0 partials (fixed order), normalise gamma, eps_p = F_pp, E_core; writes scal[0..4]
-__global__ void k_setup_finish(const SysDev* __restrict__ sys, const double* partial, int npart, double* gamma,
-                               double* eps, double* scal) {
-    const SysDev S = *sys;
-    __shared__ double s_num, s_norm;
-    if (threadIdx.x == 0) {
-        double a = 0.0, b = 0.0;
-        for (int i = 0; i < npart; i++) {
-            a += partial[2 * i];
-            b += partial[2 * i + 1];
-        }
-        s_num = a;
-        s_norm = b;
+__global__ void __launch_bounds__(1024) k_setup_finish(const SysDev* __restrict__ sys, const double* __restrict__ partial,
+                                                       const double* __restrict__ rdm, double* gamma, double* eps,
+                                                       double* scal) {
+    const SysDev& S = *sys;
+    __shared__ double s_part[2][MRQ_REF_BLOCKS], s_sum[2], s_pair[64 * 64], s_ec;      // n_core <= 64
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int i = threadIdx.x; i < 2 * MRQ_REF_BLOCKS; i += blockDim.x) s_part[i & 1][i >> 1] = partial[i];
+    for (int k = threadIdx.x; k < S.nc * S.nc; k += blockDim.x) {
+        const int i = k / S.nc, j = k - i * S.nc;
+        s_pair[k] = 2.0 * eri_g(S, i, i, j, j) - eri_g(S, i, j, j, i);
     }
     __syncthreads();
-    const int na = S.na;
-    for (int k = threadIdx.x; k < na * na; k += blockDim.x) gamma[k] /= s_norm;
-    __syncthreads();
-    for (int p = threadIdx.x; p < S.n; p += blockDim.x) {
-        double v = __ldg(S.hc + p * S.n + p);
-        for (int t = 0; t < na; t++)
-            for (int u = 0; u < na; u++)
-                v += gamma[t * na + u] * (eri_g(S, p, p, S.nc + t, S.nc + u) - 0.5 * eri_g(S, p, S.nc + t, S.nc + u, p));
-        eps[p] = v;
+    if (threadIdx.x < 64 && lane == 0) {     // two running sums over the blocks
+        double a = 0.0;
+        for (int i = 0; i < MRQ_REF_BLOCKS; i++) a += s_part[warp][i];
+        s_sum[warp] = a;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double ec = S.e_nuc, se = 0.0;
+    const double num = s_sum[0], norm = s_sum[1];
+    if (threadIdx.x == 0) {              // the core energy: one running sum over the orbitals
+        double ec = S.e_nuc;
         for (int i = 0; i < S.nc; i++) {
             ec += 2.0 * __ldg(S.h1 + i * S.n + i);
-            for (int j = 0; j < S.nc; j++) ec += 2.0 * eri_g(S, i, i, j, j) - eri_g(S, i, j, j, i);
-            se += eps[i];
+            for (int j = 0; j < S.nc; j++) ec += s_pair[i * S.nc + j];
         }
-        scal[0] = s_num / s_norm;
-        scal[1] = s_norm;
-        scal[2] = ec;
+        s_ec = ec;
+    }
+    const int na = S.na;
+    for (int k = threadIdx.x; k < na * na; k += blockDim.x) {
+        double g = 0.0;
+        for (int q = 0; q < MRQ_RDM_SLICES; q++) g += rdm[k * MRQ_RDM_SLICES + q];
+        gamma[k] = g / norm;
+    }
+    __syncthreads();
+    for (int p = warp; p < S.n; p += nw) {               // a warp per orbital, lanes over (t, u)
+        double v = 0.0;
+        for (int k = lane; k < na * na; k += 32) {
+            const int t = S.nc + k / na, u = S.nc + k % na;
+            v += gamma[k] * (eri_g(S, p, p, t, u) - 0.5 * eri_g(S, p, t, u, p));
+        }
+        v = warp_sum(v);
+        if (lane == 0) eps[p] = __ldg(S.hc + p * S.n + p) + v;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double se = 0.0;
+        for (int i = 0; i < S.nc; i++) se += eps[i];
+        scal[0] = num / norm;
+        scal[1] = norm;
+        scal[2] = s_ec;
         scal[3] = se;
     }
+}
+
+__global__ void k_default_coeffs(double* c, long long n) {
+    for (long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x; l < n; l += (long long)gridDim.x * blockDim.x)
+        c[l] = l == 0 ? 1.0 : 0.1;
 }
 
 // the race's screen and exact clock for given (k, rate, best clock) triples (parity of the move
@@ -671,6 +688,7 @@ __global__ void k_argmax_abs(const double* c, long long n, long long* out) {
     __shared__ long long bi[1024];
     double v = -1.0;
     long long idx = 0;
+#pragma unroll 8
     for (long long i = threadIdx.x; i < n; i += blockDim.x) {
         double a = fabs(c[i]);
         if (a > v) { v = a; idx = i; }
@@ -709,22 +727,26 @@ __device__ __forceinline__ int label_type(long long l, long long nPs, int nc2, i
 // A walk visits few of its labels (a few thousand of 256,038 at 56 orbitals), so one pass over the
 // accumulators finds them and the G + 1 jackknife variants read only those.  Bound by the one read
 // of accN (G x labels).
-__global__ void __launch_bounds__(256) k_fin_list(const SysDev* __restrict__ sys, long long chunk, int* __restrict__ list) {
+__global__ void __launch_bounds__(1024) k_fin_list(const SysDev* __restrict__ sys, long long chunk, int* __restrict__ list) {
     const int G = sys->G;
     const long long L = sys->nlab, lo = blockIdx.x * chunk, hi = min(L, lo + chunk);
     const double* const accN = sys->accN;
-    __shared__ int s_w[8];
+    __shared__ int s_w[32];
     int run = 0;
-    for (long long base = lo; base < hi; base += 256) {
+    for (long long base = lo; base < hi; base += 1024) {
         const long long l = base + threadIdx.x;
         bool seen = false;
-        if (l > 0 && l < hi)
-            for (int g = 0; g < G; g++) seen = seen || !(accN[(long long)g * L + l] == 0.0);
+        if (l > 0 && l < hi) {
+            unsigned long long any = 0;              // some bit of some group's sum (the sign aside) is set
+#pragma unroll 8
+            for (int g = 0; g < G; g++) any |= (unsigned long long)__double_as_longlong(accN[(long long)g * L + l]) << 1;
+            seen = any != 0;
+        }
         const unsigned m = __ballot_sync(0xffffffffu, seen);
         if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = __popc(m);
         __syncthreads();
         int at = run, all = 0;
-        for (int w = 0; w < 8; w++) {
+        for (int w = 0; w < 32; w++) {
             if (w < (int)(threadIdx.x >> 5)) at += s_w[w];
             all += s_w[w];
         }
@@ -792,8 +814,8 @@ __global__ void __launch_bounds__(256) k_fin_labels(const SysDev* __restrict__ s
     block_sum_store<FIN_NV>(acc, partial);
 }
 
-// one block: sum chunk partials in order, jackknife over groups, write the result struct.  Warp k makes the
-// sums of the (variant, quantity) pairs k, k + 32, ...; then one thread per reported quantity runs the jackknife.
+// one block: sum chunk partials in order, every reported quantity of every variant (one thread each), then
+// one thread per quantity runs the jackknife over the groups and writes the result struct
 __global__ void __launch_bounds__(1024) k_fin_reduce(const SysDev* __restrict__ sys, const double* __restrict__ partial,
                                                      int nchunk, mrq_result* res) {
     const SysDev& S = *sys;
@@ -817,40 +839,41 @@ __global__ void __launch_bounds__(1024) k_fin_reduce(const SysDev* __restrict__ 
     const double c0 = S.c[0];
     const double f = G > 1 ? (double)(G - 1) / G : NAN;
     // quantity q of variant v: 0 E^(2), 1 E_var, 2 a_0^2, then per type its norm and E^(2)
-    auto quantity = [&](int q, int v, double Wt, double Et, double N0t) {
+    constexpr int NQ = 3 + 2 * MRQ_NTYPES;
+    __shared__ double x[65][NQ];
+    for (int idx = threadIdx.x; idx < (G + 1) * NQ; idx += blockDim.x) {
+        const int v = idx / NQ, q = idx - v * NQ;
+        double y = 0.0;
         if (q == 0) {
-            double e2 = 0.0;
-            for (int t = 0; t < MRQ_NTYPES; t++) e2 += vals[v][t * FIN_Q + 1];
-            return e2;
+            for (int t = 0; t < MRQ_NTYPES; t++) y += vals[v][t * FIN_Q + 1];
+        } else if (q < 3) {
+            double Wt = 0.0, Xt = 0.0;
+            for (int g = 0; g < G; g++) {
+                Wt += sW[g];
+                Xt += q == 1 ? sE[g] : sN[g];
+            }
+            const double Wv = Wt - (v < G ? sW[v] : 0.0), Xv = Xt - (v < G ? (q == 1 ? sE[v] : sN[v]) : 0.0);
+            y = q == 1 ? Xv / Wv : c0 * c0 * Xv / Wv;
+        } else {
+            y = vals[v][(q - 3) / 2 * FIN_Q + (q - 3) % 2];
         }
-        const double Wv = Wt - (v < G ? sW[v] : 0.0);
-        if (q == 1) return (Et - (v < G ? sE[v] : 0.0)) / Wv;
-        if (q == 2) return c0 * c0 * (N0t - (v < G ? sN[v] : 0.0)) / Wv;
-        return vals[v][(q - 3) / 2 * FIN_Q + (q - 3) % 2];
-    };
-    if (threadIdx.x < 3 + 2 * MRQ_NTYPES) {
+        x[v][q] = y;
+    }
+    __syncthreads();
+    if (threadIdx.x < NQ) {
         const int q = threadIdx.x;
-        double Wt = 0.0, Et = 0.0, N0t = 0.0;
-        for (int g = 0; g < G; g++) {
-            Wt += sW[g];
-            Et += sE[g];
-            N0t += sN[g];
-        }
-        const double full = quantity(q, G, Wt, Et, N0t);
+        const double full = x[G][q];
         double m = 0.0, var = 0.0;
-        for (int g = 0; g < G; g++) m += quantity(q, g, Wt, Et, N0t);
+        for (int g = 0; g < G; g++) m += x[g][q];
         m /= G;
-        for (int g = 0; g < G; g++) {
-            const double x = quantity(q, g, Wt, Et, N0t);
-            var += (x - m) * (x - m);
-        }
+        for (int g = 0; g < G; g++) var += (x[g][q] - m) * (x[g][q] - m);
         const double sigma = sqrt(f * var);
         if (q == 0) {
             res->e0 = S.e0;
             res->e2 = full;
             res->e2_sigma = sigma;
         } else if (q == 1) {
-            const double a0 = quantity(2, G, Wt, Et, N0t);
+            const double a0 = x[G][2];
             res->e_var = full;
             res->e_var_sigma = sigma;
             res->e_mrci_q = full + (1.0 - a0) * (full - S.e0);
@@ -961,11 +984,14 @@ struct mrq_ctx {
     double *d_h1 = nullptr, *d_eri = nullptr, *d_eri4 = nullptr, *d_tab = nullptr, *d_sgl = nullptr, *d_hc = nullptr,
            *d_eps = nullptr, *d_gamma = nullptr;
     unsigned short* d_colex = nullptr;
+    size_t cap_h1 = 0, cap_eri = 0, cap_eri4 = 0, cap_tab = 0, cap_sgl = 0, cap_hc = 0, cap_eps = 0, cap_gamma = 0;   // bytes
     long long nHs = 0, nPs = 0, nlab = 0;
     // reference
     bool ref = false;
     long long nref = 0;
     HashSlot* d_hash = nullptr;
+    unsigned char* d_setup = nullptr;   // the reference's determinants and coefficients and partial sums while it is set up
+    size_t cap_hash = 0, cap_c = 0, cap_setup = 0;
     unsigned long long hcap = 0;
     unsigned long long start[4] = {0, 0, 0, 0};
     double start_c = 0.0;
@@ -1010,8 +1036,8 @@ struct mrq_ctx {
     SysDev hsys{};
     SysDev* d_sys = nullptr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-    cudaStream_t side = nullptr;     // second stream of a walk step, forked from and joined to `stream`
-    cudaEvent_t ev_fork = nullptr, ev_prep = nullptr, ev_join = nullptr;
+    cudaStream_t side[2] = {};       // side streams of a walk step, forked from and joined to `stream`
+    cudaEvent_t ev_fork = nullptr, ev_prep = nullptr, ev_join[2] = {};
     // launch configuration (mrq_set_launch, mrq_tune_batch)
     int wpb = 0;                     // warps per walk block (0: MRQ_MAXNW)
     int max_nw = MRQ_MAXNW;          // most warps per block whose candidate lists fit shared memory
@@ -1020,10 +1046,11 @@ struct mrq_ctx {
     struct GraphKey {
         const void *sys = nullptr, *wptr = nullptr, *off = nullptr, *work = nullptr;
         long long nslots = 0;
-        int k = 0, wpb = 0, spl = 0, cap = 0, gstride = 0, ns = 0, nref = 0, fg = 0;
+        int k = 0, wpb = 0, spl = 0, cap = 0, gstride = 0, ns = 0, nref = 0, fg = 0, wave = 0, fwave = 0;
         bool operator==(const GraphKey& o) const {
             return sys == o.sys && wptr == o.wptr && off == o.off && work == o.work && nslots == o.nslots &&
-                   k == o.k && wpb == o.wpb && spl == o.spl && cap == o.cap && gstride == o.gstride && ns == o.ns && nref == o.nref && fg == o.fg;
+                   k == o.k && wpb == o.wpb && spl == o.spl && cap == o.cap && gstride == o.gstride && ns == o.ns && nref == o.nref && fg == o.fg && wave == o.wave &&
+                   fwave == o.fwave;
         }
     };
     // per determinant width and warps per block (8, 4, 2, 1) of a batch launch
@@ -1110,9 +1137,24 @@ static void dfree(T*& p) {
     p = nullptr;
 }
 
+// A device buffer of at least n elements: kept when it is that large already, so that a context that is
+// loaded again (a geometry scan) allocates nothing
+template <typename T>
+static cudaError_t reserve(T*& p, size_t& cap, size_t n) {
+    if (p && cap >= n * sizeof(T)) return cudaSuccess;
+    dfree(p);
+    cap = 0;
+    const cudaError_t e = cudaMalloc(&p, n * sizeof(T));
+    if (e == cudaSuccess) cap = n * sizeof(T);
+    else p = nullptr;
+    return e;
+}
+
 static void free_reference(mrq_ctx* c) {
     dfree(c->d_hash);
     dfree(c->d_c);
+    dfree(c->d_setup);
+    c->cap_hash = c->cap_c = c->cap_setup = 0;
     c->ref = false;
 }
 static void free_walkers(mrq_ctx* c) {
@@ -1145,6 +1187,7 @@ static void free_hamiltonian(mrq_ctx* c) {
     dfree(c->d_eps);
     dfree(c->d_gamma);
     dfree(c->d_colex);
+    c->cap_h1 = c->cap_eri = c->cap_eri4 = c->cap_tab = c->cap_sgl = c->cap_hc = c->cap_eps = c->cap_gamma = 0;
     c->ham = false;
 }
 
@@ -1344,24 +1387,29 @@ static int launch_segment(mrq_ctx* ctx, const WalkSet& ws, WalkScratch sc, const
     const int sms = ctx->n_sm;
     const cudaStream_t st = ctx->stream;
     const size_t lbytes = cand_list_bytes(need.cap), rbytes = rows_warp_bytes(need.cap), fbytes = frows_warp_bytes(need.cap);
-    const cudaStream_t st2 = ctx->side;
+    const cudaStream_t st2 = ctx->side[0], st3 = ctx->side[1];
     if (ws.nsys > 1) CK(cudaMemsetAsync(sc.ctl, 0, sizeof(int) * CTL_N, st));
     k_group<W><<<(unsigned)ws.nsys, 1024, 0, st>>>(ws, sc);
-    // side stream: the determinants' constants, the neighbours inside the CAS and of first-order determinants
     CK(cudaEventRecord(ctx->ev_fork, st));
+    // first side stream: the determinants' constants, the neighbours inside the CAS, the active-only ones of
+    // first-order determinants
     CK(cudaStreamWaitEvent(st2, ctx->ev_fork, 0));
     k_prep<W><<<(unsigned)std::min<long long>(n, 8LL * sms), 128, 0, st2>>>(ws, sc);
     CK(cudaEventRecord(ctx->ev_prep, st2));
     k_int<W><<<(unsigned)std::min<long long>(n, 3LL * sms), 256, 0, st2>>>(ws, sc);
     k_fois_act<W><<<(unsigned)std::min<long long>(4 * n, 3LL * sms), 256, 0, st2>>>(ws, sc);
+    CK(cudaEventRecord(ctx->ev_join[0], st2));
+    // second side stream: the other neighbours of first-order determinants
+    CK(cudaStreamWaitEvent(st3, ctx->ev_fork, 0));
     for (long long g = 0; g < n; g += sc.fwave) {
         sc.fwave0 = (int)g;
-        if (g > 0) CK(cudaMemsetAsync(sc.ctl + CTL_FOIS, 0, sizeof(int) * (CTL_CUR - CTL_FOIS), st2));
-        k_fgroups<W><<<(unsigned)std::min<long long>(n, 4LL * sms), 256, 0, st2>>>(ws, sc);
-        k_frows<W, 3><<<(unsigned)ctx->frows_blocks, 32 * nw, nw * fbytes, st2>>>(ws, sc, (int)fbytes, need.cap);
-        k_fois<W, 3><<<3 * sms, 256, 0, st2>>>(ws, sc);
+        if (g > 0) CK(cudaMemsetAsync(sc.ctl + CTL_FOIS, 0, sizeof(int) * (CTL_CUR - CTL_FOIS), st3));
+        k_fgroups<W><<<(unsigned)std::min<long long>(n, 4LL * sms), 256, 0, st3>>>(ws, sc);
+        k_frows<W, 3><<<(unsigned)ctx->frows_blocks, 32 * nw, nw * fbytes, st3>>>(ws, sc, (int)fbytes, need.cap);
+        if (g == 0) CK(cudaStreamWaitEvent(st3, ctx->ev_prep, 0));
+        k_fois<W, 3><<<3 * sms, 256, 0, st3>>>(ws, sc);
     }
-    CK(cudaEventRecord(ctx->ev_join, st2));
+    CK(cudaEventRecord(ctx->ev_join[1], st3));
     // main stream: the CAS determinants' rows and pairs
     for (long long g = 0; g < n; g += sc.wave_groups) {
         sc.wave0 = (int)g;
@@ -1378,7 +1426,7 @@ static int launch_segment(mrq_ctx* ctx, const WalkSet& ws, WalkScratch sc, const
         cfg.dynamicSmemBytes = 0;
         CK(cudaLaunchKernelEx(&cfg, k_pairs<W, 4>, ws, sc));
     }
-    CK(cudaStreamWaitEvent(st, ctx->ev_join, 0));
+    for (int k = 0; k < 2; k++) CK(cudaStreamWaitEvent(st, ctx->ev_join[k], 0));
     k_move<W><<<(unsigned)std::min<long long>((n + nw - 1) / nw, 4LL * sms), 32 * nw, nw * lbytes, st>>>(
         ws, sc, accumulate, (int)lbytes, need.cap);
     CK(cudaGetLastError());
@@ -1583,10 +1631,12 @@ int mrq_create(mrq_ctx** out, int device) {
         cudaMalloc(&ctx->d_err, sizeof(int)) != cudaSuccess || cudaMalloc(&ctx->d_sys, sizeof(SysDev)) != cudaSuccess ||
         cudaMalloc(&ctx->d_res, sizeof(mrq_result)) != cudaSuccess || cudaEventCreate(&ctx->ev0) != cudaSuccess ||
         cudaEventCreate(&ctx->ev1) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&ctx->side[0], cudaStreamNonBlocking) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&ctx->side[1], cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->ev_prep, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->ev_join[0], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->ev_join[1], cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->ev_wait, cudaEventDisableTiming) != cudaSuccess) {
         mrq_destroy(ctx);
         return MRQ_CUDA_ERROR;
@@ -1631,8 +1681,10 @@ void mrq_destroy(mrq_ctx* ctx) {
     if (ctx->ev_wait) cudaEventDestroy(ctx->ev_wait);
     if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
     if (ctx->ev_prep) cudaEventDestroy(ctx->ev_prep);
-    if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
-    if (ctx->side) cudaStreamDestroy(ctx->side);
+    for (int k = 0; k < 2; k++) {
+        if (ctx->ev_join[k]) cudaEventDestroy(ctx->ev_join[k]);
+        if (ctx->side[k]) cudaStreamDestroy(ctx->side[k]);
+    }
     if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
     delete ctx;
 }
@@ -1670,8 +1722,9 @@ int mrq_load_hamiltonian(mrq_ctx* ctx, int n_core, int n_act, int n_virt, int n_
     if (int r_ = sync_stream(ctx)) return r_;
     DeadlinePause pause_(ctx);
     free_walkers(ctx);
-    free_reference(ctx);
-    free_hamiltonian(ctx);
+    dfree(ctx->d_work);               // the walk workspace of the last system is given back
+    ctx->work_cap = 0;
+    ctx->ref = ctx->ham = false;
     ctx->n = n;
     ctx->nc = n_core;
     ctx->na = n_act;
@@ -1685,16 +1738,16 @@ int mrq_load_hamiltonian(mrq_ctx* ctx, int n_core, int n_act, int n_virt, int n_
     ctx->nHs = 1 + 2LL * n_core + (2LL * n_core) * (2LL * n_core - 1) / 2;
     ctx->nPs = 1 + 2LL * n_virt + (2LL * n_virt) * (2LL * n_virt - 1) / 2;
     ctx->nlab = ctx->nHs * ctx->nPs;
-    CK(cudaMalloc(&ctx->d_h1, sizeof(double) * n * n));
-    CK(cudaMalloc(&ctx->d_eri, sizeof(double) * ctx->neri));
-    CK(cudaMalloc(&ctx->d_eri4, sizeof(double) * npair * n * n));
+    CK(reserve(ctx->d_h1, ctx->cap_h1, (size_t)n * n));
+    CK(reserve(ctx->d_eri, ctx->cap_eri, (size_t)ctx->neri));
+    CK(reserve(ctx->d_eri4, ctx->cap_eri4, (size_t)npair * n * n));
     const long long nca = n_core + n_act, nav = n_act + n_virt;
-    CK(cudaMalloc(&ctx->d_tab, sizeof(double) * 2 * std::max(1LL, nca * nca * nav * nav)));
-    CK(cudaMalloc(&ctx->d_sgl, sizeof(double) * 2 * std::max(1LL, n_act * nca * nav)));
-    CK(cudaMalloc(&ctx->d_hc, sizeof(double) * n * n));
-    CK(cudaMalloc(&ctx->d_eps, sizeof(double) * n));
-    CK(cudaMalloc(&ctx->d_gamma, sizeof(double) * std::max(1, n_act * n_act)));
-    {
+    CK(reserve(ctx->d_tab, ctx->cap_tab, 2 * (size_t)std::max(1LL, nca * nca * nav * nav)));
+    CK(reserve(ctx->d_sgl, ctx->cap_sgl, 2 * (size_t)std::max(1LL, n_act * nca * nav)));
+    CK(reserve(ctx->d_hc, ctx->cap_hc, (size_t)n * n));
+    CK(reserve(ctx->d_eps, ctx->cap_eps, (size_t)n));
+    CK(reserve(ctx->d_gamma, ctx->cap_gamma, (size_t)std::max(1, n_act * n_act)));
+    if (!ctx->d_colex) {
         // co-lexicographic pair table of up to 128 items: colex[j(j-1)/2 + i] = i | j << 8, i < j
         std::vector<unsigned short> colex(128 * 127 / 2);
         for (int j = 1, q = 0; j < 128; j++)
@@ -1766,26 +1819,30 @@ int mrq_load_reference(mrq_ctx* ctx, int64_t n_det, const uint64_t* dets, const 
     if (int r_ = sync_stream(ctx)) return r_;
     DeadlinePause pause_(ctx);
     free_walkers(ctx);
-    free_reference(ctx);
+    ctx->ref = false;
     const int W = ctx->W;
     unsigned long long cap = 16;
     while (cap < 4ull * (unsigned long long)n_det) cap <<= 1;
     ctx->hcap = cap;
     ctx->nref = n_det;
-    unsigned long long* d_dets = nullptr;
-    double* d_co = nullptr;
-    CK(cudaMalloc(&ctx->d_hash, sizeof(HashSlot) * cap));
-    CK(cudaMalloc(&d_dets, sizeof(unsigned long long) * 2 * W * n_det));
-    CK(cudaMalloc(&d_co, sizeof(double) * n_det));
-    CK(cudaMalloc(&ctx->d_c, sizeof(double) * ctx->nlab));
+    const int nrdm = ctx->na * ctx->na * MRQ_RDM_SLICES;
+    auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+    const size_t b_dets = up(sizeof(unsigned long long) * 2 * W * n_det), b_co = up(sizeof(double) * n_det),
+                 b_part = up(sizeof(double) * 2 * MRQ_REF_BLOCKS), b_e = b_co, b_rdm = up(sizeof(double) * std::max(1, nrdm)), b_scal = 256;
+    CK(reserve(ctx->d_hash, ctx->cap_hash, (size_t)cap));
+    CK(reserve(ctx->d_c, ctx->cap_c, (size_t)ctx->nlab));
+    CK(reserve(ctx->d_setup, ctx->cap_setup, b_dets + b_co + b_part + b_rdm + 2 * b_scal + b_e));
+    unsigned long long* const d_dets = (unsigned long long*)ctx->d_setup;
+    double* const d_co = (double*)(ctx->d_setup + b_dets);
+    double* const d_part = (double*)(ctx->d_setup + b_dets + b_co);
+    double* const d_rdm = (double*)(ctx->d_setup + b_dets + b_co + b_part);
+    double* const d_scal = (double*)(ctx->d_setup + b_dets + b_co + b_part + b_rdm);
+    long long* const d_idx = (long long*)(ctx->d_setup + b_dets + b_co + b_part + b_rdm + b_scal);
+    double* const d_e = (double*)(ctx->d_setup + b_dets + b_co + b_part + b_rdm + 2 * b_scal);
     CK(cudaMemcpyAsync(d_dets, dets, sizeof(unsigned long long) * 2 * W * n_det, cudaMemcpyDefault, ctx->stream));
     CK(cudaMemcpyAsync(d_co, coeffs, sizeof(double) * n_det, cudaMemcpyDefault, ctx->stream));
-    {
-        std::vector<double> c(ctx->nlab, 0.1);
-        c[0] = 1.0;
-        CK(cudaMemcpyAsync(ctx->d_c, c.data(), sizeof(double) * ctx->nlab, cudaMemcpyHostToDevice, ctx->stream));
-        if (int r_ = sync_stream(ctx)) return r_;
-    }
+    k_default_coeffs<<<(unsigned)std::min<long long>(1024, (ctx->nlab + 255) / 256), 256, 0, ctx->stream>>>(ctx->d_c, ctx->nlab);
+    CK(cudaGetLastError());
     CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream));
     if (int r = push_sys(ctx)) return r;
     k_hash_clear<<<(unsigned)((cap + 255) / 256), 256, 0, ctx->stream>>>(ctx->d_hash, cap);
@@ -1796,47 +1853,33 @@ int mrq_load_reference(mrq_ctx* ctx, int64_t n_det, const uint64_t* dets, const 
     int flag = 0;
     if (int r = check_err_flag(ctx, &flag)) return r;
     if (flag) {
-        cudaFree(d_dets);
-        cudaFree(d_co);
         free_reference(ctx);
         if (flag & 32) return fail(ctx, MRQ_HASH_OVERFLOW, "hash insertion ran past the probe bound");
         return fail(ctx, MRQ_BAD_REFERENCE, "reference determinant with a core hole, a virtual electron, "
                                             "a wrong electron count or a duplicate (flags %d)", flag);
     }
-    // start determinant: largest |c| (first on ties)
-    long long* d_idx = nullptr;
-    CK(cudaMalloc(&d_idx, sizeof(long long)));
+    // start determinant (largest |c|, first on ties), E0, norm, gamma, eps
     k_argmax_abs<<<1, 1024, 0, ctx->stream>>>(d_co, n_det, d_idx);
-    CK(cudaMemcpyAsync(&ctx->start_idx, d_idx, sizeof(long long), cudaMemcpyDeviceToHost, ctx->stream));
-    if (int r_ = sync_stream(ctx)) return r_;
-    cudaFree(d_idx);
-    memset(ctx->start, 0, sizeof ctx->start);
-    {
-        unsigned long long tmp[4] = {0, 0, 0, 0};
-        CK(cudaMemcpy(tmp, d_dets + ctx->start_idx * 2 * W, sizeof(unsigned long long) * 2 * W, cudaMemcpyDeviceToHost));
-        for (int w = 0; w < W; w++) {
-            ctx->start[w] = tmp[w];
-            ctx->start[2 + w] = tmp[W + w];
-        }
-        CK(cudaMemcpy(&ctx->start_c, d_co + ctx->start_idx, sizeof(double), cudaMemcpyDeviceToHost));
+    const unsigned nd = (unsigned)((n_det + 127) / 128), nw8 = (unsigned)std::min<long long>((n_det + 7) / 8, 8LL * ctx->n_sm);
+    if (W == 1) {
+        k_ref_diag<1><<<nd, 128, 0, ctx->stream>>>(ctx->d_sys, d_dets, n_det, d_e);
+        k_ref_energy<1><<<nw8, 256, 0, ctx->stream>>>(ctx->d_sys, d_dets, d_co, n_det, d_e);
+    } else {
+        k_ref_diag<2><<<nd, 128, 0, ctx->stream>>>(ctx->d_sys, d_dets, n_det, d_e);
+        k_ref_energy<2><<<nw8, 256, 0, ctx->stream>>>(ctx->d_sys, d_dets, d_co, n_det, d_e);
     }
-    // E0, norm, gamma, eps
-    const int nblk = 304;
-    double* d_part = nullptr;
-    double* d_scal = nullptr;
-    CK(cudaMalloc(&d_part, sizeof(double) * 2 * nblk));
-    CK(cudaMalloc(&d_scal, sizeof(double) * 8));
-    if (W == 1) k_ref_energy<1><<<nblk, 128, 0, ctx->stream>>>(ctx->d_sys, d_dets, d_co, n_det, d_part);
-    else k_ref_energy<2><<<nblk, 128, 0, ctx->stream>>>(ctx->d_sys, d_dets, d_co, n_det, d_part);
+    k_ref_sum<<<MRQ_REF_BLOCKS, 128, 0, ctx->stream>>>(d_e, d_co, n_det, d_part);
     CK(cudaGetLastError());
     if (ctx->na > 0) {
-        if (W == 1) k_ref_rdm<1><<<ctx->na * ctx->na, 256, 0, ctx->stream>>>(ctx->d_sys, d_dets, d_co, n_det, ctx->d_gamma);
-        else k_ref_rdm<2><<<ctx->na * ctx->na, 256, 0, ctx->stream>>>(ctx->d_sys, d_dets, d_co, n_det, ctx->d_gamma);
+        const dim3 grid(ctx->na * ctx->na, MRQ_RDM_SLICES);
+        if (W == 1) k_ref_rdm<1><<<grid, 256, 0, ctx->stream>>>(ctx->d_sys, d_dets, d_co, n_det, d_rdm);
+        else k_ref_rdm<2><<<grid, 256, 0, ctx->stream>>>(ctx->d_sys, d_dets, d_co, n_det, d_rdm);
         CK(cudaGetLastError());
     }
-    k_setup_finish<<<1, 256, 0, ctx->stream>>>(ctx->d_sys, d_part, nblk, ctx->d_gamma, ctx->d_eps, d_scal);
+    k_setup_finish<<<1, 1024, 0, ctx->stream>>>(ctx->d_sys, d_part, d_rdm, ctx->d_gamma, ctx->d_eps, d_scal);
     CK(cudaGetLastError());
     double scal[8];
+    CK(cudaMemcpyAsync(&ctx->start_idx, d_idx, sizeof(long long), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaMemcpyAsync(scal, d_scal, sizeof(double) * 4, cudaMemcpyDeviceToHost, ctx->stream));
     ctx->eps.assign(ctx->n, 0.0);
     ctx->gamma.assign((size_t)ctx->na * ctx->na, 0.0);
@@ -1845,10 +1888,18 @@ int mrq_load_reference(mrq_ctx* ctx, int64_t n_det, const uint64_t* dets, const 
         CK(cudaMemcpyAsync(ctx->gamma.data(), ctx->d_gamma, sizeof(double) * ctx->na * ctx->na, cudaMemcpyDeviceToHost,
                            ctx->stream));
     if (int r_ = sync_stream(ctx)) return r_;
-    cudaFree(d_part);
-    cudaFree(d_scal);
-    cudaFree(d_dets);
-    cudaFree(d_co);
+    memset(ctx->start, 0, sizeof ctx->start);
+    {
+        unsigned long long tmp[4] = {0, 0, 0, 0};
+        CK(cudaMemcpyAsync(tmp, d_dets + ctx->start_idx * 2 * W, sizeof(unsigned long long) * 2 * W, cudaMemcpyDeviceToHost,
+                           ctx->stream));
+        CK(cudaMemcpyAsync(&ctx->start_c, d_co + ctx->start_idx, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+        if (int r_ = sync_stream(ctx)) return r_;
+        for (int w = 0; w < W; w++) {
+            ctx->start[w] = tmp[w];
+            ctx->start[2 + w] = tmp[W + w];
+        }
+    }
     ctx->e0 = scal[0];
     ctx->norm0 = scal[1];
     ctx->e_core = scal[2];
@@ -2057,7 +2108,7 @@ static long long fin_scratch_doubles(const mrq_ctx* ctx, int* nchunk) {
 // (the device copy of the system is current since mrq_walkers_init pushed it, so nothing is copied
 // in: a copy from pageable host memory would wait for the walk and defeat the deadline)
 static int finalize_with(mrq_ctx* ctx, mrq_result* out, double* scratch, int nchunk) {
-    k_fin_list<<<nchunk, 256, 0, ctx->stream>>>(ctx->d_sys, FIN_CHUNK, ctx->d_flist);
+    k_fin_list<<<nchunk, 1024, 0, ctx->stream>>>(ctx->d_sys, FIN_CHUNK, ctx->d_flist);
     k_fin_labels<<<(ctx->G + 1) * nchunk, 256, 0, ctx->stream>>>(ctx->d_sys, ctx->tau, nchunk, FIN_CHUNK, ctx->d_flist, scratch);
     CK(cudaGetLastError());
     k_fin_reduce<<<1, 1024, 0, ctx->stream>>>(ctx->d_sys, scratch, nchunk, ctx->d_res);
@@ -2245,6 +2296,8 @@ static int batch_run(mrq_ctx* ctx, int W, const WalkSet& ws, const WalkNeed& nee
         key.ns = need.ns;
         key.nref = need.nref;
         key.fg = need.fg_max;
+        key.wave = ctx->work.wave_groups;
+        key.fwave = ctx->work.fwave;
         cudaGraphExec_t& ex = ctx->gexec[slot];
         if (!ex || !(ctx->gkey[slot] == key)) {
             if (ex) CK(cudaGraphExecDestroy(ex));

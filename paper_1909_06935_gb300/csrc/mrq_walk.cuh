@@ -1067,6 +1067,7 @@ struct StepSink {
     RaceBest* best;
     unsigned* bound;
     int count, lane;
+    bool primary;             // this task group stores the determinant's sums
     double sA, sT, sD;        // sum |t|, sum t, sum t_D   (t = H_nm psi_s(m), t_D = (H_D)_nm psi_s(m))
     template <int W>
     __device__ __forceinline__ void post(bool valid, int, const unsigned long long (&)[2][W], double hnm, double hd,
@@ -1100,10 +1101,12 @@ struct StepSink {
         __syncwarp();
     }
     __device__ __forceinline__ void take(double t0, unsigned e0, double t1, unsigned e1) {
-        sA += fabs(t0);
-        sT += t0;
-        sA += fabs(t1);
-        sT += t1;
+        if (primary) {
+            sA += fabs(t0);
+            sT += t0;
+            sA += fabs(t1);
+            sT += t1;
+        }
         for (unsigned hits = race_round(wt, t0, e0, t1, e1, count); hits; hits &= hits - 1) {
             const int j = __ffs(hits) - 1;
             race_slow(wt, best, bound, j, t0, e0, lane);
@@ -1390,7 +1393,7 @@ __global__ void __launch_bounds__(256, 3) k_int(const WalkSet ws, const WalkScra
             const unsigned long long(&n)[2][W] = *reinterpret_cast<const unsigned long long(*)[2][W]>(wt.nsh);
             if (lane == 0) wt.cw = cas_constants<W>(S, n, sc.meta[tg.group].psi);
             __syncwarp();
-            StepSink sink{wt, sc.best, sc.bound, tg.count, lane, 0.0, 0.0, 0.0};
+            StepSink sink{wt, sc.best, sc.bound, tg.count, lane, tg.primary != 0, 0.0, 0.0, 0.0};
             for (int u = slice; u < S.cas_units; u += MRQ_INT_SLICES) cas_internal_unit<W>(S, wt.cw, n, u, lane, sink, ctr);
             sink.finish();
             sA = sink.sA;
@@ -1419,7 +1422,7 @@ __global__ void __launch_bounds__(256, 3) k_fois_act(const WalkSet ws, const Wal
         const int slice = id / ntg;
         const TaskGroup tg = sc.tgf[id - slice * ntg];
         task_system(wt, ws, tg.sys, cur, lane);
-        StepSink sink{wt, sc.best, sc.bound, tg.count, lane, 0.0, 0.0, 0.0};
+        StepSink sink{wt, sc.best, sc.bound, tg.count, lane, tg.primary != 0, 0.0, 0.0, 0.0};
         if (task_begin<W>(wt, ws, sc, tg, lane)) {
             const unsigned long long(&n)[2][W] = *reinterpret_cast<const unsigned long long(*)[2][W]>(wt.nsh);
             const double* const gops = sc.gops + (long long)tg.group * sc.gstride;
@@ -1785,7 +1788,7 @@ __global__ void __launch_bounds__(256, MINB) k_fois(const WalkSet ws, const Walk
         const int g = (int)(sc.nseg - 1 - tg.group) - sc.fwave0;
         if (g < 0 || g >= sc.fwave) continue;
         task_system(wt, ws, tg.sys, cur, lane);
-        StepSink sink{wt, sc.best, sc.bound, tg.count, lane, 0.0, 0.0, 0.0};
+        StepSink sink{wt, sc.best, sc.bound, tg.count, lane, tg.primary != 0, 0.0, 0.0, 0.0};
         if (task_begin<W>(wt, ws, sc, tg, lane)) {
             const unsigned long long(&n)[2][W] = *reinterpret_cast<const unsigned long long(*)[2][W]>(wt.nsh);
             if (lane == 0) fois_outer<W>(S, n, o);
@@ -2046,7 +2049,7 @@ __global__ void __launch_bounds__(256, MINB) k_pairs(const WalkSet ws, const Wal
         if (tg.group < sc.wave0 || tg.group >= sc.wave0 + sc.wave_groups) continue;
         task_system(wt, ws, tg.sys, cur, lane);
         if (slice >= S.nslice) continue;
-        StepSink sink{wt, sc.best, sc.bound, tg.count, lane, 0.0, 0.0, 0.0};
+        StepSink sink{wt, sc.best, sc.bound, tg.count, lane, tg.primary != 0, 0.0, 0.0, 0.0};
         if (task_begin<W>(wt, ws, sc, tg, lane)) {
             const unsigned long long(&n)[2][W] = *reinterpret_cast<const unsigned long long(*)[2][W]>(wt.nsh);
             const unsigned ao0 = active_bits<W>(S, n[0]), ao1 = active_bits<W>(S, n[1]);
