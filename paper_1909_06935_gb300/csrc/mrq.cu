@@ -1030,6 +1030,8 @@ struct mrq_ctx {
     long long row_worst = 0;         // doubles of one CAS determinant's rows when none is shared
     int fg_max = 1;                  // groups of a first-order determinant's neighbours (at most)
     WalkScratch work{};
+    size_t ktab_bytes = 0;           // the table of known rows that was cleared last, and its counters
+    int* kctl_at = nullptr;
     double* d_partial = nullptr;
     long long partial_cap = 0;
     mrq_result* d_res = nullptr;
@@ -1263,7 +1265,7 @@ static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, lo
                           8LL * need.gstride + 24LL * (need.ns + MRQ_ACT_SLICES) + (long long)sizeof(RaceBest) + 4;
     const long long seg = std::min(nslots, std::max(256LL, std::min(1LL << 20, MRQ_WORK_BYTES / per)));
     *seg_out = seg;
-    const long long per_group = 8 * need.row_worst + 33LL * need.nref;
+    const long long per_group = 8 * need.row_worst + 93LL * need.nref;
     long long groups = std::max(1LL, std::min(seg, MRQ_ROW_BYTES / per_group));
     groups = std::min(groups, std::max(1LL, (1LL << 29) / need.nref));           // reference indices and the table: 32 bits
     const long long per_fois = 8 * need.fois_nb + (long long)sizeof(FGroup) * need.fg_max + 8;
@@ -1272,7 +1274,7 @@ static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, lo
     WalkScratch& w = ctx->work;
     for (;; groups = (groups + 1) / 2, fwave = (fwave + 1) / 2) {
         long long tsz = 2;
-        while (tsz < 2 * groups * need.nref) tsz <<= 1;
+        while (tsz < 2 * groups * need.nref) tsz <<= 1;      // (as many known rows as references of a wave)
         size_t off = 0;
         auto take = [&](size_t bytes) {
             const size_t at = off;
@@ -1286,12 +1288,14 @@ static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, lo
                      gops = take(8 * (size_t)need.gstride * seg), part = take(24 * (size_t)(need.ns + MRQ_ACT_SLICES) * seg),
                      best = take(sizeof(RaceBest) * seg), bound = take(4 * seg), ctl = take(4 * CTL_N), ao = take(8 * nr),
                      cls = take(nr), rrep = take(4 * nr), roff = take(8 * nr), tbl = take(4 * tsz), ul = take(4 * nr),
+                     kt = take(8 * tsz), kao = take(8 * nr), kkey = take(4 * nr), koff = take(8 * nr), kctl = take(4 * KNOWN_N),
                      fgo = take(8 * fwave), fg = take(sizeof(FGroup) * (size_t)need.fg_max * fwave),
                      rows = take(8 * (size_t)need.row_worst * groups), frows = take(8 * (size_t)need.fois_nb * fwave);
         if (off > ctx->work_cap) {
             CK(cudaStreamSynchronize(ctx->stream));
             dfree(ctx->d_work);
             ctx->work_cap = 0;
+            ctx->ktab_bytes = 0;
             const cudaError_t e = cudaMalloc(&ctx->d_work, off);
             if (e == cudaErrorMemoryAllocation && (groups > 1 || fwave > 1)) {
                 cudaGetLastError();
@@ -1325,11 +1329,25 @@ static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, lo
         w.rows = (double*)(b + rows);
         w.frows = (double*)(b + frows);
         w.table_size = (int)tsz;
+        w.ktab_size = (int)tsz;
+        w.k_ao = (unsigned long long*)(b + kao);
+        w.k_key = (int*)(b + kkey);
+        w.k_off = (long long*)(b + koff);
+        w.kctl = (int*)(b + kctl);
+        // a new layout of the workspace: nothing in it is a table of known rows yet
+        if (w.ktab != (unsigned long long*)(b + kt) || ctx->ktab_bytes != 8 * (size_t)tsz || ctx->kctl_at != w.kctl) {
+            w.ktab = (unsigned long long*)(b + kt);
+            ctx->ktab_bytes = 8 * (size_t)tsz;
+            ctx->kctl_at = w.kctl;
+            CK(cudaMemsetAsync(w.ktab, 0, ctx->ktab_bytes, ctx->stream));
+            CK(cudaMemsetAsync(w.kctl, 0, sizeof(int) * KNOWN_N, ctx->stream));
+        }
         w.fg_of = (int2*)(b + fgo);
         w.fg = (FGroup*)(b + fg);
         break;
     }
     w.nref_max = need.nref;
+    w.row_worst = need.row_worst;
     w.wave_groups = (int)groups;
     w.wave0 = 0;
     w.fg_max = need.fg_max;
@@ -1403,7 +1421,7 @@ static int launch_segment(mrq_ctx* ctx, const WalkSet& ws, WalkScratch sc, const
     CK(cudaStreamWaitEvent(st3, ctx->ev_fork, 0));
     for (long long g = 0; g < n; g += sc.fwave) {
         sc.fwave0 = (int)g;
-        if (g > 0) CK(cudaMemsetAsync(sc.ctl + CTL_FOIS, 0, sizeof(int) * (CTL_CUR - CTL_FOIS), st3));
+        if (g > 0) CK(cudaMemsetAsync(sc.ctl + CTL_FOIS, 0, sizeof(int) * (CTL_N - CTL_FOIS), st3));
         k_fgroups<W><<<(unsigned)std::min<long long>(n, 4LL * sms), 256, 0, st3>>>(ws, sc);
         k_frows<W, 3><<<(unsigned)ctx->frows_blocks, 32 * nw, nw * fbytes, st3>>>(ws, sc, (int)fbytes, need.cap);
         if (g == 0) CK(cudaStreamWaitEvent(st3, ctx->ev_prep, 0));
@@ -1413,6 +1431,7 @@ static int launch_segment(mrq_ctx* ctx, const WalkSet& ws, WalkScratch sc, const
     // main stream: the CAS determinants' rows and pairs
     for (long long g = 0; g < n; g += sc.wave_groups) {
         sc.wave0 = (int)g;
+        k_wave_begin<<<1, 1, 0, st>>>(sc);
         k_refs<W><<<(unsigned)std::min<long long>(n, 8LL * sms), 256, 0, st>>>(ws, sc);
         k_insert<<<8 * sms, 256, 0, st>>>(ws, sc);
         cfg.gridDim = dim3((unsigned)ctx->rows_blocks);
@@ -1451,6 +1470,8 @@ static int launch_walk(mrq_ctx* ctx, int W, const WalkSet& ws, int nsteps, const
         cfg.attrs = attr;
         cfg.numAttrs = 1;
     }
+    k_rows_begin<<<1, 1, 0, ctx->stream>>>(ctx->work);
+    CK(cudaGetLastError());
     for (int step = 0; step < nsteps; step++) {
         for (long long s0 = 0; s0 < ws.nslots; s0 += seg) {
             WalkScratch sc = ctx->work;
@@ -1724,6 +1745,7 @@ int mrq_load_hamiltonian(mrq_ctx* ctx, int n_core, int n_act, int n_virt, int n_
     free_walkers(ctx);
     dfree(ctx->d_work);               // the walk workspace of the last system is given back
     ctx->work_cap = 0;
+    ctx->ktab_bytes = 0;
     ctx->ref = ctx->ham = false;
     ctx->n = n;
     ctx->nc = n_core;

@@ -86,9 +86,9 @@ enum {
     CTL_BIG, CTL_SMALL,           // distinct rows of a wave: long ones (from the list's front), short ones
     CTL_FOIS, CTL_FG, CTL_FGTASK, // first-order waves: next task of k_fois, most groups of a determinant, next task
     CTL_FCUR = 14,                // (64 bits) doubles of the first-order row buffer in use
-    CTL_CUR = 16,                 // (64 bits) doubles of the row buffer in use
-    CTL_N = CTL_CUR + 2
+    CTL_N = CTL_FCUR + 2
 };
+enum { KNOWN_ROWS, KNOWN_EPOCH, KNOWN_CUR, KNOWN_N = KNOWN_CUR + 2 };   // rows, epoch, (64 bits) doubles of the buffer in use
 #define MRQ_INT_SLICES 8          // warp tasks of a CAS determinant's neighbours inside the CAS
 #define MRQ_ACT_SLICES 32         // warp tasks of a first-order determinant's active-only neighbours
 #define MRQ_FOIS_SLICES 256       // warp tasks of its other neighbours
@@ -106,6 +106,7 @@ struct FGroup {
     unsigned char ac, sac, bv, sbv, av, bc, xs, ys;
 };
 #define MRQ_NOROW 255             // a reference without entries
+#define MRQ_KNOWN 64              // flag of a reference whose row is known from an earlier step of the launch
 
 // device workspace of a walk launch, sized for the slots [seg0, seg1) of the walk set
 struct WalkScratch {
@@ -124,10 +125,19 @@ struct WalkScratch {
     unsigned long long* ref_ao;   // the row's active remnant
     unsigned char* ref_cls;       // 3 (core holes) + (virtual electrons), MRQ_NOROW
     int* ref_rep;                 // the reference that owns the row
-    long long* row_off;           // (owners) the row's place in rows
+    long long* row_off;           // (owners and rows known from earlier) the row's place in rows
     int *table, *ulist;           // open addressing over references; the owners
     double* rows;
     int table_size, nref_max, wave_groups, wave0;
+    // rows known in this launch: open addressing over row numbers (entry: epoch << 32 | row; another epoch's
+    // entry is an empty one), the rows' remnants, systems and classes, and places
+    unsigned long long* ktab;
+    unsigned long long* k_ao;
+    int* k_key;
+    long long* k_off;
+    int* kctl;                    // KNOWN_*
+    int ktab_size;
+    long long row_worst;
     // groups of a wave of at most fwave first-order determinants (fg_max each) and psi_s of their neighbours
     FGroup* fg;
     double* frows;
@@ -399,13 +409,13 @@ __device__ __forceinline__ int active_neighbour(const SysDev& S, unsigned long l
         Yb = subset_bits(S.colex, al ? ea : eb, ne, 2, x % ny);
         return 2;
     }
-    int x = idx - b3;
-    const int yb = x % ceb;
-    x /= ceb;
-    const int xb = x % cob;
-    x /= cob;
-    Xb = subset_bits(S.colex, oa, coa, 1, x / cea) | subset_bits(S.colex, ob, cob, 1, xb);
-    Yb = subset_bits(S.colex, ea, cea, 1, x % cea) | subset_bits(S.colex, eb, ceb, 1, yb);
+    int x = idx - b3;                          // the beta excitation slowest
+    const int ya = x % cea;
+    x /= cea;
+    const int xa = x % coa;
+    x /= coa;
+    Xb = subset_bits(S.colex, oa, coa, 1, xa) | subset_bits(S.colex, ob, cob, 1, x / ceb);
+    Yb = subset_bits(S.colex, ea, cea, 1, ya) | subset_bits(S.colex, eb, ceb, 1, x % ceb);
     return 2;
 }
 
@@ -1863,15 +1873,37 @@ __device__ __forceinline__ int row_len(const SysDev& S, int c, int v, int d) {
     return len;
 }
 
-// the row references of every determinant of the wave: remnant and class
+// Rows stay known through a launch's steps (they depend on the loaded system and its coefficients only;
+// every launch begins with none): most determinants of a step were there the step before.  A wave that
+// may not fit behind the known rows forgets them first.
+__global__ void k_rows_begin(const WalkScratch sc) {
+    sc.kctl[KNOWN_ROWS] = 0;
+    sc.kctl[KNOWN_EPOCH]++;
+    *reinterpret_cast<unsigned long long*>(sc.kctl + KNOWN_CUR) = 0ull;
+}
+__global__ void k_wave_begin(const WalkScratch sc) {
+    const long long ng = min(sc.wave_groups, sc.ctl[CTL_GC] - sc.wave0);
+    if (ng <= 0) return;
+    sc.ctl[CTL_PAIRS] = sc.ctl[CTL_ROWTASK] = sc.ctl[CTL_BIG] = sc.ctl[CTL_SMALL] = 0;
+    unsigned long long* const cur = reinterpret_cast<unsigned long long*>(sc.kctl + KNOWN_CUR);
+    if ((long long)*cur + ng * sc.row_worst > sc.wave_groups * sc.row_worst ||
+        sc.kctl[KNOWN_ROWS] + ng * sc.nref_max > (long long)sc.wave_groups * sc.nref_max) {
+        sc.kctl[KNOWN_ROWS] = 0;
+        sc.kctl[KNOWN_EPOCH]++;
+        *cur = 0ull;
+    }
+}
+
+__device__ __forceinline__ unsigned long long row_hash(unsigned long long ao, int key) {
+    return mix64(ao + 0x9E3779B97F4A7C15ull * (unsigned)(key + 1));
+}
+
+// the row references of every determinant of the wave: remnant and class, and the row where it is known
 template <int W>
 __global__ void __launch_bounds__(256) k_refs(const WalkSet ws, const WalkScratch sc) {
     const int ng = min(sc.wave_groups, sc.ctl[CTL_GC] - sc.wave0);
     if (ng <= 0) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        sc.ctl[CTL_PAIRS] = sc.ctl[CTL_ROWTASK] = sc.ctl[CTL_BIG] = sc.ctl[CTL_SMALL] = 0;
-        *reinterpret_cast<unsigned long long*>(sc.ctl + CTL_CUR) = 0ull;
-    }
+    const unsigned epoch = (unsigned)sc.kctl[KNOWN_EPOCH], known = (unsigned)sc.kctl[KNOWN_ROWS];
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < sc.table_size; k += gridDim.x * blockDim.x) sc.table[k] = -1;
     for (int g = blockIdx.x; g < ng; g += gridDim.x) {
         const GroupMeta& meta = sc.meta[sc.wave0 + g];
@@ -1900,17 +1932,35 @@ __global__ void __launch_bounds__(256) k_refs(const WalkSet ws, const WalkScratc
                 const unsigned long long Yb = subset_bits(S.colex, AE, cntE, kb, ya);
                 const int d = __popcll(Yb & 0xFFFFFFFFull) - __popcll(Xb & 0xFFFFFFFFull);
                 const int c = r - ka, v = r - kb;
-                sc.ref_ao[at + q] = (AO & ~Xb) | Yb;
-                if (row_len(S, c, v, d) > 0) cls = (unsigned char)(3 * c + v);
+                const unsigned long long ao = (AO & ~Xb) | Yb;
+                sc.ref_ao[at + q] = ao;
+                if (row_len(S, c, v, d) > 0) {
+                    cls = (unsigned char)(3 * c + v);
+                    const int key = 9 * meta.sys + cls;
+                    int h = (int)(row_hash(ao, key) & (unsigned)(sc.ktab_size - 1));
+                    for (int probe = 0; probe < sc.ktab_size; probe++) {
+                        const unsigned long long e = sc.ktab[h];
+                        if ((unsigned)(e >> 32) != epoch) break;
+                        const unsigned id = (unsigned)e;
+                        if (id < known && sc.k_ao[id] == ao && sc.k_key[id] == key) {
+                            cls |= MRQ_KNOWN;
+                            sc.ref_rep[at + q] = (int)(at + q);
+                            sc.row_off[at + q] = sc.k_off[id];
+                            break;
+                        }
+                        h = (h + 1) & (sc.ktab_size - 1);
+                    }
+                }
             }
             sc.ref_cls[at + q] = cls;
         }
     }
 }
 
-// Distinct rows: every reference finds or becomes the owner of its (system, class, remnant) in an
-// open-addressing table with at least twice as many entries as references; owners get a place in the
-// row buffer (which holds the worst case of a wave, every row distinct).
+// Distinct new rows: every reference whose row is not known finds or becomes the owner of its (system,
+// class, remnant) in an open-addressing table with at least twice as many entries as references; owners
+// get a place in the row buffer (which holds the worst case of a wave, every row distinct) and enter the
+// table of known rows, which k_refs reads in later waves and steps.
 __global__ void __launch_bounds__(256) k_insert(const WalkSet ws, const WalkScratch sc) {
     const int ng = min(sc.wave_groups, sc.ctl[CTL_GC] - sc.wave0);
     if (ng <= 0) return;
@@ -1919,10 +1969,13 @@ __global__ void __launch_bounds__(256) k_insert(const WalkSet ws, const WalkScra
         const int i = base + lane;
         bool owner = false;
         int len = 0;
-        if (i < total && sc.ref_cls[i] != MRQ_NOROW) {
+        int key = 0;
+        unsigned long long ao = 0;
+        if (i < total && !(sc.ref_cls[i] & MRQ_KNOWN)) {              // (MRQ_NOROW has that bit too)
             const int cls = sc.ref_cls[i], sys = sc.meta[sc.wave0 + i / sc.nref_max].sys;
-            const unsigned long long ao = sc.ref_ao[i];
-            int k = (int)(mix64(ao + 0x9E3779B97F4A7C15ull * (unsigned)(9 * sys + cls + 1)) & (unsigned)(sc.table_size - 1));
+            key = 9 * sys + cls;
+            ao = sc.ref_ao[i];
+            int k = (int)(row_hash(ao, key) & (unsigned)(sc.table_size - 1));
             for (int probe = 0; probe < sc.table_size; probe++) {
                 const int prev = atomicCAS(sc.table + k, -1, i);
                 if (prev < 0) {
@@ -1953,16 +2006,33 @@ __global__ void __launch_bounds__(256) k_insert(const WalkSet ws, const WalkScra
         const unsigned big = __ballot_sync(0xffffffffu, owner && len >= MRQ_BIG_ROW);
         const unsigned small = __ballot_sync(0xffffffffu, owner && len < MRQ_BIG_ROW);
         unsigned long long cur = 0;
-        int nb = 0, ns = 0;
-        if (lane == 31 && x > 0) cur = atomicAdd(reinterpret_cast<unsigned long long*>(sc.ctl + CTL_CUR), (unsigned long long)x);
+        int nb = 0, ns = 0, nk = 0;
+        if (lane == 31 && x > 0) cur = atomicAdd(reinterpret_cast<unsigned long long*>(sc.kctl + KNOWN_CUR), (unsigned long long)x);
+        if (lane == 0 && (big | small)) nk = atomicAdd(sc.kctl + KNOWN_ROWS, __popc(big | small));
         if (lane == 0 && big) nb = atomicAdd(sc.ctl + CTL_BIG, __popc(big));
         if (lane == 0 && small) ns = atomicAdd(sc.ctl + CTL_SMALL, __popc(small));
         cur = __shfl_sync(0xffffffffu, cur, 31);
         nb = __shfl_sync(0xffffffffu, nb, 0);
         ns = __shfl_sync(0xffffffffu, ns, 0);
+        nk = __shfl_sync(0xffffffffu, nk, 0);
         if (owner) {
-            sc.row_off[i] = (long long)cur + x - len;
+            const long long off = (long long)cur + x - len;
+            sc.row_off[i] = off;
             const unsigned lt = (1u << lane) - 1u;
+            const int id = nk + __popc((big | small) & lt);
+            sc.k_ao[id] = ao;
+            sc.k_key[id] = key;
+            sc.k_off[id] = off;
+            const unsigned long long mine = ((unsigned long long)(unsigned)sc.kctl[KNOWN_EPOCH] << 32) | (unsigned)id;
+            int h = (int)(row_hash(ao, key) & (unsigned)(sc.ktab_size - 1));
+            for (int probe = 0; probe < sc.ktab_size;) {
+                const unsigned long long e = *reinterpret_cast<volatile unsigned long long*>(sc.ktab + h);
+                if ((e >> 32) != (mine >> 32) && atomicCAS(sc.ktab + h, e, mine) == e) break;
+                if ((e >> 32) == (mine >> 32)) {
+                    h = (h + 1) & (sc.ktab_size - 1);
+                    probe++;
+                }
+            }
             const int all = sc.wave_groups * sc.nref_max;
             if (len >= MRQ_BIG_ROW) sc.ulist[nb + __popc(big & lt)] = i;
             else sc.ulist[all - 1 - (ns + __popc(small & lt))] = i;
