@@ -48,7 +48,7 @@
 struct CasWalker {
     unsigned long long AOn, AEn, keyn;
     int cntO, cntE;
-    double phin, c0, inv_psin;
+    double phin, c0;
 };
 
 __host__ __device__ __forceinline__ size_t cand_list_bytes(int cap) {
@@ -74,6 +74,8 @@ struct TaskGroup {
 struct GroupMeta {
     unsigned long long d[2][2];
     double psi, hnn, hdnn;
+    double inv_psi, phi;      // 1/psi_s(n), psi_s(n)/c_0: divided once here (an FP64 division holds its SM's pipe for
+                              // hundreds of cycles, and there are some 10^5 warp tasks per step)
     long long label;
     int h, p, sys, pad;
 };
@@ -854,7 +856,7 @@ __device__ void walker_operator(const SysDev& S, const unsigned long long (&n)[2
 }
 
 template <int W>
-__device__ __forceinline__ CasWalker cas_constants(const SysDev& S, const unsigned long long (&n)[2][W], double psin) {
+__device__ __forceinline__ CasWalker cas_constants(const SysDev& S, const unsigned long long (&n)[2][W], double phin) {
     CasWalker cw;
     const unsigned ao0 = active_bits<W>(S, n[0]), ao1 = active_bits<W>(S, n[1]);
     const unsigned amask = (S.na >= 32) ? 0xFFFFFFFFu : ((1u << S.na) - 1u);
@@ -864,8 +866,7 @@ __device__ __forceinline__ CasWalker cas_constants(const SysDev& S, const unsign
     cw.cntO = __popcll(cw.AOn);
     cw.cntE = __popcll(cw.AEn);
     cw.c0 = __ldg(S.c);
-    cw.phin = psin / cw.c0;
-    cw.inv_psin = 1.0 / psin;
+    cw.phin = phin;
     return cw;
 }
 
@@ -1247,6 +1248,8 @@ __global__ void __launch_bounds__(1024) k_group(const WalkSet ws, const WalkScra
 #pragma unroll
             for (int w = 0; w < W; w++) m.d[sg][w] = d[sg][w];
         m.psi = wk[rep[k]].psi;
+        m.inv_psi = m.psi != 0.0 ? 1.0 / m.psi : 0.0;
+        m.phi = m.psi / __ldg(S.c);
         m.hnn = m.hdnn = 0.0;
         m.label = det_label<W>(S, d, m.h, m.p);
         m.sys = sys;
@@ -1338,10 +1341,9 @@ template <int W>
 __device__ __forceinline__ bool task_begin(WarpTask& wt, const WalkSet& ws, const WalkScratch& sc, const TaskGroup& tg,
                                            int lane) {
     const GroupMeta* const meta = sc.meta + tg.group;
-    const double psin = meta->psi;
-    if (meta->label < 0 || !(psin != 0.0)) return false;
+    if (meta->label < 0 || !(meta->psi != 0.0)) return false;
     if (lane < 2 * W) wt.nsh[lane] = meta->d[lane / W][lane % W];
-    const double inv = 1.0 / psin;
+    const double inv = meta->inv_psi;
     float inv_f = abs_f32_of(inv);
     if (!(inv_f > 0.0f)) inv_f = INFINITY;
     if (lane < tg.count) {
@@ -1367,13 +1369,15 @@ __device__ __forceinline__ bool task_begin(WarpTask& wt, const WalkSet& ws, cons
     return true;
 }
 
-// partial sums of a task, stored by the determinant's primary group
+// partial sums of a task, stored by the determinant's primary group (D: with the H_D numerator)
+template <bool D>
 __device__ __forceinline__ void task_sums(const WalkScratch& sc, const TaskGroup& tg, int slice, double sA, double sT,
                                           double sD, int lane) {
+    if (!tg.primary) return;
     sA = warp_sum(sA);
     sT = warp_sum(sT);
-    sD = warp_sum(sD);
-    if (lane == 0 && tg.primary) {
+    if (D) sD = warp_sum(sD);
+    if (lane == 0) {
         double* const p = sc.part + ((long long)tg.group * (sc.ns_max + MRQ_ACT_SLICES) + slice) * 3;
         p[0] = sA;
         p[1] = sT;
@@ -1401,7 +1405,7 @@ __global__ void __launch_bounds__(256, 3) k_int(const WalkSet ws, const WalkScra
         double sA = 0.0, sT = 0.0;
         if (task_begin<W>(wt, ws, sc, tg, lane)) {
             const unsigned long long(&n)[2][W] = *reinterpret_cast<const unsigned long long(*)[2][W]>(wt.nsh);
-            if (lane == 0) wt.cw = cas_constants<W>(S, n, sc.meta[tg.group].psi);
+            if (lane == 0) wt.cw = cas_constants<W>(S, n, sc.meta[tg.group].phi);
             __syncwarp();
             StepSink sink{wt, sc.best, sc.bound, tg.count, lane, tg.primary != 0, 0.0, 0.0, 0.0};
             for (int u = slice; u < S.cas_units; u += MRQ_INT_SLICES) cas_internal_unit<W>(S, wt.cw, n, u, lane, sink, ctr);
@@ -1409,7 +1413,7 @@ __global__ void __launch_bounds__(256, 3) k_int(const WalkSet ws, const WalkScra
             sA = sink.sA;
             sT = sink.sT;
         }
-        task_sums(sc, tg, sc.ns_max + slice, sA, sT, 0.0, lane);
+        task_sums<false>(sc, tg, sc.ns_max + slice, sA, sT, 0.0, lane);
     }
 }
 
@@ -1468,7 +1472,7 @@ __global__ void __launch_bounds__(256, 3) k_fois_act(const WalkSet ws, const Wal
             }
             sink.finish();
         }
-        task_sums(sc, tg, sc.ns_max + slice, sink.sA, sink.sT, sink.sD, lane);
+        task_sums<true>(sc, tg, sc.ns_max + slice, sink.sA, sink.sT, sink.sD, lane);
     }
 }
 
@@ -1855,7 +1859,7 @@ __global__ void __launch_bounds__(256, MINB) k_fois(const WalkSet ws, const Walk
             }
             sink.finish();
         }
-        task_sums(sc, tg, slice, sink.sA, sink.sT, 0.0, lane);
+        task_sums<false>(sc, tg, slice, sink.sA, sink.sT, 0.0, lane);
     }
 }
 
@@ -2128,7 +2132,7 @@ __global__ void __launch_bounds__(256, MINB) k_pairs(const WalkSet ws, const Wal
             const unsigned long long AE = (unsigned long long)(~ao0 & amask) | ((unsigned long long)(~ao1 & amask) << 32);
             const int cntO = __popcll(AO), cntE = __popcll(AE), nc = S.nc, nv = S.nv, voff = S.nc + S.na;
             const long long refs = (long long)(tg.group - sc.wave0) * sc.nref_max;
-            const double phin = sc.meta[tg.group].psi / __ldg(S.c);
+            const double phin = sc.meta[tg.group].phi;
             for (int u = S.cas_units + slice; u < S.unit_off[8]; u += S.nslice) {
                 int k = 0;
                 while (k < 7 && u >= S.unit_off[k + 1]) k++;
@@ -2278,7 +2282,7 @@ __global__ void __launch_bounds__(256, MINB) k_pairs(const WalkSet ws, const Wal
             }
             sink.finish();
         }
-        task_sums(sc, tg, slice, sink.sA, sink.sT, 0.0, lane);
+        task_sums<false>(sc, tg, slice, sink.sA, sink.sT, 0.0, lane);
     }
 }
 
@@ -2314,7 +2318,7 @@ __global__ void __launch_bounds__(MRQ_MAXNW * 32) k_move(const WalkSet ws, const
         const TaskGroup tg = g < ntc ? sc.tgc[g] : sc.tgf[g - ntc];
         const SysDev& S = ws.systems[tg.sys];
         const GroupMeta meta = sc.meta[tg.group];
-        const double inv_psin = meta.psi != 0.0 ? 1.0 / meta.psi : 0.0;
+        const double inv_psin = meta.inv_psi;
         double A = 0.0, T = 0.0, D = 0.0;
         const double* const part = sc.part + (long long)tg.group * (sc.ns_max + MRQ_ACT_SLICES) * 3;
         const int ns = g < ntc ? S.nslice : MRQ_FOIS_SLICES;
@@ -2536,7 +2540,7 @@ __global__ void __launch_bounds__(MRQ_MAXNW * 32, 2) k_debug2(const SysDev* __re
         if (lane == 0) {
             cs.hnn = hnn;
             cs.hdnn = hdnn;
-            if (cas) cs.cw = cas_constants<W>(S, n, psin);
+            if (cas) cs.cw = cas_constants<W>(S, n, psin / c0);
 #pragma unroll
             for (int sg = 0; sg < 2; sg++)
 #pragma unroll
