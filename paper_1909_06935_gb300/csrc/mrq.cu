@@ -1321,13 +1321,13 @@ static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, lo
             off += (bytes + 255) / 256 * 256;
             return at;
         };
-        const size_t nr = (size_t)groups * need.nref;
+        const size_t nr = (size_t)groups * need.nref, nul = nr + (size_t)(need.row_worst * groups / MRQ_BIG_ROW) + 1;
         const size_t rep = take(16 * seg), cnt = take(16 * seg), start = take(16 * seg), tab = take(4 * seg),
                      pos = take(4 * seg), mem = take(4 * seg), tgc = take(sizeof(TaskGroup) * seg),
                      tgf = take(sizeof(TaskGroup) * seg), meta = take(sizeof(GroupMeta) * seg),
                      gops = take(8 * (size_t)need.gstride * seg), part = take(24 * (size_t)(need.ns + MRQ_ACT_SLICES) * seg),
                      best = take(sizeof(RaceBest) * seg), bound = take(4 * seg), ctl = take(4 * CTL_N), ao = take(8 * nr),
-                     cls = take(nr), rrep = take(4 * nr), roff = take(8 * nr), tbl = take(4 * tsz), ul = take(4 * nr),
+                     cls = take(nr), rrep = take(4 * nr), roff = take(8 * nr), tbl = take(4 * tsz), ul = take(sizeof(int2) * nul),
                      kt = take(8 * tsz), kao = take(8 * nr), kkey = take(4 * nr), koff = take(8 * nr), kctl = take(4 * KNOWN_N),
                      fgo = take(8 * fwave), fg = take(sizeof(FGroup) * (size_t)need.fg_max * fwave),
                      rows = take(8 * (size_t)need.row_worst * groups), frows = take(8 * (size_t)need.fois_nb * fwave);
@@ -1365,7 +1365,8 @@ static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, lo
         w.ref_rep = (int*)(b + rrep);
         w.row_off = (long long*)(b + roff);
         w.table = (int*)(b + tbl);
-        w.ulist = (int*)(b + ul);
+        w.ulist = (int2*)(b + ul);
+        w.ulist_size = (int)nul;
         w.rows = (double*)(b + rows);
         w.frows = (double*)(b + frows);
         w.table_size = (int)tsz;

@@ -85,7 +85,7 @@ enum {
     CTL_TGC, CTL_GC,              // CAS task groups, CAS determinants
     CTL_TGF, CTL_GF,              // first-order task groups, determinants
     CTL_INT, CTL_PAIRS, CTL_ACT, CTL_ROWTASK,   // next warp task of each kernel
-    CTL_BIG, CTL_SMALL,           // distinct rows of a wave: long ones (from the list's front), short ones
+    CTL_BIG, CTL_SMALL,           // tasks of k_rows in a wave: pieces of long rows, short rows
     CTL_FOIS, CTL_FG, CTL_FGTASK, // first-order waves: next task of k_fois, most groups of a determinant, next task
     CTL_FCUR = 14,                // (64 bits) doubles of the first-order row buffer in use
     CTL_N = CTL_FCUR + 2
@@ -94,7 +94,7 @@ enum { KNOWN_ROWS, KNOWN_EPOCH, KNOWN_CUR, KNOWN_N = KNOWN_CUR + 2 };   // rows,
 #define MRQ_INT_SLICES 8          // warp tasks of a CAS determinant's neighbours inside the CAS
 #define MRQ_ACT_SLICES 32         // warp tasks of a first-order determinant's active-only neighbours
 #define MRQ_FOIS_SLICES 256       // warp tasks of its other neighbours
-#define MRQ_BIG_ROW 1024          // entries of a long row
+#define MRQ_BIG_ROW 1024          // entries of a task of k_rows; longer rows are cut (one warp took 1.3 ms on 65,000 entries)
 #define MRQ_FG_NB 1024            // neighbours of a group of a first-order determinant (longer ones are cut)
 
 // Neighbours of a first-order determinant that share an active remnant and an outer pattern: core
@@ -128,7 +128,9 @@ struct WalkScratch {
     unsigned char* ref_cls;       // 3 (core holes) + (virtual electrons), MRQ_NOROW
     int* ref_rep;                 // the reference that owns the row
     long long* row_off;           // (owners and rows known from earlier) the row's place in rows
-    int *table, *ulist;           // open addressing over references; the owners
+    int* table;                   // open addressing over references
+    int2* ulist;                  // tasks of k_rows: owner, piece (cut rows from the front, whole ones from the back)
+    int ulist_size;
     double* rows;
     int table_size, nref_max, wave_groups, wave0;
     // rows known in this launch: open addressing over row numbers (entry: epoch << 32 | row; another epoch's
@@ -2007,16 +2009,25 @@ __global__ void __launch_bounds__(256) k_insert(const WalkSet ws, const WalkScra
             const int y = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += y;
         }
-        const unsigned big = __ballot_sync(0xffffffffu, owner && len >= MRQ_BIG_ROW);
-        const unsigned small = __ballot_sync(0xffffffffu, owner && len < MRQ_BIG_ROW);
+        const unsigned big = __ballot_sync(0xffffffffu, owner && len > MRQ_BIG_ROW);
+        const unsigned small = __ballot_sync(0xffffffffu, owner && len <= MRQ_BIG_ROW);
+        const int pieces = owner && len > MRQ_BIG_ROW ? (len + MRQ_BIG_ROW - 1) / MRQ_BIG_ROW : 0;
+        int y = pieces;
+        if (big) {
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int z = __shfl_up_sync(0xffffffffu, y, o);
+                if (lane >= o) y += z;
+            }
+        }
         unsigned long long cur = 0;
         int nb = 0, ns = 0, nk = 0;
         if (lane == 31 && x > 0) cur = atomicAdd(reinterpret_cast<unsigned long long*>(sc.kctl + KNOWN_CUR), (unsigned long long)x);
         if (lane == 0 && (big | small)) nk = atomicAdd(sc.kctl + KNOWN_ROWS, __popc(big | small));
-        if (lane == 0 && big) nb = atomicAdd(sc.ctl + CTL_BIG, __popc(big));
+        if (lane == 31 && big) nb = atomicAdd(sc.ctl + CTL_BIG, y);
         if (lane == 0 && small) ns = atomicAdd(sc.ctl + CTL_SMALL, __popc(small));
         cur = __shfl_sync(0xffffffffu, cur, 31);
-        nb = __shfl_sync(0xffffffffu, nb, 0);
+        nb = __shfl_sync(0xffffffffu, nb, 31) + y - pieces;
         ns = __shfl_sync(0xffffffffu, ns, 0);
         nk = __shfl_sync(0xffffffffu, nk, 0);
         if (owner) {
@@ -2037,14 +2048,13 @@ __global__ void __launch_bounds__(256) k_insert(const WalkSet ws, const WalkScra
                     probe++;
                 }
             }
-            const int all = sc.wave_groups * sc.nref_max;
-            if (len >= MRQ_BIG_ROW) sc.ulist[nb + __popc(big & lt)] = i;
-            else sc.ulist[all - 1 - (ns + __popc(small & lt))] = i;
+            for (int k2 = 0; k2 < pieces; k2++) sc.ulist[nb + k2] = make_int2(i, k2);
+            if (pieces == 0) sc.ulist[sc.ulist_size - 1 - (ns + __popc(small & lt))] = make_int2(i, 0);
         }
     }
 }
 
-// The distinct rows, one warp task each.  Entry q of a group (core choice slow, virtual choice fast)
+// The distinct rows, a warp task each (long ones in pieces).  Entry q of a group (core choice slow, virtual choice fast)
 // holds c_l O(m) (-1)^(core-hole positions of m): the sign that H_nm of the same neighbour carries too,
 // so k_pairs multiplies the two as they are.
 // Bound by FP64 (2 FMA per clock and SM): one read and one FMA per candidate.
@@ -2058,12 +2068,13 @@ __global__ void __launch_bounds__(MRQ_MAXNW * 32, MINB) k_rows(const WalkSet ws,
     unsigned* const ccode = reinterpret_cast<unsigned*>(cphi + cap);
     if (sc.ctl[CTL_GC] <= sc.wave0) return;
     int cur = -1;
-    const int nbig = sc.ctl[CTL_BIG], ntask = nbig + sc.ctl[CTL_SMALL], all = sc.wave_groups * sc.nref_max;
+    const int nbig = sc.ctl[CTL_BIG], ntask = nbig + sc.ctl[CTL_SMALL];
     NoCtr ctr;
     for (;;) {
         const int id = next_task(sc.ctl + CTL_ROWTASK, lane);
         if (id >= ntask) break;
-        const int i = id < nbig ? sc.ulist[id] : sc.ulist[all - 1 - (id - nbig)];
+        const int2 task = id < nbig ? sc.ulist[id] : sc.ulist[sc.ulist_size - 1 - (id - nbig)];
+        const int i = task.x, lo = task.y * MRQ_BIG_ROW, hi = lo + MRQ_BIG_ROW;      // entries of the row
         const int sys = sc.meta[sc.wave0 + i / sc.nref_max].sys;
         __syncwarp();
         if (sys != cur) {
@@ -2075,16 +2086,22 @@ __global__ void __launch_bounds__(MRQ_MAXNW * 32, MINB) k_rows(const WalkSet ws,
         const int c = sc.ref_cls[i] / 3, v = sc.ref_cls[i] - 3 * c;
         const int d = __popcll(AO & 0xFFFFFFFFull) - (S.nalpha - S.nc);
         double* row = sc.rows + sc.row_off[i];
+        int base = 0;
         for (int scn = 0; scn <= c; scn++) {
             const int sv = scn - d;
             if (sv < 0 || sv > v) continue;
             const int nvc = shape_count(S.nv, v, sv), ni = shape_count(S.nc, c, scn) * nvc;
-            if (ni == 0) continue;
+            const int q0 = max(lo, base) - base, q1 = min(hi, base + ni) - base;
+            base += ni;
+            if (q0 >= q1) {
+                row += ni;
+                continue;
+            }
             int n1;
             const int count = row_list<W>(S, AO, c, v, scn, sv, cphi, ccode, n1, lane, ctr);
             const unsigned long long mvc = ~0ull / (unsigned long long)nvc + 1ull;     // q / nvc by its high product
-            for (int qb = 0; qb < ni; qb += 32) {
-                const int nr = min(32, ni - qb), f = split_of(nr), lf = __ffs(f) - 1;
+            for (int qb = q0; qb < q1; qb += 32) {
+                const int nr = min(32, q1 - qb), f = split_of(nr), lf = __ffs(f) - 1;
                 const int qi = lane >> lf, part = lane & (f - 1);
                 const int q = qb + min(qi, nr - 1);
                 const int ic = nvc == 1 ? q : (int)__umul64hi((unsigned long long)q, mvc);
