@@ -1398,8 +1398,9 @@ static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, lo
     w.ns_max = need.ns;
     w.nseg = seg;
     // walkers per task group: 32 when there are many, fewer for small launches, so that the walkers of
-    // a crowded determinant spread over more warps
-    w.tgw = (int)std::max(4LL, std::min<long long>(MRQ_TGW, seg / 128));
+    // a crowded determinant spread over more warps (against the determinant's neighbours being formed once
+    // per group)
+    w.tgw = (int)std::max(4LL, std::min<long long>(seg <= 2048 ? 16 : MRQ_TGW, seg <= 2048 ? seg / 64 : seg / 128));
     return 0;
 }
 

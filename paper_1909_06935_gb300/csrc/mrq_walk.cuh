@@ -893,6 +893,7 @@ struct WarpTask {
     uint4 wp[MRQ_TGW];                  // per walker: Philox words (x, y) and screen scale (w, FP32)
     unsigned wid[MRQ_TGW], step[MRQ_TGW], slot[MRQ_TGW];
     float bnd[MRQ_TGW];                 // upper bound of the best clock
+    RaceBest best[MRQ_TGW];             // the task's best candidate
     double qt[96];                      // queued neighbours: t and excitation
     unsigned qe[96];
 };
@@ -942,12 +943,23 @@ __device__ __forceinline__ bool atomic_cas128(RaceBest* at, const RaceBest& cmp,
 // whether two FP32 clocks (relative error below 1e-5) leave the order of the exact ones open
 __device__ __forceinline__ bool clocks_near(float a, float b) { return !(a < b * 0.9999f) && !(b < a * 0.9999f); }
 
-// Some lane's neighbour passed walker j's screen: of those that pass the closer one (race_may_win)
-// take the smallest clock, settle near ties by
-// the exact FP64 clocks (then the smaller excitation), and replace the walker's best if it is beaten.
-// Runs a handful of times per walker and step.
-__device__ __noinline__ void race_slow(WarpTask& wt, RaceBest* best, unsigned* bound, int j, double t, unsigned exc,
-                                       int lane) {
+// Whether a candidate (FP32 clock a; draw k, rate g, excitation) beats `cur`: by the FP32 clocks, near ties
+// by the exact FP64 ones, then by the smaller excitation
+__device__ __forceinline__ bool race_better(const WarpTask& wt, int j, float a, unsigned long long k, double g, unsigned exc,
+                                            const RaceBest& cur) {
+    if (cur.exc == 0xFFFFFFFFu) return true;
+    const float ca = __uint_as_float(cur.clk);
+    if (!clocks_near(a, ca)) return a < ca;
+    const double tm = race_clock_f64(k, g);
+    const double tb = race_clock_f64(race_bits(wt.sys.seed, cur.exc, wt.step[j], wt.wid[j]), fabs(cur.t * wt.inv_psin));
+    return tm < tb || (tm == tb && exc < cur.exc);
+}
+
+// Some lane's neighbour passed walker j's screen: of those that pass the closer one (race_may_win) take
+// the smallest clock (near ties by the exact FP64 clocks, then the smaller excitation) as the task's best
+// candidate if it beats that.  Runs a handful of times per walker and task and touches shared memory only;
+// the tasks' candidates meet in race_publish.
+__device__ __noinline__ void race_slow(WarpTask& wt, int j, double t, unsigned exc, int lane) {
     const unsigned long long seed = wt.sys.seed;
     const unsigned step = wt.step[j], wid = wt.wid[j];
     const unsigned long long k = race_bits(seed, exc, step, wid);
@@ -987,45 +999,41 @@ __device__ __noinline__ void race_slow(WarpTask& wt, RaceBest* best, unsigned* b
         src = __ffs(__ballot_sync(0xffffffffu, (near >> lane & 1u) && tc == tm && e == em)) - 1;
         if (src < 0) src = __ffs(near) - 1;
     }
-    float b = 0.0f;
-    if (lane == src) {
-        RaceBest mine, cur, old;
-        mine.clk = __float_as_uint(a);
-        mine.exc = exc;
-        mine.t = t;
-        const int slot = (int)wt.slot[j];
-        RaceBest* at = best + slot;
-        {
-            unsigned lo, hi;
-            asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-                         : "=r"(cur.clk), "=r"(cur.exc), "=r"(lo), "=r"(hi)
-                         : "l"(at));
-            cur.t = __hiloint2double((int)hi, (int)lo);
-        }
-        for (;;) {                                      // every turn but the last, another warp's candidate won
-            bool better = cur.exc == 0xFFFFFFFFu;
-            if (!better) {
-                const float ca = __uint_as_float(cur.clk);
-                if (!clocks_near(a, ca)) better = a < ca;
-                else {
-                    const double tm = race_clock_f64(k, g);
-                    const double tb = race_clock_f64(race_bits(seed, cur.exc, step, wid), fabs(cur.t * wt.inv_psin));
-                    better = tm < tb || (tm == tb && exc < cur.exc);
-                }
-            }
-            if (!better) break;
-            if (atomic_cas128(at, cur, mine, old)) break;
-            cur = old;
-        }
+    if (lane == src && race_better(wt, j, a, k, g, exc, wt.best[j])) {
+        wt.best[j].clk = __float_as_uint(a);
+        wt.best[j].exc = exc;
+        wt.best[j].t = t;
         const float up = a * 1.0001f;
-        b = fminf(up, __uint_as_float(atomicMin(bound + slot, __float_as_uint(up))));
-    }
-    b = __shfl_sync(0xffffffffu, b, src);
-    if (lane == 0) {
-        wt.bnd[j] = b;
-        wt.wp[j].w = __float_as_uint(race_scale(b, wt.inv_f));
+        if (up < wt.bnd[j]) {
+            wt.bnd[j] = up;
+            wt.wp[j].w = __float_as_uint(race_scale(up, wt.inv_f));
+        }
     }
     __syncwarp();
+}
+
+// the task's best candidates against the walkers' (one walker per lane): replaced by a 128-bit
+// compare-and-swap, and the bounds lowered for the tasks that begin later
+__device__ __noinline__ void race_publish(const WarpTask& wt, RaceBest* best, unsigned* bound, int count, int lane) {
+    if (lane >= count || wt.best[lane].exc == 0xFFFFFFFFu) return;
+    const RaceBest mine = wt.best[lane];
+    const float a = __uint_as_float(mine.clk);
+    const unsigned long long k = race_bits(wt.sys.seed, mine.exc, wt.step[lane], wt.wid[lane]);
+    const double g = fabs(mine.t * wt.inv_psin);
+    RaceBest* const at = best + (int)wt.slot[lane];
+    RaceBest cur, old;
+    {
+        unsigned lo, hi;
+        asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(cur.clk), "=r"(cur.exc), "=r"(lo), "=r"(hi)
+                     : "l"(at));
+        cur.t = __hiloint2double((int)hi, (int)lo);
+    }
+    while (race_better(wt, lane, a, k, g, mine.exc, cur)) {     // every turn but the last, another task's candidate won
+        if (atomic_cas128(at, cur, mine, old)) break;
+        cur = old;
+    }
+    atomicMin(bound + (int)wt.slot[lane], __float_as_uint(a * 1.0001f));
 }
 
 // the FP32 |t| of the screen
@@ -1122,8 +1130,8 @@ struct StepSink {
         }
         for (unsigned hits = race_round(wt, t0, e0, t1, e1, count); hits; hits &= hits - 1) {
             const int j = __ffs(hits) - 1;
-            race_slow(wt, best, bound, j, t0, e0, lane);
-            race_slow(wt, best, bound, j, t1, e1, lane);
+            race_slow(wt, j, t0, e0, lane);
+            race_slow(wt, j, t1, e1, lane);
         }
     }
     __device__ __forceinline__ void finish() {
@@ -1131,6 +1139,9 @@ struct StepSink {
         if (qn > 0)
             take(lane < qn ? wt.qt[lane] : 0.0, lane < qn ? wt.qe[lane] : 0u, 32 + lane < qn ? wt.qt[32 + lane] : 0.0,
                  32 + lane < qn ? wt.qe[32 + lane] : 0u);
+        __syncwarp();
+        race_publish(wt, best, bound, count, lane);
+        __syncwarp();
     }
 };
 
@@ -1361,6 +1372,7 @@ __device__ __forceinline__ bool task_begin(WarpTask& wt, const WalkSet& ws, cons
         wt.wid[lane] = wid;
         wt.step[lane] = step;
         wt.slot[lane] = (unsigned)slot;
+        wt.best[lane].exc = 0xFFFFFFFFu;
     }
     if (lane == 0) {
         wt.inv_psin = inv;
