@@ -29,10 +29,6 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 WORKLOAD = "cas10_56o"
-# DRAM bytes (read + write) per walker-step of the walk kernel, from an ncu capture of one
-# steady-state launch of the current kernel: dram__bytes_read.sum + dram__bytes_write.sum =
-# 183.68 MB + 6630.77 MB for 4,096 walkers on the 56-orbital workload
-TRAFFIC_PER_WALKER_STEP = {"cas10_56o": (183.676416e6 + 6630.774e6) / 4096}
 METRIC = "walker-steps/s"
 # FP64 FMA pipe of GB300: 2 FMA per clock per SM, 152 SMs, 2.07 GHz maximum SM clock
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
@@ -321,14 +317,19 @@ def run_ours(args):
     units = nw * inner * args.steps
     value = job_rate(units, world, ms)
 
-    # algorithmic work per walker-step, counted exactly by the debug kernel on walker snapshots taken
-    # before and after the timed region: every reach-back term H_mk phi0(k) is one FP64 FMA (2 flops),
-    # every neighbour adds <n|H|m>, the ratio, the rate and three sums (8 flops)
+    # algorithmic work, counted exactly by the debug kernel on walker snapshots taken before and after the
+    # timed region: every reach-back term H_mk phi0(k) is one FP64 FMA (2 flops), every neighbour adds
+    # <n|H|m>, the ratio, the rate and three sums (8 flops).  A step evaluates each distinct determinant
+    # once for all walkers on it, so the work is that of the distinct determinants (the terms that they
+    # share among each other are counted for each).
     locs = [ctx.debug_local(snap)[0] for snap in (snap0, snap1)]
-    terms = float(np.mean([np.mean(l["n_terms"]) for l in locs]))
+    once = [np.unique(snap, axis=0, return_index=True)[1] for snap in (snap0, snap1)]
+    distinct = float(np.mean([len(u) for u in once]))
+    terms = float(np.mean([np.sum(l["n_terms"][u]) for l, u in zip(locs, once)])) / nw
     nbrs = float(np.mean([np.mean(l["n_neighbours"]) for l in locs]))
-    gathers = float(np.mean([np.mean(l["n_gathers"] + l["n_probes"]) for l in locs]))
-    flops_per_step = 2.0 * terms + 8.0 * nbrs
+    nbrs_once = float(np.mean([np.sum(l["n_neighbours"][u]) for l, u in zip(locs, once)])) / nw
+    gathers = float(np.mean([np.sum((l["n_gathers"] + l["n_probes"])[u]) for l, u in zip(locs, once)])) / nw
+    flops_per_step = 2.0 * terms + 8.0 * nbrs_once
     launch_s = walk_s / max(walk_launches, 1)
     units_per_launch = nw * inner
     achieved = flops_per_step * units_per_launch / launch_s / 1e12
@@ -337,15 +338,16 @@ def run_ours(args):
     sectors_per_s = gathers * units_per_launch / launch_s
     roof = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
             "frac": achieved / FP64_PEAK_TFLOPS,
-            "traffic": (TRAFFIC_PER_WALKER_STEP[args.system] * units_per_launch
-                        if args.system in TRAFFIC_PER_WALKER_STEP else None),
-            "kernel": "k_walk2",
+            "traffic": None,
+            "kernel": "k_pairs, k_rows, k_frows, k_fois, k_fois_act (one walk step)",
             "peak_source": "FP64 FMA pipe: 152 SMs x 2 FMA/clk x 2 flop x 2.07 GHz (derived from unit counts and the "
                            "maximum SM clock)",
             "peak_measured": probe["fp64_flops"] / 1e12,
             "frac_of_measured": achieved / (probe["fp64_flops"] / 1e12),
             "flops_per_walker_step": flops_per_step, "terms_per_walker_step": terms,
-            "neighbours_per_walker_step": nbrs, "launch_seconds": launch_s, "launches_timed": int(walk_launches),
+            "neighbours_per_walker_step": nbrs, "distinct_determinants": distinct,
+            # the move race draws one Philox clock per neighbour and walker
+            "race_draws_per_s": nbrs * units_per_launch / launch_s, "launch_seconds": launch_s, "launches_timed": int(walk_launches),
             # the gather view of the same launches: every integral / table gather and hash-slot read is
             # one random 32-byte sector (the algorithmic sectors of the walk)
             "sectors_per_walker_step": gathers, "sectors_per_s": sectors_per_s,
@@ -429,8 +431,9 @@ def run_ours(args):
             "clocks": clk.summary(),
             "roofline": roof,
             "e2e": e2e,
-            # per step: slot keys, slot sort, walk, accumulate; finalize labels, finalize reduce
-            "gpu_launches": 6 * args.steps,
+            # per step: group, prep, int, fois_act, fgroups, frows, fois, rows_begin, wave_begin, refs, insert,
+            # rows, pairs, move, accumulate; finalize list, labels, reduce (empty waves not counted)
+            "gpu_launches": 18 * args.steps,
             "cpu_baseline": cpu,
             "batched": batched,
             "served": served,
@@ -448,7 +451,7 @@ def measure_batched(n_systems: int, total_walkers: int, R: int, steps: int, warm
     6-max_act, references of 400 to 5e5 determinants, walkers proportional to the reference size)
     run three ways with the same reporting interval of R walker steps (one finalize per system):
     plain (one system per launch, one after the other), batched (every system in one launch per
-    determinant width and occupancy class) and batched with the autotuned launch configuration and
+    determinant width) and batched with the autotuned launch configuration and
     CUDA-graph replay."""
     os.environ.setdefault("OPENBLAS_NUM_THREADS", "1")
     import synthetic as S

@@ -9,7 +9,7 @@
  *
  * Conventions shared by every call:
  *  - n = n_core + n_act + n_virt spatial orbitals (n <= 128), ordered core, active, virtual;
- *    n_core <= 64, n_act <= 32.  A walker's block keeps one reach-back candidate list per warp in
+ *    n_core <= 64, n_act <= 32.  The walk's blocks keep one reach-back candidate list per warp in
  *    shared memory: systems whose lists are too long for eight warps run with four, two or one
  *    (mrq_load_hamiltonian returns MRQ_TOO_LARGE only when one warp's list does not fit).
  *  - A determinant is 2W uint64 words, W = ceil(n/64): alpha occupation bits (bit p of word
@@ -69,9 +69,9 @@ typedef struct {
     int32_t n_groups;       /* G walker groups for jackknife errors (walker w is in group w mod G) */
     int32_t method;         /* mrq_method: informative; both estimators are always accumulated */
     double screen_tau;      /* perturbers with N_l/N_0 below this are screened out (Sec. II C) */
-    int32_t warps_per_walker;  /* 1, 2, 4 or 8 warps in each walker's thread block (at most what the
+    int32_t warps_per_walker;  /* 1, 2, 4 or 8 warps in the walk's list-building blocks (at most what the
                                   system's candidate lists allow); 0 keeps the context's setting (by
-                                  default chosen from the system's size, see mrq_set_launch) */
+                                  default 8, see mrq_set_launch) */
     int32_t steps_per_check;   /* mrq_sample with target_sigma: steps between error checks (0: n_steps/16) */
     double target_sigma;    /* mrq_sample stops early once the jackknife sigma of E^(2) (method
                                SC_NEVPT2) or of E (SC_MRCI) is at or below this; 0 = off */
@@ -193,7 +193,11 @@ int mrq_walkers_init(mrq_ctx* ctx, const mrq_sample_params* p);
  * Advance every walker by n_steps continuous-time steps (Sec. II B; first-reaction form of
  * Gillespie's algorithm with Philox4x32-10 clocks keyed on (seed; exc, step, walker)),
  * accumulating the estimators of Eq. 4, 12 and 16 after each walker's burn-in.  Asynchronous
- * on the context stream.  Errors: MRQ_NOT_LOADED, MRQ_CUDA_ERROR.
+ * on the context stream (two more streams of the context are forked from it and joined to it).  The
+ * first advance allocates the walk's workspace - per distinct determinant of a step, the overlaps of
+ * its neighbours: at most about 12 GiB, less for small systems or few walkers or where the device has
+ * less - which the context keeps until the next mrq_load_hamiltonian or mrq_destroy.
+ * Errors: MRQ_NOT_LOADED, MRQ_OOM, MRQ_CUDA_ERROR.
  */
 int mrq_walkers_advance(mrq_ctx* ctx, int64_t n_steps);
 
@@ -222,10 +226,9 @@ int mrq_finalize_noalloc(mrq_ctx* ctx, mrq_result* out);
 
 /*
  * Batched walk: advance the walkers of n contexts (independent systems, each initialised with
- * mrq_walkers_init) by n_steps in one walk launch per determinant width and occupancy class (the
- * walk blocks per SM a system's shared memory allows, so that small systems are not held to the
- * occupancy of the largest), so that many small systems fill the GPU together (the paper runs each
- * system on its own; walkers are independent Markov chains, Sec. II B).  Walker ids, seeds and accumulators stay per context, so every
+ * mrq_walkers_init) by n_steps in one walk launch per determinant width (and number of warps per
+ * block, where a system's candidate lists limit it), so that many small systems fill the GPU together
+ * (the paper runs each system on its own; walkers are independent Markov chains, Sec. II B).  Walker ids, seeds and accumulators stay per context, so every
  * trajectory is the same as when its context advances alone.  All contexts must be on one device;
  * the launch uses ctxs[0]'s stream after waiting for every context's stream, and returns after it
  * completes.  The walk time is reported by mrq_finalize on ctxs[0] only.
@@ -236,14 +239,12 @@ int mrq_batch_advance(mrq_ctx* const* ctxs, int n, int64_t n_steps);
 /*
  * Launch configuration of a context's walks (no counterpart in the paper: a GPU scheduling
  * choice that leaves every trajectory and accumulator the same, up to the order of the FP64
- * additions).  warps_per_walker in {1, 2, 4, 8}: the warps of the thread block that takes one walker's
- * step (they split its neighbours into interleaved work units); 0, the default, chooses from the
- * system's work units per CAS walker (8 for 512 or more, 4 for 128 or more, else 2; a batch takes
- * the largest of its systems' choices);
- * steps_per_launch >= 1 splits an advance into launches of that many steps, each re-ordering the
- * walker slots first (0, the default: one launch per advance); use_graph != 0 makes
+ * additions).  warps_per_walker in {1, 2, 4, 8}: the warps of the thread blocks that build the
+ * candidate lists (every warp takes its own work units); 0, the default, is 8;
+ * steps_per_launch >= 1 splits an advance into launches of that many steps, each of which computes
+ * the overlaps it needs anew (0, the default: one launch per advance); use_graph != 0 makes
  * mrq_batch_advance, with ctxs[0] this context, capture one launch of steps_per_launch steps (the
- * reporting interval: slot sort + walk) into a CUDA graph once per batch layout and replay it.
+ * reporting interval) into a CUDA graph once per batch layout and replay it.
  * Errors: MRQ_INVALID_ARG.
  */
 int mrq_set_launch(mrq_ctx* ctx, int warps_per_walker, int steps_per_launch, int use_graph);
@@ -287,7 +288,8 @@ enum mrq_request_state { MRQ_REQ_QUEUED = 0, MRQ_REQ_RUNNING = 1, MRQ_REQ_DONE =
 typedef struct {
     int32_t device;
     int32_t max_active;          /* requests resident at once */
-    int64_t hbm_budget_bytes;    /* device bytes the resident requests may use (estimated per request) */
+    int64_t hbm_budget_bytes;    /* device bytes the resident requests may use (estimated per request); the
+                                    batch's walk workspace takes at most what they leave of it */
     int64_t steps_per_round;     /* walker steps per batched launch */
 } mrq_server_params;
 

@@ -387,7 +387,7 @@ class Context:
                                                     int(total_steps)))
 
     def set_launch(self, warps_per_walker=0, steps_per_launch=0, use_graph=False):
-        """Walk launch configuration: warps per walker block (0 = chosen from the system's size),
+        """Walk launch configuration: warps per list-building block (0 = 8),
         steps per launch (0 = one launch per advance), CUDA-graph replay of batched reporting
         intervals."""
         self._check(self._lib.mrq_set_launch(self._h, warps_per_walker, steps_per_launch, int(bool(use_graph))))
@@ -499,8 +499,7 @@ def _ctx_array(ctxs):
 
 
 def batch_advance(ctxs, n_steps: int):
-    """Advance the walkers of several contexts together (one walk launch per determinant width and
-    occupancy class)."""
+    """Advance the walkers of several contexts together (one walk launch per determinant width)."""
     lib = load_library()
     rc = lib.mrq_batch_advance(C.cast(_ctx_array(ctxs), C.c_void_p), len(ctxs), n_steps)
     if rc:
@@ -508,7 +507,7 @@ def batch_advance(ctxs, n_steps: int):
 
 
 def tune_batch(ctxs, trial_steps: int = 4):
-    """Autotune walkers per block and steps per launch for this batch (on scratch walkers; the
+    """Autotune warps per block and steps per launch for this batch (on scratch walkers; the
     contexts' state is unchanged) and set the fastest on every context.  Returns the timings."""
     lib = load_library()
     out = TuneResult()

@@ -1067,6 +1067,7 @@ struct mrq_ctx {
     // workspace of this context's walk launches (WalkScratch), kept between calls
     unsigned char* d_work = nullptr;
     size_t work_cap = 0;
+    long long work_limit = 1LL << 40;   // mrq_internal_work_limit
     long long row_worst = 0;         // doubles of one CAS determinant's rows when none is shared
     int fg_max = 1;                  // groups of a first-order determinant's neighbours (at most)
     WalkScratch work{};
@@ -1303,13 +1304,13 @@ struct WalkNeed {
 static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, long long* seg_out) {
     const long long per = 12 * 4 + 3 * 4 + 2 * (long long)sizeof(TaskGroup) + (long long)sizeof(GroupMeta) +
                           8LL * need.gstride + 24LL * (need.ns + MRQ_ACT_SLICES) + (long long)sizeof(RaceBest) + 4;
-    const long long seg = std::min(nslots, std::max(256LL, std::min(1LL << 20, MRQ_WORK_BYTES / per)));
+    const long long seg = std::min(nslots, std::max(256LL, std::min(1LL << 20, std::min(MRQ_WORK_BYTES, ctx->work_limit / 5) / per)));
     *seg_out = seg;
     const long long per_group = 8 * need.row_worst + 93LL * need.nref;
-    long long groups = std::max(1LL, std::min(seg, MRQ_ROW_BYTES / per_group));
+    long long groups = std::max(1LL, std::min(seg, std::min(MRQ_ROW_BYTES, ctx->work_limit / 5 * 3) / per_group));
     groups = std::min(groups, std::max(1LL, (1LL << 29) / need.nref));           // reference indices and the table: 32 bits
     const long long per_fois = 8 * need.fois_nb + (long long)sizeof(FGroup) * need.fg_max + 8;
-    long long fwave = std::max(1LL, std::min(seg, MRQ_FROW_BYTES / per_fois));
+    long long fwave = std::max(1LL, std::min(seg, std::min(MRQ_FROW_BYTES, ctx->work_limit / 5) / per_fois));
     fwave = std::min(fwave, std::max(1LL, (1LL << 30) / need.fg_max));           // group indices: 32 bits
     WalkScratch& w = ctx->work;
     for (;; groups = (groups + 1) / 2, fwave = (fwave + 1) / 2) {
@@ -1331,7 +1332,8 @@ static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, lo
                      kt = take(8 * tsz), kao = take(8 * nr), kkey = take(4 * nr), koff = take(8 * nr), kctl = take(4 * KNOWN_N),
                      fgo = take(8 * fwave), fg = take(sizeof(FGroup) * (size_t)need.fg_max * fwave),
                      rows = take(8 * (size_t)need.row_worst * groups), frows = take(8 * (size_t)need.fois_nb * fwave);
-        if (off > ctx->work_cap) {
+        // (a workspace well above a lowered limit is given back)
+        if (off > ctx->work_cap || ((long long)ctx->work_cap > ctx->work_limit && off < ctx->work_cap / 2)) {
             CK(cudaStreamSynchronize(ctx->stream));
             dfree(ctx->d_work);
             ctx->work_cap = 0;
@@ -2764,6 +2766,8 @@ int mrq_internal_fail(mrq_ctx* ctx, int code, const char* fmt, ...) {
     }
     return code;
 }
+
+void mrq_internal_work_limit(mrq_ctx* ctx, long long bytes) { ctx->work_limit = std::max(0LL, bytes); }
 
 int mrq_internal_sync(mrq_ctx* ctx) { return sync_stream(ctx); }
 

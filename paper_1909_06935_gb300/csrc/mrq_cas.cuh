@@ -121,52 +121,6 @@ __device__ __forceinline__ double neg_if(double x, int odd) {
     return __longlong_as_double(__double_as_longlong(x) ^ ((long long)(odd & 1) << 63));
 }
 
-// the two removed (or added) spin orbitals of a candidate: `cnt` lane orbitals l0, l1 first, then
-// the candidate's active orbitals from its code (bit positions b0, b1); returned sorted
-__device__ __forceinline__ void merge_pair(const SysDev& S, int cnt, int l0, int l1, unsigned b0, unsigned b1,
-                                           int& x0, int& x1) {
-    const int c0 = act_so(S, (int)(b0 & 63u)), c1 = act_so(S, (int)(b1 & 63u));
-    x0 = cnt >= 1 ? l0 : c0;
-    x1 = cnt == 2 ? l1 : (cnt == 1 ? c0 : c1);
-    if (x0 > x1) {
-        int t = x0;
-        x0 = x1;
-        x1 = t;
-    }
-}
-
-// <m|H|k> for a double candidate: removed = lane's virtual electrons yv + candidate's R',
-// added = lane's core holes xc + candidate's A' (pairing by sorted order, spin conserving)
-template <int W, class C>
-__device__ __forceinline__ double dbl_elem_code(const SysDev& S, const unsigned long long (&m)[2][W], unsigned code,
-                                                int nyv, int yv0, int yv1, int nxc, int xc0, int xc1, C& ctr) {
-    int r1, r2, a1, a2;
-    merge_pair(S, nyv, yv0, yv1, code & 127u, (code >> 7) & 127u, r1, r2);
-    merge_pair(S, nxc, xc0, xc1, (code >> 14) & 127u, (code >> 21) & 127u, a1, a2);
-    const int n = S.n;
-    const int s_r1 = r1 >= n, s_r2 = r2 >= n;
-    const int pr1 = r1 - s_r1 * n, pr2 = r2 - s_r2 * n, pa1 = a1 - (a1 >= n) * n, pa2 = a2 - (a2 >= n) * n;
-    int c1 = popc_sel<W>(m, s_r1, min(pr1, pa1), max(pr1, pa1));
-    int c2;
-    if (s_r2 == s_r1) {
-        unsigned long long t[W];
-#pragma unroll
-        for (int w = 0; w < W; w++) t[w] = s_r1 ? m[1][w] : m[0][w];
-        flip<W>(t, pr1);
-        flip<W>(t, pa1);
-        c2 = popc_between<W>(t, min(pr2, pa2), max(pr2, pa2));
-    } else {
-        c2 = popc_sel<W>(m, s_r2, min(pr2, pa2), max(pr2, pa2));
-    }
-    double v = __ldg(S.eri4 + eri_idx(S, pa1, pr1, pa2, pr2));
-    ctr.g();
-    if (s_r1 == s_r2) {
-        v -= __ldg(S.eri4 + eri_idx(S, pa1, pr2, pa2, pr1));
-        ctr.g();
-    }
-    return neg_if(v, c1 + c2);
-}
-
 // A double candidate of a group as a signed table lookup.  With the added pair A = (A0, A1) and the
 // removed pair R = (R0, R1) of m -> k ordered "candidate's active orbitals first, lane's core /
 // virtual orbitals last", <m|H|k> = sgn (-1)^(piA + piR) <A0 A1||R0 R1>, where <A0 A1||R0 R1> is
@@ -241,50 +195,6 @@ __device__ __forceinline__ void lane_offsets(const SysDev& S, int c, int v, int 
     off_d = core + (v == 2 ? v0 * sv + v1 : (v == 1 ? v0 : 0u));
     off_x = core + (v == 2 ? v1 * sv + v0 : (v == 1 ? v0 * sv : 0u));
     par = (c >= 1 ? (int)p0 : 0) + (c == 2 ? (int)p1 : 0);
-}
-
-// sum over the table-form double candidates e0, e0 + stride, ... < e1 (list order)
-template <class C>
-__device__ __forceinline__ double tab_sum(const SysDev& S, const double* cphi, const unsigned* ccode, int e0, int e1,
-                                          int stride, unsigned off_d, unsigned off_x, C& ctr) {
-#ifndef MRQ_TAB_UNROLL
-#define MRQ_TAB_UNROLL 4
-#endif
-    double p[MRQ_TAB_UNROLL];
-#pragma unroll
-    for (int k = 0; k < MRQ_TAB_UNROLL; k++) p[k] = 0.0;
-    int e = e0;
-    for (; e + (MRQ_TAB_UNROLL - 1) * stride < e1; e += MRQ_TAB_UNROLL * stride) {
-        double x[MRQ_TAB_UNROLL];
-#pragma unroll
-        for (int k = 0; k < MRQ_TAB_UNROLL; k++) {
-            const unsigned bp = ccode[e + k * stride];
-            x[k] = __ldg(S.tab + (bp & 0x7FFFFFFFu) + ((bp & 0x80000000u) ? off_x : off_d));
-        }
-#pragma unroll
-        for (int k = 0; k < MRQ_TAB_UNROLL; k++) p[k] = fma(cphi[e + k * stride], x[k], p[k]);
-        ctr.g(MRQ_TAB_UNROLL);
-    }
-    for (; e < e1; e += stride) {
-        const unsigned bp = ccode[e];
-        p[0] = fma(cphi[e], __ldg(S.tab + (bp & 0x7FFFFFFFu) + ((bp & 0x80000000u) ? off_x : off_d)), p[0]);
-        ctr.g();
-    }
-    double t = p[0];
-#pragma unroll
-    for (int k = 1; k < MRQ_TAB_UNROLL; k++) t += p[k];
-    return t;
-}
-
-// sum over double candidates e0, e0 + stride, ... < e1 of phi_e <m|H|k_e> (list order)
-template <int W, class C>
-__device__ __forceinline__ double cand_sum(const SysDev& S, const unsigned long long (&m)[2][W], const double* cphi,
-                                           const unsigned* ccode, int e0, int e1, int stride, int nyv, int yv0, int yv1,
-                                           int nxc, int xc0, int xc1, C& ctr) {
-    double p0 = 0.0;
-    for (int e = e0; e < e1; e += stride)
-        p0 = fma(cphi[e], dbl_elem_code<W>(S, m, ccode[e], nyv, yv0, yv1, nxc, xc0, xc1, ctr), p0);
-    return p0;
 }
 
 // The walker's single-excitation operator, for every hole y (core or active) and electron x (active

@@ -22,6 +22,9 @@ struct MrqHamView {
 int mrq_internal_ham(mrq_ctx* ctx, MrqHamView* out);
 // record a message in the context's error slot and return code
 int mrq_internal_fail(mrq_ctx* ctx, int code, const char* fmt, ...);
+// Bytes the context's walk workspace may take (the launch works in smaller segments and waves within
+// them; a floor of 256 walkers and one determinant per wave remains)
+void mrq_internal_work_limit(mrq_ctx* ctx, long long bytes);
 // the context's host-wait (deadline-aware) synchronisation
 int mrq_internal_sync(mrq_ctx* ctx);
 

@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "../../include/mrq.h"
+#include "mrq_internal.h"
 
 namespace {
 
@@ -176,6 +177,10 @@ static int server_round(mrq_server* s) {
     std::vector<mrq_ctx*> ctxs;
     for (Request* r : act) ctxs.push_back(r->ctx);
     const int64_t steps = s->p.steps_per_round;
+    {
+        std::lock_guard<std::mutex> g(s->mu);        // the workspace is the first context's; it takes what is left
+        mrq_internal_work_limit(ctxs[0], s->p.hbm_budget_bytes - s->used_bytes);
+    }
     int rc = mrq_batch_advance(ctxs.data(), (int)ctxs.size(), steps);
     if (rc) snprintf(s->err, sizeof s->err, "batched advance failed: %s", mrq_last_error(ctxs[0]));
     // 3. finalize with the lock released (only this thread uses an active request's context, and

@@ -461,7 +461,8 @@ __device__ __noinline__ void cas_internal_unit(const SysDev& S, const CasWalker&
     }
 }
 
-// one (X_a, Y_a) pair chunk [lo, hi) of a CAS walker
+// one (X_a, Y_a) pair chunk [lo, hi) of a CAS walker with the lists of its own groups (the debug evaluation,
+// which counts a determinant's own terms; the walk takes the shared rows, k_pairs)
 template <int W, class Sink, class C>
 __device__ void cas_pair_unit(const SysDev& S, const CasWalker& cw, const double* __restrict__ gops, double* cphi,
                               unsigned* ccode, const unsigned long long (&n)[2][W], int u, int lane, Sink& sink, C& ctr) {
@@ -586,7 +587,7 @@ __device__ void cas_pair_unit(const SysDev& S, const CasWalker& cw, const double
 
 // ------------------------------------------------------------------ FOIS units
 
-// neighbours [i0, i1) of the class-block enumeration, reach-back per lane
+// neighbours [i0, i1) of the class-block enumeration, reach-back per lane (the debug evaluation)
 template <int W, class Sink, class C>
 __device__ __noinline__ void fois_unit(const SysDev& S, const WarpLists& sh, const double* __restrict__ gops,
                                        const unsigned long long (&n)[2][W], long long ln, double c0,
