@@ -348,8 +348,9 @@ def run_ours(args):
             "neighbours_per_walker_step": nbrs, "distinct_determinants": distinct,
             # the move race draws one Philox clock per neighbour and walker
             "race_draws_per_s": nbrs * units_per_launch / launch_s, "launch_seconds": launch_s, "launches_timed": int(walk_launches),
-            # the gather view of the same launches: every integral / table gather and hash-slot read is
-            # one random 32-byte sector (the algorithmic sectors of the walk)
+            # the gather view of the same launches: every integral / table gather and hash-slot read of the
+            # distinct determinants, each for itself, is one random 32-byte sector; determinants that share
+            # rows read less, so this rate can lie above the probe's
             "sectors_per_walker_step": gathers, "sectors_per_s": sectors_per_s,
             "l2_gather_peak_per_s": probe["l2_gathers_per_s"], "hbm_gather_peak_per_s": probe["hbm_gathers_per_s"],
             "l2_frac": sectors_per_s / probe["l2_gathers_per_s"],

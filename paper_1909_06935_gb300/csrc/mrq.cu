@@ -1011,6 +1011,8 @@ static double* noalloc_scratch_address(int device) {
 
 // ============================================================================ host runtime
 
+#define MRQ_MAX_SMEM (227 * 1024)      // dynamic shared memory of a block, at most
+
 struct mrq_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -1406,9 +1408,11 @@ static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, lo
     return 0;
 }
 
+// (a kernel's limit is the process's, so it is always set to the most a block may have: contexts on other
+// threads launch with other sizes)
 template <int W, int B>
 static int rows_fits(mrq_ctx* ctx, size_t smem, int threads, int& blocks) {
-    CK(cudaFuncSetAttribute(k_rows<W, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CK(cudaFuncSetAttribute(k_rows<W, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, MRQ_MAX_SMEM));
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_rows<W, B>, threads, smem));
     return 0;
 }
@@ -1416,20 +1420,20 @@ static int rows_fits(mrq_ctx* ctx, size_t smem, int threads, int& blocks) {
 // k_rows' build for this launch: the most resident warps per SM (4 or 2 blocks' worth of MRQ_MAXNW warps)
 // that the candidate lists in shared memory allow, and a grid that fills the chip once
 static int rows_prepare(mrq_ctx* ctx, int W, int nw, int cap) {
-    const size_t smem = nw * rows_warp_bytes(cap), lsm = nw * cand_list_bytes(cap);
+    const size_t smem = nw * rows_warp_bytes(cap);
     const size_t fsm = nw * frows_warp_bytes(cap);
     int b4 = 0, b2 = 0, bf = 0;
     if (W == 1) {
         if (int r = rows_fits<1, 4>(ctx, smem, 32 * nw, b4)) return r;
         if (int r = rows_fits<1, 2>(ctx, smem, 32 * nw, b2)) return r;
-        CK(cudaFuncSetAttribute(k_move<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm));
-        CK(cudaFuncSetAttribute(k_frows<1, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm));
+        CK(cudaFuncSetAttribute(k_move<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, MRQ_MAX_SMEM));
+        CK(cudaFuncSetAttribute(k_frows<1, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, MRQ_MAX_SMEM));
         CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bf, k_frows<1, 3>, 32 * nw, fsm));
     } else {
         if (int r = rows_fits<2, 4>(ctx, smem, 32 * nw, b4)) return r;
         if (int r = rows_fits<2, 2>(ctx, smem, 32 * nw, b2)) return r;
-        CK(cudaFuncSetAttribute(k_move<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm));
-        CK(cudaFuncSetAttribute(k_frows<2, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm));
+        CK(cudaFuncSetAttribute(k_move<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, MRQ_MAX_SMEM));
+        CK(cudaFuncSetAttribute(k_frows<2, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, MRQ_MAX_SMEM));
         CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bf, k_frows<2, 3>, 32 * nw, fsm));
     }
     ctx->rows_minb = b4 > b2 ? 4 : 2;
@@ -1652,7 +1656,7 @@ static int walk_plan(mrq_ctx* ctx, SysDev& s) {
     // warp the active space is too large for the walk
     ctx->max_nw = 0;
     for (int nw = MRQ_MAXNW; nw >= 1 && ctx->max_nw == 0; nw >>= 1)
-        if (debug_smem_bytes(nw, (int)cap, s.gstride) <= 227 * 1024 && nw * frows_warp_bytes((int)cap) <= 227 * 1024)
+        if (debug_smem_bytes(nw, (int)cap, s.gstride) <= MRQ_MAX_SMEM && nw * frows_warp_bytes((int)cap) <= MRQ_MAX_SMEM)
             ctx->max_nw = nw;
     if (ctx->max_nw == 0)
         return fail(ctx, MRQ_TOO_LARGE, "active space too large for the shared-memory candidate lists");
@@ -2037,11 +2041,11 @@ int mrq_debug_local(mrq_ctx* ctx, int64_t n, const uint64_t* dets, mrq_local* lo
     }
     long long* pre = nb ? ctx->d_nbpre : nullptr;
     if (W == 1) {
-        CK(cudaFuncSetAttribute(k_debug2<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        CK(cudaFuncSetAttribute(k_debug2<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, MRQ_MAX_SMEM));
         k_debug2<1><<<(unsigned)n, 32 * nw, smem, ctx->stream>>>(ctx->d_sys, d_dets, n, d_loc, max_nb, d_nb, pre,
                                                                  (int)stride);
     } else {
-        CK(cudaFuncSetAttribute(k_debug2<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        CK(cudaFuncSetAttribute(k_debug2<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, MRQ_MAX_SMEM));
         k_debug2<2><<<(unsigned)n, 32 * nw, smem, ctx->stream>>>(ctx->d_sys, d_dets, n, d_loc, max_nb, d_nb, pre,
                                                                  (int)stride);
     }
