@@ -1088,20 +1088,18 @@ struct mrq_ctx {
     int max_nw = MRQ_MAXNW;          // most warps per block whose candidate lists fit shared memory
     int spl = 0;                     // steps per launch (0: every advance is one launch)
     int use_graph = 0;               // batches replay one reporting interval from a CUDA graph
+    // everything a captured launch holds by value: the walk set, the workspace's layout and bounds, and the
+    // launch shapes.  Compared and copied as bytes (made by graph_key, which clears the padding).
     struct GraphKey {
-        const void *sys = nullptr, *wptr = nullptr, *off = nullptr, *work = nullptr;
-        long long nslots = 0;
-        int k = 0, wpb = 0, spl = 0, cap = 0, gstride = 0, ns = 0, nref = 0, fg = 0, wave = 0, fwave = 0;
-        bool operator==(const GraphKey& o) const {
-            return sys == o.sys && wptr == o.wptr && off == o.off && work == o.work && nslots == o.nslots &&
-                   k == o.k && wpb == o.wpb && spl == o.spl && cap == o.cap && gstride == o.gstride && ns == o.ns && nref == o.nref && fg == o.fg && wave == o.wave &&
-                   fwave == o.fwave;
-        }
+        const void *sys, *wptr, *off;
+        long long nslots;
+        int k, wpb, spl, cap, rows_minb, rows_blocks, frows_blocks, pad;
+        WalkScratch work;
     };
     // per determinant width and warps per block (8, 4, 2, 1) of a batch launch
     static constexpr int NSLOT = 8;
     cudaGraphExec_t gexec[NSLOT] = {};
-    GraphKey gkey[NSLOT];
+    GraphKey gkey[NSLOT] = {};
     int n_sm = 0;                    // SMs of the device
     long long graph_replays = 0;
     long long* d_nbpre = nullptr;    // debug records: neighbour offsets of a determinant's units
@@ -1193,6 +1191,18 @@ static cudaError_t reserve(T*& p, size_t& cap, size_t n) {
     if (e == cudaSuccess) cap = n * sizeof(T);
     else p = nullptr;
     return e;
+}
+
+// Give the walk's workspace back, and with it the graphs captured on it (the caller has waited for the
+// context's stream)
+static void free_work(mrq_ctx* c) {
+    for (int w = 0; w < mrq_ctx::NSLOT; w++) {
+        if (c->gexec[w]) cudaGraphExecDestroy(c->gexec[w]);
+        c->gexec[w] = nullptr;
+    }
+    dfree(c->d_work);
+    c->work_cap = 0;
+    c->ktab_bytes = 0;
 }
 
 static void free_reference(mrq_ctx* c) {
@@ -1337,9 +1347,7 @@ static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, lo
         // (a workspace well above a lowered limit is given back)
         if (off > ctx->work_cap || ((long long)ctx->work_cap > ctx->work_limit && off < ctx->work_cap / 2)) {
             CK(cudaStreamSynchronize(ctx->stream));
-            dfree(ctx->d_work);
-            ctx->work_cap = 0;
-            ctx->ktab_bytes = 0;
+            free_work(ctx);
             const cudaError_t e = cudaMalloc(&ctx->d_work, off);
             if (e == cudaErrorMemoryAllocation && (groups > 1 || fwave > 1)) {
                 cudaGetLastError();
@@ -1733,7 +1741,7 @@ void mrq_destroy(mrq_ctx* ctx) {
     dfree(ctx->d_err);
     dfree(ctx->d_sys);
     dfree(ctx->d_res);
-    dfree(ctx->d_work);
+    free_work(ctx);
     dfree(ctx->d_wptr);
     dfree(ctx->d_woff);
     dfree(ctx->d_bsys);
@@ -1742,8 +1750,6 @@ void mrq_destroy(mrq_ctx* ctx) {
     dfree(ctx->d_tune);
     dfree(ctx->d_tptr);
     dfree(ctx->d_nbpre);
-    for (int w = 0; w < mrq_ctx::NSLOT; w++)
-        if (ctx->gexec[w]) cudaGraphExecDestroy(ctx->gexec[w]);
     for (auto e : ctx->evs) cudaEventDestroy(e);
     if (ctx->ev0) cudaEventDestroy(ctx->ev0);
     if (ctx->ev1) cudaEventDestroy(ctx->ev1);
@@ -1791,9 +1797,7 @@ int mrq_load_hamiltonian(mrq_ctx* ctx, int n_core, int n_act, int n_virt, int n_
     if (int r_ = sync_stream(ctx)) return r_;
     DeadlinePause pause_(ctx);
     free_walkers(ctx);
-    dfree(ctx->d_work);               // the walk workspace of the last system is given back
-    ctx->work_cap = 0;
-    ctx->ktab_bytes = 0;
+    free_work(ctx);                   // the walk workspace of the last system is given back
     ctx->ref = ctx->ham = false;
     ctx->n = n;
     ctx->nc = n_core;
@@ -2339,6 +2343,23 @@ static int batch_tables(mrq_ctx* const* ctxs, int n, int W, Walker* const* walke
     return 0;
 }
 
+// the key of a graph of this launch; the workspace and the launch shapes are prepared
+static void graph_key(const mrq_ctx* ctx, const WalkSet& ws, const WalkNeed& need, int wpb, int spl, mrq_ctx::GraphKey& key) {
+    memset((void*)&key, 0, sizeof key);
+    key.sys = ws.systems;
+    key.wptr = ws.walkers;
+    key.off = ws.offsets;
+    key.nslots = ws.nslots;
+    key.k = ws.nsys;
+    key.wpb = wpb;
+    key.spl = spl;
+    key.cap = need.cap;
+    key.rows_minb = ctx->rows_minb;
+    key.rows_blocks = ctx->rows_blocks;
+    key.frows_blocks = ctx->frows_blocks;
+    memcpy((void*)&key.work, (const void*)&ctx->work, sizeof(WalkScratch));
+}
+
 // n_steps steps of one width's walk set: launches of `spl` steps (the reporting interval), replayed
 // from a CUDA graph when the lead context asks for it
 static int batch_run(mrq_ctx* ctx, int W, const WalkSet& ws, const WalkNeed& need, int64_t n_steps, int wpb, int64_t spl,
@@ -2353,23 +2374,9 @@ static int batch_run(mrq_ctx* ctx, int W, const WalkSet& ws, const WalkNeed& nee
         if (int r = work_prepare(ctx, ws.nslots, need, &seg)) return r;
         if (int r = rows_prepare(ctx, W, std::min(wpb, MRQ_MAXNW), need.cap)) return r;
         mrq_ctx::GraphKey key;
-        key.sys = ws.systems;
-        key.wptr = ws.walkers;
-        key.off = ws.offsets;
-        key.work = ctx->d_work;
-        key.nslots = ws.nslots;
-        key.k = ws.nsys;
-        key.wpb = wpb;
-        key.spl = (int)spl;
-        key.cap = need.cap;
-        key.gstride = need.gstride;
-        key.ns = need.ns;
-        key.nref = need.nref;
-        key.fg = need.fg_max;
-        key.wave = ctx->work.wave_groups;
-        key.fwave = ctx->work.fwave;
+        graph_key(ctx, ws, need, wpb, (int)spl, key);
         cudaGraphExec_t& ex = ctx->gexec[slot];
-        if (!ex || !(ctx->gkey[slot] == key)) {
+        if (!ex || memcmp(&ctx->gkey[slot], &key, sizeof key) != 0) {
             if (ex) CK(cudaGraphExecDestroy(ex));
             ex = nullptr;
             CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
@@ -2387,7 +2394,7 @@ static int batch_run(mrq_ctx* ctx, int W, const WalkSet& ws, const WalkNeed& nee
                 ex = nullptr;
                 return fail(ctx, MRQ_CUDA_ERROR, "cudaGraphInstantiate: %s", cudaGetErrorString(ei));
             }
-            ctx->gkey[slot] = key;
+            memcpy(&ctx->gkey[slot], &key, sizeof key);
         }
         for (int64_t i = 0; i < nfull; i++) CK(cudaGraphLaunch(ex, ctx->stream));
         ctx->graph_replays += nfull;
