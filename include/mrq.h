@@ -400,6 +400,18 @@ int mrq_debug_race_screen(mrq_ctx* ctx, int64_t n, const uint64_t* k53, const do
                           uint8_t* pass, double* exact);
 
 /*
+ * The walk's move race alone, for parity: n neighbours of one determinant with psi_s = psi (excitation
+ * codes exc as in mrq_neighbour, distinct, and t = H_nm psi_s(m), zeros never win) against the clocks of
+ * n_walkers walkers (Philox4x32-10 words keyed on (seed; exc, step, walker)).  The neighbours are dealt to
+ * `slices` (1 ... 4096) warp tasks per group of walkers, whose candidates meet as in a walk step; the result does
+ * not depend on it.  winner[i] receives the excitation with walker i's smallest clock -ln(u)/|t / psi|
+ * (ties: the smaller excitation), 0xFFFFFFFF when every t is zero.
+ * Errors: MRQ_INVALID_ARG, MRQ_OOM, MRQ_CUDA_ERROR.
+ */
+int mrq_debug_race(mrq_ctx* ctx, int64_t n, const uint32_t* exc, const double* t, double psi, uint64_t seed,
+                   int32_t n_walkers, const uint32_t* walker, const uint32_t* step, int32_t slices, uint32_t* winner);
+
+/*
  * Persisting-L2 window of this context's walk launches (no counterpart in the paper; a GB300
  * cache setting).  With fraction > 0 every walk launch marks the physicists' integral tables (the
  * entries every reach-back term reads) as persisting in L2, with a hit ratio that fits them into

@@ -150,6 +150,7 @@ def load_library(build_if_missing: bool = True):
     lib.mrq_read_gradient_sums.argtypes = [P, P, P]
     lib.mrq_sample_batch.argtypes = [P, C.c_int, P, P]
     lib.mrq_debug_race_screen.argtypes = [P, I64, P, P, P, P, P]
+    lib.mrq_debug_race.argtypes = [P, I64, P, P, C.c_double, C.c_uint64, C.c_int32, P, P, C.c_int32, P]
     lib.mrq_set_deadline.argtypes = [P, C.c_double]
     lib.mrq_probe_peaks.argtypes = [C.c_int, P]
     lib.mrq_set_l2_window.argtypes = [P, C.c_double]
@@ -162,7 +163,7 @@ def load_library(build_if_missing: bool = True):
                "mrq_setup_info", "mrq_debug_local", "mrq_walkers_init", "mrq_walkers_advance", "mrq_finalize",
                "mrq_finalize_noalloc", "mrq_batch_advance", "mrq_sample_batch", "mrq_mrci_gradient",
                "mrq_amsgrad_step", "mrq_read_coeffs", "mrq_read_gradient_sums", "mrq_sample", "mrq_set_launch",
-               "mrq_tune_batch", "mrq_read_accumulators", "mrq_read_walkers", "mrq_debug_race_screen",
+               "mrq_tune_batch", "mrq_read_accumulators", "mrq_read_walkers", "mrq_debug_race_screen", "mrq_debug_race",
                "mrq_set_deadline", "mrq_debug_set_limits", "mrq_probe_peaks",
                "mrq_set_l2_window", "mrq_read_hamiltonian", "mrq_sci_reference", "mrq_load_accumulators", "mrq_set_heat_bath_cutoff"):
         getattr(lib, fn).restype = C.c_int
@@ -452,6 +453,20 @@ class Context:
         self._check(self._lib.mrq_debug_race_screen(self._h, k.size, _addr(k), _addr(r), _addr(tb), _addr(ok),
                                                     _addr(ex)))
         return ok.astype(bool), ex
+
+    def race(self, exc, t, psi, seed, walker, step, slices=8):
+        """Winners (excitation codes) of the walk's move race: neighbours (exc, t = H_nm psi_s(m)) of a
+        determinant with psi_s = psi, one winner per (walker, step), the neighbours in `slices` warp tasks."""
+        e = np.ascontiguousarray(exc, np.uint32)
+        v = np.ascontiguousarray(t, np.float64)
+        w = np.ascontiguousarray(walker, np.uint32)
+        s = np.ascontiguousarray(step, np.uint32)
+        if e.shape != v.shape or w.shape != s.shape or e.ndim != 1 or w.ndim != 1:
+            raise ValueError("exc and t, and walker and step, must be vectors of one length")
+        out = np.zeros(len(w), np.uint32)
+        self._check(self._lib.mrq_debug_race(self._h, len(e), _addr(e), _addr(v), float(psi), int(seed), len(w), _addr(w),
+                                             _addr(s), int(slices), _addr(out)))
+        return out
 
     def set_heat_bath_cutoff(self, eps: float):
         """Drop double excitations with |<ab||ij>| < eps from the walk (0: exact)."""

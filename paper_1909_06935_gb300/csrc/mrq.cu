@@ -717,8 +717,8 @@ __global__ void k_race_screen(const unsigned long long* __restrict__ k, const do
     if (i >= n) return;
     const float btf = isinf(tbest[i]) ? INFINITY : (float)tbest[i];
     const float gf = abs_f32_of(rate[i]);
-    pass[i] = race_pass((unsigned)(k[i] >> 21), gf > 0.0f ? gf : INFINITY, race_scale(btf * 1.0001f, 1.0f)) &&
-              race_may_win(k[i], gf, btf * 1.0001f);
+    pass[i] = race_pass((unsigned)(k[i] >> 21), gf > 0.0f ? gf : INFINITY, race_scale(race_bound(btf), 1.0f)) &&
+              race_may_win(k[i], gf, race_bound(btf));
     exact[i] = race_clock_f64(k[i], rate[i]);
 }
 
@@ -2683,6 +2683,46 @@ int mrq_debug_race_screen(mrq_ctx* ctx, int64_t n, const uint64_t* k53, const do
     cudaFree(d_e);
     cudaFree(d_p);
     return 0;
+}
+
+int mrq_debug_race(mrq_ctx* ctx, int64_t n, const uint32_t* exc, const double* t, double psi, uint64_t seed, int32_t n_walkers,
+                   const uint32_t* walker, const uint32_t* step, int32_t slices, uint32_t* winner) {
+    if (!ctx) return MRQ_INVALID_ARG;
+    ctx->err[0] = 0;
+    if (n <= 0 || !exc || !t || !(psi != 0.0) || !std::isfinite(psi) || n_walkers <= 0 || !walker || !step || slices < 1 || slices > 4096 || !winner)
+        return fail(ctx, MRQ_INVALID_ARG, "bad arguments");
+    CK(cudaSetDevice(ctx->device));
+    if (int r = sync_stream(ctx)) return r;
+    const size_t nw = (size_t)n_walkers;
+    auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+    const size_t o_exc = up(8 * (size_t)n), o_wid = o_exc + up(4 * (size_t)n), o_step = o_wid + up(4 * nw),
+                 o_best = o_step + up(4 * nw), o_bound = o_best + up(sizeof(RaceBest) * nw);
+    std::vector<RaceBest> best(nw);
+    for (RaceBest& b : best) b = RaceBest{0x7F800000u, 0xFFFFFFFFu, 0.0};
+    const std::vector<unsigned> bound(nw, 0x7F800000u);
+    unsigned char* d = nullptr;
+    CK(cudaMalloc(&d, o_bound + 4 * nw));
+    const auto run = [&]() -> int {
+        CK(cudaMemcpyAsync(d, t, 8 * (size_t)n, cudaMemcpyDefault, ctx->stream));
+        CK(cudaMemcpyAsync(d + o_exc, exc, 4 * (size_t)n, cudaMemcpyDefault, ctx->stream));
+        CK(cudaMemcpyAsync(d + o_wid, walker, 4 * nw, cudaMemcpyDefault, ctx->stream));
+        CK(cudaMemcpyAsync(d + o_step, step, 4 * nw, cudaMemcpyDefault, ctx->stream));
+        CK(cudaMemcpyAsync(d + o_best, best.data(), sizeof(RaceBest) * nw, cudaMemcpyHostToDevice, ctx->stream));
+        CK(cudaMemcpyAsync(d + o_bound, bound.data(), 4 * nw, cudaMemcpyHostToDevice, ctx->stream));
+        const long long warps = (long long)((nw + MRQ_TGW - 1) / MRQ_TGW) * slices;
+        if ((warps + 7) / 8 > 0x7FFFFFFFLL) return fail(ctx, MRQ_INVALID_ARG, "too many walkers");
+        k_debug_race<<<(unsigned)((warps + 7) / 8), 256, 0, ctx->stream>>>(
+            (const unsigned*)(d + o_exc), (const double*)d, n, 1.0 / psi, seed, (const unsigned*)(d + o_wid),
+            (const unsigned*)(d + o_step), n_walkers, slices, (RaceBest*)(d + o_best), (unsigned*)(d + o_bound));
+        CK(cudaGetLastError());
+        CK(cudaMemcpyAsync(best.data(), d + o_best, sizeof(RaceBest) * nw, cudaMemcpyDeviceToHost, ctx->stream));
+        CK(cudaStreamSynchronize(ctx->stream));
+        for (size_t i = 0; i < nw; i++) winner[i] = best[i].exc;
+        return 0;
+    };
+    const int r = run();
+    cudaFree(d);
+    return r;
 }
 
 int mrq_set_l2_window(mrq_ctx* ctx, double fraction) {

@@ -941,8 +941,15 @@ __device__ __forceinline__ bool atomic_cas128(RaceBest* at, const RaceBest& cmp,
     return o0 == c0 && o1 == c1;
 }
 
-// whether two FP32 clocks (relative error below 1e-5) leave the order of the exact ones open
-__device__ __forceinline__ bool clocks_near(float a, float b) { return !(a < b * 0.9999f) && !(b < a * 0.9999f); }
+// Whether two FP32 clocks leave the order of the exact ones open.  Their relative error is below 1e-5 within
+// FP32's normal range; below and above it (rates near 1e38 or 1e-38 and beyond) the exact clocks always decide.
+__device__ __forceinline__ bool clocks_near(float a, float b) {
+    return (!(a < b * 0.9999f) && !(b < a * 0.9999f)) || fmaxf(a, b) < 1e-30f || fminf(a, b) > 1e37f;
+}
+
+// FP32 upper bound of the clock whose FP32 image is a.  Images below the normal range may have lost all their
+// bits, so the bound never falls below 1e-37 (which keeps race_scale away from 0 times infinity, too).
+__device__ __forceinline__ float race_bound(float a) { return fmaxf(a * 1.0001f, 1e-37f); }
 
 // Whether a candidate (FP32 clock a; draw k, rate g, excitation) beats `cur`: by the FP32 clocks, near ties
 // by the exact FP64 ones, then by the smaller excitation
@@ -976,7 +983,7 @@ __device__ __noinline__ void race_slow(WarpTask& wt, int j, double t, unsigned e
     float amin = a;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) amin = fminf(amin, __shfl_xor_sync(0xffffffffu, amin, o));
-    unsigned near = __ballot_sync(0xffffffffu, ok && !(amin < a * 0.9999f));
+    unsigned near = __ballot_sync(0xffffffffu, ok && clocks_near(a, amin));
     if (near == 0u) return;
     int src = __ffs(near) - 1;
     if (near & (near - 1u)) {
@@ -1004,7 +1011,7 @@ __device__ __noinline__ void race_slow(WarpTask& wt, int j, double t, unsigned e
         wt.best[j].clk = __float_as_uint(a);
         wt.best[j].exc = exc;
         wt.best[j].t = t;
-        const float up = a * 1.0001f;
+        const float up = race_bound(a);
         if (up < wt.bnd[j]) {
             wt.bnd[j] = up;
             wt.wp[j].w = __float_as_uint(race_scale(up, wt.inv_f));
@@ -1034,7 +1041,7 @@ __device__ __noinline__ void race_publish(const WarpTask& wt, RaceBest* best, un
         if (atomic_cas128(at, cur, mine, old)) break;
         cur = old;
     }
-    atomicMin(bound + (int)wt.slot[lane], __float_as_uint(a * 1.0001f));
+    atomicMin(bound + (int)wt.slot[lane], __float_as_uint(race_bound(a)));
 }
 
 // the FP32 |t| of the screen
@@ -1349,6 +1356,26 @@ __device__ __forceinline__ void task_system(WarpTask& wt, const WalkSet& ws, int
     }
 }
 
+// walker `lane` of a task: its Philox words and its screen, from the bound of its best clock so far
+__device__ __forceinline__ void race_walker(WarpTask& wt, int lane, unsigned step, unsigned wid, int slot, const unsigned* bound,
+                                            float inv_f) {
+    uint4 a = race_walker_words(wt.sys.seed, step, wid);
+    const float b = __uint_as_float(__ldcg(bound + slot));
+    a.w = __float_as_uint(race_scale(b, inv_f));
+    wt.bnd[lane] = b;
+    wt.wp[lane] = a;
+    wt.wid[lane] = wid;
+    wt.step[lane] = step;
+    wt.slot[lane] = (unsigned)slot;
+    wt.best[lane].exc = 0xFFFFFFFFu;
+}
+
+// FP32 |1/psi_s(n)| of the screen; INFINITY (every neighbour passes) where FP32 cannot carry it
+__device__ __forceinline__ float race_inv(double inv) {
+    const float f = abs_f32_of(inv);
+    return f > 0.0f ? f : INFINITY;
+}
+
 // the determinant of a task group and the Philox words and screens of its walkers; false when it cannot
 // be evaluated (outside the first-order space, or psi_s = 0)
 template <int W>
@@ -1358,22 +1385,11 @@ __device__ __forceinline__ bool task_begin(WarpTask& wt, const WalkSet& ws, cons
     if (meta->label < 0 || !(meta->psi != 0.0)) return false;
     if (lane < 2 * W) wt.nsh[lane] = meta->d[lane / W][lane % W];
     const double inv = meta->inv_psi;
-    float inv_f = abs_f32_of(inv);
-    if (!(inv_f > 0.0f)) inv_f = INFINITY;
+    const float inv_f = race_inv(inv);
     if (lane < tg.count) {
         const int i = sc.members[tg.first + lane];
         const Walker* const wk = ws.walkers[tg.sys] + i;
-        const int slot = (int)(ws.offsets[tg.sys] + i - sc.seg0);
-        const unsigned step = wk->step, wid = wk->wid;
-        uint4 a = race_walker_words(wt.sys.seed, step, wid);
-        const float b = __uint_as_float(__ldcg(sc.bound + slot));
-        a.w = __float_as_uint(race_scale(b, inv_f));
-        wt.bnd[lane] = b;
-        wt.wp[lane] = a;
-        wt.wid[lane] = wid;
-        wt.step[lane] = step;
-        wt.slot[lane] = (unsigned)slot;
-        wt.best[lane].exc = 0xFFFFFFFFu;
+        race_walker(wt, lane, wk->step, wk->wid, (int)(ws.offsets[tg.sys] + i - sc.seg0), sc.bound, inv_f);
     }
     if (lane == 0) {
         wt.inv_psin = inv;
@@ -2491,6 +2507,43 @@ __global__ void __launch_bounds__(1024) k_accum(const WalkSet ws) {
         S.accW[g] += wsum;
         S.accE[g] += esum;
     }
+}
+
+// The race alone, for parity: the neighbours (t, excitation) of one determinant against nw walkers' clocks, the
+// neighbours in rounds of 64 dealt to `slices` warp tasks per group of MRQ_TGW walkers, as in a walk step.
+__global__ void __launch_bounds__(256) k_debug_race(const unsigned* __restrict__ exc, const double* __restrict__ t, long long n,
+                                                    double inv_psi, unsigned long long seed, const unsigned* __restrict__ wid,
+                                                    const unsigned* __restrict__ step, int nw, int slices, RaceBest* best,
+                                                    unsigned* bound) {
+    __shared__ WarpTask tasks[8];
+    const int lane = threadIdx.x & 31;
+    WarpTask& wt = tasks[threadIdx.x >> 5];
+    const long long id = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const long long first = id / slices * MRQ_TGW;
+    if (first >= nw) return;
+    const int count = (int)min((long long)MRQ_TGW, nw - first);
+    if (lane == 0) {
+        wt.sys.seed = seed;
+        wt.inv_psin = inv_psi;
+        wt.inv_f = race_inv(inv_psi);
+        wt.qn = 0;
+    }
+    __syncwarp();
+    if (lane < count) race_walker(wt, lane, step[first + lane], wid[first + lane], (int)(first + lane), bound, wt.inv_f);
+    __syncwarp();
+    StepSink sink{wt, best, bound, count, lane, false, 0.0, 0.0, 0.0};
+    for (long long q = 64 * (id % slices); q < n; q += 64LL * slices) {
+        const long long q0 = q + lane, q1 = q0 + 32;
+        const double t0 = q0 < n ? t[q0] : 0.0, t1 = q1 < n ? t[q1] : 0.0;
+        const unsigned e0 = q0 < n ? exc[q0] : 0u, e1 = q1 < n ? exc[q1] : 0u;
+        if (q + 64 <= n) {
+            sink.take(t0, e0, t1, e1);
+        } else {
+            sink.push(q0 < n, t0, e0);
+            sink.push(q1 < n, t1, e1);
+        }
+    }
+    sink.finish();
 }
 
 // ------------------------------------------------------------------ debug evaluation (parity)
