@@ -941,6 +941,23 @@ __device__ __forceinline__ bool atomic_cas128(RaceBest* at, const RaceBest& cmp,
     return o0 == c0 && o1 == c1;
 }
 
+// one 128-bit access: a vector load is four scalar ones to the memory model, and could mix the clock and
+// excitation of one candidate with the t of another
+__device__ __forceinline__ RaceBest load_best128(const RaceBest* at) {
+    unsigned long long o0, o1;
+    asm volatile("{\n\t.reg .b128 d;\n\t"
+                 "ld.relaxed.gpu.global.b128 d, [%2];\n\t"
+                 "mov.b128 {%0, %1}, d;\n\t}"
+                 : "=l"(o0), "=l"(o1)
+                 : "l"(at)
+                 : "memory");
+    RaceBest b;
+    b.clk = (unsigned)o0;
+    b.exc = (unsigned)(o0 >> 32);
+    b.t = __longlong_as_double((long long)o1);
+    return b;
+}
+
 // Whether two FP32 clocks leave the order of the exact ones open.  Their relative error is below 1e-5 within
 // FP32's normal range; below and above it (rates near 1e38 or 1e-38 and beyond) the exact clocks always decide.
 __device__ __forceinline__ bool clocks_near(float a, float b) {
@@ -1029,14 +1046,7 @@ __device__ __noinline__ void race_publish(const WarpTask& wt, RaceBest* best, un
     const unsigned long long k = race_bits(wt.sys.seed, mine.exc, wt.step[lane], wt.wid[lane]);
     const double g = fabs(mine.t * wt.inv_psin);
     RaceBest* const at = best + (int)wt.slot[lane];
-    RaceBest cur, old;
-    {
-        unsigned lo, hi;
-        asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-                     : "=r"(cur.clk), "=r"(cur.exc), "=r"(lo), "=r"(hi)
-                     : "l"(at));
-        cur.t = __hiloint2double((int)hi, (int)lo);
-    }
+    RaceBest cur = load_best128(at), old;
     while (race_better(wt, lane, a, k, g, mine.exc, cur)) {     // every turn but the last, another task's candidate won
         if (atomic_cas128(at, cur, mine, old)) break;
         cur = old;
