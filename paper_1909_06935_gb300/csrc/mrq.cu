@@ -1044,7 +1044,8 @@ struct mrq_ctx {
     double* d_c = nullptr;
     // walkers / accumulators
     Walker* d_walk = nullptr;
-    long long nwalk = 0, walk_cap = 0;
+    long long nwalk = 0;
+    size_t cap_walk = 0;             // (all cap_*: bytes of a kept buffer, 0 when there is none)
     int G = 0;
     long long burn = 0;
     unsigned long long seed = 0;
@@ -1065,7 +1066,7 @@ struct mrq_ctx {
     SysDev* d_bsys = nullptr;
     Walker** d_bwptr = nullptr;
     long long* d_boff = nullptr;
-    int bcap = 0;
+    size_t cap_bsys = 0, cap_bwptr = 0, cap_boff = 0;
     // workspace of this context's walk launches (WalkScratch), kept between calls
     unsigned char* d_work = nullptr;
     size_t work_cap = 0;
@@ -1076,7 +1077,7 @@ struct mrq_ctx {
     size_t ktab_bytes = 0;           // the table of known rows that was cleared last, and its counters
     int* kctl_at = nullptr;
     double* d_partial = nullptr;
-    long long partial_cap = 0;
+    size_t cap_partial = 0;
     mrq_result* d_res = nullptr;
     SysDev hsys{};
     SysDev* d_sys = nullptr;
@@ -1103,11 +1104,9 @@ struct mrq_ctx {
     int n_sm = 0;                    // SMs of the device
     long long graph_replays = 0;
     long long* d_nbpre = nullptr;    // debug records: neighbour offsets of a determinant's units
-    long long nbpre_cap = 0;
+    size_t cap_nbpre = 0;
     Walker* d_tune = nullptr;        // the tuner's scratch copy of a batch's walkers
-    long long tune_cap = 0;
-    Walker** d_tptr = nullptr;
-    int tptr_cap = 0;
+    size_t cap_tune = 0;
     std::vector<cudaEvent_t> evs;    // start/stop pairs of the walk launches since the last finalize
     int launches = 0;
     long long launches_total = 0;
@@ -1137,9 +1136,11 @@ static int fail(mrq_ctx* c, int code, const char* fmt, ...) {
 #define CK(call)                                                                                      \
     do {                                                                                              \
         cudaError_t e_ = (call);                                                                      \
-        if (e_ != cudaSuccess)                                                                        \
+        if (e_ != cudaSuccess) {                                                                      \
+            cudaGetLastError(); /* a failed allocation is not the next launch's error */              \
             return fail(ctx, e_ == cudaErrorMemoryAllocation ? MRQ_OOM : MRQ_CUDA_ERROR, "%s: %s (%s:%d)", \
                         #call, cudaGetErrorString(e_), __FILE__, __LINE__);                           \
+        }                                                                                             \
     } while (0)
 
 // Wait for the context stream.  With a deadline set (mrq_set_deadline) the wait polls an event
@@ -1184,9 +1185,11 @@ static void dfree(T*& p) {
 // loaded again (a geometry scan) allocates nothing
 template <typename T>
 static cudaError_t reserve(T*& p, size_t& cap, size_t n) {
-    if (p && cap >= n * sizeof(T)) return cudaSuccess;
+    const bool fits = n <= SIZE_MAX / sizeof(T);
+    if (p && fits && cap >= n * sizeof(T)) return cudaSuccess;
     dfree(p);
     cap = 0;
+    if (!fits) return cudaErrorMemoryAllocation;
     const cudaError_t e = cudaMalloc(&p, n * sizeof(T));
     if (e == cudaSuccess) cap = n * sizeof(T);
     else p = nullptr;
@@ -1212,25 +1215,56 @@ static void free_reference(mrq_ctx* c) {
     c->cap_hash = c->cap_c = c->cap_setup = 0;
     c->ref = false;
 }
-static void free_walkers(mrq_ctx* c) {
-    dfree(c->d_walk);
+static void free_accumulators(mrq_ctx* c) {
     dfree(c->d_accN);
     dfree(c->d_accU);
     dfree(c->d_accA);
     dfree(c->d_accB);
-    dfree(c->d_grad);
-    dfree(c->d_am_m);
-    dfree(c->d_am_v);
-    dfree(c->d_am_vh);
     dfree(c->d_accW);
     dfree(c->d_accE);
     dfree(c->d_types);
     dfree(c->d_flist);
-    dfree(c->d_partial);
-    c->nwalk = c->walk_cap = 0;
     c->acc_lab = 0;
     c->acc_G = 0;
-    c->partial_cap = 0;
+}
+
+// Accumulators of G groups, all or none: a context whose allocation failed holds none and can be started again
+static int alloc_accumulators(mrq_ctx* ctx, int G) {
+    if (ctx->acc_lab == ctx->nlab && ctx->acc_G == G) return 0;
+    free_accumulators(ctx);
+    const size_t L = (size_t)ctx->nlab;
+    const auto all = [&]() -> int {
+        CK(cudaMalloc(&ctx->d_accN, sizeof(double) * L * G));
+        CK(cudaMalloc(&ctx->d_accU, sizeof(double) * L * G));
+        CK(cudaMalloc(&ctx->d_accA, sizeof(double) * L * G));
+        CK(cudaMalloc(&ctx->d_accB, sizeof(double) * L * G));
+        CK(cudaMalloc(&ctx->d_accW, sizeof(double) * G));
+        CK(cudaMalloc(&ctx->d_accE, sizeof(double) * G));
+        CK(cudaMalloc(&ctx->d_types, sizeof(unsigned long long) * MRQ_NTYPES));
+        CK(cudaMalloc(&ctx->d_flist, sizeof(int) * (L + (size_t)((ctx->nlab + FIN_CHUNK - 1) / FIN_CHUNK))));
+        return 0;
+    };
+    if (int r = all()) {
+        free_accumulators(ctx);
+        ctx->nwalk = 0;
+        return r;
+    }
+    ctx->acc_lab = ctx->nlab;
+    ctx->acc_G = G;
+    return 0;
+}
+
+static void free_walkers(mrq_ctx* c) {
+    dfree(c->d_walk);
+    c->cap_walk = 0;
+    c->nwalk = 0;
+    free_accumulators(c);
+    dfree(c->d_grad);
+    dfree(c->d_am_m);
+    dfree(c->d_am_v);
+    dfree(c->d_am_vh);
+    dfree(c->d_partial);
+    c->cap_partial = 0;
 }
 static void free_hamiltonian(mrq_ctx* c) {
     dfree(c->d_h1);
@@ -1748,7 +1782,6 @@ void mrq_destroy(mrq_ctx* ctx) {
     dfree(ctx->d_bwptr);
     dfree(ctx->d_boff);
     dfree(ctx->d_tune);
-    dfree(ctx->d_tptr);
     dfree(ctx->d_nbpre);
     for (auto e : ctx->evs) cudaEventDestroy(e);
     if (ctx->ev0) cudaEventDestroy(ctx->ev0);
@@ -2038,11 +2071,7 @@ int mrq_debug_local(mrq_ctx* ctx, int64_t n, const uint64_t* dets, mrq_local* lo
     const size_t smem = debug_smem_bytes(nw, cap, ctx->hsys.gstride);
     // neighbour offsets of the CAS units, for the records
     const long long stride = nb ? std::max(1, ctx->hsys.unit_off[8]) : 0;
-    if (nb && n * stride > ctx->nbpre_cap) {
-        dfree(ctx->d_nbpre);
-        CK(cudaMalloc(&ctx->d_nbpre, sizeof(long long) * n * stride));
-        ctx->nbpre_cap = n * stride;
-    }
+    if (nb) CK(reserve(ctx->d_nbpre, ctx->cap_nbpre, (size_t)(n * stride)));
     long long* pre = nb ? ctx->d_nbpre : nullptr;
     if (W == 1) {
         CK(cudaFuncSetAttribute(k_debug2<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, MRQ_MAX_SMEM));
@@ -2081,31 +2110,9 @@ int mrq_walkers_init(mrq_ctx* ctx, const mrq_sample_params* p) {
     if (p->warps_per_walker) ctx->wpb = p->warps_per_walker;
     CK(cudaSetDevice(ctx->device));
     DeadlinePause pause_(ctx);
-    if (p->n_walkers > ctx->walk_cap) {
-        dfree(ctx->d_walk);
-        CK(cudaMalloc(&ctx->d_walk, sizeof(Walker) * p->n_walkers));
-        ctx->walk_cap = p->n_walkers;
-    }
-    if (ctx->acc_lab != ctx->nlab || ctx->acc_G != p->n_groups) {
-        dfree(ctx->d_accN);
-        dfree(ctx->d_accU);
-        dfree(ctx->d_accW);
-        dfree(ctx->d_accE);
-        dfree(ctx->d_types);
-        dfree(ctx->d_flist);
-        CK(cudaMalloc(&ctx->d_accN, sizeof(double) * ctx->nlab * p->n_groups));
-        CK(cudaMalloc(&ctx->d_accU, sizeof(double) * ctx->nlab * p->n_groups));
-        dfree(ctx->d_accA);
-        dfree(ctx->d_accB);
-        CK(cudaMalloc(&ctx->d_accA, sizeof(double) * ctx->nlab * p->n_groups));
-        CK(cudaMalloc(&ctx->d_accB, sizeof(double) * ctx->nlab * p->n_groups));
-        CK(cudaMalloc(&ctx->d_accW, sizeof(double) * p->n_groups));
-        CK(cudaMalloc(&ctx->d_accE, sizeof(double) * p->n_groups));
-        CK(cudaMalloc(&ctx->d_types, sizeof(unsigned long long) * MRQ_NTYPES));
-        CK(cudaMalloc(&ctx->d_flist, sizeof(int) * (ctx->nlab + (ctx->nlab + FIN_CHUNK - 1) / FIN_CHUNK)));
-        ctx->acc_lab = ctx->nlab;
-        ctx->acc_G = p->n_groups;
-    }
+    ctx->nwalk = 0;                   // (none, should an allocation fail)
+    CK(reserve(ctx->d_walk, ctx->cap_walk, (size_t)p->n_walkers));
+    if (int r = alloc_accumulators(ctx, p->n_groups)) return r;
     ctx->nwalk = p->n_walkers;
     ctx->G = p->n_groups;
     ctx->burn = p->burn_in;
@@ -2127,10 +2134,8 @@ int mrq_walkers_init(mrq_ctx* ctx, const mrq_sample_params* p) {
     double c0 = 1.0;
     CK(cudaMemcpyAsync(&c0, ctx->d_c, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     if (int r_ = sync_stream(ctx)) return r_;
-    if (!ctx->d_wptr) {
-        CK(cudaMalloc(&ctx->d_wptr, sizeof(Walker*)));
-        CK(cudaMalloc(&ctx->d_woff, 2 * sizeof(long long)));
-    }
+    if (!ctx->d_wptr) CK(cudaMalloc(&ctx->d_wptr, sizeof(Walker*)));
+    if (!ctx->d_woff) CK(cudaMalloc(&ctx->d_woff, 2 * sizeof(long long)));
     {
         ctx->h_wset_ptr = ctx->d_walk;
         ctx->h_wset_off[0] = 0;
@@ -2213,11 +2218,7 @@ int mrq_finalize(mrq_ctx* ctx, mrq_result* out) {
     CK(cudaSetDevice(ctx->device));
     int nchunk = 0;
     const long long need = fin_scratch_doubles(ctx, &nchunk);
-    if (need > ctx->partial_cap) {
-        dfree(ctx->d_partial);
-        CK(cudaMalloc(&ctx->d_partial, sizeof(double) * need));
-        ctx->partial_cap = need;
-    }
+    CK(reserve(ctx->d_partial, ctx->cap_partial, (size_t)need));
     return finalize_with(ctx, out, ctx->d_partial, nchunk);
 }
 
@@ -2267,10 +2268,9 @@ int mrq_amsgrad_step(mrq_ctx* ctx, double lr, double beta1, double beta2, double
     if (!(lr > 0.0) || !(beta1 >= 0.0 && beta1 < 1.0) || !(beta2 >= 0.0 && beta2 < 1.0) || !(eps > 0.0))
         return fail(ctx, MRQ_INVALID_ARG, "need lr > 0, 0 <= beta < 1, eps > 0");
     CK(cudaSetDevice(ctx->device));
-    if (!ctx->d_am_m) {
-        CK(cudaMalloc(&ctx->d_am_m, sizeof(double) * ctx->nlab));
-        CK(cudaMalloc(&ctx->d_am_v, sizeof(double) * ctx->nlab));
-        CK(cudaMalloc(&ctx->d_am_vh, sizeof(double) * ctx->nlab));
+    if (!ctx->d_am_m || !ctx->d_am_v || !ctx->d_am_vh) {     // (the last one is missing where a call ran out of memory)
+        for (double** p : {&ctx->d_am_m, &ctx->d_am_v, &ctx->d_am_vh})
+            if (!*p) CK(cudaMalloc(p, sizeof(double) * ctx->nlab));
         CK(cudaMemsetAsync(ctx->d_am_m, 0, sizeof(double) * ctx->nlab, ctx->stream));
         CK(cudaMemsetAsync(ctx->d_am_v, 0, sizeof(double) * ctx->nlab, ctx->stream));
         CK(cudaMemsetAsync(ctx->d_am_vh, 0, sizeof(double) * ctx->nlab, ctx->stream));
@@ -2314,15 +2314,9 @@ static int batch_check(mrq_ctx* const* ctxs, int n) {
 static int batch_tables(mrq_ctx* const* ctxs, int n, int W, Walker* const* walkers, WalkSet& ws, WalkNeed& need, int nw,
                         int nw_eff) {
     mrq_ctx* ctx = ctxs[0];
-    if (n > ctx->bcap) {
-        dfree(ctx->d_bsys);
-        dfree(ctx->d_bwptr);
-        dfree(ctx->d_boff);
-        CK(cudaMalloc(&ctx->d_bsys, sizeof(SysDev) * n));
-        CK(cudaMalloc(&ctx->d_bwptr, sizeof(Walker*) * n));
-        CK(cudaMalloc(&ctx->d_boff, sizeof(long long) * (n + 1)));
-        ctx->bcap = n;
-    }
+    CK(reserve(ctx->d_bsys, ctx->cap_bsys, (size_t)n));
+    CK(reserve(ctx->d_bwptr, ctx->cap_bwptr, (size_t)n));
+    CK(reserve(ctx->d_boff, ctx->cap_boff, (size_t)n + 1));
     std::vector<SysDev> sys;
     std::vector<Walker*> wp;
     std::vector<long long> off(1, 0);
@@ -2465,11 +2459,7 @@ int mrq_tune_batch(mrq_ctx* const* ctxs, int n, int64_t trial_steps, mrq_tune_re
     // scratch copies of every system's walkers: the trials move those, never the real ones
     long long tot = 0;
     for (int i = 0; i < n; i++) tot += ctxs[i]->nwalk;
-    if (tot > ctx->tune_cap) {
-        dfree(ctx->d_tune);
-        CK(cudaMalloc(&ctx->d_tune, sizeof(Walker) * tot));
-        ctx->tune_cap = tot;
-    }
+    CK(reserve(ctx->d_tune, ctx->cap_tune, (size_t)tot));
     std::vector<Walker*> scratch(n);
     {
         long long o = 0;
@@ -2601,26 +2591,7 @@ int mrq_load_accumulators(mrq_ctx* ctx, int32_t n_groups, const double* accN, co
     CK(cudaSetDevice(ctx->device));
     if (int r = sync_stream(ctx)) return r;
     DeadlinePause pause_(ctx);
-    if (ctx->acc_lab != ctx->nlab || ctx->acc_G != n_groups) {
-        dfree(ctx->d_accN);
-        dfree(ctx->d_accU);
-        dfree(ctx->d_accA);
-        dfree(ctx->d_accB);
-        dfree(ctx->d_accW);
-        dfree(ctx->d_accE);
-        dfree(ctx->d_types);
-        dfree(ctx->d_flist);
-        CK(cudaMalloc(&ctx->d_accN, sizeof(double) * ctx->nlab * n_groups));
-        CK(cudaMalloc(&ctx->d_accU, sizeof(double) * ctx->nlab * n_groups));
-        CK(cudaMalloc(&ctx->d_accA, sizeof(double) * ctx->nlab * n_groups));
-        CK(cudaMalloc(&ctx->d_accB, sizeof(double) * ctx->nlab * n_groups));
-        CK(cudaMalloc(&ctx->d_accW, sizeof(double) * n_groups));
-        CK(cudaMalloc(&ctx->d_accE, sizeof(double) * n_groups));
-        CK(cudaMalloc(&ctx->d_types, sizeof(unsigned long long) * MRQ_NTYPES));
-        CK(cudaMalloc(&ctx->d_flist, sizeof(int) * (ctx->nlab + (ctx->nlab + FIN_CHUNK - 1) / FIN_CHUNK)));
-        ctx->acc_lab = ctx->nlab;
-        ctx->acc_G = n_groups;
-    }
+    if (int r = alloc_accumulators(ctx, n_groups)) return r;
     const long long L = ctx->nlab * n_groups;
     CK(cudaMemcpyAsync(ctx->d_accN, accN, sizeof(double) * L, cudaMemcpyDefault, ctx->stream));
     CK(cudaMemcpyAsync(ctx->d_accU, accU, sizeof(double) * L, cudaMemcpyDefault, ctx->stream));
