@@ -195,8 +195,11 @@ int mrq_walkers_init(mrq_ctx* ctx, const mrq_sample_params* p);
  * accumulating the estimators of Eq. 4, 12 and 16 after each walker's burn-in.  Asynchronous
  * on the context stream (two more streams of the context are forked from it and joined to it).  The
  * first advance allocates the walk's workspace - per distinct determinant of a step, the overlaps of
- * its neighbours: at most about 12 GiB, less for small systems or few walkers or where the device has
- * less - which the context keeps until the next mrq_load_hamiltonian or mrq_destroy.
+ * its neighbours - and a later one a larger workspace where a finalized walk has spread over more
+ * determinants: at most about 12 GiB, at most an eighth of the memory that is free then, and less for
+ * small systems or few walkers.  (A least size for 256 walkers and one determinant at a time remains;
+ * MRQ_OOM where that does not fit.)  The context keeps it until the next mrq_load_hamiltonian or
+ * mrq_destroy.
  * Errors: MRQ_NOT_LOADED, MRQ_OOM, MRQ_CUDA_ERROR.
  */
 int mrq_walkers_advance(mrq_ctx* ctx, int64_t n_steps);

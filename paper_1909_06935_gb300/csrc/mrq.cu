@@ -1057,7 +1057,8 @@ struct mrq_ctx {
     int* d_flist = nullptr;                             // visited labels of the finalize, by chunk, and their counts
     long long acc_lab = 0;
     int acc_G = 0;
-    int* d_err = nullptr;
+    int* d_err = nullptr;                        // error flags; most CAS determinants of a step (WalkScratch::seen)
+    int seen = 0;                                // the latter as last read (it sizes the workspace)
     Walker** d_wptr = nullptr;                   // this context's walk set: one walker array
     Walker* h_wset_ptr = nullptr;                // (host staging of the copies above)
     long long h_wset_off[2] = {0, 0};
@@ -1306,11 +1307,12 @@ static int push_sys(mrq_ctx* ctx) {
 }
 
 static int check_err_flag(mrq_ctx* ctx, int* flag_out) {
-    int f = 0;
+    int f[2] = {0, 0};
     if (int r = sync_stream(ctx)) return r;
-    CK(cudaMemcpyAsync(&f, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaMemcpyAsync(f, ctx->d_err, sizeof f, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));    // idle already: returns at once
-    *flag_out = f;
+    *flag_out = f[0];
+    ctx->seen = f[1];
     return 0;
 }
 
@@ -1328,8 +1330,10 @@ struct WalkLaunch {
 struct WalkNeed {
     int cap = 1, gstride = 0, ns = MRQ_FOIS_SLICES, nref = 1, fg_max = 1;
     long long row_worst = 1, fois_nb = 1;
+    long long ncas = 0;              // CAS determinants with walkers, at most: those of the references (psi_s is 0 on others)
     void add(const mrq_ctx* c) {
         const SysDev& s = c->hsys;
+        ncas += c->nref;
         nref = std::max(nref, s.ref_off[8]);
         row_worst = std::max(row_worst, c->row_worst);
         fg_max = std::max(fg_max, c->fg_max);
@@ -1341,112 +1345,183 @@ struct WalkNeed {
 };
 
 // Workspace of a launch over nslots walkers.  A launch takes its walkers in segments, and a segment's
-// CAS determinants in waves, so that the workspace stays below MRQ_WORK_BYTES and MRQ_ROW_BYTES whatever
-// the number of walkers: a segment's arrays hold one entry per walker, a wave's row buffer the worst
-// case that none of its determinants share a row.  When the device cannot give that much, waves shrink.
+// determinants in waves, so that the workspace stays within bounds whatever the number of walkers: a segment's
+// arrays hold one entry per walker, a wave's row buffer the worst case that none of its determinants share a row.
+// Walkers crowd (56 orbitals: 4,096 walkers on 640 CAS determinants), so a wave starts at a third of the walkers, or
+// whatever MRQ_ROW_START holds, and grows in steps of a half to 1.5 times the most CAS determinants that a step of
+// this context has had.  (Steps, since a count that creeps up would make it anew again and again: 2 % of the time of a
+// running 56-orbital walk.  One determinant for every walker: 8 GiB of rows there instead of 4, and no faster.)
+// A workspace takes at most an eighth of the memory that is free when it is made, so that other contexts and
+// libraries find room; where that or a lowered limit is less, waves and segments shrink.
 #define MRQ_WORK_BYTES (1LL << 30)
 #define MRQ_ROW_BYTES (8LL << 30)
-#define MRQ_FROW_BYTES (2LL << 30)     // likewise for the first-order determinants
-static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, long long* seg_out) {
+#define MRQ_ROW_START (2LL << 30)
+#define MRQ_FROW_BYTES (2LL << 30)
+
+// sizes of a workspace and the places of its arrays
+struct WorkPlan {
+    long long seg, groups, fwave, tsz;
+    bool least;                      // the floor: 256 walkers per segment, one determinant per wave
+    size_t rep, cnt, start, tab, pos, mem, tgc, tgf, meta, gops, part, best, bound, ctl, ao, cls, rrep, roff, tbl, ul, kt, kao, kkey,
+        koff, kctl, fgo, fg, rows, frows, nul, bytes;
+};
+
+static WorkPlan work_layout(const WalkNeed& need, long long seg, long long groups, long long fwave) {
+    WorkPlan p{};
+    p.seg = seg;
+    p.groups = groups;
+    p.fwave = fwave;
+    p.tsz = 2;
+    while (p.tsz < 2 * groups * need.nref) p.tsz <<= 1;      // (as many known rows as references of a wave)
+    auto take = [&](size_t bytes) {
+        const size_t at = p.bytes;
+        p.bytes += (bytes + 255) / 256 * 256;
+        return at;
+    };
+    const size_t nr = (size_t)groups * need.nref;
+    p.nul = nr + (size_t)(need.row_worst * groups / MRQ_BIG_ROW) + 1;
+    p.rep = take(16 * seg);
+    p.cnt = take(16 * seg);
+    p.start = take(16 * seg);
+    p.tab = take(4 * seg);
+    p.pos = take(4 * seg);
+    p.mem = take(4 * seg);
+    p.tgc = take(sizeof(TaskGroup) * seg);
+    p.tgf = take(sizeof(TaskGroup) * seg);
+    p.meta = take(sizeof(GroupMeta) * seg);
+    p.gops = take(8 * (size_t)need.gstride * seg);
+    p.part = take(24 * (size_t)(need.ns + MRQ_ACT_SLICES) * seg);
+    p.best = take(sizeof(RaceBest) * seg);
+    p.bound = take(4 * seg);
+    p.ctl = take(4 * CTL_N);
+    p.ao = take(8 * nr);
+    p.cls = take(nr);
+    p.rrep = take(4 * nr);
+    p.roff = take(8 * nr);
+    p.tbl = take(4 * p.tsz);
+    p.ul = take(sizeof(int2) * p.nul);
+    p.kt = take(8 * p.tsz);
+    p.kao = take(8 * nr);
+    p.kkey = take(4 * nr);
+    p.koff = take(8 * nr);
+    p.kctl = take(4 * KNOWN_N);
+    p.fgo = take(8 * fwave);
+    p.fg = take(sizeof(FGroup) * (size_t)need.fg_max * fwave);
+    p.rows = take(8 * (size_t)need.row_worst * groups);
+    p.frows = take(8 * (size_t)need.fois_nb * fwave);
+    return p;
+}
+
+// the workspace for nslots walkers within `limit` bytes (or the floor); seen: the most CAS determinants of a step
+// so far
+static WorkPlan work_size(long long nslots, const WalkNeed& need, int seen, long long limit) {
     const long long per = 12 * 4 + 3 * 4 + 2 * (long long)sizeof(TaskGroup) + (long long)sizeof(GroupMeta) +
                           8LL * need.gstride + 24LL * (need.ns + MRQ_ACT_SLICES) + (long long)sizeof(RaceBest) + 4;
-    const long long seg = std::min(nslots, std::max(256LL, std::min(1LL << 20, std::min(MRQ_WORK_BYTES, ctx->work_limit / 5) / per)));
-    *seg_out = seg;
     const long long per_group = 8 * need.row_worst + 93LL * need.nref;
-    long long groups = std::max(1LL, std::min(seg, std::min(MRQ_ROW_BYTES, ctx->work_limit / 5 * 3) / per_group));
-    groups = std::min(groups, std::max(1LL, (1LL << 29) / need.nref));           // reference indices and the table: 32 bits
     const long long per_fois = 8 * need.fois_nb + (long long)sizeof(FGroup) * need.fg_max + 8;
-    long long fwave = std::max(1LL, std::min(seg, std::min(MRQ_FROW_BYTES, ctx->work_limit / 5) / per_fois));
-    fwave = std::min(fwave, std::max(1LL, (1LL << 30) / need.fg_max));           // group indices: 32 bits
-    WalkScratch& w = ctx->work;
-    for (;; groups = (groups + 1) / 2, fwave = (fwave + 1) / 2) {
-        long long tsz = 2;
-        while (tsz < 2 * groups * need.nref) tsz <<= 1;      // (as many known rows as references of a wave)
-        size_t off = 0;
-        auto take = [&](size_t bytes) {
-            const size_t at = off;
-            off += (bytes + 255) / 256 * 256;
-            return at;
-        };
-        const size_t nr = (size_t)groups * need.nref, nul = nr + (size_t)(need.row_worst * groups / MRQ_BIG_ROW) + 1;
-        const size_t rep = take(16 * seg), cnt = take(16 * seg), start = take(16 * seg), tab = take(4 * seg),
-                     pos = take(4 * seg), mem = take(4 * seg), tgc = take(sizeof(TaskGroup) * seg),
-                     tgf = take(sizeof(TaskGroup) * seg), meta = take(sizeof(GroupMeta) * seg),
-                     gops = take(8 * (size_t)need.gstride * seg), part = take(24 * (size_t)(need.ns + MRQ_ACT_SLICES) * seg),
-                     best = take(sizeof(RaceBest) * seg), bound = take(4 * seg), ctl = take(4 * CTL_N), ao = take(8 * nr),
-                     cls = take(nr), rrep = take(4 * nr), roff = take(8 * nr), tbl = take(4 * tsz), ul = take(sizeof(int2) * nul),
-                     kt = take(8 * tsz), kao = take(8 * nr), kkey = take(4 * nr), koff = take(8 * nr), kctl = take(4 * KNOWN_N),
-                     fgo = take(8 * fwave), fg = take(sizeof(FGroup) * (size_t)need.fg_max * fwave),
-                     rows = take(8 * (size_t)need.row_worst * groups), frows = take(8 * (size_t)need.fois_nb * fwave);
-        // (a workspace well above a lowered limit is given back)
-        if (off > ctx->work_cap || ((long long)ctx->work_cap > ctx->work_limit && off < ctx->work_cap / 2)) {
-            CK(cudaStreamSynchronize(ctx->stream));
-            free_work(ctx);
-            const cudaError_t e = cudaMalloc(&ctx->d_work, off);
-            if (e == cudaErrorMemoryAllocation && (groups > 1 || fwave > 1)) {
-                cudaGetLastError();
-                ctx->d_work = nullptr;
-                continue;
-            }
-            CK(e);
-            ctx->work_cap = off;
-        }
-        unsigned char* const b = ctx->d_work;
-        w.rep = (int*)(b + rep);
-        w.cnt = (int*)(b + cnt);
-        w.start = (int*)(b + start);
-        w.tab_of = (int*)(b + tab);
-        w.pos_of = (int*)(b + pos);
-        w.members = (int*)(b + mem);
-        w.tgc = (TaskGroup*)(b + tgc);
-        w.tgf = (TaskGroup*)(b + tgf);
-        w.meta = (GroupMeta*)(b + meta);
-        w.gops = (double*)(b + gops);
-        w.part = (double*)(b + part);
-        w.best = (RaceBest*)(b + best);
-        w.bound = (unsigned*)(b + bound);
-        w.ctl = (int*)(b + ctl);
-        w.ref_ao = (unsigned long long*)(b + ao);
-        w.ref_cls = b + cls;
-        w.ref_rep = (int*)(b + rrep);
-        w.row_off = (long long*)(b + roff);
-        w.table = (int*)(b + tbl);
-        w.ulist = (int2*)(b + ul);
-        w.ulist_size = (int)nul;
-        w.rows = (double*)(b + rows);
-        w.frows = (double*)(b + frows);
-        w.table_size = (int)tsz;
-        w.ktab_size = (int)tsz;
-        w.k_ao = (unsigned long long*)(b + kao);
-        w.k_key = (int*)(b + kkey);
-        w.k_off = (long long*)(b + koff);
-        w.kctl = (int*)(b + kctl);
-        // a new layout of the workspace: nothing in it is a table of known rows yet
-        if (w.ktab != (unsigned long long*)(b + kt) || ctx->ktab_bytes != 8 * (size_t)tsz || ctx->kctl_at != w.kctl) {
-            w.ktab = (unsigned long long*)(b + kt);
-            ctx->ktab_bytes = 8 * (size_t)tsz;
-            ctx->kctl_at = w.kctl;
-            CK(cudaMemsetAsync(w.ktab, 0, ctx->ktab_bytes, ctx->stream));
-            CK(cudaMemsetAsync(w.kctl, 0, sizeof(int) * KNOWN_N, ctx->stream));
-        }
-        w.fg_of = (int2*)(b + fgo);
-        w.fg = (FGroup*)(b + fg);
-        break;
+    const long long seg0 = std::min(256LL, nslots);
+    long long seg = std::min(nslots, std::max(seg0, std::min(1LL << 20, std::min(MRQ_WORK_BYTES, limit / 5) / per)));
+    long long groups = std::max({1LL, MRQ_ROW_START / per_group, (seg + 2) / 3});
+    while (2 * groups < 3LL * seen) groups += (groups + 1) / 2;
+    groups = std::min({groups, seg, need.ncas, std::min(MRQ_ROW_BYTES, limit / 5 * 3) / per_group,
+                       (1LL << 29) / need.nref});                                  // (reference indices and the table: 32 bits)
+    long long fwave = std::min(MRQ_FROW_BYTES, limit / 5) / per_fois;
+    fwave = std::min({fwave, seg, (1LL << 30) / need.fg_max});                     // (group indices: 32 bits)
+    groups = std::max(1LL, groups);
+    fwave = std::max(1LL, fwave);
+    for (;;) {
+        WorkPlan p = work_layout(need, seg, groups, fwave);
+        p.least = groups == 1 && fwave == 1 && seg == seg0;
+        if ((long long)p.bytes <= limit || p.least) return p;
+        groups = (groups + 1) / 2;
+        fwave = (fwave + 1) / 2;
+        seg = std::max(seg0, (seg + 1) / 2);
     }
+}
+
+static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need) {
+    const long long limit = ctx->work_limit;
+    WorkPlan p = work_size(nslots, need, ctx->seen, limit);
+    const auto renew = [&]() { return p.bytes > ctx->work_cap || ((long long)ctx->work_cap > limit && p.bytes < ctx->work_cap); };
+    if (renew()) {
+        size_t free_b = 0, total_b = 0;
+        CK(cudaMemGetInfo(&free_b, &total_b));
+        long long room = (long long)((free_b + ctx->work_cap) / 8);
+        if (room < limit) {
+            // (one that is nearly as large stays)
+            if ((long long)ctx->work_cap <= limit && (long long)ctx->work_cap >= room - room / 4) room = (long long)ctx->work_cap;
+            p = work_size(nslots, need, ctx->seen, room);
+        }
+        if (renew()) {
+            if (int r = sync_stream(ctx)) return r;
+            free_work(ctx);
+            for (;;) {
+                const cudaError_t e = cudaMalloc(&ctx->d_work, p.bytes);
+                if (e == cudaSuccess) break;
+                ctx->d_work = nullptr;
+                if (e != cudaErrorMemoryAllocation || p.least) CK(e);
+                cudaGetLastError();
+                p = work_size(nslots, need, ctx->seen, (long long)(p.bytes / 2));
+            }
+            ctx->work_cap = p.bytes;
+        }
+    }
+    unsigned char* const b = ctx->d_work;
+    WalkScratch& w = ctx->work;
+    w.rep = (int*)(b + p.rep);
+    w.cnt = (int*)(b + p.cnt);
+    w.start = (int*)(b + p.start);
+    w.tab_of = (int*)(b + p.tab);
+    w.pos_of = (int*)(b + p.pos);
+    w.members = (int*)(b + p.mem);
+    w.tgc = (TaskGroup*)(b + p.tgc);
+    w.tgf = (TaskGroup*)(b + p.tgf);
+    w.meta = (GroupMeta*)(b + p.meta);
+    w.gops = (double*)(b + p.gops);
+    w.part = (double*)(b + p.part);
+    w.best = (RaceBest*)(b + p.best);
+    w.bound = (unsigned*)(b + p.bound);
+    w.ctl = (int*)(b + p.ctl);
+    w.seen = ctx->d_err + 1;
+    w.ref_ao = (unsigned long long*)(b + p.ao);
+    w.ref_cls = b + p.cls;
+    w.ref_rep = (int*)(b + p.rrep);
+    w.row_off = (long long*)(b + p.roff);
+    w.table = (int*)(b + p.tbl);
+    w.ulist = (int2*)(b + p.ul);
+    w.ulist_size = (int)p.nul;
+    w.rows = (double*)(b + p.rows);
+    w.frows = (double*)(b + p.frows);
+    w.table_size = (int)p.tsz;
+    w.ktab_size = (int)p.tsz;
+    w.k_ao = (unsigned long long*)(b + p.kao);
+    w.k_key = (int*)(b + p.kkey);
+    w.k_off = (long long*)(b + p.koff);
+    w.kctl = (int*)(b + p.kctl);
+    // a new layout of the workspace: nothing in it is a table of known rows yet
+    if (w.ktab != (unsigned long long*)(b + p.kt) || ctx->ktab_bytes != 8 * (size_t)p.tsz || ctx->kctl_at != w.kctl) {
+        w.ktab = (unsigned long long*)(b + p.kt);
+        ctx->ktab_bytes = 8 * (size_t)p.tsz;
+        ctx->kctl_at = w.kctl;
+        CK(cudaMemsetAsync(w.ktab, 0, ctx->ktab_bytes, ctx->stream));
+        CK(cudaMemsetAsync(w.kctl, 0, sizeof(int) * KNOWN_N, ctx->stream));
+    }
+    w.fg_of = (int2*)(b + p.fgo);
+    w.fg = (FGroup*)(b + p.fg);
     w.nref_max = need.nref;
     w.row_worst = need.row_worst;
-    w.wave_groups = (int)groups;
+    w.wave_groups = (int)p.groups;
     w.wave0 = 0;
     w.fg_max = need.fg_max;
-    w.fwave = (int)fwave;
+    w.fwave = (int)p.fwave;
     w.fwave0 = 0;
     w.gstride = need.gstride;
     w.ns_max = need.ns;
-    w.nseg = seg;
+    w.nseg = p.seg;
     // walkers per task group: 32 when there are many, fewer for small launches, so that the walkers of
     // a crowded determinant spread over more warps (against the determinant's neighbours being formed once
     // per group)
-    w.tgw = (int)std::max(4LL, std::min<long long>(seg <= 2048 ? 16 : MRQ_TGW, seg <= 2048 ? seg / 64 : seg / 128));
+    w.tgw = (int)std::max(4LL, std::min<long long>(p.seg <= 2048 ? 16 : MRQ_TGW, p.seg <= 2048 ? p.seg / 64 : p.seg / 128));
     return 0;
 }
 
@@ -1519,7 +1594,7 @@ static int launch_segment(mrq_ctx* ctx, const WalkSet& ws, WalkScratch sc, const
     }
     CK(cudaEventRecord(ctx->ev_join[1], st3));
     // main stream: the CAS determinants' rows and pairs
-    for (long long g = 0; g < n; g += sc.wave_groups) {
+    for (long long g = 0; g < std::min(n, need.ncas); g += sc.wave_groups) {
         sc.wave0 = (int)g;
         k_wave_begin<<<1, 1, 0, st>>>(sc);
         k_refs<W><<<(unsigned)std::min<long long>(n, 8LL * sms), 256, 0, st>>>(ws, sc);
@@ -1547,10 +1622,11 @@ static int launch_segment(mrq_ctx* ctx, const WalkSet& ws, WalkScratch sc, const
 static int launch_walk(mrq_ctx* ctx, int W, const WalkSet& ws, int nsteps, const WalkNeed& need,
                        const WalkLaunch& L = WalkLaunch()) {
     const int nw = std::min(L.wpb, MRQ_MAXNW);
-    long long seg = 0;
-    if (int r = work_prepare(ctx, ws.nslots, need, &seg)) return r;
-    if (!L.captured)
+    if (!L.captured) {
+        if (int r = work_prepare(ctx, ws.nslots, need)) return r;
         if (int r = rows_prepare(ctx, W, nw, need.cap)) return r;
+    }
+    const long long seg = ctx->work.nseg;
     cudaLaunchConfig_t cfg = {};
     cfg.stream = ctx->stream;
     cudaLaunchAttribute attr[1];
@@ -1739,7 +1815,7 @@ int mrq_create(mrq_ctx** out, int device) {
         return MRQ_CUDA_ERROR;
     }
     if (cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaMalloc(&ctx->d_err, sizeof(int)) != cudaSuccess || cudaMalloc(&ctx->d_sys, sizeof(SysDev)) != cudaSuccess ||
+        cudaMalloc(&ctx->d_err, 2 * sizeof(int)) != cudaSuccess || cudaMalloc(&ctx->d_sys, sizeof(SysDev)) != cudaSuccess ||
         cudaMalloc(&ctx->d_res, sizeof(mrq_result)) != cudaSuccess || cudaEventCreate(&ctx->ev0) != cudaSuccess ||
         cudaEventCreate(&ctx->ev1) != cudaSuccess ||
         cudaStreamCreateWithFlags(&ctx->side[0], cudaStreamNonBlocking) != cudaSuccess ||
@@ -1753,7 +1829,7 @@ int mrq_create(mrq_ctx** out, int device) {
         return MRQ_CUDA_ERROR;
     }
     ctx->own_stream = true;
-    cudaMemset(ctx->d_err, 0, sizeof(int));
+    cudaMemset(ctx->d_err, 0, 2 * sizeof(int));
     if (cudaDeviceGetAttribute(&ctx->n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
         mrq_destroy(ctx);
         return MRQ_CUDA_ERROR;
@@ -1831,6 +1907,8 @@ int mrq_load_hamiltonian(mrq_ctx* ctx, int n_core, int n_act, int n_virt, int n_
     DeadlinePause pause_(ctx);
     free_walkers(ctx);
     free_work(ctx);                   // the walk workspace of the last system is given back
+    CK(cudaMemsetAsync(ctx->d_err, 0, 2 * sizeof(int), ctx->stream));
+    ctx->seen = 0;
     ctx->ref = ctx->ham = false;
     ctx->n = n;
     ctx->nc = n_core;
@@ -2364,8 +2442,7 @@ static int batch_run(mrq_ctx* ctx, int W, const WalkSet& ws, const WalkNeed& nee
     if (spl <= 0 || spl > n_steps) spl = n_steps;
     const int64_t nfull = n_steps / spl, rem = n_steps % spl;
     if (graph && nfull > 0) {
-        long long seg = 0;
-        if (int r = work_prepare(ctx, ws.nslots, need, &seg)) return r;
+        if (int r = work_prepare(ctx, ws.nslots, need)) return r;
         if (int r = rows_prepare(ctx, W, std::min(wpb, MRQ_MAXNW), need.cap)) return r;
         mrq_ctx::GraphKey key;
         graph_key(ctx, ws, need, wpb, (int)spl, key);

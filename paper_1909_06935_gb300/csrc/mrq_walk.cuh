@@ -122,6 +122,7 @@ struct WalkScratch {
     RaceBest* best;           // per slot
     unsigned* bound;          // per slot: FP32 bits of an upper bound of the best clock
     int* ctl;
+    int* seen;                // most CAS determinants of a step so far
     // rows of a wave of at most wave_groups CAS determinants; a reference is (determinant of the wave,
     // row number in it), index determinant * nref_max + row number
     unsigned long long* ref_ao;   // the row's active remnant
@@ -1927,6 +1928,7 @@ __global__ void k_rows_begin(const WalkScratch sc) {
     *reinterpret_cast<unsigned long long*>(sc.kctl + KNOWN_CUR) = 0ull;
 }
 __global__ void k_wave_begin(const WalkScratch sc) {
+    if (sc.wave0 == 0) *sc.seen = max(*sc.seen, sc.ctl[CTL_GC]);
     const long long ng = min(sc.wave_groups, sc.ctl[CTL_GC] - sc.wave0);
     if (ng <= 0) return;
     sc.ctl[CTL_PAIRS] = sc.ctl[CTL_ROWTASK] = sc.ctl[CTL_BIG] = sc.ctl[CTL_SMALL] = 0;
