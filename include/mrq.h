@@ -291,8 +291,10 @@ enum mrq_request_state { MRQ_REQ_QUEUED = 0, MRQ_REQ_RUNNING = 1, MRQ_REQ_DONE =
 typedef struct {
     int32_t device;
     int32_t max_active;          /* requests resident at once */
-    int64_t hbm_budget_bytes;    /* device bytes the resident requests may use (estimated per request); the
-                                    batch's walk workspace takes at most what they leave of it */
+    int64_t hbm_budget_bytes;    /* device bytes the resident requests and the batch's walk workspace may use: the
+                                    former are estimated, the latter takes what they leave, and room for its
+                                    least size is kept at every admission (but a request that fits alone without
+                                    it is run alone) */
     int64_t steps_per_round;     /* walker steps per batched launch */
 } mrq_server_params;
 
@@ -334,7 +336,8 @@ int mrq_server_step(mrq_server* s);
 /* Start / stop a background thread that runs rounds while there is work. */
 int mrq_server_start(mrq_server* s);
 int mrq_server_stop(mrq_server* s);
-/* out4 = queued, active, estimated resident bytes, walker steps advanced so far. */
+/* out4 = queued, active, estimated resident bytes (with the least workspace of each request), walker steps
+ * advanced so far. */
 int mrq_server_info(mrq_server* s, int64_t* out4);
 const char* mrq_server_last_error(const mrq_server* s);
 /* Stop, free every resident request, destroy. */

@@ -1433,9 +1433,9 @@ static WorkPlan work_size(long long nslots, const WalkNeed& need, int seen, long
         WorkPlan p = work_layout(need, seg, groups, fwave);
         p.least = groups == 1 && fwave == 1 && seg == seg0;
         if ((long long)p.bytes <= limit || p.least) return p;
-        groups = (groups + 1) / 2;
-        fwave = (fwave + 1) / 2;
-        seg = std::max(seg0, (seg + 1) / 2);
+        groups = std::max(1LL, groups * 7 / 8);
+        fwave = std::max(1LL, fwave * 7 / 8);
+        seg = std::max(seg0, seg * 7 / 8);
     }
 }
 
@@ -2866,7 +2866,36 @@ int mrq_internal_fail(mrq_ctx* ctx, int code, const char* fmt, ...) {
     return code;
 }
 
-void mrq_internal_work_limit(mrq_ctx* ctx, long long bytes) { ctx->work_limit = std::max(0LL, bytes); }
+int mrq_internal_work_limit(mrq_ctx* ctx, long long bytes) {
+    ctx->work_limit = std::max(0LL, bytes);
+    if ((long long)ctx->work_cap <= ctx->work_limit) return 0;
+    CK(cudaSetDevice(ctx->device));
+    if (int r = sync_stream(ctx)) return r;
+    free_work(ctx);
+    return 0;
+}
+
+long long mrq_internal_work_floor(int n_core, int n_act, int n_virt, int n_alpha, int n_beta, long long n_ref) {
+    const int n = n_core + n_act + n_virt;
+    if (n_core < 0 || n_act < 0 || n_virt < 0 || n <= 0 || n > MRQ_MAXN || n_core > 64 || n_act > 32 || n_alpha < n_core ||
+        n_beta < n_core || n_alpha > n_core + n_act || n_beta > n_core + n_act)
+        return 0;
+    mrq_ctx c;                        // (host side only)
+    SysDev& s = c.hsys;
+    s.n = n;
+    s.nc = n_core;
+    s.na = n_act;
+    s.nv = n_virt;
+    s.nalpha = n_alpha;
+    s.nbeta = n_beta;
+    s.nca = n_core + n_act;
+    s.nav = n_act + n_virt;
+    if (walk_plan(&c, s)) return 0;
+    c.nref = n_ref;
+    WalkNeed need;
+    need.add(&c);
+    return (long long)work_size(256, need, 0, 0).bytes;
+}
 
 int mrq_internal_sync(mrq_ctx* ctx) { return sync_stream(ctx); }
 

@@ -22,9 +22,11 @@ struct MrqHamView {
 int mrq_internal_ham(mrq_ctx* ctx, MrqHamView* out);
 // record a message in the context's error slot and return code
 int mrq_internal_fail(mrq_ctx* ctx, int code, const char* fmt, ...);
-// Bytes the context's walk workspace may take (the launch works in smaller segments and waves within
-// them; a floor of 256 walkers and one determinant per wave remains)
-void mrq_internal_work_limit(mrq_ctx* ctx, long long bytes);
+// Bytes the context's walk workspace may take from now on (a launch works in smaller segments and waves within
+// them; a floor of 256 walkers and one determinant per wave remains).  A workspace above that is given back.
+int mrq_internal_work_limit(mrq_ctx* ctx, long long bytes);
+// Bytes of the floor for a system (0 where its sizes are out of range); that of a batch is below the sum over its systems
+long long mrq_internal_work_floor(int n_core, int n_act, int n_virt, int n_alpha, int n_beta, long long n_ref);
 // the context's host-wait (deadline-aware) synchronisation
 int mrq_internal_sync(mrq_ctx* ctx);
 

@@ -44,7 +44,8 @@ struct Request {
     int state = MRQ_REQ_QUEUED;
     int status = 0;
     int64_t steps_done = 0;
-    int64_t footprint = 0;
+    int64_t footprint = 0;        // resident device bytes
+    int64_t floor = 0;            // least walk workspace it can run in
     mrq_ctx* ctx = nullptr;
     mrq_result result{};
     clk::time_point t_submit, t_admit, t_done;
@@ -52,8 +53,8 @@ struct Request {
 
 int64_t nsub2(int64_t k) { return k * (k - 1) / 2; }
 
-// device bytes a request keeps resident while active (integral tables, hash, coefficients,
-// accumulators, walkers, candidate scratch) - an estimate used for admission
+// device bytes a request keeps resident while active (integral tables, hash, reference, coefficients,
+// accumulators, walkers; the walk's workspace is the batch's) - an estimate used for admission
 int64_t footprint_of(const Request& r) {
     const int64_t n = r.n_core + r.n_act + r.n_virt;
     const int64_t npair = n * (n + 1) / 2;
@@ -66,13 +67,13 @@ int64_t footprint_of(const Request& r) {
     int64_t b = 0;
     const int64_t nca = r.n_core + r.n_act, nav = r.n_act + r.n_virt;
     b += 8 * (2 * n * n + neri + npair * n * n + 2 * nca * nca * nav * nav + n + r.n_act * r.n_act);
+    b += 16 * r.n_act * nca * nav;      // terms of the single-excitation operator
     b += 16 * cap + 8 * nlab;
+    b += 8 * (int64_t)r.dets.size() + 16 * (int64_t)r.coeffs.size() + 128 * r.n_act * r.n_act;   // set-up buffers, kept
     b += 32 * G * nlab + 16 * G;        // N, U and the SC-MRCI gradient sums A, B per group
-    b += 112 * r.params.n_walkers;     // walkers with their step records
-    int64_t npad = 1;
-    while (npad < r.params.n_walkers) npad <<= 1;
-    b += 12 * npad;                     // slot ordering keys and indices
-    b += 8 * (G + 1) * ((nlab + 8191) / 8192) * 45;   // finalize partial sums
+    b += 96 * r.params.n_walkers;       // walkers with their step records
+    const int64_t chunks = (nlab + 8191) / 8192;
+    b += 4 * (nlab + chunks) + 8 * (G + 1) * chunks * 45;   // finalize: visited labels, partial sums
     return b;
 }
 
@@ -86,7 +87,8 @@ struct mrq_server {
     std::vector<Request*> active;
     std::map<int64_t, Request*> all;
     int64_t next_ticket = 1;
-    int64_t used_bytes = 0;
+    int64_t used_bytes = 0;       // footprints and workspace floors of the resident requests
+    int64_t floor_bytes = 0;      // the floors among them
     std::thread worker;
     std::atomic<bool> stop{false};
     bool running = false;
@@ -94,11 +96,16 @@ struct mrq_server {
     int64_t rounds = 0, total_walker_steps = 0;
 };
 
+static void release_bytes(mrq_server* s, const Request* r) {
+    s->used_bytes -= r->footprint + r->floor;
+    s->floor_bytes -= r->floor;
+}
+
 static void retire_locked(mrq_server* s, Request* r, int state) {
     if (r->ctx) {
         mrq_destroy(r->ctx);
         r->ctx = nullptr;
-        s->used_bytes -= r->footprint;
+        release_bytes(s, r);
     }
     r->state = state;
     r->t_done = clk::now();
@@ -137,8 +144,32 @@ static int admit(mrq_server* s, Request* r) {
     return 0;
 }
 
+// requests cancelled while they ran leave, and give their memory back (the first one's holds the walk's workspace)
+static void drop_cancelled_locked(mrq_server* s) {
+    std::vector<Request*> keep;
+    for (Request* r : s->active) {
+        if (r->state == MRQ_REQ_CANCELLED) retire_locked(s, r, MRQ_REQ_CANCELLED);
+        else keep.push_back(r);
+    }
+    s->active.swap(keep);
+}
+
+// The walk's workspace is the first active request's context's; it takes what the footprints leave of the budget.
+// The floors are reserved for it: each is enough for any walkers of its request, and the batch's least workspace
+// is below their sum.
+static void limit_workspace_locked(mrq_server* s) {
+    if (s->active.empty()) return;
+    const int64_t rest = s->p.hbm_budget_bytes - (s->used_bytes - s->floor_bytes);
+    mrq_internal_work_limit(s->active[0]->ctx, std::max(rest, s->floor_bytes));
+}
+
 static int server_round(mrq_server* s) {
-    // 1. admission (FIFO; stop at the first request that does not fit)
+    // 1. admission (FIFO; stop at the first request that does not fit).  The workspace shrinks before a request
+    //    is loaded, so that the two never exceed the budget together.
+    {
+        std::lock_guard<std::mutex> g(s->mu);
+        drop_cancelled_locked(s);
+    }
     for (;;) {
         Request* r = nullptr;
         {
@@ -149,16 +180,18 @@ static int server_round(mrq_server* s) {
                 s->queue.pop_front();
                 continue;
             }
-            if (s->used_bytes + head->footprint > s->p.hbm_budget_bytes && !s->active.empty()) break;
+            if (s->used_bytes + head->footprint + head->floor > s->p.hbm_budget_bytes && !s->active.empty()) break;
             s->queue.pop_front();
             r = head;
-            s->used_bytes += r->footprint;
+            s->used_bytes += r->footprint + r->floor;
+            s->floor_bytes += r->floor;
+            limit_workspace_locked(s);
         }
         const int rc = admit(s, r);
         std::lock_guard<std::mutex> g(s->mu);
         if (rc) {
             r->status = rc;
-            s->used_bytes -= r->footprint;
+            release_bytes(s, r);
             retire_locked(s, r, MRQ_REQ_FAILED);
         } else {
             r->state = MRQ_REQ_RUNNING;
@@ -170,17 +203,14 @@ static int server_round(mrq_server* s) {
     std::vector<Request*> act;
     {
         std::lock_guard<std::mutex> g(s->mu);
-        for (Request* r : s->active)
-            if (r->state == MRQ_REQ_RUNNING) act.push_back(r);
+        drop_cancelled_locked(s);
+        act = s->active;
+        limit_workspace_locked(s);
     }
     if (act.empty()) return 0;
     std::vector<mrq_ctx*> ctxs;
     for (Request* r : act) ctxs.push_back(r->ctx);
     const int64_t steps = s->p.steps_per_round;
-    {
-        std::lock_guard<std::mutex> g(s->mu);        // the workspace is the first context's; it takes what is left
-        mrq_internal_work_limit(ctxs[0], s->p.hbm_budget_bytes - s->used_bytes);
-    }
     int rc = mrq_batch_advance(ctxs.data(), (int)ctxs.size(), steps);
     if (rc) snprintf(s->err, sizeof s->err, "batched advance failed: %s", mrq_last_error(ctxs[0]));
     // 3. finalize with the lock released (only this thread uses an active request's context, and
@@ -258,6 +288,7 @@ int mrq_server_submit(mrq_server* s, const mrq_request* q, int64_t* ticket) {
     r->target_sigma = q->target_sigma;
     r->max_steps = q->max_steps;
     r->footprint = footprint_of(*r);
+    r->floor = mrq_internal_work_floor(r->n_core, r->n_act, r->n_virt, r->n_alpha, r->n_beta, (int64_t)r->coeffs.size());
     r->t_submit = clk::now();
     std::lock_guard<std::mutex> g(s->mu);
     if (r->footprint > s->p.hbm_budget_bytes) {
