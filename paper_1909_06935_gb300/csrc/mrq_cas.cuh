@@ -1,17 +1,13 @@
-// Local evaluation at a CAS walker, organised by active remnant (included by mrq.cu).
+// Reach-back by active remnant: candidate lists, the physicists' tables and single elements (included by mrq.cu).
 //
-// Every neighbour m of a CAS determinant n is n with active electrons X_a -> active holes Y_a
-// and core electrons X_c -> virtual orbitals Y_v (|X_a|+|X_c| = |Y_a|+|Y_v| <= 2).  Its reach-back
-// candidates k (Eq. 6-7: the reference determinants H-connected to m) are
+// Every neighbour m of a determinant has an active remnant A_m, c core holes and v virtual electrons (at most two
+// each).  Its reach-back candidates k (Eq. 6-7: the reference determinants H-connected to m) are
 //     k = m - (Y_v u R') + (X_c u A'),   R' active electrons of m, A' active holes of m,
-// and which (R', A') occur, and phi0(k), depend only on the active remnant A_m = A_n - X_a + Y_a and
-// on the counts and spins of X_c and Y_v - not on which core / virtual orbitals they are.  So the
-// neighbours are processed in groups (X_a, Y_a, spins of X_c and Y_v): the warp builds the group's
-// candidate list once (lanes probe distinct keys in parallel, compacted into shared memory), then
-// the lanes run over the group's core / virtual orbital choices and evaluate
-//     O(m) = H_nm phi0(n) + sum_{k in list} <m|H|k> phi0(k)
-// in lockstep; the k = n term needs no lookup.  Every neighbour and every candidate of the plain
-// enumeration is visited exactly once, so the sums are the same as in local_eval.
+// and which (R', A') occur, and phi0(k), depend only on A_m and on the numbers and spins of m's core holes X_c and
+// virtual electrons Y_v - not on which orbitals they are.  So one candidate list serves every m of a class
+// (A_m, c, v, spins): the walk builds it once per row (k_rows) or group of first-order neighbours (k_frows) and
+// runs over the orbitals; the debug evaluation builds it per (X_a, Y_a) pair of one determinant n = m + X - Y.
+// Every candidate of the plain enumeration is visited exactly once.
 
 __device__ __forceinline__ int nsub(int cnt, int size) {
     return size == 0 ? 1 : (size == 1 ? cnt : cnt * (cnt - 1) / 2);
@@ -197,13 +193,13 @@ __device__ __forceinline__ void lane_offsets(const SysDev& S, int c, int v, int 
     par = (c >= 1 ? (int)p0 : 0) + (c == 2 ? (int)p1 : 0);
 }
 
-// The walker's single-excitation operator, for every hole y (core or active) and electron x (active
-// or virtual) of one spin s:  G^s_yx(n) = hc_yx + sum_{j in act occ(n)} (yx|jj) - sum_{j in act occ_s(n)} (yj|jx)
-// (n a CAS determinant: full core, empty virtuals), tabulated per walker step by the walk block
-// (2 x nca x nav doubles, [s][y][x - nc]; the active-active block is not needed).  Slater-Condon
-// gives, for a neighbour m = n - R + A and its single x -> y,  <k|H|m> = sign (G^s_yx(n) +
-// sum_{j in A} f(j) - sum_{j in R} f(j)), f(j) = (yx|jj) - d_{s_j s} (yj|jx): the same sum as
-// single_elem over occ(m), with <= 4 corrections in place of one term per occupied orbital.
+// A determinant's single-excitation operator, for every hole y (core or active) and electron x (active or virtual)
+// of one spin s:  G^s_yx(n) = hc_yx + sum_{j in act occ(n)} (yx|jj) - sum_{j in act occ_s(n)} (yj|jx)
+// (n a CAS determinant: full core, empty virtuals; first-order ones add their virtual electrons' terms and take
+// their core holes' out), made once per determinant (k_prep; 2 x nca x nav doubles, [s][y][x - nc]; the
+// active-active block is not needed).  Slater-Condon gives, for a neighbour m = n - R + A and its single x -> y,
+// <k|H|m> = sign (G^s_yx(n) + sum_{j in A} f(j) - sum_{j in R} f(j)), f(j) = (yx|jj) - d_{s_j s} (yj|jx): the
+// same sum as single_elem over occ(m), with <= 4 corrections in place of one term per occupied orbital.
 
 // f(j) of one orbital j (spin orbital) for the single x -> y of spin sx (spatial px, py)
 __device__ __forceinline__ double single_corr(const SysDev& S, int sx, int px, int py, int j) {

@@ -385,7 +385,7 @@ __device__ double hd_single_elem(const SysDev& S, const unsigned long long (&d)[
 // needs no lookup: its term is H_nm phi0(n), both already known (pass self_key = ~0 otherwise).
 // Single elements from a walker's operator: <k|H|m> for the single x -> y of m (x in active +
 // virtual, y in core + active, not both active) is G_yx(m) = h_yx + sum_{j in m} [(yx|jj) - delta
-// (yj|jx)], taken as the walker n's G_yx(n) (g, in shared memory) plus the terms of the <= 4 spin
+// (yj|jx)], taken as the walker n's G_yx(n) (g, made by k_prep) plus the terms of the <= 4 spin
 // orbitals in which m differs from n (removed rm*, added ad*; r of each), with m's sign.
 struct SglFromWalker {
     const double* g;        // nullptr: full Slater-Condon sums

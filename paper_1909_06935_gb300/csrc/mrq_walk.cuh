@@ -2582,7 +2582,9 @@ __host__ __device__ __forceinline__ size_t rows_warp_bytes(int cap) {
     return (sizeof(SysDev) + 15) / 16 * 16 + cand_list_bytes(cap);
 }
 
-// local quantities of arbitrary determinants: one block per determinant, the walk's unit code
+// Local quantities of arbitrary determinants: one block per determinant, every neighbour with the lists of its own
+// group or lane (cas_pair_unit, fois_unit).  The walk shares rows and groups between determinants instead; the two
+// meet in the tests, which hold the walk's per-walker sums against this evaluation and both against the oracle.
 template <int W>
 __global__ void __launch_bounds__(MRQ_MAXNW * 32, 2) k_debug2(const SysDev* __restrict__ sys,
                                                               const unsigned long long* __restrict__ dets, long long ndet,
