@@ -30,7 +30,10 @@ sys.path.insert(0, ROOT)
 
 WORKLOAD = "cas10_56o"
 METRIC = "walker-steps/s"
-# FP64 FMA pipe of GB300: 2 FMA per clock per SM, 152 SMs, 2.07 GHz maximum SM clock
+# The race draws one Philox clock per neighbour and walker: about 22 logic operations, on 64 lanes per clock and SM
+# (152 SMs, 2.07 GHz maximum SM clock)
+RACE_PEAK = 152 * 64 / 22 * 2.07e9
+# FP64 FMA pipe of GB300: 2 FMA per clock per SM
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 
 
@@ -256,6 +259,28 @@ def run_reference(args):
 
 # ----------------------------------------------------------------------------- our arm
 
+def roofline(neighbours: float, walker_steps: float, seconds: float, distinct: float, terms: float, neighbours_once: float,
+             steps_per_launch: int = 1) -> dict:
+    """Roofline object of one walk launch of `walker_steps` walker steps in `seconds`.
+
+    The rate is that of work that is really done: the race draws a clock per neighbour and walker (`neighbours` per
+    walker step), against the integer pipes' rate.  Overlaps are shared between determinants through their rows, so
+    the FP64 work of evaluating each of the `distinct` determinants of a step by itself (`terms` reach-back products, 2
+    flops each, and 8 flops per neighbour) is reported as the algorithm's work without sharing, and is no rate of the
+    FP64 pipe."""
+    draws = neighbours * walker_steps / seconds
+    return {"bound": "alu", "achieved": draws / 1e12, "peak": RACE_PEAK / 1e12, "unit": "1e12 race draws/s",
+            "frac": draws / RACE_PEAK, "traffic": None,
+            "kernel": "k_pairs, k_int, k_fois, k_fois_act: the move race, over the time of the whole step",
+            "peak_source": "152 SMs x 64 lanes/clk x 2.07 GHz / 22 logic operations a draw (derived from unit counts and "
+                           "the maximum SM clock)",
+            "neighbours_per_walker_step": neighbours, "distinct_determinants": distinct, "launch_seconds": seconds,
+            "unshared_work": {"terms_per_step": terms, "flops_per_step": 2.0 * terms + 8.0 * neighbours_once,
+                              "tflops_if_nothing_were_shared":
+                                  (2.0 * terms + 8.0 * neighbours_once) * steps_per_launch / seconds / 1e12,
+                              "fp64_peak_tflops": FP64_PEAK_TFLOPS}}
+
+
 def run_ours(args):
     import torch
     import paper_1909_06935_gb300 as P
@@ -296,6 +321,7 @@ def run_ours(args):
         res_w = ctx.finalize()
         flush.zero_()
     snap0 = ctx.walkers(nw)[0]
+    kernels0 = ctx.kernel_launches
     # timed region
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     res = None
@@ -308,6 +334,7 @@ def run_ours(args):
             flush.zero_()
         ev1.record(stream)
         barrier()
+    kernels = ctx.kernel_launches - kernels0
     ms = max_over_ranks(ev0.elapsed_time(ev1), world, dev)
     # walk-kernel time of the timed launches (CUDA events recorded by the library on its stream)
     walk_s = res["seconds"] - (res_w["seconds"] if res_w else 0.0)
@@ -317,44 +344,23 @@ def run_ours(args):
     units = nw * inner * args.steps
     value = job_rate(units, world, ms)
 
-    # algorithmic work, counted exactly by the debug kernel on walker snapshots taken before and after the
-    # timed region: every reach-back term H_mk phi0(k) is one FP64 FMA (2 flops), every neighbour adds
-    # <n|H|m>, the ratio, the rate and three sums (8 flops).  A step evaluates each distinct determinant
-    # once for all walkers on it, so the work is that of the distinct determinants (the terms that they
-    # share among each other are counted for each).
+    # neighbours and the work of evaluating each distinct determinant by itself, counted exactly by the debug kernel
+    # on walker snapshots taken before and after the timed region
     locs = [ctx.debug_local(snap)[0] for snap in (snap0, snap1)]
     once = [np.unique(snap, axis=0, return_index=True)[1] for snap in (snap0, snap1)]
-    distinct = float(np.mean([len(u) for u in once]))
-    terms = float(np.mean([np.sum(l["n_terms"][u]) for l, u in zip(locs, once)])) / nw
     nbrs = float(np.mean([np.mean(l["n_neighbours"]) for l in locs]))
-    nbrs_once = float(np.mean([np.sum(l["n_neighbours"][u]) for l, u in zip(locs, once)])) / nw
-    gathers = float(np.mean([np.sum((l["n_gathers"] + l["n_probes"])[u]) for l, u in zip(locs, once)])) / nw
-    flops_per_step = 2.0 * terms + 8.0 * nbrs_once
     launch_s = walk_s / max(walk_launches, 1)
-    units_per_launch = nw * inner
-    achieved = flops_per_step * units_per_launch / launch_s / 1e12
+    roof = roofline(nbrs, nw * inner, launch_s,
+                    distinct=float(np.mean([len(u) for u in once])),
+                    terms=float(np.mean([np.sum(l["n_terms"][u]) for l, u in zip(locs, once)])),
+                    neighbours_once=float(np.mean([np.sum(l["n_neighbours"][u]) for l, u in zip(locs, once)])),
+                    steps_per_launch=inner)
+    roof["launches_timed"] = int(walk_launches)
     peaks, peak_kind = load_peaks()
     probe = P.probe_peaks(local)
-    sectors_per_s = gathers * units_per_launch / launch_s
-    roof = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-            "frac": achieved / FP64_PEAK_TFLOPS,
-            "traffic": None,
-            "kernel": "k_pairs, k_rows, k_frows, k_fois, k_fois_act (one walk step)",
-            "peak_source": "FP64 FMA pipe: 152 SMs x 2 FMA/clk x 2 flop x 2.07 GHz (derived from unit counts and the "
-                           "maximum SM clock)",
-            "peak_measured": probe["fp64_flops"] / 1e12,
-            "frac_of_measured": achieved / (probe["fp64_flops"] / 1e12),
-            "flops_per_walker_step": flops_per_step, "terms_per_walker_step": terms,
-            "neighbours_per_walker_step": nbrs, "distinct_determinants": distinct,
-            # the move race draws one Philox clock per neighbour and walker
-            "race_draws_per_s": nbrs * units_per_launch / launch_s, "launch_seconds": launch_s, "launches_timed": int(walk_launches),
-            # the gather view of the same launches: every integral / table gather and hash-slot read of the
-            # distinct determinants, each for itself, is one random 32-byte sector; determinants that share
-            # rows read less, so this rate can lie above the probe's
-            "sectors_per_walker_step": gathers, "sectors_per_s": sectors_per_s,
-            "l2_gather_peak_per_s": probe["l2_gathers_per_s"], "hbm_gather_peak_per_s": probe["hbm_gathers_per_s"],
-            "l2_frac": sectors_per_s / probe["l2_gathers_per_s"],
-            "hbm_peak_gbs": float(peaks.get("hbm_gbs", 6800.0)), "hbm_peak_source": peak_kind}
+    roof["peaks_measured"] = {"fp64_tflops": probe["fp64_flops"] / 1e12, "l2_gathers_per_s": probe["l2_gathers_per_s"],
+                              "hbm_gathers_per_s": probe["hbm_gathers_per_s"],
+                              "hbm_gbs": float(peaks.get("hbm_gbs", 6800.0)), "hbm_source": peak_kind}
     cand_per_step = float(np.mean([np.mean(l["n_candidates"]) for l in locs]))
     nb_per_step = nbrs
 
@@ -407,7 +413,8 @@ def run_ours(args):
     # the metric's other half: batched and served against plain, on their own workloads
     batched = served = None
     if rank == 0 and world == 1 and not args.no_batched:
-        batched = measure_batched(args.n_systems, args.batch_walkers, R=1, steps=1, warmup=1, tuned=False)
+        # (from walkers that have left their start determinants)
+        batched = measure_batched(args.n_systems, args.batch_walkers, R=1, steps=4, warmup=8, tuned=False)
     if rank == 0 and world == 1 and not args.no_served:
         served = measure_served(args.n_requests, args.rate, args.target_sigma, args.req_walkers, args.req_max_steps,
                                 args.max_active, args.budget_gb)
@@ -432,9 +439,8 @@ def run_ours(args):
             "clocks": clk.summary(),
             "roofline": roof,
             "e2e": e2e,
-            # per step: group, prep, int, fois_act, fgroups, frows, fois, rows_begin, wave_begin, refs, insert,
-            # rows, pairs, move, accumulate; finalize list, labels, reduce (empty waves not counted)
-            "gpu_launches": 18 * args.steps,
+            # kernels of the timed walks and finalizes, counted where they are launched
+            "gpu_launches": int(kernels),
             "cpu_baseline": cpu,
             "batched": batched,
             "served": served,

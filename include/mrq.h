@@ -417,6 +417,10 @@ int mrq_debug_race_screen(mrq_ctx* ctx, int64_t n, const uint64_t* k53, const do
 int mrq_debug_race(mrq_ctx* ctx, int64_t n, const uint32_t* exc, const double* t, double psi, uint64_t seed,
                    int32_t n_walkers, const uint32_t* walker, const uint32_t* step, int32_t slices, uint32_t* winner);
 
+/* Kernels that this context's walks and finalizes have launched so far, those of replayed graphs and of waves that
+ * turned out empty included (a batch counts on its first context). */
+int64_t mrq_kernel_launches(const mrq_ctx* ctx);
+
 /*
  * Persisting-L2 window of this context's walk launches (no counterpart in the paper; a GB300
  * cache setting).  With fraction > 0 every walk launch marks the physicists' integral tables (the

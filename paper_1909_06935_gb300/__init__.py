@@ -151,6 +151,8 @@ def load_library(build_if_missing: bool = True):
     lib.mrq_sample_batch.argtypes = [P, C.c_int, P, P]
     lib.mrq_debug_race_screen.argtypes = [P, I64, P, P, P, P, P]
     lib.mrq_debug_race.argtypes = [P, I64, P, P, C.c_double, C.c_uint64, C.c_int32, P, P, C.c_int32, P]
+    lib.mrq_kernel_launches.argtypes = [P]
+    lib.mrq_kernel_launches.restype = I64
     lib.mrq_set_deadline.argtypes = [P, C.c_double]
     lib.mrq_probe_peaks.argtypes = [C.c_int, P]
     lib.mrq_set_l2_window.argtypes = [P, C.c_double]
@@ -306,6 +308,11 @@ class Context:
     @property
     def n_labels(self) -> int:
         return int(self._lib.mrq_n_labels(self._h))
+
+    @property
+    def kernel_launches(self) -> int:
+        """Kernels launched by this context's walks and finalizes so far."""
+        return int(self._lib.mrq_kernel_launches(self._h))
 
     def setup_info(self):
         out = np.zeros(5)

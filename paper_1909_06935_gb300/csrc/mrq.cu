@@ -1104,6 +1104,8 @@ struct mrq_ctx {
     GraphKey gkey[NSLOT] = {};
     int n_sm = 0;                    // SMs of the device
     long long graph_replays = 0;
+    long long kernels = 0;           // kernels of walks and finalizes launched so far (mrq_kernel_launches)
+    long long gkernels[NSLOT] = {};  // kernels of one replay of a graph
     long long* d_nbpre = nullptr;    // debug records: neighbour offsets of a determinant's units
     size_t cap_nbpre = 0;
     Walker* d_tune = nullptr;        // the tuner's scratch copy of a batch's walkers
@@ -1571,6 +1573,7 @@ static int launch_segment(mrq_ctx* ctx, const WalkSet& ws, WalkScratch sc, const
     const cudaStream_t st = ctx->stream;
     const size_t lbytes = cand_list_bytes(need.cap), rbytes = rows_warp_bytes(need.cap), fbytes = frows_warp_bytes(need.cap);
     const cudaStream_t st2 = ctx->side[0], st3 = ctx->side[1];
+    ctx->kernels += 5;                // k_group, k_prep, k_int, k_fois_act, k_move; the waves' are added below
     if (ws.nsys > 1) CK(cudaMemsetAsync(sc.ctl, 0, sizeof(int) * CTL_N, st));
     k_group<W><<<(unsigned)ws.nsys, 1024, 0, st>>>(ws, sc);
     CK(cudaEventRecord(ctx->ev_fork, st));
@@ -1586,6 +1589,7 @@ static int launch_segment(mrq_ctx* ctx, const WalkSet& ws, WalkScratch sc, const
     CK(cudaStreamWaitEvent(st3, ctx->ev_fork, 0));
     for (long long g = 0; g < n; g += sc.fwave) {
         sc.fwave0 = (int)g;
+        ctx->kernels += 3;
         if (g > 0) CK(cudaMemsetAsync(sc.ctl + CTL_FOIS, 0, sizeof(int) * (CTL_N - CTL_FOIS), st3));
         k_fgroups<W><<<(unsigned)std::min<long long>(n, 4LL * sms), 256, 0, st3>>>(ws, sc);
         k_frows<W, 3><<<(unsigned)ctx->frows_blocks, 32 * nw, nw * fbytes, st3>>>(ws, sc, (int)fbytes, need.cap);
@@ -1596,6 +1600,7 @@ static int launch_segment(mrq_ctx* ctx, const WalkSet& ws, WalkScratch sc, const
     // main stream: the CAS determinants' rows and pairs
     for (long long g = 0; g < std::min(n, need.ncas); g += sc.wave_groups) {
         sc.wave0 = (int)g;
+        ctx->kernels += 5;
         k_wave_begin<<<1, 1, 0, st>>>(sc);
         k_refs<W><<<(unsigned)std::min<long long>(n, 8LL * sms), 256, 0, st>>>(ws, sc);
         k_insert<<<8 * sms, 256, 0, st>>>(ws, sc);
@@ -1638,6 +1643,7 @@ static int launch_walk(mrq_ctx* ctx, int W, const WalkSet& ws, int nsteps, const
     }
     k_rows_begin<<<1, 1, 0, ctx->stream>>>(ctx->work);
     CK(cudaGetLastError());
+    ctx->kernels++;
     for (int step = 0; step < nsteps; step++) {
         for (long long s0 = 0; s0 < ws.nslots; s0 += seg) {
             WalkScratch sc = ctx->work;
@@ -1650,6 +1656,7 @@ static int launch_walk(mrq_ctx* ctx, int W, const WalkSet& ws, int nsteps, const
         if (L.accumulate) {
             k_accum<<<dim3((unsigned)ws.nsys, 2), 1024, 0, ctx->stream>>>(ws);
             CK(cudaGetLastError());
+            ctx->kernels++;
         }
     }
     return 0;
@@ -2270,6 +2277,7 @@ static int finalize_with(mrq_ctx* ctx, mrq_result* out, double* scratch, int nch
     CK(cudaGetLastError());
     k_fin_reduce<<<1, 1024, 0, ctx->stream>>>(ctx->d_sys, scratch, nchunk, ctx->d_res);
     CK(cudaGetLastError());
+    ctx->kernels += 3;
     if (int r = sync_stream(ctx)) return r;
     CK(cudaMemcpyAsync(out, ctx->d_res, sizeof(mrq_result), cudaMemcpyDeviceToHost, ctx->stream));
     int flag = 0;
@@ -2452,7 +2460,10 @@ static int batch_run(mrq_ctx* ctx, int W, const WalkSet& ws, const WalkNeed& nee
             ex = nullptr;
             CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
             L.captured = true;
+            const long long before = ctx->kernels;
             const int r = launch_walk(ctx, W, ws, (int)spl, need, L);
+            ctx->gkernels[slot] = ctx->kernels - before;
+            ctx->kernels = before;
             cudaGraph_t g = nullptr;
             const cudaError_t e = cudaStreamEndCapture(ctx->stream, &g);
             if (r || e != cudaSuccess) {
@@ -2469,6 +2480,7 @@ static int batch_run(mrq_ctx* ctx, int W, const WalkSet& ws, const WalkNeed& nee
         }
         for (int64_t i = 0; i < nfull; i++) CK(cudaGraphLaunch(ex, ctx->stream));
         ctx->graph_replays += nfull;
+        ctx->kernels += nfull * ctx->gkernels[slot];
         L.captured = false;
     } else {
         for (int64_t i = 0; i < nfull; i++)
@@ -2772,6 +2784,8 @@ int mrq_debug_race(mrq_ctx* ctx, int64_t n, const uint32_t* exc, const double* t
     cudaFree(d);
     return r;
 }
+
+int64_t mrq_kernel_launches(const mrq_ctx* ctx) { return ctx ? ctx->kernels : 0; }
 
 int mrq_set_l2_window(mrq_ctx* ctx, double fraction) {
     if (!ctx) return MRQ_INVALID_ARG;
