@@ -199,7 +199,7 @@ int mrq_walkers_init(mrq_ctx* ctx, const mrq_sample_params* p);
  * determinants: at most about 12 GiB, at most an eighth of the memory that is free then, and less for
  * small systems or few walkers.  (A least size for 256 walkers and one determinant at a time remains;
  * MRQ_OOM where that does not fit.)  The context keeps it until the next mrq_load_hamiltonian or
- * mrq_destroy.
+ * mrq_destroy, or until a batch that it is not the first of walks where memory is short.
  * Errors: MRQ_NOT_LOADED, MRQ_OOM, MRQ_CUDA_ERROR.
  */
 int mrq_walkers_advance(mrq_ctx* ctx, int64_t n_steps);

@@ -1318,12 +1318,20 @@ static int check_err_flag(mrq_ctx* ctx, int* flag_out) {
     return 0;
 }
 
+// The other contexts of a batch walk in its first one's workspace; where memory is short they give theirs back
+// (their streams have been waited for).
+struct WorkPeers {
+    mrq_ctx* const* ctxs = nullptr;
+    int n = 0;
+};
+
 // launch-time options of a walk: warps per block, whether to accumulate, and whether the one-time
 // set-up (workspace growth, function attributes) has been done already (inside a stream capture)
 struct WalkLaunch {
     int wpb = 8;
     int accumulate = 1;
     bool captured = false;
+    WorkPeers peers;                     // (a batch's contexts)
     cudaAccessPolicyWindow l2win = {};   // num_bytes 0: no persisting-L2 window
 };
 
@@ -1441,7 +1449,7 @@ static WorkPlan work_size(long long nslots, const WalkNeed& need, int seen, long
     }
 }
 
-static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need) {
+static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need, const WorkPeers& peers) {
     const long long limit = ctx->work_limit;
     WorkPlan p = work_size(nslots, need, ctx->seen, limit);
     const auto renew = [&]() { return p.bytes > ctx->work_cap || ((long long)ctx->work_cap > limit && p.bytes < ctx->work_cap); };
@@ -1449,6 +1457,14 @@ static int work_prepare(mrq_ctx* ctx, long long nslots, const WalkNeed& need) {
         size_t free_b = 0, total_b = 0;
         CK(cudaMemGetInfo(&free_b, &total_b));
         long long room = (long long)((free_b + ctx->work_cap) / 8);
+        if ((long long)p.bytes > room) {
+            for (int i = 0; i < peers.n; i++) {
+                if (peers.ctxs[i] == ctx) continue;
+                free_b += peers.ctxs[i]->work_cap;
+                free_work(peers.ctxs[i]);
+            }
+            room = (long long)((free_b + ctx->work_cap) / 8);
+        }
         if (room < limit) {
             // (one that is nearly as large stays)
             if ((long long)ctx->work_cap <= limit && (long long)ctx->work_cap >= room - room / 4) room = (long long)ctx->work_cap;
@@ -1628,7 +1644,7 @@ static int launch_walk(mrq_ctx* ctx, int W, const WalkSet& ws, int nsteps, const
                        const WalkLaunch& L = WalkLaunch()) {
     const int nw = std::min(L.wpb, MRQ_MAXNW);
     if (!L.captured) {
-        if (int r = work_prepare(ctx, ws.nslots, need)) return r;
+        if (int r = work_prepare(ctx, ws.nslots, need, L.peers)) return r;
         if (int r = rows_prepare(ctx, W, nw, need.cap)) return r;
     }
     const long long seg = ctx->work.nseg;
@@ -2442,15 +2458,18 @@ static void graph_key(const mrq_ctx* ctx, const WalkSet& ws, const WalkNeed& nee
 
 // n_steps steps of one width's walk set: launches of `spl` steps (the reporting interval), replayed
 // from a CUDA graph when the lead context asks for it
-static int batch_run(mrq_ctx* ctx, int W, const WalkSet& ws, const WalkNeed& need, int64_t n_steps, int wpb, int64_t spl,
-                     int accumulate, bool graph, int slot) {
+static int batch_run(mrq_ctx* const* ctxs, int n, int W, const WalkSet& ws, const WalkNeed& need, int64_t n_steps, int wpb,
+                     int64_t spl, int accumulate, bool graph, int slot) {
+    mrq_ctx* const ctx = ctxs[0];
     WalkLaunch L;
+    L.peers.ctxs = ctxs;
+    L.peers.n = n;
     L.wpb = wpb;
     L.accumulate = accumulate;
     if (spl <= 0 || spl > n_steps) spl = n_steps;
     const int64_t nfull = n_steps / spl, rem = n_steps % spl;
     if (graph && nfull > 0) {
-        if (int r = work_prepare(ctx, ws.nslots, need)) return r;
+        if (int r = work_prepare(ctx, ws.nslots, need, L.peers)) return r;
         if (int r = rows_prepare(ctx, W, std::min(wpb, MRQ_MAXNW), need.cap)) return r;
         mrq_ctx::GraphKey key;
         graph_key(ctx, ws, need, wpb, (int)spl, key);
@@ -2516,7 +2535,7 @@ int mrq_batch_advance(mrq_ctx* const* ctxs, int n, int64_t n_steps) {
             ctx->evs.push_back(ev);
         }
         CK(cudaEventRecord(ctx->evs[q], ctx->stream));
-        if (int r = batch_run(ctx, W, ws, need, n_steps, nw_eff, lead->spl, 1, lead->use_graph != 0, slot))
+        if (int r = batch_run(ctxs, n, W, ws, need, n_steps, nw_eff, lead->spl, 1, lead->use_graph != 0, slot))
             return r;
         CK(cudaEventRecord(ctx->evs[q + 1], ctx->stream));
         ctx->launches++;
@@ -2583,7 +2602,7 @@ int mrq_tune_batch(mrq_ctx* const* ctxs, int n, int64_t trial_steps, mrq_tune_re
                 WalkNeed need;
                 if (int r = batch_tables(ctxs, n, W, scratch.data(), ws, need, wpb, nw_eff)) return r;
                 if (ws.nsys == 0) continue;
-                if (int r = batch_run(ctx, W, ws, need, trial_steps, nw_eff, spl, 0, false, slot)) return r;
+                if (int r = batch_run(ctxs, n, W, ws, need, trial_steps, nw_eff, spl, 0, false, slot)) return r;
                 if (int r_ = sync_stream(ctx)) return r_;
             }
             CK(cudaEventRecord(ctx->ev1, ctx->stream));

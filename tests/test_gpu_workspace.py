@@ -56,6 +56,14 @@ def test_contexts_on_a_nearly_full_device_all_walk():
             _same((c.walkers(4096)[0], c.accumulators(G)), want)
         for c in ctxs:                                                  # and once more on what they have
             _same(_walk(c, 4096, 3, 8), want)
+        # together they walk in the first one's workspace, and the others give theirs back
+        for c in ctxs:
+            c.walkers_init(c.params(4096, 3, burn_in=1, seed=8, n_groups=G))
+        before = _free()
+        P.batch_advance(ctxs, 3)
+        assert _free() > before
+        for c in ctxs:
+            _same((c.walkers(4096)[0], c.accumulators(G)), want)
     finally:
         for c in ctxs:
             c.close()
