@@ -1825,6 +1825,35 @@ static int l2_window(mrq_ctx* ctx, cudaAccessPolicyWindow& w) {
     return 0;
 }
 
+// Load the code of every kernel of a walk on the current device, once.  A step runs on three streams, and the runtime
+// otherwise uploads a kernel's code at its first launch, beside kernels of the other streams that are running.
+template <int W>
+static cudaError_t load_walk_kernels() {
+    const void* const kernels[] = {
+        (const void*)k_group<W>, (const void*)k_prep<W>, (const void*)k_int<W>, (const void*)k_fois_act<W>,
+        (const void*)k_fgroups<W>, (const void*)k_frows<W, 3>, (const void*)k_fois<W, 3>, (const void*)k_refs<W>,
+        (const void*)k_rows<W, 2>, (const void*)k_rows<W, 4>, (const void*)k_pairs<W, 4>, (const void*)k_move<W>,
+        (const void*)k_rows_begin, (const void*)k_wave_begin, (const void*)k_insert, (const void*)k_accum,
+        (const void*)k_fin_list, (const void*)k_fin_labels, (const void*)k_fin_reduce, (const void*)k_walkers_init};
+    for (const void* k : kernels) {
+        cudaFuncAttributes a;
+        const cudaError_t e = cudaFuncGetAttributes(&a, k);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+static cudaError_t load_kernels(int device) {
+    static std::mutex mu;
+    static bool done[MRQ_MAX_DEVICES];
+    std::lock_guard<std::mutex> lock(mu);
+    if (device >= 0 && device < MRQ_MAX_DEVICES && done[device]) return cudaSuccess;
+    cudaError_t e = load_walk_kernels<1>();
+    if (e == cudaSuccess) e = load_walk_kernels<2>();
+    if (e == cudaSuccess && device >= 0 && device < MRQ_MAX_DEVICES) done[device] = true;
+    return e;
+}
+
 extern "C" {
 
 int mrq_create(mrq_ctx** out, int device) {
@@ -1853,7 +1882,8 @@ int mrq_create(mrq_ctx** out, int device) {
     }
     ctx->own_stream = true;
     cudaMemset(ctx->d_err, 0, 2 * sizeof(int));
-    if (cudaDeviceGetAttribute(&ctx->n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
+    if (cudaDeviceGetAttribute(&ctx->n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+        load_kernels(device) != cudaSuccess) {
         mrq_destroy(ctx);
         return MRQ_CUDA_ERROR;
     }
