@@ -962,7 +962,8 @@ __device__ __forceinline__ RaceBest load_best128(const RaceBest* at) {
 // Whether two FP32 clocks leave the order of the exact ones open.  Their relative error is below 1e-5 within
 // FP32's normal range; below and above it (rates near 1e38 or 1e-38 and beyond) the exact clocks always decide.
 __device__ __forceinline__ bool clocks_near(float a, float b) {
-    return (!(a < b * 0.9999f) && !(b < a * 0.9999f)) || fmaxf(a, b) < 1e-30f || fminf(a, b) > 1e37f;
+    const float lo = fminf(a, b), hi = fmaxf(a, b);
+    return !(lo < hi * 0.9999f) | (hi < 1e-30f) | (lo > 1e37f);
 }
 
 // FP32 upper bound of the clock whose FP32 image is a.  Images below the normal range may have lost all their
