@@ -2,7 +2,7 @@
 //
 // A walker's local evaluation (Eq. 5, Eq. 16, the reach-back overlaps of Eq. 6-7) depends on its
 // determinant only, and the walkers of a system crowd on few of them: at 56 orbitals 4,096 walkers
-// in the steady state sit on about 340 determinants of the CAS and 250 of the first-order space.
+// in the steady state sit on about 640 determinants of the CAS and 230 of the first-order space.
 // So a step
 //   k_group   finds the distinct determinants (a hash table over the walkers) and cuts each one's
 //             walkers into task groups of at most MRQ_TGW;
